@@ -52,14 +52,15 @@ typedef struct pulda_handle pulda_handle;
 /* Launch options.  Zero-initialise and set what you need; NULL = defaults. */
 typedef struct {
     void *stream;           /* cudaStream_t to run on; NULL = a stream the handle creates */
-    int32_t zstep_path;     /* 0 = auto (iterate the smaller of the document's and the
-                               word's nonzero topics), 1 = always iterate the word's Phi
-                               column, 2 = iterate the document's topics whenever K <= 2048 */
+    int32_t zstep_path;     /* 0 = auto (a word with few nonzero topics is summed over its Phi
+                               column, the others over a dense row of its weights), 1 = always
+                               over the column, 2 = over the dense row wherever there is one;
+                               results are identical */
     int32_t warps_per_block;/* warp-per-document z-step: warps per CTA, 1..4; 0 = 4, halved
                                while the CTA's shared memory would pass 160 KB */
     int32_t docs_per_warp;  /* z-step documents per warp: 0 = auto (one: measured faster at
                                every K), 1 = one, 4 = four (needs K <= 1024; falls back to
-                               one when every word's dense q row does not fit 2 GB;
+                               one when V K 4-byte weights do not fit 2 GB;
                                documents longer than 65,535 tokens still go one per warp,
                                the longest to CTAs as coop_min_len says); results are
                                identical */
@@ -74,16 +75,19 @@ typedef struct {
                                slices, a different sampler from the paper's (AD-LDA's
                                approximation within a document).  Needs docs_per_warp 0 or 1;
                                fold-in, serving and the batched form ignore/reject it */
-    int32_t coop_min_len;   /* corpus z-step and pulda_infer: a document at least this long is
-                               resampled by the 4 warps of one CTA together, token by token
-                               (its intersections split over 128 lanes), concurrently with the
-                               other documents' one-warp kernel; results are identical.
-                               0 = auto (documents longer than max(256, N / 8000) tokens,
+    int32_t coop_min_len;   /* z-step and fold-in: a document of at least this many tokens (and
+                               at most 65,535) gets a CTA of its own, in which one warp draws
+                               the tokens and two others prepare and record them -- the least
+                               time per token -- concurrently with the other documents' one-warp
+                               kernel; results are identical.
+                               0 = auto (documents longer than max(256, N / 4500) tokens,
                                N / 16000 beside four documents per warp: those that would
-                               outlast the rest of the pass), -1 = never, > 0 = this length.
-                               Not used with slice_len > 0; the batched form takes 0 or -1
-                               (one warp per document); a server on the handle uses it for
-                               requests (0 = requests of at least 1,024 tokens) */
+                               outlast the rest of the pass; where a pass has at most two
+                               documents for every such CTA the GPU holds, all of them run in
+                               that form), -1 = never, > 0 = this length.
+                               Not used with slice_len > 0; a server on the handle uses it for
+                               requests (0 = requests of at least 1,024 tokens, and all of them
+                               while a CTA is free for each) */
     int32_t count_path;     /* how the Phi-step rebuilds n_{k,v}: 0 = shared-memory histogram of
                                each word's topics (the default, measured faster), 1 = radix sort
                                of every token's key w K + z and its runs (needs V K < 2^32; the
@@ -295,8 +299,8 @@ typedef struct pulda_batch pulda_batch;
  * set, is used for all chains; opt->warps_per_block in 1..8 fixes the z-step
  * CTA size instead of tuning it over {2, 4, 8}; opt->coop_min_len -1 keeps
  * every document on one warp, > 0 sends the documents at least that long (of
- * every chain) to the cooperative z-step, 0 sends those of at least
- * max(256, N / 8000) tokens (N = tokens of all chains), the single-chain rule;
+ * every chain) to CTAs of their own, 0 sends those of at least
+ * max(256, N / 4500) tokens (N = tokens of all chains), the single-chain rule;
  * docs_per_warp must be 0 or 1; batch_form picks the launch form and
  * alias_layout the alias tables' layout (see pulda_options).  Tuning times
  * each CTA size on two real sweeps (in order, then in reverse), together with
@@ -342,11 +346,10 @@ void pulda_batch_free(pulda_batch *b);
  * worker thread admits waiting requests while a slot and a contiguous range
  * of the token arena are free (memory-based admission, first come first
  * served), advances every admitted request by up to `slice_tokens` tokens per
- * launch (one warp per request; one CTA of the cooperative z-step per request
- * of at least the handle's coop_min_len tokens -- 1,024 when it is 0, none
- * when -1 -- on a second stream while the active requests fill at most an
- * eighth of the resident warps; sweeps continuing within a launch) and
- * copies finished topics out.  A request's result equals pulda_infer on that
+ * launch (one warp per request; one CTA per request of at least the handle's
+ * coop_min_len tokens, beside the others on a second stream -- when it is 0,
+ * 1,024, and all requests while a CTA is free for each; none when -1; sweeps
+ * continuing within a launch) and copies finished topics out.  A request's result equals pulda_infer on that
  * document alone with the same seed and n_sweeps: its random streams are keyed
  * by its own seed and token positions, never by its neighbours.
  * Do not run pulda_sweep / pulda_phi_step on the handle while a server is open
@@ -400,8 +403,8 @@ pulda_status pulda_serve_close(pulda_server *s);
 
 /* pulda_z_layout -- how the handle's corpus z-step is laid out (launch shape
  * only: results never depend on it): documents per warp of the main z-step
- * kernel (1 or 4), the number of (longest) documents resampled by one CTA
- * each, and, beside four per warp, the documents too long for it that run one
+ * kernel (1 or 4), the number of (longest) documents that coop_min_len puts on
+ * CTAs of their own, and, beside four per warp, the documents too long for it that run one
  * per warp (otherwise every document not on a CTA).  Any pointer may be NULL.
  * Errors: PULDA_ERR_INVALID (NULL handle). */
 pulda_status pulda_z_layout(pulda_handle *h, int32_t *docs_per_warp, int64_t *coop_docs, int64_t *one_warp_docs);

@@ -128,15 +128,6 @@ cudaError_t clear_z_counters(pulda_handle *h) {
 
 // Documents in decreasing length (ties by index), so the persistent z-step
 // starts the long ones first.
-// Whether every document from position `from` of a length order (longest
-// first) has at most kNarrowMaxLen tokens: the one-warp z-step over them can
-// hold its counts in 16 bits.
-bool narrow_from(const int64_t *off, const std::vector<int32_t> &order, int64_t from) {
-    if (from >= static_cast<int64_t>(order.size())) return true;
-    const int32_t d = order[static_cast<size_t>(from)];
-    return off[d + 1] - off[d] <= kNarrowMaxLen;
-}
-
 std::vector<int32_t> length_order(const int64_t *off, int64_t D) {
     std::vector<int32_t> o(D);
     std::iota(o.begin(), o.end(), 0);
@@ -144,72 +135,21 @@ std::vector<int32_t> length_order(const int64_t *off, int64_t D) {
     return o;
 }
 
-// Number of leading documents of a length-ordered schedule that the grouped
-// z-step cannot take (longer than kMaxGroupDocLen tokens).
-int64_t count_long(const int64_t *off, const std::vector<int32_t> &order) {
+// Number of leading documents of a length-ordered schedule with 2^16 tokens
+// or more: their counts take three planes, which the one-warp kernel alone has.
+int64_t count_wide(const int64_t *off, const std::vector<int32_t> &order) {
     int64_t n = 0;
-    while (n < static_cast<int64_t>(order.size()) && off[order[n] + 1] - off[order[n]] > kMaxGroupDocLen) ++n;
+    while (n < static_cast<int64_t>(order.size()) && off[order[n] + 1] - off[order[n]] > kNarrowMaxLen) ++n;
     return n;
 }
 
-// Number of leading documents of a length-ordered schedule that the
-// cooperative z-step takes: at least coop_min_len tokens (0 = automatic:
-// longer than max(256, N / 8000), or N / 16000 beside the grouped z-step);
-// none with coop_min_len < 0 or slices.
-int64_t count_coop(const pulda_handle *h, const int64_t *off, const std::vector<int32_t> &order, int64_t N) {
-    if (h->opt.coop_min_len < 0 || h->opt.slice_len > 0) return 0;
-    const int64_t div = h->z_groups ? kCoopAutoDivGrouped : kCoopAutoDiv;
-    const int64_t L = h->opt.coop_min_len > 0 ? h->opt.coop_min_len : std::max<int64_t>(kCoopAutoMin, N / div + 1);
-    int64_t n = 0;
+// Number of documents, after the n_wide widest of a length-ordered schedule,
+// that the long-document z-step takes.
+int64_t count_coop(const pulda_handle *h, const int64_t *off, const std::vector<int32_t> &order, int64_t n_wide, int64_t N) {
+    const int64_t L = long_document_tokens(h, N);
+    int64_t n = n_wide;
     while (n < static_cast<int64_t>(order.size()) && off[order[n] + 1] - off[order[n]] >= L) ++n;
-    return n;
-}
-
-// One z-step over the documents doc_order[0..D) (longest first).  The
-// first n_coop go to the cooperative kernel (a CTA each); with the grouped
-// kernel, the documents after them that are too long for it (up to n_long)
-// then run one per warp on the same stream, while the rest run four per warp
-// (grouped) or one per warp on a second stream, joined back before the next
-// step.
-// `narrow`: every document the one-warp kernel gets (those after the first
-// n_coop) has at most kNarrowMaxLen tokens.
-pulda_status run_z(pulda_handle *h, const int64_t *doc_off, const int32_t *doc_order, int64_t D, int64_t n_long,
-                   int64_t n_coop, const int32_t *w, int16_t *z, uint64_t seed, uint32_t sweep, int64_t index_base,
-                   bool narrow) {
-    CU(h, cudaMemsetAsync(h->work + 1, 0, 3 * sizeof(int), h->stream));
-    ZArgs a = z_args(h, doc_off, doc_order, D, w, z, seed, sweep, index_base);
-    a.narrow = narrow ? 1 : 0;
-    const int64_t n_head = h->z_groups ? std::max(n_coop, n_long) : n_coop;
-    auto launch_rest = [&](cudaStream_t st) {
-        if (D <= n_head) return;
-        ZArgs ar = a;
-        ar.doc_order = doc_order + n_head;
-        ar.D = D - n_head;
-        if (h->z_groups) {
-            ar.work = h->work + 2;
-            launch_z_step_groups(ar, h->zg_grid, st);
-        } else {
-            launch_z_step(ar, h->z_warps, h->z_grid, st);
-        }
-    };
-    if (n_head > 0) {
-        CU(h, cudaEventRecord(h->ev_fork, h->stream));
-        if (n_coop > 0) launch_z_step_coop(a, static_cast<int>(n_coop), h->work + 3, h->coop_grid, h->stream);
-        if (n_head > n_coop) {
-            ZArgs al = a;
-            al.doc_order = doc_order + n_coop;
-            al.D = n_head - n_coop;
-            launch_z_step(al, h->z_warps, h->z_grid, h->stream);
-        }
-        CU(h, cudaStreamWaitEvent(h->stream2, h->ev_fork, 0));
-        launch_rest(h->stream2);
-        CU(h, cudaEventRecord(h->ev_join, h->stream2));
-        CU(h, cudaStreamWaitEvent(h->stream, h->ev_join, 0));
-    } else {
-        launch_rest(h->stream);
-    }
-    CU(h, cudaGetLastError());
-    return PULDA_OK;
+    return n - n_wide;
 }
 
 }  // namespace
@@ -247,7 +187,7 @@ PhiArgs phi_args(pulda_handle *h) {
     a.S = h->S; a.rowbuf = h->rowbuf; a.col_ptr = h->col_ptr;
     a.topic = h->topic; a.c = h->c; a.q = h->q; a.athr = h->athr; a.atopic = h->atopic; a.apack = h->apack;
     a.A = h->A; a.vose_p = h->vose_p; a.vose_stack = h->vose_stack; a.bits = h->bits; a.KW = h->KW; a.KWp = h->KWp;
-    a.qdense = h->qdense; a.dense_slot = h->dense_slot;
+    a.qrow = h->qrow; a.row_slot = h->row_slot; a.drow = h->drow; a.qdense = h->qdense;
     a.alpha = h->alpha; a.work = h->work; a.stats = h->stats;
     a.heavy_row = h->heavy_row; a.heavy_hist = h->heavy_hist; a.n_heavy = h->n_heavy;
     a.gam = h->gam; a.Sd = h->Sd; a.invS = h->invS; a.invSf = h->invSf; a.dpart = h->dpart;
@@ -261,11 +201,71 @@ ZArgs z_args(pulda_handle *h, const int64_t *doc_off, const int32_t *doc_order, 
     a.col_ptr = h->col_ptr; a.topic = h->topic; a.q = h->q; a.A = h->A; a.athr = h->athr; a.atopic = h->atopic;
     a.apack = h->apack;
     a.bits = h->bits; a.K = h->K; a.KW = h->KW; a.KWp = h->KWp; a.seed = seed; a.sweep = sweep; a.index_base = index_base;
-    a.qdense = h->qdense; a.dense_slot = h->dense_slot;
+    a.qrow = h->qrow; a.drow = h->drow; a.qdense = h->qdense;
     a.path = h->opt.zstep_path; a.work = h->work + 1; a.stats = h->stats;
     return a;
 }
 
+
+// At least coop_min_len tokens (0 = automatic: longer than max(256, N / 4500),
+// or N / 16000 beside the grouped z-step); none with coop_min_len < 0 or slices.
+int64_t long_document_tokens(const pulda_handle *h, int64_t N) {
+    if (h->opt.coop_min_len < 0 || h->opt.slice_len > 0) return INT64_MAX;
+    if (h->opt.coop_min_len > 0) return h->opt.coop_min_len;
+    return std::max<int64_t>(kCoopAutoMin, N / (h->z_groups ? kCoopAutoDivGrouped : kCoopAutoDiv) + 1);
+}
+
+// The n_wide widest documents one per warp, the next n_coop on a CTA each,
+// both on the handle's stream; beside them, on a second stream joined back
+// before the next step, the rest four per warp (grouped) or one per warp.
+// Few documents (at most two for every CTA the GPU holds) all go to CTAs: each
+// is a chain of its own, and there a token takes a third of the time (1,000
+// documents of 100 tokens at K = 20: 85 us against 136).
+cudaError_t run_z(pulda_handle *h, ZArgs a, int64_t n_wide, int64_t n_coop, int *work) {
+    cudaError_t e = cudaMemsetAsync(work, 0, 5 * sizeof(int), h->stream);
+    if (e != cudaSuccess) return e;
+    const int64_t D = a.D;
+    if (h->opt.coop_min_len == 0 && h->opt.slice_len == 0 && !h->z_groups && D - n_wide <= 2 * static_cast<int64_t>(h->coop_grid))
+        n_coop = D - n_wide;
+    const int64_t n_head = n_wide + n_coop;
+    const int32_t *order = a.doc_order;
+    auto launch_rest = [&](cudaStream_t st) {
+        if (D <= n_head) return;
+        ZArgs ar = a;
+        ar.doc_order = order + n_head;
+        ar.D = D - n_head;
+        ar.narrow = 1;
+        ar.work = work + (h->z_groups ? 1 : 0);
+        if (h->z_groups) launch_z_step_groups(ar, h->zg_grid, st);
+        else launch_z_step(ar, h->z_warps, h->z_grid, st);
+    };
+    auto launch_head = [&](cudaStream_t st) {
+        if (n_wide > 0) {
+            ZArgs aw = a;
+            aw.D = n_wide;
+            aw.narrow = 0;
+            aw.work = work + 2;
+            launch_z_step(aw, h->z_warps, h->z_grid, st);
+        }
+        if (n_coop > 0) {
+            ZArgs ac = a;
+            ac.doc_order = order + n_wide;
+            launch_z_step_coop(ac, static_cast<int>(n_coop), work + 3, h->coop_grid, st);
+        }
+    };
+    if (n_head > 0 && n_head < D) {
+        if ((e = cudaEventRecord(h->ev_fork, h->stream)) != cudaSuccess) return e;
+        launch_head(h->stream);
+        if ((e = cudaStreamWaitEvent(h->stream2, h->ev_fork, 0)) != cudaSuccess) return e;
+        launch_rest(h->stream2);
+        if ((e = cudaEventRecord(h->ev_join, h->stream2)) != cudaSuccess) return e;
+        if ((e = cudaStreamWaitEvent(h->stream, h->ev_join, 0)) != cudaSuccess) return e;
+    } else {
+        launch_head(h->stream);
+        launch_rest(h->stream);
+    }
+    return cudaGetLastError();
+}
 
 // Read-only view of a handle for other translation units of the library.
 bool handle_view(pulda_handle *h, HandleView *out) {
@@ -381,12 +381,12 @@ pulda_status pulda_init(pulda_handle **out, const int32_t *word_ids, const int64
     ALLOC(h->topic, h->cap); ALLOC(h->c, h->cap); ALLOC(h->q, h->cap); ALLOC(h->athr, h->cap); ALLOC(h->atopic, h->cap);
     if (h->opt.alias_layout == 2) ALLOC(h->apack, h->cap);
     ALLOC(h->A, V); ALLOC(h->vose_p, h->cap); ALLOC(h->vose_stack, h->cap);
-    if (K <= kMaxKBitmap) ALLOC(h->bits, static_cast<size_t>(V) * h->KWp);
+    ALLOC(h->bits, static_cast<size_t>(V) * h->KWp);
     if (h->opt.phi_mode == 1) {
         ALLOC(h->gam, h->cap); ALLOC(h->Sd, K); ALLOC(h->invS, K); ALLOC(h->invSf, K);
         ALLOC(h->dpart, dir_part_count(V, K));
     }
-    ALLOC(h->work, 4); ALLOC(h->stats, ST_TOTAL_SLOTS);
+    ALLOC(h->work, 6); ALLOC(h->stats, ST_TOTAL_SLOTS);
     if (h->opt.count_path == 1) ALLOC(h->sort_scratch, count_sort_scratch_words(N));
     cudaStream_t st = h->stream;
     CUI(cudaMemcpyAsync(h->w, word_ids, sizeof(int32_t) * N, cudaMemcpyHostToDevice, st));
@@ -448,27 +448,22 @@ pulda_status pulda_init(pulda_handle **out, const int32_t *word_ids, const int64
     std::stable_sort(word_order.begin(), word_order.end(),
                      [&](int32_t a, int32_t b) { return woff[a + 1] - woff[a] > woff[b + 1] - woff[b]; });
     CUI(cudaMemcpyAsync(h->word_order, word_order.data(), sizeof(int32_t) * V, cudaMemcpyHostToDevice, st));
-    // dense q rows for the most frequent words, within kDenseBytes
-    if (K <= kMaxKBitmap && kDenseBytes > 0) {
-        const int64_t cap = std::min<int64_t>(V, kDenseBytes / (static_cast<int64_t>(sizeof(uint32_t)) * K));
+    // dense rows for the most frequent words, within kDenseBytes
+    {
+        const int64_t cap = std::min<int64_t>(V, kDenseBytes / dense_row_bytes(K));
         std::vector<int32_t> slot(V, -1);
-        int32_t n = 0;
-        for (int32_t v : word_order) {   // every word, most frequent first, while the budget lasts
-            if (n >= cap) break;
-            slot[v] = n++;
-        }
-        if (n > 0) {
-            ALLOC(h->dense_slot, V);
-            // 32 words before the first row: the document side's empty gather
-            // slots read the word before a lane's segment (times a zero count)
-            ALLOC(h->qdense, static_cast<size_t>(n) * K + 32);
-            CUI(cudaMemsetAsync(h->qdense, 0, 32 * sizeof(uint32_t), st));
-            h->qdense += 32;
-            CUI(cudaMemcpyAsync(h->dense_slot, slot.data(), sizeof(int32_t) * V, cudaMemcpyHostToDevice, st));
-            CUI(cudaStreamSynchronize(st));
-        }
-        h->n_dense = n;
+        for (int64_t i = 0; i < cap; ++i) slot[word_order[i]] = static_cast<int32_t>(i);
+        ALLOC(h->row_slot, V);
+        ALLOC(h->drow, V);
+        ALLOC(h->qrow, static_cast<size_t>(cap) * dense_row_bytes(K));
+        CUI(cudaMemcpyAsync(h->row_slot, slot.data(), sizeof(int32_t) * V, cudaMemcpyHostToDevice, st));
+        CUI(cudaStreamSynchronize(st));
     }
+    // four documents per warp read q by topic for every word
+    const bool groups_ok = K <= kMaxKGrouped && static_cast<int64_t>(V) * K * static_cast<int64_t>(sizeof(uint32_t)) <= kDenseBytes &&
+                           h->opt.slice_len == 0 && h->opt.zstep_path != 1;
+    h->z_groups = groups_ok && h->opt.docs_per_warp == 4;
+    if (h->z_groups) ALLOC(h->qdense, static_cast<size_t>(V) * K);
     // the most frequent words are histogrammed in chunks by many CTAs
     {
         std::vector<int32_t> row(V, -1);
@@ -505,26 +500,11 @@ pulda_status pulda_init(pulda_handle **out, const int32_t *word_ids, const int64
     while (wpb > 1 && z_step_smem(K, wpb) > 160 * 1024) wpb >>= 1;
     h->z_warps = wpb;
     CUI(cudaGetLastError());
-    // Four documents per warp share each token's fixed work (record, count
-    // updates, scan, draw) over four tokens, but each lane then walks four
-    // times the topics, so a token's intersection costs more and a document's
-    // tokens advance about 3x slower.  Once the one-warp z-step spread small K
-    // over 8 or 16 topics per lane it was faster at every K measured (z-step
-    // ms, 100,000 documents of the large corpus: K = 50 10.2 vs 14.7 four per
-    // warp, K = 100 10.4 vs 13.7, K = 200 10.3 vs 13.0), so auto takes one
-    // per warp and four per warp is an explicit choice.  That needs every
-    // word's dense q row; not with slices or the column-only path.
-    const bool groups_ok = K <= kMaxKGrouped && h->n_dense == V && h->opt.slice_len == 0 && h->opt.zstep_path != 1;
-    h->z_groups = groups_ok && h->opt.docs_per_warp == 4;
-    h->n_long = count_long(doc_offsets, dord);
-    h->n_coop = count_coop(h, doc_offsets, dord, N);
-    h->narrow_z = narrow_from(doc_offsets, dord, h->n_coop);
-    h->narrow_all = narrow_from(doc_offsets, dord, 0);
-    // as many one-warp CTAs as fit with the corpus pass's count width (16-bit
-    // counts halve the shared memory, which limits residency at large K); a
-    // launch with 32-bit counts (a fold-in of long documents) queues the
-    // CTAs that do not fit, each taking documents from the same counter
-    h->z_grid = sms * z_step_blocks_per_sm(K, wpb, h->narrow_z);
+    h->n_wide = count_wide(doc_offsets, dord);
+    h->n_coop = count_coop(h, doc_offsets, dord, h->n_wide, N);
+    // as many one-warp CTAs as fit with two count planes; a launch with three
+    // queues the CTAs that do not fit, each taking documents from the same counter
+    h->z_grid = sms * z_step_blocks_per_sm(K, wpb, true);
     CUI(cudaGetLastError());
     h->coop_grid = sms * z_coop_blocks_per_sm(K);
     CUI(cudaGetLastError());
@@ -587,16 +567,18 @@ pulda_status pulda_z_step(pulda_handle *h) {
         launch_slice_counts(h->doc_off, h->sliced_docs, h->n_sliced, h->z, h->K, h->m0, h->stream);
         ZArgs a = z_args(h, h->doc_off, h->doc_order_short, h->D_short, h->w, h->z, h->seed,
                          static_cast<uint32_t>(h->sweep), 0);
+        a.work = h->work + 1;
         a.slices = h->slices;
         a.n_slices = h->n_slices;
         a.m0 = h->m0;
-        a.narrow = h->narrow_all ? 1 : 0;      // the slices start from whole documents' counts
+        a.narrow = h->n_wide == 0 ? 1 : 0;     // the slices start from whole documents' counts
         launch_z_step(a, h->z_warps, h->z_grid, h->stream);
         CU(h, cudaGetLastError());
         return PULDA_OK;
     }
-    return run_z(h, h->doc_off, h->doc_order, h->D, h->n_long, h->n_coop, h->w, h->z, h->seed,
-                 static_cast<uint32_t>(h->sweep), 0, h->narrow_z);
+    CU(h, run_z(h, z_args(h, h->doc_off, h->doc_order, h->D, h->w, h->z, h->seed, static_cast<uint32_t>(h->sweep), 0), h->n_wide,
+                h->n_coop, h->work + 1));
+    return PULDA_OK;
 }
 
 pulda_status pulda_sweep(pulda_handle *h, int32_t n_sweeps) {
@@ -780,13 +762,10 @@ pulda_status pulda_infer(pulda_handle *h, const int32_t *word_ids, const int64_t
     CU(h, cudaMemcpyAsync(dord, ord.data(), sizeof(int32_t) * D_new, cudaMemcpyHostToDevice, st));
     launch_init_z(N, h->K, seed, 0, dz, st);
     CU(h, clear_z_counters(h));
-    const int64_t n_long = count_long(doc_offsets, ord);
-    const int64_t n_coop = count_coop(h, doc_offsets, ord, N);
-    const bool narrow = narrow_from(doc_offsets, ord, n_coop);
-    for (int32_t sw = 1; sw <= n_sweeps; ++sw) {
-        s = run_z(h, doff, dord, D_new, n_long, n_coop, dw, dz, seed, static_cast<uint32_t>(sw), 0, narrow);
-        if (s != PULDA_OK) return s;
-    }
+    const int64_t n_wide = count_wide(doc_offsets, ord);
+    const int64_t n_coop = count_coop(h, doc_offsets, ord, n_wide, N);
+    for (int32_t sw = 1; sw <= n_sweeps; ++sw)
+        CU(h, run_z(h, z_args(h, doff, dord, D_new, dw, dz, seed, static_cast<uint32_t>(sw), 0), n_wide, n_coop, h->work + 1));
     if (z_out) CU(h, cudaMemcpyAsync(z_out, dz, sizeof(int16_t) * N, cudaMemcpyDeviceToHost, st));
     if (m_out) {
         CU(h, tm.get(&dm, static_cast<size_t>(D_new) * h->K));
@@ -801,10 +780,7 @@ pulda_status pulda_z_layout(pulda_handle *h, int32_t *docs_per_warp, int64_t *co
     if (!h) return PULDA_ERR_INVALID;
     if (docs_per_warp) *docs_per_warp = h->z_groups ? 4 : 1;
     if (coop_docs) *coop_docs = h->n_coop;
-    if (one_warp_docs) {
-        const int64_t head = h->z_groups ? std::max(h->n_coop, h->n_long) : h->n_coop;
-        *one_warp_docs = h->z_groups ? head - h->n_coop : h->D - h->n_coop;
-    }
+    if (one_warp_docs) *one_warp_docs = h->z_groups ? h->n_wide : h->D - h->n_coop;
     return PULDA_OK;
 }
 

@@ -81,12 +81,13 @@ cudaError_t balloc(pulda_batch *b, T **p, size_t n) {
 
 thread_local std::string g_batch_init_error;
 
-// Documents the cooperative z-step takes at threshold L (the work list is longest first).
+// Documents the long-document z-step takes at threshold L (the work list is
+// longest first; the n_wide widest are the one-warp kernel's).
 int count_coop_items(const pulda_batch *b, int64_t L) {
     if (L <= 0) return 0;
-    int n = 0;
+    int n = b->bl.n_wide;
     while (n < static_cast<int>(b->dlen.size()) && b->dlen[n] >= L) ++n;
-    return n;
+    return n - b->bl.n_wide;
 }
 
 // Starts a tuning phase over candidates [first, cand.size()): forward, then backward.
@@ -259,7 +260,7 @@ pulda_status pulda_batch_init(pulda_batch **out, const pulda_chain_desc *chains,
             hz[c].apack = nullptr;
         }
         kmax = std::max(kmax, h->K);
-        narrow = narrow && h->narrow_all;
+        narrow = narrow && h->n_wide == 0;
         for (HeavyChunk hc : h->heavy_chunks) {
             hc.chain = c;
             heavy.push_back(hc);
@@ -287,6 +288,7 @@ pulda_status pulda_batch_init(pulda_batch **out, const pulda_chain_desc *chains,
         b->dlen[i] = di[i].first;
         n_tokens += di[i].first;
     }
+    while (b->bl.n_wide < static_cast<int>(b->dlen.size()) && b->dlen[b->bl.n_wide] > kNarrowMaxLen) ++b->bl.n_wide;
     int2 *d_wl = nullptr, *d_dl = nullptr;
     HeavyChunk *d_heavy = nullptr;
     if ((ea = balloc(b, &d_wl, wlist.size())) != cudaSuccess || (ea = balloc(b, &d_dl, dlist.size())) != cudaSuccess ||
@@ -296,6 +298,7 @@ pulda_status pulda_batch_init(pulda_batch **out, const pulda_chain_desc *chains,
     }
     cudaStream_t st = b->stream;
     const uint32_t zero = 0;
+    for (ZArgs &z : hz) z.narrow = narrow ? 1 : 0;      // one width of the counts for the whole launch
     if (cudaMemcpyAsync(d_phi, hp.data(), sizeof(PhiArgs) * n_chains, cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaMemcpyAsync(d_z, hz.data(), sizeof(ZArgs) * n_chains, cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaMemcpyAsync(d_wl, wlist.data(), sizeof(int2) * wlist.size(), cudaMemcpyHostToDevice, st) != cudaSuccess ||
@@ -325,7 +328,7 @@ pulda_status pulda_batch_init(pulda_batch **out, const pulda_chain_desc *chains,
     bl.phi_grid = b->sms * batch_phi_blocks_per_sm(kmax);
     bl.coop_grid = b->sms * batch_coop_blocks_per_sm(kmax);
     bl.bar = d_bar;
-    bl.persist_grid = b->sms * batch_persistent_blocks_per_sm(kmax, narrow);
+    bl.persist_grid = b->sms * batch_persistent_blocks_per_sm(kmax, narrow, &bl.persist_z_warps, &bl.table_stage);
     // The cooperative threshold: fixed, none, or the automatic rule of the
     // single-chain z-step over all chains' tokens (documents that would outlast
     // the pass on one warp).  It is not timed: on the 32-chain workload, timing
@@ -348,7 +351,9 @@ pulda_status pulda_batch_init(pulda_batch **out, const pulda_chain_desc *chains,
         }
         b->cand.push_back({kMultiWarps, 0, true, pk});
     } else if (o.warps_per_block > 0) {
-        b->cand.push_back({o.warps_per_block, fixed_coop, false, pk});
+        int w = o.warps_per_block;
+        while (w > 1 && z_step_smem(kmax, w, narrow) > static_cast<size_t>(smem_optin())) --w;
+        b->cand.push_back({w, fixed_coop, false, pk});
     } else {
         for (int w : {2, 4, 8})
             if (w <= kMultiWarps && z_step_smem(kmax, w) <= 160 * 1024) b->cand.push_back({w, fixed_coop, false, pk});

@@ -25,10 +25,8 @@ struct pulda_handle {
     int z_warps = 8, z_grid = 0, phi_grid = 0;
     bool z_groups = false;      // grouped z-step (four documents per warp) in use
     int zg_grid = 0;
-    int64_t n_long = 0;         // documents too long for the grouped z-step (first in doc_order)
-    int64_t n_coop = 0;         // documents the cooperative z-step takes (first in doc_order)
-    bool narrow_z = false;      // the one-warp z-step's documents (after n_coop) fit 16-bit counts
-    bool narrow_all = false;    // every document does
+    int64_t n_wide = 0;         // documents of 2^16 tokens or more (first in doc_order)
+    int64_t n_coop = 0;         // documents the long-document z-step takes (next in doc_order)
     int coop_grid = 0;
     cudaStream_t stream2 = nullptr;                       // the one-warp z-step beside the cooperative one
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
@@ -50,8 +48,10 @@ struct pulda_handle {
     int4 *slices = nullptr; int n_slices = 0;
     uint32_t *m0 = nullptr;
     int32_t *doc_order_short = nullptr; int64_t D_short = 0;
-    // dense q rows of the most frequent words (z-step document side)
-    uint32_t *qdense = nullptr; int32_t *dense_slot = nullptr; int n_dense = 0;
+    // dense rows of the most frequent words, and every word's row or -1 (fixed,
+    // and as the current Phi allows); q by topic for four documents per warp
+    uint8_t *qrow = nullptr; int32_t *row_slot = nullptr, *drow = nullptr;
+    uint32_t *qdense = nullptr;
     // Dirichlet Phi (Algorithm 1), allocated in that mode only
     float *gam = nullptr, *invSf = nullptr; double *Sd = nullptr, *invS = nullptr, *dpart = nullptr;
     uint16_t *topic = nullptr; uint32_t *c = nullptr, *q = nullptr, *athr = nullptr; uint16_t *atopic = nullptr;
@@ -96,6 +96,13 @@ struct DevTemp {
         return e;
     }
 };
+// Tokens from which a document of an N-token pass goes to a CTA of its own
+// (INT64_MAX: none do).
+int64_t long_document_tokens(const pulda_handle *h, int64_t N);
+// One z-step over a's documents doc_order[0 .. D) on the handle's streams: the
+// first n_wide have 2^16 tokens or more, the next n_coop go to a CTA each, and
+// so do the others when they are few.  work: five counters.
+cudaError_t run_z(pulda_handle *h, ZArgs a, int64_t n_wide, int64_t n_coop, int *work);
 PhiArgs phi_args(pulda_handle *h);
 ZArgs z_args(pulda_handle *h, const int64_t *doc_off, const int32_t *doc_order, int64_t D, const int32_t *w,
              int16_t *z, uint64_t seed, uint32_t sweep, int64_t index_base);

@@ -28,6 +28,7 @@
 
 #include "device_rng.cuh"
 #include "pulda_internal.h"
+#include "zdense.cuh"
 #include "zstep.cuh"
 #include "checks.cuh"
 
@@ -498,7 +499,7 @@ __global__ void k_colptr_scan_multi(const PhiArgs *chains) {
 // the word's nonzero topics.
 // The same per-word tables, one warp per word: the per-entry arithmetic in
 // parallel, the Vose pairing (sequential by definition) in lane 0.
-__device__ void phi_tables_word_warp(const PhiArgs &a, int v) {
+__device__ void phi_tables_word_warp(const PhiArgs &a, int v, uint8_t *stage) {
     const int lane = threadIdx.x & 31;
     const int n = a.nnz_c[v];
     const int64_t src = static_cast<int64_t>(v) * a.K;
@@ -514,16 +515,22 @@ __device__ void phi_tables_word_warp(const PhiArgs &a, int v) {
             bm[wi] = bits;
         }
     }
-    // a word with a dense q row: zero it (the column's entries are written below)
-    uint32_t *qrow = nullptr;
-    if (a.dense_slot) {
-        const int slot = a.dense_slot[v];
-        if (slot >= 0) {
-            qrow = a.qdense + static_cast<int64_t>(slot) * a.K;
-            for (int k = lane; k < a.K; k += 32) qrow[k] = 0;
-            __syncwarp();
-        }
+    uint32_t *q32 = a.qdense ? a.qdense + static_cast<int64_t>(v) * a.K : nullptr;
+    if (q32) {
+        for (int k = lane; k < a.K; k += 32) q32[k] = 0;
+        __syncwarp();
     }
+    // the word's dense row is put together in `stage` (zero between words),
+    // else in place
+    const int slot = a.row_slot[v];
+    const int RB = dense_row_bytes(a.K), PB = RB / 3;
+    uint8_t *row = slot >= 0 ? a.qrow + static_cast<int64_t>(slot) * RB : nullptr;
+    if (row && (n == 0 || !stage)) {
+        for (int i = lane; i < RB / 16; i += 32) reinterpret_cast<uint4 *>(row)[i] = make_uint4(0u, 0u, 0u, 0u);
+        __syncwarp();
+    }
+    uint8_t *rw = stage ? stage : row;
+    if (n == 0 && lane == 0) a.drow[v] = slot;
     if (n == 0) {
         if (lane == 0) a.A[v] = 0;
         return;
@@ -547,6 +554,7 @@ __device__ void phi_tables_word_warp(const PhiArgs &a, int v) {
     const int e = static_cast<int>((bits >> 52) & 0x7FF) - 1022;
     const double scale = __longlong_as_double(static_cast<long long>(1023 + 24 - e) << 52);
     u64 asum = 0;
+    uint32_t qtop = 0;                  // a q of 2^24 does not fit a row's three bytes
     for (int j = lane; j < n; j += 32) {
         const int k = a.cst_k[src + j];
         const uint32_t c = a.cst_c[src + j];
@@ -558,7 +566,14 @@ __device__ void phi_tables_word_warp(const PhiArgs &a, int v) {
         a.topic[out + j] = static_cast<uint16_t>(k);
         a.c[out + j] = c;
         a.q[out + j] = qv;
-        if (qrow) qrow[k] = qv;
+        if (q32) q32[k] = qv;
+        if (row) {
+            const int at = dense_pos(a.K, k);
+            rw[at] = static_cast<uint8_t>(qv);
+            rw[at + PB] = static_cast<uint8_t>(qv >> 8);
+            rw[at + 2 * PB] = static_cast<uint8_t>(qv >> 16);
+        }
+        qtop |= qv >> 24;
         a.vose_p[out + j] = am * static_cast<u64>(n);   // scaled so each slot holds A units
         a.athr[out + j] = 0xFFFFFFFFu;
         a.atopic[out + j] = static_cast<uint16_t>(k);
@@ -566,8 +581,19 @@ __device__ void phi_tables_word_warp(const PhiArgs &a, int v) {
         asum += am;
     }
     asum = warp_sum64(asum);
-    if (lane == 0) a.A[v] = asum;
+    const bool fits = !__any_sync(0xFFFFFFFFu, qtop != 0);
+    if (lane == 0) {
+        a.A[v] = asum;
+        a.drow[v] = fits ? slot : -1;
+    }
     __syncwarp();
+    if (row && stage) {
+        for (int i = lane; i < RB / 16; i += 32) {
+            reinterpret_cast<uint4 *>(row)[i] = reinterpret_cast<uint4 *>(stage)[i];
+            reinterpret_cast<uint4 *>(stage)[i] = make_uint4(0u, 0u, 0u, 0u);
+        }
+        __syncwarp();
+    }
     if (asum == 0) return;
     // Vose: small stack grows up from 0, large stack down from n-1, each in
     // ascending slot order.  The warp builds the two stacks with a ballot per
@@ -633,400 +659,52 @@ __device__ void phi_tables_word_warp(const PhiArgs &a, int v) {
     }
 }
 
-// One warp per word, most frequent first (their columns are the longest).
-__global__ void k_phi_tables(PhiArgs a) {
-    const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    for (int i = wid; i < a.V; i += nwarps) phi_tables_word_warp(a, a.word_order[i]);
+// A warp's stage of the dense row it puts together: RB bytes each, zeroed;
+// null when the CTA has no room (bytes = 0).
+__device__ __forceinline__ uint8_t *table_stage(uint32_t *sm, int stage_bytes) {
+    if (stage_bytes == 0) return nullptr;
+    const int lane = threadIdx.x & 31;
+    uint8_t *st = reinterpret_cast<uint8_t *>(sm) + static_cast<size_t>(threadIdx.x >> 5) * stage_bytes;
+    for (int i = lane; i < stage_bytes / 16; i += 32) reinterpret_cast<uint4 *>(st)[i] = make_uint4(0u, 0u, 0u, 0u);
+    __syncwarp();
+    return st;
 }
 
-__global__ void k_phi_tables_multi(const PhiArgs *chains, const int2 *items, int n_items) {
+// One warp per word, most frequent first (their columns are the longest).
+__global__ void k_phi_tables(PhiArgs a, int stage_bytes) {
+    extern __shared__ __align__(16) uint32_t tsm[];
+    uint8_t *stage = table_stage(tsm, stage_bytes);
+    const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int nwarps = (gridDim.x * blockDim.x) >> 5;
+    for (int i = wid; i < a.V; i += nwarps) phi_tables_word_warp(a, a.word_order[i], stage);
+}
+
+__global__ void k_phi_tables_multi(const PhiArgs *chains, const int2 *items, int n_items, int stage_bytes) {
+    extern __shared__ __align__(16) uint32_t tsm[];
+    uint8_t *stage = table_stage(tsm, stage_bytes);
     const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     for (int i = wid; i < n_items; i += nwarps) {
         const int2 it = items[i];
-        phi_tables_word_warp(chains[it.x], it.y);
+        phi_tables_word_warp(chains[it.x], it.y, stage);
     }
 }
 
 // ============================================================== z-step
-// Entries of the document-side intersection each lane gathers with
-// independent loads before consuming them.
-#ifndef PULDA_ZGATHER
-#define PULDA_ZGATHER 7
-#endif
-// 4-warp CTAs, 8 per SM: the kernel fits 64 registers without
-// spilling and 32 warps share each SM (issue slots are what bound it; fewer
-// warps leave them idle while each warp waits on its dependent chain).
+// 4-warp CTAs, 7 per SM: 72 registers, 28 warps per SM.
 #ifndef PULDA_ZMINBLOCKS
-#define PULDA_ZMINBLOCKS 8
+#define PULDA_ZMINBLOCKS 7
 #endif
-constexpr int kGather = PULDA_ZGATHER;
-// the same for 16 and 8 topics per lane (fewer bits per lane)
-#ifndef PULDA_ZGATHER16
-#define PULDA_ZGATHER16 5
-#endif
-#ifndef PULDA_ZGATHER8
-#define PULDA_ZGATHER8 4
-#endif
-constexpr int kGather16 = PULDA_ZGATHER16;
-constexpr int kGather8 = PULDA_ZGATHER8;
-
-// Index of topic k's count with TPL topics per lane: a gap word after each
-// lane's TPL slots keeps the lanes' slots on distinct banks.
-template <int TPL>
-__device__ __forceinline__ int mit(int k) { return k + k / TPL; }
-
-// A lane's bits of its TPL topics: 32 bits, or 64 for 64 topics per lane.
-template <int TPL>
-using lane_word_t = typename std::conditional<TPL == 64, uint64_t, uint32_t>::type;
-
-// This lane's TPL bits of a bitmap row starting at word `row`.
-template <int TPL>
-__device__ __forceinline__ lane_word_t<TPL> lane_bits(const uint32_t *bits, int64_t row, int lane) {
-    if constexpr (TPL == 64) {
-        const uint32_t *p = bits + row + 2 * lane;
-        return static_cast<uint64_t>(p[0]) | (static_cast<uint64_t>(p[1]) << 32);
-    } else if constexpr (TPL == 32) {
-        return bits[row + lane];
-    } else {
-        const uint32_t w = bits[row + (lane * TPL >> 5)];
-        return (w >> ((lane * TPL) & 31)) & ((1u << (TPL & 31)) - 1u);
-    }
-}
-
-// 1 << b in a lane word, 0 for b = -1.
-template <int TPL>
-__device__ __forceinline__ lane_word_t<TPL> lane_bit(int b) {
-    if constexpr (TPL == 64) return bit_or_zero64(b);
-    else return bit_or_zero(b);
-}
-
-// 1 << b in a lane word for b in [0, TPL).
-template <int TPL>
-__device__ __forceinline__ lane_word_t<TPL> lane_bit_at(int b) {
-    return static_cast<lane_word_t<TPL>>(1) << b;
-}
-
-__device__ __forceinline__ int popc_word(uint32_t x) { return __popc(x); }
-__device__ __forceinline__ int popc_word(uint64_t x) { return __popcll(x); }
-
-// One warp per document (dynamically scheduled, longest first).  m_d lives
-// in shared memory as a dense count array; for K <= 2048 each lane also holds
-// the bits of m_d's nonzero topics among the TPL it owns (TPL = 64 above 1024
-// topics, 32, or 16 / 8 for K <= 512 / 256, so that small K still spreads
-// over the warp), and the document side reads q of topic TPL lane + b from
-// the word's dense q row.  Tokens are visited in position order: remove token i (m^{-i}),
-// compute sigma_b = sum_k q_{k,v} m_k over the smaller of {k : m_k > 0} and
-// {k : phi_{k,v} > 0} (complexity theorem), draw r = floor(u (A + 2^16 B)),
-// take the alias draw if r < A, else the first topic where the running sum
-// of q m passes (r - A) / 2^16; add the token back.
-//
-// Latency matters as much as throughput: a document's tokens are strictly
-// sequential, so the longest documents bound the kernel.  Everything that
-// depends only on the token (its word, Philox words, alias outcome, the
-// word's bitmap) is fetched ahead; the only loads on the critical path are
-// the q values of the intersection, issued together.
-// Resamples the tokens of one document, by one warp, in position order,
-// pass after pass, until `budget` tokens are done or `max_pass_end` passes
-// have been completed.  m (K entries of shared memory) is rebuilt from the
-// current topics first: with positions < pos already resampled in this pass
-// that is exactly m of the sequential sampler at `pos`.  Returns the run's
-// final (sweep, pos) through r.
-// With m0 set, m starts from those K counts (a slice of a longer document,
-// from the document's counts at the start of the pass) instead of the run's
-// own topics.
-template <int TPL, typename CT>
-__device__ void z_doc_warp_t(const ZArgs &a, uint32_t *m, DocRun &r, u64 *wcnt, const uint32_t *m0) {
-    static_assert(TPL == 8 || TPL == 16 || TPL == 32 || TPL == 64, "8, 16, 32 or 64 topics per lane");
-    using BT = lane_word_t<TPL>;
-    static_assert(sizeof(CT) == 2 || sizeof(CT) == 4, "16- or 32-bit counts");
-    constexpr int kLead = 4 / static_cast<int>(sizeof(CT));    // counts before mt[0]: the leading zero's word
-    constexpr int G = TPL >= 32 ? kGather : TPL == 16 ? kGather16 : kGather8;
-    const int lane = threadIdx.x & 31;
-    const int K = a.K;
-    const bool use_bm = a.bits != nullptr && a.path != 1;
-    if (r.len == 0 || r.budget <= 0) return;
-    // Lane l owns topics [TPL l, TPL l + TPL) (TPL = 64, 32, 16 or 8 by K, so
-    // that small K spreads over more lanes).  Topic k's count is
-    // mt[mit<TPL>(k)]: lane l's topics sit at mt[(TPL + 1) l + b], and the word
-    // before each lane's slots is a zero (mt[-1] for lane 0 and for the lanes
-    // without topics, the gap word after lane l - 1's slots otherwise), so an
-    // empty gather slot (bit -1) reads a zero count.  Counts are CT (16-bit
-    // when every document of the launch is shorter than 2^16 tokens).
-    CT *mt = reinterpret_cast<CT *>(m) + kLead;
-    const int nl = TPL == 32 ? a.KW : (K + TPL - 1) / TPL;      // lanes that own topics
-    const bool own = lane < nl;
-    const int mo = own ? (TPL + 1) * lane : 0;   // this lane's count slots (document side)
-    const int qo = own ? TPL * lane : 0;         // and its segment of a dense q row
-    if (m0) {
-        for (int k = lane; k < K; k += 32) mt[mit<TPL>(k)] = m0[k];
-    } else {
-        for (int k = lane; k < K; k += 32) mt[mit<TPL>(k)] = 0;
-        __syncwarp();
-        for (int i = lane; i < r.len; i += 32) {
-            const int k = guard_index(r.z[i], K, a.stats);
-            if (sizeof(CT) == 4) {
-                atomicAdd(reinterpret_cast<uint32_t *>(&mt[mit<TPL>(k)]), 1u);
-            } else {        // the 32-bit word holding the count: no carry, counts stay below 2^16
-                const int h = mit<TPL>(k) + kLead;
-                atomicAdd(m + (h >> 1), 1u << ((h & 1) * 16));
-            }
-        }
-    }
-    if (lane == 0) mt[-1] = 0;
-    if (lane + 1 < nl) mt[(TPL + 1) * lane + TPL] = 0;
-    __syncwarp();
-    BT mbits = 0;
-    int kd = 0;
-    if (use_bm && TPL == 32) {
-        for (int g = 0; g < a.KW; ++g) {
-            const int k = g * 32 + lane;
-            const uint32_t bal = __ballot_sync(0xFFFFFFFFu, k < K && mt[mit<TPL>(k)] > 0);
-            if (lane == g) mbits = bal;
-            kd += __popc(bal);
-        }
-    } else if (use_bm) {
-        if (own) {
-            for (int b = 0; b < TPL; ++b) {
-                const int k = TPL * lane + b;
-                if (k < K && mt[mit<TPL>(k)] > 0) mbits |= lane_bit_at<TPL>(b);
-            }
-        }
-        kd = static_cast<int>(__reduce_add_sync(0xFFFFFFFFu, static_cast<uint32_t>(popc_word(mbits))));
-    } else {
-        int cnt = 0;
-        for (int k = lane; k < K; k += 32) cnt += mt[mit<TPL>(k)] > 0;
-#pragma unroll
-        for (int o = 16; o; o >>= 1) cnt += __shfl_xor_sync(0xFFFFFFFFu, cnt, o);
-        kd = cnt;
-    }
-    // The run's state lives in the warp's shared memory while its tokens are
-    // drawn (it is read and advanced once per 32-token block), which keeps it
-    // out of the registers of the token loop.
-    DocRun &rs = *z_warp_run(wcnt);
-    if (lane == 0) rs = r;
-    __syncwarp();
-    const uint32_t sweep_end = rs.sweep + static_cast<uint32_t>(rs.max_pass_end);
-    bool first = true;
-    while (rs.budget > 0 && rs.sweep != sweep_end) {
-        if (rs.deadline != ~0ull && !first) {
-            uint64_t now = 0;
-            if (lane == 0) now = global_ns();
-            if (__shfl_sync(0xFFFFFFFFu, now, 0) >= rs.deadline) break;
-        }
-        first = false;
-        const int i0 = rs.pos;
-        const int64_t left = static_cast<int64_t>(rs.len - i0);
-        const int cnt = static_cast<int>(min(static_cast<int64_t>(32), min(left, rs.budget)));
-        const int i = i0 + lane;
-        const bool valid = lane < cnt;
-        int znew = 0;
-        // Everything that depends only on the token is fetched for 32 tokens at
-        // once, one per lane, and staged in shared memory:
-        //   rec[2t]   = {column start (low 32), column start >> 32 | alias outcome << 16, sigma_a (lo, hi)}
-        //   rec[2t+1] = {Philox x0, x1, word, K_v | old topic << 16}
-        // (column starts are below 2^48, K_v <= 16384, topics < 16384).
-        uint4 *rec = reinterpret_cast<uint4 *>(m + z_count_words<CT>(K));
-        uint32_t *drow_of = reinterpret_cast<uint32_t *>(rec + 64);   // q row offset of the token's word, or ~0
-        if (valid) znew = stage_token(a, rs, i, rec + 2 * lane, drow_of + lane);
-        __syncwarp();
-        // the word's bitmap row (TPL topics per lane)
-        const uint32_t *bits = a.bits;
-        BT bm_next = 0u;
-        if (use_bm && own) bm_next = lane_bits<TPL>(bits, static_cast<int64_t>(rec[1].z) * a.KWp, lane);
-        // this block's counters, in 32 bits (at most 32 tokens of K <= 16384),
-        // added to the warp's 64-bit counters once per block
-        // (c_min: sum of min(K_d, K_v), the same in every lane; c_cnt: tokens
-        // with K_d < K_v in bits 0-5, alias draws in 6-11, zero-mass tokens in
-        // 12-17 -- each at most 32 -- and this lane's share of |J| (at most
-        // 32 x 32) from bit 18)
-        uint32_t c_min = 0, c_cnt = 0;
-        for (int tt = 0; tt < cnt; ++tt) {
-            const uint4 t0 = rec[2 * tt], t1 = rec[2 * tt + 1];
-            const int kold = static_cast<int>(t1.w >> 16);
-            const int64_t col = static_cast<int64_t>((static_cast<u64>(t0.y & 0xFFFFu) << 32) | t0.x);
-            const int n_w = static_cast<int>(t1.w & 0xFFFFu);
-            const u64 At = (static_cast<u64>(t0.w) << 32) | t0.z;
-            const u64 U = (static_cast<u64>(t1.x) << 32) | t1.y;
-            const int ka = static_cast<int>(t0.y >> 16);
-            const BT bm = bm_next;
-            if (use_bm && tt + 1 < cnt && own)   // the next token's bitmap word, fetched while this one is drawn
-                bm_next = lane_bits<TPL>(bits, static_cast<int64_t>(rec[2 * tt + 3].z) * a.KWp, lane);
-            // remove token i: m^{-i}
-            if (use_bm) {
-                // the lane owning topic kold updates its count and bitmap word
-                // (lanes read only their own counts on the document side)
-                const bool me = lane == kold / TPL;
-                const uint32_t old = me ? mt[mit<TPL>(kold)] : 0u;
-                if (me) mt[mit<TPL>(kold)] = old - 1;
-                const bool died = me && old == 1;
-                if (died) mbits &= ~lane_bit_at<TPL>(kold % TPL);
-                kd -= __any_sync(0xFFFFFFFFu, died) ? 1 : 0;
-            } else {
-                const uint32_t old = mt[mit<TPL>(kold)];
-                __syncwarp();
-                if (lane == 0) mt[mit<TPL>(kold)] = old - 1;
-                if (old == 1) --kd;
-                __syncwarp();
-            }
-            c_min += static_cast<uint32_t>(kd < n_w ? kd : n_w);
-            c_cnt += kd < n_w ? 1u : 0u;
-            // |J| from the bitmaps on either side (the column side's topics with
-            // m > 0 are the same set); without bitmaps the column loop counts it
-            if (use_bm) c_cnt += static_cast<uint32_t>(popc_word(bm & mbits)) << 18;
-            // The document side needs the word's dense q row (q of topic TPL lane + b
-            // at qd[b]); a word without one is iterated on the column side.
-            const uint32_t drow = drow_of[tt];
-            const bool docside = use_bm && drow != 0xFFFFFFFFu && (a.path == 2 || kd * kDocRatio < n_w * 16);
-            const uint32_t *qcol = a.q + col;
-            const uint32_t *qd = a.qdense + drow + qo;
-            const CT *ml = mt + mo;
-            // per-lane partial sums of q m, in ascending topic order across lanes
-            u64 acc = 0;
-            uint32_t qv[G];
-            int bp[G];
-            BT rest = 0;               // docside: bits below the first G
-            int seg = 0, seg0 = 0;     // column side: this lane's contiguous segment
-            if (docside) {
-                // The lane's bits from the highest down; a slot past the last
-                // bit gets b = -1 and q = 0 (no load), and its count read hits
-                // the zero before the lane's slots.
-                BT rem = bm & mbits;
-#pragma unroll
-                for (int t = 0; t < G; ++t) {
-                    const int b = msb_or_neg1(rem);
-                    rem ^= lane_bit<TPL>(b);
-                    bp[t] = b;
-                    qv[t] = b >= 0 ? qd[b] : 0u;
-                }
-#pragma unroll
-                for (int t = 0; t < G; ++t) acc += static_cast<u64>(qv[t]) * ml[bp[t]];
-                rest = rem;
-                for (BT bb = rest; bb;) {
-                    const int b = msb_or_neg1(bb);
-                    bb ^= lane_bit<TPL>(b);
-                    acc += static_cast<u64>(qd[b]) * ml[b];
-                }
-            } else {
-                __syncwarp();   // the column side reads every lane's counts
-                seg = (n_w + 31) >> 5;
-                seg0 = seg * lane;
-                const int seg1 = min(seg0 + seg, n_w);
-                unsigned nj = 0;
-#pragma unroll 4
-                for (int j = seg0; j < seg1; ++j) {
-                    const uint32_t mk = mt[mit<TPL>(guard_index(a.topic[col + j], K, a.stats))];
-                    acc += static_cast<u64>(qcol[j]) * mk;
-                    if (!use_bm) nj += mk != 0u;
-                }
-                if (!use_bm) c_cnt += nj << 18;
-            }
-            const u64 incl = warp_incl_scan64(acc);
-            const u64 B = __shfl_sync(0xFFFFFFFFu, incl, 31);
-            const u64 T = At + (B << kFracBits);
-            int knew = kold;
-            if (T == 0) {
-                c_cnt += 1u << 12;
-            } else {
-                const u64 rr = __umul64hi(U, T);
-                if (rr < At) {
-                    knew = ka;
-                    c_cnt += 1u << 6;
-                } else {
-                    const u64 rb = (rr - At) >> kFracBits;
-                    const uint32_t bal = __ballot_sync(0xFFFFFFFFu, rb < incl);
-                    int found = -1;
-                    if (bal) {
-                        const int L = __ffs(bal) - 1;
-                        int f = -1;
-                        if (lane == L) {
-                            if (docside) {
-                                // walk down from the lane's inclusive sum: the
-                                // topic whose term takes it to rb or below (an
-                                // empty slot adds nothing, so the walk stops at
-                                // one of the lane's bits)
-                                u64 run = incl;
-#pragma unroll
-                                for (int t = 0; t < G; ++t) {
-                                    run -= static_cast<u64>(qv[t]) * ml[bp[t]];
-                                    if (rb >= run) { f = TPL * lane + bp[t]; break; }
-                                }
-                                for (BT bb = rest; f < 0 && bb;) {
-                                    const int b = msb_or_neg1(bb);
-                                    bb ^= lane_bit<TPL>(b);
-                                    run -= static_cast<u64>(qd[b]) * ml[b];
-                                    if (rb >= run) f = TPL * lane + b;
-                                }
-                            } else {
-                                u64 run = incl - acc;
-                                const int seg1 = min(seg0 + seg, n_w);
-                                for (int j = seg0; j < seg1; ++j) {
-                                    const int k = guard_index(a.topic[col + j], K, a.stats);
-                                    run += static_cast<u64>(qcol[j]) * mt[mit<TPL>(k)];
-                                    if (rb < run) { f = k; break; }
-                                }
-                            }
-                        }
-                        found = __shfl_sync(0xFFFFFFFFu, f, L);
-                    }
-                    if (found < 0) {
-                        if (lane == 0) atomicOr(&a.stats[ST_ERROR], ERR_INTERNAL);
-                    } else {
-                        knew = found;
-                    }
-                }
-            }
-            // add token i back with its new topic
-            knew = guard_index(knew, K, a.stats);
-            if (use_bm) {
-                const bool me = lane == knew / TPL;
-                const uint32_t old2 = me ? mt[mit<TPL>(knew)] : 0u;
-                if (me) mt[mit<TPL>(knew)] = old2 + 1;
-                const bool born = me && old2 == 0;
-                if (born) mbits |= lane_bit_at<TPL>(knew % TPL);
-                kd += __any_sync(0xFFFFFFFFu, born) ? 1 : 0;
-            } else {
-                const uint32_t old2 = mt[mit<TPL>(knew)];
-                __syncwarp();
-                if (lane == 0) mt[mit<TPL>(knew)] = old2 + 1;
-                if (old2 == 0) ++kd;
-                __syncwarp();
-            }
-            if (lane == tt) znew = knew;
-        }
-        if (valid) rs.z[i] = static_cast<int16_t>(znew);
-        {   // the block's counts into the warp's 64-bit counters, lane j its counter j
-            const uint32_t jsum = __reduce_add_sync(0xFFFFFFFFu, c_cnt >> 18);
-            const uint32_t v = lane == 0 ? static_cast<uint32_t>(cnt)
-                             : lane == 1 ? (c_cnt >> 6) & 63u
-                             : lane == 2 ? c_min
-                             : lane == 3 ? (c_cnt >> 12) & 63u
-                             : lane == 4 ? jsum : c_cnt & 63u;
-            if (lane < 6) wcnt[lane] += v;
-        }
-        __syncwarp();
-        if (lane == 0) {
-            rs.budget -= cnt;
-            rs.pos += cnt;
-            if (rs.pos == rs.len) { rs.pos = 0; rs.sweep += 1; }
-        }
-        __syncwarp();
-    }
-    r = rs;
-    __syncwarp();
-}
 
 // One chain, one document per warp (dynamically scheduled, longest first),
 // one pass.
-// TPL topics per lane (z_lane_topics(K)) and CT counts, one instantiation
-// per kernel.
-template <int TPL, typename CT>
+// NW = z_nw(K) words per lane and plane, one instantiation per kernel.
+template <int NW>
 __global__ void __launch_bounds__(32 * kZWarps, PULDA_ZMINBLOCKS) k_z_step(ZArgs a) {
-    extern __shared__ uint32_t zsm[];
+    extern __shared__ __align__(16) uint32_t zsm[];
     const int lane = threadIdx.x & 31;
-    uint32_t *m = zsm + static_cast<size_t>(threadIdx.x >> 5) * z_warp_words_t<CT>(a.K);
-    u64 *wcnt = z_warp_counters_t<CT>(m, a.K);
+    uint32_t *m = zsm + static_cast<size_t>(threadIdx.x >> 5) * z_dense_warp_words(a.K, a.narrow != 0);
+    u64 *wcnt = z_dense_counters(m, a.K, a.narrow != 0);
     zero_warp_counters(wcnt);
     const uint32_t sweep = sweep_of(a);
     for (;;) {
@@ -1049,7 +727,7 @@ __global__ void __launch_bounds__(32 * kZWarps, PULDA_ZMINBLOCKS) k_z_step(ZArgs
             len = static_cast<int>(a.doc_off[d + 1] - s);
         }
         DocRun r{a.w + s, a.z + s, len, a.seed, a.index_base + s, sweep, 0, len, 1};
-        z_doc_warp_t<TPL, CT>(a, m, r, wcnt, m0);
+        z_doc<NW>(a, m, r, wcnt, m0);
     }
     flush_warp_counters(a.stats, wcnt);
 }
@@ -1072,16 +750,13 @@ __global__ void k_slice_counts(const int64_t *doc_off, const int32_t *sliced_doc
 
 // Many chains: the work list holds (chain, document) pairs, longest first
 // across all chains; shared memory per warp is sized for the largest K.
-// TPL = z_lane_topics(kmax): every chain of the batch that carries bitmaps has
-// K <= kmax <= 32 TPL (the others iterate their columns);
-// CT 16-bit when every document of every chain is shorter than 2^16 tokens.
-template <int TPL, typename CT>
+// Chains take the form of their own K.
 __global__ void __launch_bounds__(32 * kMultiWarps, PULDA_MULTI_MINB) k_z_step_multi(const ZArgs *chains, const int2 *items,
-                                                                        int n_items, int *work, int kmax) {
-    extern __shared__ uint32_t zsm[];
+                                                                        int n_items, int *work, int kmax, int narrow) {
+    extern __shared__ __align__(16) uint32_t zsm[];
     const int lane = threadIdx.x & 31;
-    uint32_t *m = zsm + static_cast<size_t>(threadIdx.x >> 5) * z_warp_words_t<CT>(kmax);
-    u64 *wcnt = z_warp_counters_t<CT>(m, kmax);     // beyond every chain's m and token records
+    uint32_t *m = zsm + static_cast<size_t>(threadIdx.x >> 5) * z_dense_warp_words(kmax, narrow != 0);
+    u64 *wcnt = z_dense_counters(m, kmax, narrow != 0);     // beyond every chain's counts and token records
     zero_warp_counters(wcnt);
     for (;;) {
         int item = 0;
@@ -1091,9 +766,7 @@ __global__ void __launch_bounds__(32 * kMultiWarps, PULDA_MULTI_MINB) k_z_step_m
         const int2 it = items[item];
         const ZArgs &a = chains[it.x];
         const int64_t s = a.doc_off[it.y];
-        DocRun r{a.w + s, a.z + s, static_cast<int>(a.doc_off[it.y + 1] - s), a.seed, a.index_base + s, sweep_of(a),
-                 0, a.doc_off[it.y + 1] - s, 1};
-        z_doc_warp_t<TPL, CT>(a, m, r, wcnt, nullptr);
+        z_doc_any(&a, m, s, static_cast<int>(a.doc_off[it.y + 1] - s), sweep_of(a), wcnt);
         flush_warp_counters(a.stats, wcnt);
     }
 }
@@ -1128,15 +801,15 @@ __global__ void k_batch_begin_sweep(const PhiArgs *chains, int n_chains, uint32_
 // With window_ns > 0 a slot also stops at the first 32-token block boundary
 // window_ns after its warp took it up, having done at least one block (a slot
 // taken up in a later wave of a crowded launch gets the same time as the first).
-template <int TPL, typename CT>
+template <int NW>
 __global__ void __launch_bounds__(32 * kZWarps, 7) k_serve_step(ZArgs a, ServeSlot *slots, const int32_t *active,
                                                                      int n_active, const int32_t *arena_w,
                                                                      int16_t *arena_z, int64_t slice, int *work,
                                                                      uint64_t window_ns) {
-    extern __shared__ uint32_t zsm[];
+    extern __shared__ __align__(16) uint32_t zsm[];
     const int lane = threadIdx.x & 31;
-    uint32_t *m = zsm + static_cast<size_t>(threadIdx.x >> 5) * z_warp_words_t<CT>(a.K);
-    u64 *wcnt = z_warp_counters_t<CT>(m, a.K);
+    uint32_t *m = zsm + static_cast<size_t>(threadIdx.x >> 5) * z_dense_warp_words(a.K, a.narrow != 0);
+    u64 *wcnt = z_dense_counters(m, a.K, a.narrow != 0);
     zero_warp_counters(wcnt);
     for (;;) {
         int item = 0;
@@ -1164,7 +837,7 @@ __global__ void __launch_bounds__(32 * kZWarps, 7) k_serve_step(ZArgs a, ServeSl
         }
         DocRun r{arena_w + sl.off, z, sl.len, sl.seed, 0, sweep, pos, slice,
                  static_cast<int>(sl.sweep_end - sweep), deadline};
-        z_doc_warp_t<TPL, CT>(a, m, r, wcnt, nullptr);
+        z_doc<NW>(a, m, r, wcnt, nullptr);
         if (lane == 0) {
             slots[idx].sweep = r.sweep;
             slots[idx].pos = r.pos;
@@ -1267,14 +940,34 @@ void launch_colptr_scan(const PhiArgs &a, cudaStream_t st) {
     k_scan_single<int32_t><<<1, 1024, 0, st>>>(a.nnz_c, a.V, a.col_ptr, &a.stats[ST_NNZPHI]);
 }
 
-void launch_phi_tables(const PhiArgs &a, cudaStream_t st) {
-    const int grid = static_cast<int>(std::min<int64_t>((static_cast<int64_t>(a.V) * 32 + 255) / 256, 16LL * sm_count()));
-    k_phi_tables<<<std::max(grid, 1), 256, 0, st>>>(a);
+// Warps per CTA and stage bytes per warp of the table pass: eight warps while
+// their stages stay within 96 KB, fewer for the longest rows.
+static int table_warps(int K) {
+    int w = 8;
+    while (w > 1 && w * dense_row_bytes(K) > 96 * 1024) w >>= 1;
+    return w;
 }
 
-void launch_phi_tables_multi(const PhiArgs *chains, const int2 *items, int n_items, cudaStream_t st) {
-    const int grid = static_cast<int>(std::min<int64_t>((static_cast<int64_t>(n_items) * 32 + 255) / 256, 16LL * sm_count()));
-    k_phi_tables_multi<<<std::max(grid, 1), 256, 0, st>>>(chains, items, n_items);
+static std::atomic<bool> g_tables_opted{false};
+static void opt_in_tables() {
+    if (g_tables_opted.load(std::memory_order_acquire)) return;
+    allow_dynamic_smem(k_phi_tables);
+    allow_dynamic_smem(k_phi_tables_multi);
+    g_tables_opted.store(true, std::memory_order_release);
+}
+
+void launch_phi_tables(const PhiArgs &a, cudaStream_t st) {
+    opt_in_tables();
+    const int w = table_warps(a.K), rb = dense_row_bytes(a.K);
+    const int grid = static_cast<int>(std::min<int64_t>((a.V + w - 1) / w, 128LL / w * sm_count()));
+    k_phi_tables<<<std::max(grid, 1), 32 * w, static_cast<size_t>(w) * rb, st>>>(a, rb);
+}
+
+void launch_phi_tables_multi(const PhiArgs *chains, const int2 *items, int n_items, int kmax, cudaStream_t st) {
+    opt_in_tables();
+    const int w = table_warps(kmax), rb = dense_row_bytes(kmax);
+    const int grid = static_cast<int>(std::min<int64_t>((n_items + w - 1) / w, 128LL / w * sm_count()));
+    k_phi_tables_multi<<<std::max(grid, 1), 32 * w, static_cast<size_t>(w) * rb, st>>>(chains, items, n_items, rb);
 }
 
 void launch_heavy_hist(const PhiArgs *chains, const HeavyChunk *chunks, int n_chunks, int kmax, cudaStream_t st) {
@@ -1285,22 +978,23 @@ void launch_heavy_hist(const PhiArgs *chains, const HeavyChunk *chunks, int n_ch
 }
 
 size_t z_step_smem(int K, int warps_per_block, bool narrow) {
-    return sizeof(uint32_t) * static_cast<size_t>(z_warp_words_n(K, narrow)) * warps_per_block;
+    return sizeof(uint32_t) * static_cast<size_t>(z_dense_warp_words(K, narrow)) * warps_per_block;
 }
 
 using ZStepKernel = void (*)(ZArgs);
-static ZStepKernel z_step_kernel(int K, bool narrow) {
-    switch (z_lane_topics(K)) {
-        case 8: return narrow ? k_z_step<8, uint16_t> : k_z_step<8, uint32_t>;
-        case 16: return narrow ? k_z_step<16, uint16_t> : k_z_step<16, uint32_t>;
-        case 32: return narrow ? k_z_step<32, uint16_t> : k_z_step<32, uint32_t>;
-        default: return narrow ? k_z_step<64, uint16_t> : k_z_step<64, uint32_t>;
+static ZStepKernel z_step_kernel(int K) {
+    switch (z_nw(K)) {
+        case 1: return k_z_step<1>;
+        case 2: return k_z_step<2>;
+        case 4: return k_z_step<4>;
+        case 8: return k_z_step<8>;
+        default: return k_z_step<0>;
     }
 }
 
 int z_step_blocks_per_sm(int K, int warps_per_block, bool narrow) {
     const size_t smem = z_step_smem(K, warps_per_block, narrow);
-    ZStepKernel kern = z_step_kernel(K, narrow);
+    ZStepKernel kern = z_step_kernel(K);
     allow_dynamic_smem(kern);
     int b = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kern, 32 * warps_per_block, smem);
@@ -1315,32 +1009,13 @@ void launch_slice_counts(const int64_t *doc_off, const int32_t *sliced_docs, int
 }
 
 void launch_z_step(const ZArgs &a, int warps_per_block, int grid, cudaStream_t st) {
-    ZStepKernel kern = z_step_kernel(a.K, a.narrow != 0);
-    // each instantiation opts in to large dynamic shared memory once
-    static std::atomic<bool> opted[4][2];
-    const int tpl = z_lane_topics(a.K);
-    std::atomic<bool> &o = opted[tpl == 8 ? 0 : tpl == 16 ? 1 : tpl == 32 ? 2 : 3][a.narrow != 0];
-    if (!o.load(std::memory_order_acquire)) {
-        allow_dynamic_smem(kern);
-        o.store(true, std::memory_order_release);
-    }
-    kern<<<grid, 32 * warps_per_block, z_step_smem(a.K, warps_per_block, a.narrow != 0), st>>>(a);
+    z_step_kernel(a.K)<<<grid, 32 * warps_per_block, z_step_smem(a.K, warps_per_block, a.narrow != 0), st>>>(a);
 }
 
-using ZMultiKernel = void (*)(const ZArgs *, const int2 *, int, int *, int);
-static ZMultiKernel z_multi_kernel(int kmax, bool narrow) {
-    switch (z_lane_topics(kmax)) {
-        case 8: return narrow ? k_z_step_multi<8, uint16_t> : k_z_step_multi<8, uint32_t>;
-        case 16: return narrow ? k_z_step_multi<16, uint16_t> : k_z_step_multi<16, uint32_t>;
-        case 32: return narrow ? k_z_step_multi<32, uint16_t> : k_z_step_multi<32, uint32_t>;
-        default: return narrow ? k_z_step_multi<64, uint16_t> : k_z_step_multi<64, uint32_t>;
-    }
-}
-
-static void launch_z_step_multi(const BatchLaunch &b, const int2 *items, int n, cudaStream_t st) {
-    ZMultiKernel kern = z_multi_kernel(b.kmax, b.narrow != 0);
-    kern<<<b.z_grid, 32 * b.z_warps, z_step_smem(b.kmax, b.z_warps, b.narrow != 0), st>>>(b.z, items, n, b.work + 1,
-                                                                                       b.kmax);
+static void launch_z_step_multi(const BatchLaunch &b, const int2 *items, int n, int *work, cudaStream_t st) {
+    if (n <= 0) return;
+    k_z_step_multi<<<b.z_grid, 32 * b.z_warps, z_step_smem(b.kmax, b.z_warps, b.narrow != 0), st>>>(
+        b.z, items, n, work, b.kmax, b.narrow);
 }
 
 void launch_batch_sweep(const BatchLaunch &b, cudaStream_t st) {
@@ -1350,18 +1025,19 @@ void launch_batch_sweep(const BatchLaunch &b, cudaStream_t st) {
                                                                                 b.work, b.kmax, true);
     k_phi_fixup_multi<<<b.n_chains, kFixBlock, 0, st>>>(b.phi);
     k_colptr_scan_multi<<<b.n_chains, 1024, 0, st>>>(b.phi);
-    launch_phi_tables_multi(b.phi, b.phi_items, b.n_phi_items, st);
+    launch_phi_tables_multi(b.phi, b.phi_items, b.n_phi_items, b.kmax, st);
     if (b.n_coop > 0) {
         // the longest documents on CTAs, the rest one per warp beside them
+        const int head = b.n_wide + b.n_coop;
         cudaEventRecord(b.ev_fork, st);
-        launch_z_step_coop_multi(b.z, b.z_items, b.n_coop, b.work + 2, b.kmax, b.coop_grid, st);
+        launch_z_step_multi(b, b.z_items, b.n_wide, b.work + 3, st);
+        launch_z_step_coop_multi(b.z, b.z_items + b.n_wide, b.n_coop, b.work + 2, b.kmax, b.coop_grid, st);
         cudaStreamWaitEvent(b.stream2, b.ev_fork, 0);
-        if (b.n_z_items > b.n_coop)
-            launch_z_step_multi(b, b.z_items + b.n_coop, b.n_z_items - b.n_coop, b.stream2);
+        launch_z_step_multi(b, b.z_items + head, b.n_z_items - head, b.work + 1, b.stream2);
         cudaEventRecord(b.ev_join, b.stream2);
         cudaStreamWaitEvent(st, b.ev_join, 0);
     } else {
-        launch_z_step_multi(b, b.z_items, b.n_z_items, st);
+        launch_z_step_multi(b, b.z_items, b.n_z_items, b.work + 1, st);
     }
 }
 
@@ -1422,9 +1098,8 @@ __global__ void k_barrier_selftest(GridBarrier *bar, unsigned expect, int rounds
     }
 }
 
-template <int TPL, typename CT>
 __global__ void __launch_bounds__(kPersistThreads, PULDA_PERSIST_MINB) k_batch_sweep_persistent(BatchLaunch b) {
-    extern __shared__ uint32_t psm[];
+    extern __shared__ __align__(16) uint32_t psm[];
     __shared__ int scan_tmp[kPersistThreads / 32 + 1];
     __shared__ int s_item;
     __shared__ uint32_t geo[kGeoLen];
@@ -1467,19 +1142,21 @@ __global__ void __launch_bounds__(kPersistThreads, PULDA_PERSIST_MINB) k_batch_s
     {
         const int wid = static_cast<int>(blockIdx.x) * kPersistWarps + (threadIdx.x >> 5);
         const int nw = static_cast<int>(nb) * kPersistWarps;
+        uint8_t *stage = table_stage(psm, b.table_stage);
         for (int i = wid; i < b.n_phi_items; i += nw) {
             const int2 it = b.phi_items[i];
-            phi_tables_word_warp(b.phi[it.x], it.y);
+            phi_tables_word_warp(b.phi[it.x], it.y, stage);
         }
     }
     if (!grid_barrier(b.bar, nb, err)) return;
     // z-step, one warp per (chain, document), longest first
     {
         const int lane = threadIdx.x & 31;
-        uint32_t *m = psm + static_cast<size_t>(threadIdx.x >> 5) * z_warp_words_t<CT>(b.kmax);
-        u64 *wcnt = z_warp_counters_t<CT>(m, b.kmax);
-        zero_warp_counters(wcnt);
-        for (;;) {
+        uint32_t *m = psm + static_cast<size_t>(threadIdx.x >> 5) * z_dense_warp_words(b.kmax, b.narrow != 0);
+        u64 *wcnt = z_dense_counters(m, b.kmax, b.narrow != 0);
+        const bool in = static_cast<int>(threadIdx.x >> 5) < b.persist_z_warps;
+        if (in) zero_warp_counters(wcnt);
+        while (in) {
             int item = 0;
             if (lane == 0) item = atomicAdd(&b.work[1], 1);
             item = __shfl_sync(0xFFFFFFFFu, item, 0);
@@ -1487,9 +1164,7 @@ __global__ void __launch_bounds__(kPersistThreads, PULDA_PERSIST_MINB) k_batch_s
             const int2 it = b.z_items[item];
             const ZArgs &a = b.z[it.x];
             const int64_t s0 = a.doc_off[it.y];
-            DocRun r{a.w + s0, a.z + s0, static_cast<int>(a.doc_off[it.y + 1] - s0), a.seed, a.index_base + s0,
-                     sweep_of(a), 0, a.doc_off[it.y + 1] - s0, 1};
-            z_doc_warp_t<TPL, CT>(a, m, r, wcnt, nullptr);
+            z_doc_any(&a, m, s0, static_cast<int>(a.doc_off[it.y + 1] - s0), sweep_of(a), wcnt);
             flush_warp_counters(a.stats, wcnt);
         }
     }
@@ -1510,26 +1185,22 @@ cudaError_t launch_barrier_selftest(GridBarrier *bar, int blocks, int missing, i
                               passed);
 }
 
-size_t batch_persistent_smem(int kmax, bool narrow) {
+// The z-step phase runs on all of a CTA's warps, or on one fewer where eight
+// warps' counts just do not fit.
+static size_t batch_persistent_smem(int kmax, int z_warps, bool narrow) {
     return std::max({phi_counts_smem(kmax), sizeof(uint32_t) * static_cast<size_t>(kmax),
-                     z_step_smem(kmax, kPersistWarps, narrow)});
+                     z_step_smem(kmax, z_warps, narrow)});
 }
 
-using PersistKernel = void (*)(BatchLaunch);
-static PersistKernel persistent_kernel(int kmax, bool narrow) {
-    switch (z_lane_topics(kmax)) {
-        case 8: return narrow ? k_batch_sweep_persistent<8, uint16_t> : k_batch_sweep_persistent<8, uint32_t>;
-        case 16: return narrow ? k_batch_sweep_persistent<16, uint16_t> : k_batch_sweep_persistent<16, uint32_t>;
-        case 32: return narrow ? k_batch_sweep_persistent<32, uint16_t> : k_batch_sweep_persistent<32, uint32_t>;
-        default: return narrow ? k_batch_sweep_persistent<64, uint16_t> : k_batch_sweep_persistent<64, uint32_t>;
-    }
-}
-
-int batch_persistent_blocks_per_sm(int kmax, bool narrow) {
-    PersistKernel kern = persistent_kernel(kmax, narrow);
-    allow_dynamic_smem(kern);
+int batch_persistent_blocks_per_sm(int kmax, bool narrow, int *z_warps, int *table_stage) {
+    allow_dynamic_smem(k_batch_sweep_persistent);
     int n = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, kPersistThreads, batch_persistent_smem(kmax, narrow));
+    for (int w = kPersistWarps; w >= kPersistWarps - 1 && n <= 0; --w) {
+        const size_t smem = batch_persistent_smem(kmax, w, narrow);
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_batch_sweep_persistent, kPersistThreads, smem) != cudaSuccess) n = 0;
+        *z_warps = w;
+        *table_stage = static_cast<size_t>(kPersistWarps) * dense_row_bytes(kmax) <= smem ? dense_row_bytes(kmax) : 0;
+    }
     return n;
 }
 
@@ -1537,14 +1208,14 @@ cudaError_t launch_batch_sweep_persistent(const BatchLaunch &b, cudaStream_t st)
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(b.persist_grid));
     cfg.blockDim = dim3(kPersistThreads);
-    cfg.dynamicSmemBytes = batch_persistent_smem(b.kmax, b.narrow != 0);
+    cfg.dynamicSmemBytes = batch_persistent_smem(b.kmax, b.persist_z_warps, b.narrow != 0);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, persistent_kernel(b.kmax, b.narrow != 0), b);
+    return cudaLaunchKernelEx(&cfg, k_batch_sweep_persistent, b);
 }
 
 int batch_phi_blocks_per_sm(int kmax) {
@@ -1555,21 +1226,21 @@ int batch_phi_blocks_per_sm(int kmax) {
 }
 
 int batch_z_blocks_per_sm(int kmax, int warps, bool narrow) {
-    ZMultiKernel kern = z_multi_kernel(kmax, narrow);
-    allow_dynamic_smem(kern);
+    allow_dynamic_smem(k_z_step_multi);
     int n = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, 32 * warps, z_step_smem(kmax, warps, narrow));
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_z_step_multi, 32 * warps, z_step_smem(kmax, warps, narrow));
     return n > 0 ? n : 1;
 }
 
 using ServeKernel = void (*)(ZArgs, ServeSlot *, const int32_t *, int, const int32_t *, int16_t *, int64_t, int *,
                             uint64_t);
-static ServeKernel serve_kernel(int K, bool narrow) {
-    switch (z_lane_topics(K)) {
-        case 8: return narrow ? k_serve_step<8, uint16_t> : k_serve_step<8, uint32_t>;
-        case 16: return narrow ? k_serve_step<16, uint16_t> : k_serve_step<16, uint32_t>;
-        case 32: return narrow ? k_serve_step<32, uint16_t> : k_serve_step<32, uint32_t>;
-        default: return narrow ? k_serve_step<64, uint16_t> : k_serve_step<64, uint32_t>;
+static ServeKernel serve_kernel(int K) {
+    switch (z_nw(K)) {
+        case 1: return k_serve_step<1>;
+        case 2: return k_serve_step<2>;
+        case 4: return k_serve_step<4>;
+        case 8: return k_serve_step<8>;
+        default: return k_serve_step<0>;
     }
 }
 
@@ -1579,15 +1250,16 @@ void launch_serve_step(const ZArgs &a, ServeSlot *slots, const int32_t *active, 
     if (n_active <= 0) return;
     cudaMemsetAsync(work, 0, sizeof(int), st);
     const int need = (n_active + warps_per_block - 1) / warps_per_block;
-    ServeKernel kern = serve_kernel(a.K, narrow);
-    kern<<<std::min(grid, need), 32 * warps_per_block, z_step_smem(a.K, warps_per_block, narrow), st>>>(
-        a, slots, active, n_active, arena_w, arena_z, slice, work, window_ns);
+    ZArgs an = a;
+    an.narrow = narrow ? 1 : 0;
+    serve_kernel(a.K)<<<std::min(grid, need), 32 * warps_per_block, z_step_smem(a.K, warps_per_block, narrow), st>>>(
+        an, slots, active, n_active, arena_w, arena_z, slice, work, window_ns);
 }
 
 int serve_blocks_per_sm(int K, int warps_per_block) {
-    // the 32-bit instantiation: its shared memory bounds the 16-bit one's
-    for (bool narrow : {true, false}) allow_dynamic_smem(serve_kernel(K, narrow));
-    ServeKernel kern = serve_kernel(K, false);
+    // three count planes: their shared memory bounds the launches with two
+    ServeKernel kern = serve_kernel(K);
+    allow_dynamic_smem(kern);
     int n = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, 32 * warps_per_block, z_step_smem(K, warps_per_block));
     return n > 0 ? n : 1;

@@ -19,6 +19,7 @@
 #include <mutex>
 
 #include "../../include/pulda.h"
+#include "handle.h"
 #include "pulda_internal.h"
 
 namespace pulda {
@@ -29,12 +30,14 @@ constexpr int64_t kNoAllocMaxDocs = 65536;
 
 // Layout of the scratch array (bytes, each part 256-byte aligned).
 constexpr size_t kOffStats = 0;                                       // u64[ST_TOTAL_SLOTS]
-constexpr size_t kOffWork = 256;                                      // int[4]: z-step work counter
+constexpr size_t kOffWork = 256;                                      // int[5]: z-step work counters
+constexpr size_t kOffCount = 320;                                     // int[4]: documents by length class
 constexpr size_t kOffFlag = 512;                                      // u64[2]: first bad token, first bad document
 constexpr size_t kOffOrder = 768;                                     // int32[kNoAllocMaxDocs]
 constexpr size_t kScratchBytes = kOffOrder + sizeof(int32_t) * kNoAllocMaxDocs;   // 262,912 bytes
 static_assert(ST_TOTAL_SLOTS * sizeof(unsigned long long) <= kOffWork, "the counters overlap the work counter");
-static_assert(4 * sizeof(int) <= kOffFlag - kOffWork, "the work counters overlap the input check");
+static_assert(5 * sizeof(int) <= kOffCount - kOffWork, "the work counters overlap the class counts");
+static_assert(4 * sizeof(int) <= kOffFlag - kOffCount, "the class counts overlap the input check");
 static_assert(2 * sizeof(unsigned long long) <= kOffOrder - kOffFlag, "the input check overlaps the schedule");
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
@@ -62,22 +65,36 @@ cudaError_t scratch_on_device(int dev, unsigned char **out) {
     return cudaSuccess;
 }
 
+// A document's class: 0 with 2^16 tokens or more (one warp), 1 at least coop_len
+// (a CTA each), 2 the rest.
+__device__ __forceinline__ int length_class(int64_t len, int64_t coop_len) {
+    return len > kNarrowMaxLen ? 0 : len >= coop_len ? 1 : 2;
+}
+
 // Checks the caller's device inputs (ids in [0, V), offsets nondecreasing from
-// 0 to N) and writes the identity document schedule.  first[0] becomes the
+// 0 to N) and counts the documents of each length class.  first[0] becomes the
 // smallest position of a word id outside [0, V), first[1] the smallest
 // document with bad offsets; both start at ~0 (none).
 __global__ void k_noalloc_check(const int32_t *w, int64_t N, const int64_t *off, int64_t D, int V,
-                                unsigned long long *first, int32_t *order) {
+                                unsigned long long *first, int *count, int64_t coop_len) {
     const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
     const int64_t t0 = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
     for (int64_t i = t0; i < N; i += stride)
         if (w[i] < 0 || w[i] >= V) atomicMin(&first[0], static_cast<unsigned long long>(i));
     for (int64_t d = t0; d < D; d += stride) {
-        order[d] = static_cast<int32_t>(d);
         const int64_t a = off[d], b = off[d + 1];
         if (a < 0 || b < a || b > N || (d == 0 && a != 0) || (d == D - 1 && b != N) || b - a > (int64_t(1) << 22))
             atomicMin(&first[1], static_cast<unsigned long long>(d));
+        atomicAdd(&count[length_class(b - a, coop_len)], 1);
     }
+}
+
+// The document schedule, class by class (within a class in any order: the
+// results do not depend on it).  cursor: where each class starts.
+__global__ void k_noalloc_order(const int64_t *off, int64_t D, int64_t coop_len, int *cursor, int32_t *order) {
+    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+    for (int64_t d = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; d < D; d += stride)
+        order[atomicAdd(&cursor[length_class(off[d + 1] - off[d], coop_len)], 1)] = static_cast<int32_t>(d);
 }
 
 }  // namespace
@@ -118,14 +135,18 @@ extern "C" pulda_status pulda_infer_noalloc(pulda_handle *h, const int32_t *word
     auto *work = reinterpret_cast<int *>(scratch + kOffWork);
     auto *first = reinterpret_cast<unsigned long long *>(scratch + kOffFlag);
     auto *order = reinterpret_cast<int32_t *>(scratch + kOffOrder);
+    auto *count = reinterpret_cast<int *>(scratch + kOffCount);
+    const int64_t coop_len = long_document_tokens(h, N_new);
     // the array keeps the previous call's contents: clear what counts from
     // zero, and set the input check's "first bad index" slots to ~0 (none)
     e = cudaMemsetAsync(scratch, 0, kOffFlag, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(first, 0xFF, 2 * sizeof(unsigned long long), st);
     if (e == cudaSuccess) {
-        k_noalloc_check<<<64, 256, 0, st>>>(word_ids_dev, N_new, doc_offsets_dev, D_new, hv.V, first, order);
+        k_noalloc_check<<<64, 256, 0, st>>>(word_ids_dev, N_new, doc_offsets_dev, D_new, hv.V, first, count, coop_len);
         e = cudaGetLastError();
     }
+    int hcount[3] = {0, 0, 0};
+    if (e == cudaSuccess) e = cudaMemcpyAsync(hcount, count, sizeof hcount, cudaMemcpyDeviceToHost, st);
     unsigned long long hfirst[2] = {~0ull, ~0ull};
     if (e == cudaSuccess) e = cudaMemcpyAsync(hfirst, first, sizeof hfirst, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -141,6 +162,12 @@ extern "C" pulda_status pulda_infer_noalloc(pulda_handle *h, const int32_t *word
         snprintf(msg, sizeof msg, "the word id at token %llu is outside [0, %d)", hfirst[0], hv.V);
         return static_cast<pulda_status>(handle_fail(h, PULDA_ERR_INVALID, msg));
     }
+    const int cursor[3] = {0, hcount[0], hcount[0] + hcount[1]};
+    e = cudaMemcpyAsync(count, cursor, sizeof cursor, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) {
+        k_noalloc_order<<<64, 256, 0, st>>>(doc_offsets_dev, D_new, coop_len, count, order);
+        e = cudaGetLastError();
+    }
     launch_init_z(N_new, hv.K, seed, 0, z_out_dev, st);
     ZArgs a = hv.zargs;
     a.doc_off = doc_offsets_dev;
@@ -150,15 +177,10 @@ extern "C" pulda_status pulda_infer_noalloc(pulda_handle *h, const int32_t *word
     a.z = z_out_dev;
     a.seed = seed;
     a.index_base = 0;
-    a.work = work;
     a.stats = stats;
     for (int32_t sw = 1; sw <= n_sweeps && e == cudaSuccess; ++sw) {
-        e = cudaMemsetAsync(work, 0, sizeof(int), st);
         a.sweep = static_cast<uint32_t>(sw);
-        if (e == cudaSuccess) {
-            launch_z_step(a, hv.z_warps, hv.z_grid, st);
-            e = cudaGetLastError();
-        }
+        e = run_z(h, a, hcount[0], hcount[1], work);
     }
     unsigned long long err = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&err, stats + ST_ERROR, sizeof err, cudaMemcpyDeviceToHost, st);

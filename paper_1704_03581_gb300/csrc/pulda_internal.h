@@ -21,9 +21,7 @@ constexpr int kFracBits = 16;
 constexpr uint32_t kMaxRedraw = 1u << 20;
 // Largest K the kernels' shared-memory layouts accept.
 constexpr int kMaxK = 16384;
-// The bitmap intersection path of the z-step: the one-warp kernel's lane
-// holds up to two 32-topic words (64 topics), the cooperative kernel's slot
-// part of one.
+// Bitmap rows are laid out for the grouped z-step's lanes up to here.
 constexpr int kMaxKBitmap = 2048;
 // Four documents per warp: each of a document's 8 lanes holds up to four
 // words.
@@ -31,10 +29,28 @@ constexpr int kMaxKGrouped = 1024;
 // Words of a word's bitmap row: ceil(K / 32) rounded up to 8 times a power
 // of two, so each of the grouped z-step's 8 lanes per document reads 1, 2 or
 // 4 consecutive words with one aligned load (the words past ceil(K / 32) are
-// zero); 64 above 1024 topics.
+// zero); 64 above 1024 topics, and above 2048 what the dense rows cover (16
+// words for every 512 topics).
 __host__ __device__ inline int bitmap_row_words(int K) {
     const int per_lane = (((K + 31) / 32) + 7) / 8;
+    if (per_lane > 8) return 16 * ((K + 511) / 512);
     return 8 * (per_lane <= 1 ? 1 : per_lane <= 2 ? 2 : per_lane <= 4 ? 4 : 8);
+}
+// Dense rows of the z-step (zdense.cuh): a word's weights q as three planes of
+// bytes, and a document's counts as planes of bytes in the same order.  Lane l
+// of a warp owns the 4 NW consecutive topics [4 NW l, 4 NW l + 4 NW); a plane
+// is 128 NW bytes.  Up to 512 topics a lane's bytes are consecutive; above,
+// they lie in chunks of 16 bytes, chunk c of all lanes before chunk c + 1, so
+// that a warp's 16-byte loads are consecutive and free of bank conflicts.
+__host__ __device__ inline int dense_words(int K) {
+    return K <= 128 ? 1 : K <= 256 ? 2 : K <= 512 ? 4 : 4 * ((K + 511) / 512);
+}
+__host__ __device__ inline int dense_row_bytes(int K) { return 3 * 128 * dense_words(K); }
+__host__ __device__ inline int dense_pos(int K, int k) {
+    if (K <= 512) return k;
+    const int tpl = 4 * dense_words(K);
+    const int l = k / tpl, b = k - l * tpl;
+    return ((b >> 4) << 9) + (l << 4) + (b & 15);
 }
 // Warps per CTA of the warp-per-document z-step: the default and the largest
 // accepted (the kernel's launch bounds are sized for it).
@@ -52,10 +68,9 @@ constexpr int kZWarps = PULDA_ZWARPS;
 #define PULDA_MULTI_MINB 3
 #endif
 constexpr int kMultiWarps = PULDA_MULTI_WARPS;
-// Words with tokens, most frequent first, also keep their fixed-point
-// weights q as dense K-entry rows, up to this many bytes (K <= kMaxKBitmap):
-// the z-step's document side reads q at topic k there.  A word without a row
-// is always iterated on its column side (the same sums).
+// Words also keep their fixed-point weights q as dense rows, most frequent
+// words first, up to this many bytes.  A word without a row is summed over its
+// column (the same sums).
 #ifndef PULDA_DENSE_BYTES
 #define PULDA_DENSE_BYTES (2048ll << 20)
 #endif
@@ -127,10 +142,12 @@ struct PhiArgs {
     unsigned long long *A;      // [V]
     unsigned long long *vose_p; // [cap] scratch
     uint16_t *vose_stack;       // [cap] scratch
-    uint32_t *bits;             // [V * KWp] nonzero-topic bits of each word's column, or null
+    uint32_t *bits;             // [V * KWp] nonzero-topic bits of each word's column
     int KW, KWp;
-    uint32_t *qdense;           // [n_dense * K] q by topic (0 off the column) or null
-    const int32_t *dense_slot;  // [V] row of the word in qdense, or -1
+    uint8_t *qrow;              // dense rows of byte planes, dense_row_bytes(K) each
+    const int32_t *row_slot;    // [V] the word's row in qrow, or -1
+    int32_t *drow;              // [V] the same as the current Phi has it: -1 too where a q is 2^24 (25 bits)
+    uint32_t *qdense;           // [V * K] q by topic (0 off the column): four documents per warp only, else null
     const float *alpha;         // [K]
     int *work;                  // dynamic word counter
     unsigned long long *stats;  // [ST_COUNT]
@@ -158,7 +175,7 @@ struct HeavyChunk {
     int64_t begin, end;
 };
 void launch_heavy_hist(const PhiArgs *chains, const HeavyChunk *chunks, int n_chunks, int kmax, cudaStream_t st);
-void launch_phi_tables_multi(const PhiArgs *chains, const int2 *items, int n_items, cudaStream_t st);
+void launch_phi_tables_multi(const PhiArgs *chains, const int2 *items, int n_items, int kmax, cudaStream_t st);
 
 struct ZArgs {
     const int64_t *doc_off;     // [D+1]
@@ -173,9 +190,10 @@ struct ZArgs {
     const uint32_t *athr;
     const uint16_t *atopic;
     const uint2 *apack;         // packed alias slots (PhiArgs::apack) or null: read athr / topic / atopic
-    const uint32_t *bits;       // [V * KWp] nonzero-topic bits of each word's column; null when K > kMaxKBitmap
-    const uint32_t *qdense;     // dense q rows of the most frequent words, or null
-    const int32_t *dense_slot;  // [V] row in qdense or -1
+    const uint32_t *bits;       // [V * KWp] nonzero-topic bits of each word's column
+    const uint8_t *qrow;        // dense rows (PhiArgs::qrow) and each word's, or -1
+    const int32_t *drow;
+    const uint32_t *qdense;     // [V * K] q by topic: four documents per warp only
     // stale-count slices of long documents (k_z_step only): {row in m0, the
     // document, first token, tokens} is {y, x, z, w}; taken before the D documents
     const int4 *slices;
@@ -187,7 +205,7 @@ struct ZArgs {
     const uint32_t *sweep_ptr;  // if set, the sweep counter is read here (graph replay)
     int64_t index_base;         // RNG index of token 0
     int path;                   // 0 auto, 1 column, 2 document topics
-    int narrow;                 // 1: every document of the launch has fewer than 2^16 tokens (16-bit counts)
+    int narrow;                 // 1: every document of the launch has fewer than 2^16 tokens (two count planes, else three)
     int *work;
     unsigned long long *stats;
 };
@@ -201,15 +219,18 @@ void launch_phi_fixup(const PhiArgs &a, cudaStream_t st);
 void launch_colptr_scan(const PhiArgs &a, cudaStream_t st);
 void launch_phi_tables(const PhiArgs &a, cudaStream_t st);
 void launch_z_step(const ZArgs &a, int warps_per_block, int grid, cudaStream_t st);
-// The longest documents, doc_order[0 .. n_coop), one CTA of four warps each;
-// `work` is a counter zeroed before the launch.
+// The documents doc_order[0 .. n_coop), of at most kNarrowMaxLen tokens, one
+// CTA each (zchain.cuh); `work` is a counter zeroed before the launch.
 void launch_z_step_coop(const ZArgs &a, int n_coop, int *work, int grid, cudaStream_t st);
 int z_coop_blocks_per_sm(int K);
-// Automatic threshold of the cooperative z-step: a document on one warp that
-// shares its SM with the rest of the pass takes about 3.3 us per token while
-// the pass streams ~2.4 G tokens/s, so one longer than N / 8000 tokens would
-// outlast the pass.
-constexpr int64_t kCoopAutoDiv = 8000;
+// Automatic threshold of the long-document z-step: a document on one warp
+// among 27 others on its SM takes about 1 us per token while the pass streams
+// a token in 0.32 ns (K = 1000), so one longer than N / 3100 tokens would
+// outlast the pass; the line lies a little below.  z-step ms at K = 1000,
+// threshold 1,000 / 1,500 / 2,500 / none: N = 12.4M 4.93 / 4.62 / 4.18 / 7.14,
+// N = 9.9M 4.04 / 3.85 / 3.48 / 6.02; K = 3000, N = 6.5M, threshold 500 /
+// 1,000 / 2,000 / none: 8.88 / 6.90 / 7.27 / 16.1.
+constexpr int64_t kCoopAutoDiv = 4500;
 constexpr int64_t kCoopAutoMin = 256;
 // The same beside the grouped z-step, whose pass is faster and whose
 // documents each advance more slowly (four share a warp's issue slots).
@@ -220,6 +241,8 @@ constexpr int64_t kCoopAutoDivGrouped = PULDA_COOP_DIV_GROUPED;
 // Pass-start topic counts of the documents that the z-step takes in slices.
 void launch_slice_counts(const int64_t *doc_off, const int32_t *sliced_docs, int n, const int16_t *z, int K,
                          uint32_t *m0, cudaStream_t st);
+// Largest dynamic shared memory a CTA may opt in to (device attribute).
+int smem_optin();
 size_t z_step_smem(int K, int warps_per_block, bool narrow = false);
 size_t phi_counts_smem(int K);
 void launch_doc_topic(const int64_t *doc_off, int64_t D, const int16_t *z, int K, int32_t *m_dk, cudaStream_t st);
@@ -285,21 +308,24 @@ struct BatchLaunch {
     int kmax;                    // largest K of the chains
     int narrow;                  // 1: every document of every chain has fewer than 2^16 tokens
     int phi_grid, z_grid, z_warps;
-    // the first n_coop z_items go to the cooperative z-step on `st`, the rest
-    // to the one-warp kernel on stream2 (forked and joined with the events)
-    int n_coop, coop_grid;
+    // the n_coop z_items after the first n_wide (2^16 tokens or more) go to the
+    // long-document z-step on `st`, the others to the one-warp kernel, the
+    // shorter ones on stream2 (forked and joined with the events)
+    int n_wide, n_coop, coop_grid;
     cudaStream_t stream2;
     cudaEvent_t ev_fork, ev_join;
     // the one-launch form: its grid (all CTAs resident) and barrier
     int persist_grid;
     GridBarrier *bar;
+    int persist_z_warps;         // warps of a CTA in its z-step phase
+    int table_stage;             // bytes of a warp's stage in its table phase (0: rows are written in place)
 };
 void launch_batch_sweep(const BatchLaunch &b, cudaStream_t st);
 // The same sweep as one cooperative launch (no cooperative z-step: every
 // document one per warp); needs persist_grid <= SMs x
 // batch_persistent_blocks_per_sm(kmax).
 cudaError_t launch_batch_sweep_persistent(const BatchLaunch &b, cudaStream_t st);
-int batch_persistent_blocks_per_sm(int kmax, bool narrow);
+int batch_persistent_blocks_per_sm(int kmax, bool narrow, int *z_warps, int *table_stage);
 // The grid barrier's self-test: `blocks` resident CTAs pass `rounds`
 // barriers that expect blocks + missing arrivals.
 cudaError_t launch_barrier_selftest(GridBarrier *bar, int blocks, int missing, int rounds, unsigned long long *err,
@@ -307,7 +333,6 @@ cudaError_t launch_barrier_selftest(GridBarrier *bar, int blocks, int missing, i
 int batch_phi_blocks_per_sm(int kmax);
 int batch_z_blocks_per_sm(int kmax, int warps, bool narrow);
 int batch_coop_blocks_per_sm(int kmax);
-size_t z_coop_multi_smem(int kmax);
 // The cooperative z-step over (chain, document) items (coop.cu).
 void launch_z_step_coop_multi(const ZArgs *chains, const int2 *items, int n_items, int *work, int kmax, int grid,
                               cudaStream_t st);
@@ -334,8 +359,8 @@ void launch_serve_step_coop(const ZArgs &a, ServeSlot *slots, const int32_t *act
                             const int32_t *arena_w, int16_t *arena_z, int64_t slice, int *work, int grid,
                             uint64_t window_ns, cudaStream_t st);
 int serve_coop_blocks_per_sm(int K);
-// Requests at least this long are served by the cooperative kernel when the
-// handle's coop_min_len is 0 (automatic).
+// With the handle's coop_min_len 0 (automatic), requests at least this long
+// are served on CTAs, and all of them while a CTA is free for each.
 constexpr int64_t kServeCoopAuto = 1024;
 
 // What another translation unit needs to launch the z-step on a handle's

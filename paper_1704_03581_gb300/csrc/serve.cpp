@@ -77,11 +77,6 @@ private:
 };
 
 constexpr size_t kMaxPending = size_t(1) << 22;
-#ifndef PULDA_SERVE_COOP_GATE
-#define PULDA_SERVE_COOP_GATE 8
-#endif
-constexpr int64_t kServeCoopGate = PULDA_SERVE_COOP_GATE;   // cooperative while n_active * this <= resident warps
-
 }  // namespace
 
 struct pulda_server {
@@ -90,7 +85,8 @@ struct pulda_server {
     cudaStream_t stream = nullptr, stream2 = nullptr;   // the cooperative launch, the one-warp launch
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     int64_t budget = 0, slice = 0;
-    int64_t coop_len = 0;                 // requests at least this long go to the cooperative kernel (0 = none)
+    int64_t coop_len = 0;                 // requests at least this long go to CTAs (0 = none)
+    bool coop_auto = false;               // every request while a CTA is free for each
     uint64_t window_ns = 0;               // automatic slice: the launch's time window
     int32_t max_slots = 0;
     int z_warps = 8, grid = 1, coop_grid = 1;
@@ -188,20 +184,18 @@ void worker_loop(pulda_server *s) {
         for (int32_t slot : newly) s->active.push_back(slot);
         newly.clear();
         const int n = static_cast<int>(s->active.size());
-        // long requests first (the cooperative kernel's), then the others.  A
-        // cooperative token costs about four times the issue slots of a
-        // one-warp token, which pays while the SMs have idle issue slots: only
-        // while the active requests fill at most an eighth of the resident warps
-        // (measured: at a quarter, 20k requests/s doubled p50).
-        const bool coop = s->coop_len > 0 &&
-                          static_cast<int64_t>(n) * kServeCoopGate <= static_cast<int64_t>(s->grid) * s->z_warps;
+        // requests on CTAs first (the long ones, and all while a CTA is free
+        // for each: there a token takes a third of the time), then the others
+        const bool coop = s->coop_len > 0;
+        const int64_t coop_len = s->coop_auto && n <= s->coop_grid ? 1 : s->coop_len;
         int nc = 0;
+        auto on_cta = [&](int32_t slot) { return coop && s->h_slots_len[slot] >= coop_len && s->h_slots_len[slot] <= kNarrowMaxLen; };
         for (int32_t slot : s->active)
-            if (coop && s->h_slots_len[slot] >= s->coop_len) s->h_active[nc++] = slot;
+            if (on_cta(slot)) s->h_active[nc++] = slot;
         int j = nc;
         bool narrow = true;     // every request on the one-warp kernel fits 16-bit counts
         for (int32_t slot : s->active)
-            if (!(coop && s->h_slots_len[slot] >= s->coop_len)) {
+            if (!on_cta(slot)) {
                 s->h_active[j++] = slot;
                 narrow = narrow && s->h_slots_len[slot] <= kNarrowMaxLen;
             }
@@ -305,6 +299,7 @@ pulda_status pulda_serve_open(pulda_handle *h, int64_t token_budget, int32_t max
     // short enough that new requests start soon), however far each request gets
     s->slice = slice_tokens == 0 ? (int64_t(1) << 22) : slice_tokens;
     s->window_ns = slice_tokens == 0 ? 2000000ull : 0ull;
+    s->coop_auto = h->opt.coop_min_len == 0;
     s->coop_len = h->opt.coop_min_len < 0 ? 0 : (h->opt.coop_min_len > 0 ? h->opt.coop_min_len : kServeCoopAuto);
     s->max_slots = max_slots;
     s->h_slots_len.assign(max_slots, 0);

@@ -1,0 +1,621 @@
+// The z-step of one long document by a CTA of three warps, for the least time
+// per token.
+//
+// A document's tokens are strictly sequential, so a long document is one
+// chain of draws, and what bounds it is the instructions and latencies from
+// one token's topic to the next's.  Warp 0 carries that chain and nothing
+// else:
+//   - warp 1 stages the tokens' records two to three blocks of 32 ahead, and
+//     has the words' dense rows copied into a ring of shared-memory slots
+//     (bulk copies, one group of tokens ahead), so no load on the chain goes
+//     past shared memory;
+//   - warp 2 replays the drawn topics one group behind, on counts of its own,
+//     for the sweep's counters, and writes them out.
+// On the chain itself, the sum q m of token t + 1 is taken while token t is
+// drawn, from the counts without token t; the token's own weight is taken off
+// beforehand, and the one thing missing, the weight of token t's new topic, is
+// added to the scanned prefixes afterwards.  All sums are exact integers, so
+// they are those of the sequential order.  The topic within the found lane
+// comes from masked dp4a, every lane summing the lane's topics up to its own
+// (no scan), and the steps of token t + 1's scan stand between the votes,
+// shuffles and loads of token t's draw: they issue in program order, and each
+// would otherwise be waited for by itself.
+// The warps meet once per group.
+#pragma once
+#include <cstdint>
+
+#include <cuda_runtime.h>
+
+#include "zdense.cuh"
+
+namespace pulda {
+
+constexpr int kChainThreads = 96;
+
+// Tokens of a group: the ring holds three groups' rows (drawn, landed, on
+// their way), within what leaves room for several CTAs per SM where rows are
+// short.
+__host__ __device__ __forceinline__ int chain_group(int K) {
+    const int rb = dense_row_bytes(K);
+    return rb <= 1536 ? 8 : rb <= 3072 ? 4 : rb <= 24576 ? 2 : 1;
+}
+
+// One token's record: {sigma_a, u}, {position of its topic | of the alias
+// outcome << 16, its row's offset in shared memory or ~0, K_v, word}, {its
+// column's start}.
+constexpr int kChainRecWords = 12;
+
+// Shared memory of a CTA, in bytes: the barriers and counters; the drawn
+// topics of two groups; three blocks of records; two sets of counts (two
+// planes each) and, above 1024 topics, the lanes' bits; the ring.
+struct ChainCtl {
+    u64 full[3];                // a group's rows have arrived
+    u64 cnt[6];                 // the counters
+    u64 deadline;
+    int item, stop;
+    int stops[2];               // after an even / odd group: a fast warp may already set the next one
+    uint32_t drawn[16];         // two groups: position | flags
+};
+constexpr int kChainRecOff = 256;
+static_assert(sizeof(ChainCtl) <= kChainRecOff, "the control block must fit");
+constexpr int kChainCountOff = kChainRecOff + 3 * 32 * 4 * kChainRecWords;
+static_assert(kChainCountOff % 16 == 0, "counts and rows are read 16 bytes at a time");
+__host__ __device__ __forceinline__ int chain_ring_off(int K) {
+    return kChainCountOff + 4 * 128 * dense_words(K) + (K > 1024 ? 16 * dense_words(K) : 0);
+}
+__host__ __device__ __forceinline__ int chain_smem_bytes(int K) { return chain_ring_off(K) + 3 * chain_group(K) * dense_row_bytes(K); }
+// The same for chains of any K up to kmax in one launch (shorter groups can
+// take less room than the longer ones below them).
+__host__ __device__ __forceinline__ int chain_smem_bytes_upto(int kmax) {
+    int most = 0;
+    const int edge[4] = {512, 1024, 8192, 16384};
+    for (int e : edge) {
+        const int b = chain_smem_bytes(kmax < e ? kmax : e);
+        most = b > most ? b : most;
+    }
+    return most;
+}
+// Flags of a drawn topic: taken from the alias table, kept for want of mass.
+constexpr uint32_t kDrawnAlias = 1u << 14, kDrawnZero = 1u << 15;
+static_assert(kMaxK <= (1 << 14), "positions must leave room for the flags");
+
+__device__ __forceinline__ uint32_t smem_addr(const void *p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
+__device__ __forceinline__ void bar_init(u64 *bar) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bar)) : "memory");
+}
+__device__ __forceinline__ bool bar_try_wait(u64 *bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+                 : "=r"(ok) : "r"(smem_addr(bar)), "r"(parity) : "memory");
+    return ok != 0;
+}
+// Waits for a slot, at most some seconds: false then.
+__device__ __forceinline__ bool bar_wait(u64 *bar, uint32_t parity) {
+    for (int i = 0; i < (1 << 22); ++i)
+        if (bar_try_wait(bar, parity)) return true;
+    return false;
+}
+__device__ __forceinline__ void bulk_copy(void *dst, const void *src, uint32_t bytes, u64 *bar) {
+    asm volatile("cp.async.bulk.shared::cta.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_addr(dst)),
+                 "l"(src), "r"(bytes), "r"(smem_addr(bar)) : "memory");
+}
+__device__ __forceinline__ void bar_expect(u64 *bar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
+}
+
+// Counts of the chain: one plane, or two (P = 2), with no test in between.
+template <int P>
+__device__ __forceinline__ uint32_t chain_count(const uint8_t *m, int PB, int p) {
+    return P == 1 ? m[p] : m[p] | (static_cast<uint32_t>(m[p + PB]) << 8);
+}
+template <int P>
+__device__ __forceinline__ void chain_set(uint8_t *m, int PB, int p, uint32_t c) {
+    m[p] = static_cast<uint8_t>(c);
+    if (P == 2) m[p + PB] = static_cast<uint8_t>(c >> 8);
+}
+__device__ __forceinline__ uint32_t row_weight(const uint8_t *row, int PB, int p) {
+    return row[p] | (static_cast<uint32_t>(row[p + PB]) << 8) | (static_cast<uint32_t>(row[p + 2 * PB]) << 16);
+}
+
+__device__ __forceinline__ u64 shfl_up64(u64 v, int o) {
+    const uint32_t lo = __shfl_up_sync(0xFFFFFFFFu, static_cast<uint32_t>(v), o);
+    const uint32_t hi = __shfl_up_sync(0xFFFFFFFFu, static_cast<uint32_t>(v >> 32), o);
+    return (static_cast<u64>(hi) << 32) | lo;
+}
+
+// What the two ranges of K do differently: NW words per lane and plane, or
+// (NW = 0, K > 1024) C chunks of four.
+template <int NW>
+struct ChainForm {
+    using G = DenseGeo<NW>;
+    uint32_t mbits;             // this lane's topics with m > 0 (warp 1)
+    __device__ __forceinline__ ChainForm(int) {}
+    __device__ __forceinline__ static constexpr int plane() { return G::PB; }
+    __device__ __forceinline__ static int pos(int k) { return G::pos(k); }
+    __device__ __forceinline__ static int topic(int p) { return G::topic(p); }
+    __device__ __forceinline__ static int owner(int p) { return G::owner(p); }
+    __device__ __forceinline__ static uint32_t weight(const uint8_t *row, int p) { return row_weight(row, G::PB, p); }
+    __device__ __forceinline__ int init_bits(const DocCounts &m, uint8_t *, int lane) {
+        mbits = 0;
+#pragma unroll 1
+        for (int b = 0; b < G::TPL; ++b)
+            if (m.get(G::lane0(b) + G::STRIDE * lane) > 0) mbits |= 1u << b;
+        return __popc(mbits);
+    }
+    __device__ __forceinline__ void flip(int p, int lane, bool on) { mbits ^= on && lane == G::owner(p) ? 1u << G::bit(p) : 0u; }
+    __device__ __forceinline__ uint32_t shared_topics(const uint32_t *bits, int lane) const {
+        return static_cast<uint32_t>(__popc(lane_bits<G::TPL>(bits, 0, lane) & mbits));
+    }
+    template <int P>
+    __device__ __forceinline__ u64 dot(const uint8_t *row, const uint8_t *m, int lane) const {
+        uint32_t q[3][NW];
+#pragma unroll
+        for (int p = 0; p < 3; ++p) load_words<NW>(row + p * G::PB, lane, q[p]);
+        u64 sum = 0;
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            uint32_t w[NW];
+            load_words<NW>(m + p * G::PB, lane, w);
+            uint32_t s0 = 0, s1 = 0, s2 = 0;
+#pragma unroll
+            for (int x = 0; x < NW; ++x) {
+                s0 = __dp4a(w[x], q[0][x], s0);
+                s1 = __dp4a(w[x], q[1][x], s1);
+                s2 = __dp4a(w[x], q[2][x], s2);
+            }
+            sum += (static_cast<u64>(s0 + (s1 << 8)) + (static_cast<u64>(s2) << 16)) << (8 * p);
+        }
+        return sum;
+    }
+    // Masks of the first `j + 1` of a lane's topics, j = this lane's number
+    // among them.
+    __device__ __forceinline__ static void topic_masks(int lane, uint32_t (&mask)[NW]) {
+        const int j = lane & (G::TPL - 1);
+#pragma unroll
+        for (int x = 0; x < NW; ++x) {
+            const int t = j - 4 * x;                // last topic of word x that counts
+            mask[x] = t >= 3 ? 0xFFFFFFFFu : t < 0 ? 0u : (1u << (8 * (t & 3) + 8)) - 1u;
+        }
+    }
+    // the running sum of q m over lane L's topics up to this lane's
+    template <int P>
+    __device__ __forceinline__ u64 prefix(int L, const uint8_t *row, const uint8_t *m, const uint32_t (&mask)[NW]) const {
+        uint32_t q[3][NW];
+#pragma unroll
+        for (int p = 0; p < 3; ++p) load_words<NW>(row + p * G::PB, L, q[p]);
+        u64 sum = 0;
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            uint32_t w[NW];
+            load_words<NW>(m + p * G::PB, L, w);
+            uint32_t s0 = 0, s1 = 0, s2 = 0;
+#pragma unroll
+            for (int x = 0; x < NW; ++x) {
+                s0 = __dp4a(w[x] & mask[x], q[0][x], s0);
+                s1 = __dp4a(w[x] & mask[x], q[1][x], s1);
+                s2 = __dp4a(w[x] & mask[x], q[2][x], s2);
+            }
+            sum += (static_cast<u64>(s0 + (s1 << 8)) + (static_cast<u64>(s2) << 16)) << (8 * p);
+        }
+        return sum;
+    }
+    // lane L's topic whose running sum passes res (position, or -1)
+    template <int P>
+    __device__ __forceinline__ int find(int L, u64 res, const uint8_t *row, const uint8_t *m, int lane) const {
+        uint32_t mask[NW];
+        topic_masks(lane, mask);
+        const uint32_t f = __ballot_sync(0xFFFFFFFFu, res < prefix<P>(L, row, m, mask));
+        return f ? G::lane0(__ffs(f) - 1) + L * G::STRIDE : -1;
+    }
+};
+template <>
+struct ChainForm<0> {
+    int C, TPL, PB;
+    uint32_t recip;
+    uint16_t *mb;               // this lane's bits (warp 1), chunk c at mb[32 c]
+    __device__ __forceinline__ ChainForm(int K) {
+        C = (K + 511) >> 9;
+        TPL = 16 * C;
+        PB = 512 * C;
+        recip = static_cast<uint32_t>((0x100000000ull + TPL - 1) / TPL);
+        mb = nullptr;
+    }
+    __device__ __forceinline__ int plane() const { return PB; }
+    __device__ __forceinline__ int pos(int k) const {
+        const int l = static_cast<int>(__umulhi(static_cast<uint32_t>(k), recip));
+        const int b = k - l * TPL;
+        return ((b >> 4) << 9) + (l << 4) + (b & 15);
+    }
+    __device__ __forceinline__ int topic(int p) const { return ((p >> 4) & 31) * TPL + ((p >> 9) << 4) + (p & 15); }
+    __device__ __forceinline__ static int owner(int p) { return (p >> 4) & 31; }
+    __device__ __forceinline__ uint32_t weight(const uint8_t *row, int p) const { return row_weight(row, PB, p); }
+    __device__ __forceinline__ int init_bits(const DocCounts &m, uint8_t *area, int lane) {
+        mb = reinterpret_cast<uint16_t *>(area) + lane;
+        int n = 0;
+        for (int c = 0; c < C; ++c) {
+            uint32_t bits = 0;
+            for (int b = 0; b < 16; ++b)
+                if (m.get(512 * c + 16 * lane + b) > 0) bits |= 1u << b;
+            mb[32 * c] = static_cast<uint16_t>(bits);
+            n += __popc(bits);
+        }
+        return n;
+    }
+    __device__ __forceinline__ void flip(int p, int lane, bool on) {
+        if (on && lane == owner(p)) mb[(p >> 9) << 5] ^= static_cast<uint16_t>(1u << (p & 15));
+    }
+    __device__ __forceinline__ uint32_t shared_topics(const uint32_t *bits, int lane) const {
+        const uint16_t *wb = reinterpret_cast<const uint16_t *>(bits) + C * lane;
+        uint32_t n = 0;
+        for (int c = 0; c < C; ++c) n += static_cast<uint32_t>(__popc(wb[c] & mb[32 * c]));
+        return n;
+    }
+    template <int P>
+    __device__ __forceinline__ u64 dot(const uint8_t *row, const uint8_t *m, int lane) const {
+        u64 sum = big_plane_dot(row, m, PB, C, lane);
+        if (P == 2) sum += big_plane_dot(row, m + PB, PB, C, lane) << 8;
+        return sum;
+    }
+    template <int P>
+    __device__ __forceinline__ int find(int L, u64 res, const uint8_t *row, uint8_t *m, int lane) const {
+        return big_find(L, res, row, DocCounts{m, PB, P - 1}, PB, C, lane);
+    }
+};
+
+// What warp 0 carries from token to token.
+struct ChainState {
+    u64 sum, incl, B;           // the coming token's: this lane's sum, its prefix, the total; all without `prev`
+    int prev;                   // the last token's new topic, not in the counts yet (at a document's
+                                // start the first token's topic, taken out of the counts)
+    uint32_t top;               // a bound on every count
+    uint32_t bad;               // a draw found no topic
+};
+
+// The lane's sum for the token of record part r1 from the counts at hand, less
+// the token itself.
+template <int NW, int P>
+__device__ __forceinline__ u64 chain_ahead(const ChainForm<NW> &form, const uint8_t *sm, const uint8_t *m, const uint4 r1, int lane) {
+    const uint32_t own = lane == form.owner(static_cast<int>(r1.x & 0xFFFFu)) ? r1.z : 0u;
+    return form.template dot<P>(sm + r1.y, m, lane) - own;
+}
+
+// Warp 0: tokens [t, t + cnt) of a pass, every one of them and the one after
+// with a dense row (after the last token of a pass a stand-in, whose sums go
+// unused).
+template <int NW, int P>
+__device__ __forceinline__ void chain_group_fast(const ChainForm<NW> &form, uint8_t *sm, uint8_t *m, int t, int cnt, uint32_t *drawn,
+                                                 ChainState &st) {
+    using G = DenseGeo<NW>;
+    const int lane = threadIdx.x & 31;
+    const uint4 *recs = reinterpret_cast<const uint4 *>(sm + kChainRecOff);
+    uint32_t mask[NW];
+    form.topic_masks(lane, mask);
+    const uint4 *rec = recs + 3 * (t % 96), *last = recs + 3 * 95;
+    uint4 r1 = rec[1];
+#pragma unroll 1
+    for (int u = 0; u < cnt; ++u) {
+        const uint4 r0 = rec[0];
+        rec = rec == last ? recs : rec + 3;
+        const uint4 n1 = rec[1];                // the next token's
+        const u64 At = (static_cast<u64>(r0.y) << 32) | r0.x, U = (static_cast<u64>(r0.w) << 32) | r0.z;
+        const int kold = static_cast<int>(r1.x & 0xFFFFu);
+        const uint8_t *row = sm + r1.y, *nrow = sm + n1.y;
+        const uint32_t delta = form.weight(row, st.prev), dn = form.weight(nrow, st.prev);
+        const int ow = G::owner(st.prev);
+        // the next token's sum: from the counts as they were before this token
+        // (these loads do not wait for the previous draw), less this token's
+        // and its own topic, and with the previous one's new topic
+        const u64 before = form.template dot<P>(nrow, m, lane);
+        // the last token's topic in, this one out: m^{-i}.  Every lane stores
+        // the same bytes
+        const uint32_t c1 = chain_count<P>(m, G::PB, st.prev) + 1u;
+        const uint32_t c0 = (st.prev == kold ? c1 : chain_count<P>(m, G::PB, kold)) - 1u;
+        __syncwarp();                           // every lane has read the old counts
+        chain_set<P>(m, G::PB, st.prev, c1);
+        chain_set<P>(m, G::PB, kold, c0);
+        st.top = max(st.top, c1);
+        const u64 upto = st.incl + (lane >= ow ? delta : 0u), mine = st.sum + (lane == ow ? delta : 0u);
+        st.sum = before + (lane == ow ? dn : 0u) - (lane == G::owner(kold) ? n1.w : 0u) -
+                 (lane == G::owner(static_cast<int>(n1.x & 0xFFFFu)) ? n1.z : 0u);
+        u64 v = st.sum;
+        const u64 T = At + ((st.B + delta) << kFracBits);
+        const u64 rr = __umul64hi(U, T);
+        const u64 rb = (rr - At) >> kFracBits;
+        u64 w = shfl_up64(v, 1);
+        // no lane passes for an alias draw (rr < At wraps round) or without any mass
+        const uint32_t bal = __ballot_sync(0xFFFFFFFFu, rb < upto);
+        v += lane >= 1 ? w : 0u;
+        w = shfl_up64(v, 2);
+        const int L = (__ffs(bal) - 1) & 31;
+        v += lane >= 2 ? w : 0u;
+        w = shfl_up64(v, 4);
+        const u64 res = __shfl_sync(0xFFFFFFFFu, rb - (upto - mine), L);
+        v += lane >= 4 ? w : 0u;
+        w = shfl_up64(v, 8);
+        const u64 pre = form.template prefix<P>(L, row, m, mask);
+        v += lane >= 8 ? w : 0u;
+        w = shfl_up64(v, 16);
+        const uint32_t f = __ballot_sync(0xFFFFFFFFu, res < pre);
+        v += lane >= 16 ? w : 0u;
+        st.incl = v;
+        st.B = __shfl_sync(0xFFFFFFFFu, v, 31);
+        uint32_t knew = static_cast<uint32_t>(G::lane0((__ffs(f) - 1) & 31) + L * G::STRIDE);
+        knew = rr < At ? (r1.x >> 16) | kDrawnAlias : bal ? knew : static_cast<uint32_t>(kold) | kDrawnZero;
+        st.bad |= bal != 0 && f == 0 ? 1u : 0u;
+        drawn[u] = knew;
+        st.prev = static_cast<int>(knew & 0x3FFFu);
+        r1 = n1;
+    }
+    __syncwarp();
+}
+
+// The same for any group: tokens without a dense row among them, or K > 1024.
+template <int NW, int P>
+__device__ __forceinline__ void chain_group_any(const ZArgs &a, const ChainForm<NW> &form, uint8_t *sm, uint8_t *m, int t, int cnt,
+                                                uint32_t *drawn, ChainState &st) {
+    const int lane = threadIdx.x & 31;
+    const int PB = form.plane();
+    const uint4 *recs = reinterpret_cast<const uint4 *>(sm + kChainRecOff);
+#pragma unroll 1
+    for (int u = 0; u < cnt; ++u, ++t) {
+        const uint4 *rec = recs + 3 * (t % 96);
+        const uint4 r0 = rec[0], r1 = rec[1], n1 = recs[3 * ((t + 1) % 96) + 1];
+        const u64 At = (static_cast<u64>(r0.y) << 32) | r0.x, U = (static_cast<u64>(r0.w) << 32) | r0.z;
+        const int kold = static_cast<int>(r1.x & 0xFFFFu);
+        const bool dense = r1.y != 0xFFFFFFFFu, ahead = n1.y != 0xFFFFFFFFu;
+        const uint8_t *row = sm + r1.y;
+        const uint32_t delta = dense ? form.weight(row, st.prev) : 0u;
+        const int ow = form.owner(st.prev);
+        const uint32_t c1 = chain_count<P>(m, PB, st.prev) + 1u;
+        const uint32_t c0 = (st.prev == kold ? c1 : chain_count<P>(m, PB, kold)) - 1u;
+        __syncwarp();
+        chain_set<P>(m, PB, st.prev, c1);
+        chain_set<P>(m, PB, kold, c0);
+        __syncwarp();
+        st.top = max(st.top, c1);
+        const u64 upto = st.incl + (lane >= ow ? delta : 0u), mine = st.sum + (lane == ow ? delta : 0u), B = st.B + delta;
+        if (ahead) st.sum = chain_ahead<NW, P>(form, sm, m, n1, lane);
+        uint32_t knew;
+        if (dense) {
+            const u64 rr = __umul64hi(U, At + (B << kFracBits));
+            if (rr < At) {
+                knew = (r1.x >> 16) | kDrawnAlias;
+            } else {
+                const u64 rb = (rr - At) >> kFracBits;
+                const uint32_t bal = __ballot_sync(0xFFFFFFFFu, rb < upto);
+                knew = static_cast<uint32_t>(kold) | kDrawnZero;
+                if (bal) {
+                    const int L = __ffs(bal) - 1;
+                    const u64 res = __shfl_sync(0xFFFFFFFFu, rb - (upto - mine), L);
+                    const int k = form.template find<P>(L, res, row, m, lane);
+                    st.bad |= k < 0 ? 1u : 0u;
+                    knew = static_cast<uint32_t>(k < 0 ? kold : k);
+                }
+            }
+        } else {
+            const uint4 r2 = rec[2];
+            uint32_t c = 0;
+            DocCounts mc{m, PB, P - 1};
+            const TokenDraw td{At, U, static_cast<int>(r1.x >> 16), kold};
+            const int k = column_draw(a, td, static_cast<int64_t>((static_cast<u64>(r2.y) << 32) | r2.x), static_cast<int>(r2.z), mc, lane, c,
+                                      [&](int x) { return form.pos(x); });
+            knew = static_cast<uint32_t>(k) | (c & (1u << 6) ? kDrawnAlias : 0u) | (c & (1u << 12) ? kDrawnZero : 0u);
+        }
+        if (ahead) {
+            st.incl = warp_incl_scan<32>(st.sum);
+            st.B = __shfl_sync(0xFFFFFFFFu, st.incl, 31);
+        }
+        drawn[u] = knew;
+        st.prev = static_cast<int>(knew & 0x3FFFu);
+        __syncwarp();
+    }
+}
+
+// All threads of the CTA; sm: chain_smem_bytes(K) bytes.  phases: the parities
+// of the groups' barriers, kept from one document to the next.  Documents of
+// at most kNarrowMaxLen tokens.
+template <int NW>
+__device__ __forceinline__ void z_doc_chain(const ZArgs &a, uint8_t *sm, DocRun &r, uint32_t &phases) {
+    const int lane = threadIdx.x & 31;
+    const int role = threadIdx.x >> 5;      // 0: the chain, 1: records and rows, 2: counters and topics
+    const int K = a.K;
+    if (r.len == 0 || r.budget <= 0) return;
+    ChainCtl &ctl = *reinterpret_cast<ChainCtl *>(sm);
+    uint4 *recs = reinterpret_cast<uint4 *>(sm + kChainRecOff);
+    const int ring = chain_ring_off(K), RB = dense_row_bytes(K), G = chain_group(K);
+    ChainForm<NW> form(K);
+    const int PB = form.plane();
+    auto pos = [&](int k) { return form.pos(k); };
+    // warps 0 and 2 each keep the document's counts
+    DocCounts m{sm + kChainCountOff + role * PB, PB, 0};
+    if (role != 1) build_counts(a, m, r, nullptr, 2, pos);
+    ChainState st{};
+    st.prev = -1;
+    int kd = 0;
+    if (role == 0) {
+        uint32_t top = 0;
+        for (int p = lane; p < PB; p += 32) top = max(top, m.b[p] | (static_cast<uint32_t>(m.b[p + PB]) << 8));
+        st.top = __reduce_max_sync(0xFFFFFFFFu, top);
+    } else if (role == 2) {
+        kd = static_cast<int>(__reduce_add_sync(0xFFFFFFFFu, static_cast<unsigned>(form.init_bits(m, sm + kChainCountOff + 4 * PB, lane))));
+    }
+    const int colmax = a.path == 1 ? 0x7FFFFFFF : -1;
+    const uint32_t sweep_end = r.sweep + static_cast<uint32_t>(r.max_pass_end);
+    bool stop = false;
+    while (!stop && r.budget > 0 && r.sweep != sweep_end) {
+        // one pass, or what of it the budget allows: n tokens from r.pos
+        const int p0 = r.pos;
+        const int n = static_cast<int>(min(static_cast<int64_t>(r.len - p0), r.budget));
+        const int ng = (n + G - 1) / G;
+        auto stage = [&](int b) {
+            const int t = 32 * b + lane;
+            uint4 *rec = recs + 3 * (t % 96);
+            if (t == n) rec[1] = make_uint4(0u, static_cast<uint32_t>(ring), 0u, 0u);     // the stand-in after the last token
+            if (t >= n) return;
+            uint4 x[2];
+            uint32_t d;
+            stage_token(a, r, p0 + t, x, &d, colmax, pos);
+            rec[0] = make_uint4(x[0].z, x[0].w, x[1].y, x[1].x);
+            rec[1] = make_uint4((x[1].w >> 16) | (x[0].y & 0xFFFF0000u),
+                                d == 0xFFFFFFFFu ? d : static_cast<uint32_t>(ring + (t % (3 * G)) * RB), 0u, d);
+            rec[2] = make_uint4(x[0].x, x[0].y & 0xFFFFu, x[1].w & 0xFFFFu, x[1].z);
+        };
+        // group g's rows on their way (lane u < G its token u)
+        auto fetch = [&](int g) {
+            const int t = g * G + lane;
+            uint32_t at = 0xFFFFFFFFu, d = 0;
+            if (lane < G && t < n) {
+                at = recs[3 * (t % 96) + 1].y;
+                d = recs[3 * (t % 96) + 1].w;
+            }
+            const int rows = __popc(__ballot_sync(0xFFFFFFFFu, at != 0xFFFFFFFFu));
+            u64 *bar = &ctl.full[g % 3];
+            if (lane == 0) bar_expect(bar, static_cast<uint32_t>(rows * RB));
+            __syncwarp();
+            if (at != 0xFFFFFFFFu) bulk_copy(sm + at, a.qrow + static_cast<size_t>(d) * RB, static_cast<uint32_t>(RB), bar);
+        };
+        auto landed = [&](int g) {
+            const int s = g % 3;
+            const bool ok = bar_wait(&ctl.full[s], (phases >> s) & 1u);
+            phases ^= 1u << s;
+            if (!ok && lane == 0) atomicOr(&a.stats[ST_ERROR], ERR_BARRIER);
+            // the weights of the tokens' own and previous topics, now that their rows are here
+            const int t = g * G + lane;
+            if (ok && lane < G && t < n) {
+                uint4 *r1 = recs + 3 * (t % 96) + 1;
+                if (r1->y != 0xFFFFFFFFu) {
+                    r1->z = form.weight(sm + r1->y, static_cast<int>(r1->x & 0xFFFFu));
+                    if (t > 0) r1->w = form.weight(sm + r1->y, static_cast<int>(recs[3 * ((t - 1) % 96) + 1].x & 0xFFFFu));
+                }
+            }
+            return ok;
+        };
+        // the counters and topics of group g, as drawn
+        auto replay = [&](int g) {
+            const int t0 = g * G, cnt = min(G, n - t0);
+            constexpr int GM = NW == 0 ? 1 : NW == 8 ? 4 : 8;       // chain_group(K), K <= 1024
+            uint32_t wb[GM];
+            if constexpr (NW > 0) {
+#pragma unroll
+                for (int u = 0; u < GM; ++u)
+                    if (u < cnt) wb[u] = lane_bits<DenseGeo<NW>::TPL>(a.bits, static_cast<int64_t>(recs[3 * ((t0 + u) % 96) + 2].w) * a.KWp, lane);
+            }
+            uint32_t c_min = 0, c_cnt = 0, c_int = 0;
+            auto token = [&](int u, uint32_t bits) {
+                const int kold = static_cast<int>(recs[3 * ((t0 + u) % 96) + 1].x & 0xFFFFu);
+                const uint4 r2 = recs[3 * ((t0 + u) % 96) + 2];
+                const uint32_t x = ctl.drawn[8 * (g & 1) + u];
+                const int knew = static_cast<int>(x & 0x3FFFu), n_w = static_cast<int>(r2.z);
+                const uint32_t co = chain_count<2>(m.b, PB, kold) - 1u;
+                __syncwarp();
+                chain_set<2>(m.b, PB, kold, co);
+                if (co == 0) --kd;
+                form.flip(kold, lane, co == 0);
+                c_min += static_cast<uint32_t>(kd < n_w ? kd : n_w);
+                c_cnt += (kd < n_w ? 1u : 0u) + (x & kDrawnAlias ? 1u << 6 : 0u) + (x & kDrawnZero ? 1u << 12 : 0u);
+                if constexpr (NW > 0) c_int += static_cast<uint32_t>(__popc(bits & form.mbits));
+                else c_int += form.shared_topics(a.bits + static_cast<int64_t>(r2.w) * a.KWp, lane);
+                const uint32_t cn = chain_count<2>(m.b, PB, knew) + 1u;
+                __syncwarp();
+                chain_set<2>(m.b, PB, knew, cn);
+                if (cn == 1) ++kd;
+                form.flip(knew, lane, cn == 1);
+            };
+            if constexpr (NW > 0) {
+#pragma unroll
+                for (int u = 0; u < GM; ++u)
+                    if (u < cnt) token(u, wb[u]);
+            } else {
+                for (int u = 0; u < cnt; ++u) token(u, 0u);
+            }
+            if (lane < cnt) {
+                const int k = form.topic(static_cast<int>(ctl.drawn[8 * (g & 1) + lane] & 0x3FFFu));
+                r.z[p0 + t0 + lane] = static_cast<int16_t>(guard_index(k, K, a.stats));
+            }
+            add_block_counts(ctl.cnt, lane, cnt, c_min, c_cnt, c_int);
+        };
+        __syncthreads();            // the last pass's topics are written and its records done with
+        stage(role);
+        __syncthreads();
+        bool ok = true;
+        if (role == 1) {
+            fetch(0);
+            if (ng > 1) fetch(1);
+            ok = landed(0);
+            if (ng > 1) ok = landed(1) && ok;
+            if (lane == 0) ctl.stop = ok ? 0 : 1;
+        }
+        __syncthreads();
+        stop = ctl.stop != 0;
+        int done = 0;
+        if (role == 0 && !stop) {
+            const uint4 r1 = recs[1];
+            if (st.prev < 0) {
+                st.prev = static_cast<int>(r1.x & 0xFFFFu);
+                chain_set<2>(m.b, PB, st.prev, chain_count<2>(m.b, PB, st.prev) - 1u);
+                __syncwarp();
+            }
+            if (r1.y != 0xFFFFFFFFu) {
+                st.sum = chain_ahead<NW, 2>(form, sm, m.b, r1, lane);
+                st.incl = warp_incl_scan<32>(st.sum);
+                st.B = __shfl_sync(0xFFFFFFFFu, st.incl, 31);
+            }
+        }
+        for (int g = 0; g < ng && !stop; ++g) {
+            const int t0 = g * G, cnt = min(G, n - t0);
+            if (role == 0) {
+                uint32_t *drawn = ctl.drawn + 8 * (g & 1);
+                const bool one = st.top + static_cast<uint32_t>(G) <= 255u;      // counts stay in one plane
+                if constexpr (NW > 0) {
+                    // every token and the next group's first with a row
+                    const uint32_t y = lane <= cnt ? recs[3 * ((t0 + lane) % 96) + 1].y : 0u;
+                    if (!__any_sync(0xFFFFFFFFu, y == 0xFFFFFFFFu)) {
+                        if (one) chain_group_fast<NW, 1>(form, sm, m.b, t0, cnt, drawn, st);
+                        else chain_group_fast<NW, 2>(form, sm, m.b, t0, cnt, drawn, st);
+                    } else {
+                        chain_group_any<NW, 2>(a, form, sm, m.b, t0, cnt, drawn, st);
+                    }
+                } else {
+                    if (one) chain_group_any<NW, 1>(a, form, sm, m.b, t0, cnt, drawn, st);
+                    else chain_group_any<NW, 2>(a, form, sm, m.b, t0, cnt, drawn, st);
+                }
+            } else if (role == 1) {
+                if (g + 2 < ng) fetch(g + 2);
+                // block b - 1 was drawn before the last group, and is replayed
+                const int b = (t0 - G) >> 5;
+                if (g > 0 && ((t0 - G) & 31) == 0 && b > 0 && 32 * (b + 2) <= n) {
+                    stage(b + 2);
+                    __syncwarp();
+                }
+                if (g + 2 < ng) ok = landed(g + 2);
+                const bool late = ((t0 + cnt) & 31) == 0 && r.deadline != ~0ull && global_ns() >= r.deadline;
+                if (lane == 0) ctl.stops[g & 1] = late || !ok;
+            } else if (g > 0) {
+                replay(g - 1);
+            }
+            done += cnt;
+            __syncthreads();
+            stop = ctl.stops[g & 1] != 0;
+        }
+        if (role == 2 && done > 0) replay((done - 1) / G);
+        if (role == 0 && lane == 0 && st.bad) atomicOr(&a.stats[ST_ERROR], ERR_INTERNAL);
+        r.budget -= done;
+        r.pos += done;
+        if (r.pos == r.len) { r.pos = 0; r.sweep += 1; }
+    }
+    __syncthreads();
+}
+
+// Before the first document: the groups' barriers and the counters.
+__device__ __forceinline__ void chain_begin(uint8_t *sm) {
+    ChainCtl &ctl = *reinterpret_cast<ChainCtl *>(sm);
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < 3; ++s) bar_init(&ctl.full[s]);
+        for (int s = 0; s < 6; ++s) ctl.cnt[s] = 0;
+        ctl.stop = 0;
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    __syncthreads();
+}
+
+}  // namespace pulda

@@ -109,12 +109,7 @@ __device__ __forceinline__ int zg_stage(const ZArgs &a, uint32_t sweep, int64_t 
         const uint32_t sl = __umulhi(x.z, static_cast<uint32_t>(nw));
         ta = alias_outcome(a, cb + sl, x.w);
     }
-    int ds = a.dense_slot[wv];
-    if (ds < 0) {                 // the host sends only corpora whose every word has a row
-        atomicOr(&a.stats[ST_ERROR], ERR_INTERNAL);
-        ds = 0;
-    }
-    const uint32_t qoff = static_cast<uint32_t>(ds) * static_cast<uint32_t>(a.K);
+    const uint32_t qoff = static_cast<uint32_t>(wv) * static_cast<uint32_t>(a.K);
     rec[0] = make_uint4(x.x, x.y, static_cast<uint32_t>(Av), static_cast<uint32_t>(Av >> 32));
     rec[1] = make_uint4(qoff, static_cast<uint32_t>(wv) * static_cast<uint32_t>(a.KWp),
                         static_cast<uint32_t>(nw) | (static_cast<uint32_t>(zo) << 16), static_cast<uint32_t>(ta));
