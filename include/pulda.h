@@ -300,7 +300,7 @@ typedef struct pulda_batch pulda_batch;
  * CTA size instead of tuning it over {2, 4, 8}; opt->coop_min_len -1 keeps
  * every document on one warp, > 0 sends the documents at least that long (of
  * every chain) to CTAs of their own, 0 sends those of at least
- * max(256, N / 4500) tokens (N = tokens of all chains), the single-chain rule;
+ * max(256, N / 8000) tokens (N = tokens of all chains);
  * docs_per_warp must be 0 or 1; batch_form picks the launch form and
  * alias_layout the alias tables' layout (see pulda_options).  Tuning times
  * each CTA size on two real sweeps (in order, then in reverse), together with

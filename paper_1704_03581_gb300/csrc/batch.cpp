@@ -4,7 +4,8 @@
 // and replayed.  The z-step CTA size, the launch form and then the alias
 // tables' layout are picked by timing the candidates on the first sweeps
 // (none of them changes a result, so tuning costs no extra sweeps); the
-// longest documents go to the cooperative z-step by the single-chain rule.
+// longest documents go to CTAs of their own, the others one per warp, the chains
+// of one form of the z-step in one launch each.
 #include <algorithm>
 #include <cstdio>
 #include <numeric>
@@ -49,7 +50,7 @@ struct pulda_batch {
     PhiArgs *d_phi = nullptr;
     ZArgs *d_z = nullptr;
     int64_t coop_len = 0;           // in use
-    std::vector<int64_t> dlen;      // document lengths in work-list order (longest first)
+    std::vector<int64_t> form_len;  // document lengths, form by form, longest first in each
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
@@ -81,13 +82,24 @@ cudaError_t balloc(pulda_batch *b, T **p, size_t n) {
 
 thread_local std::string g_batch_init_error;
 
-// Documents the long-document z-step takes at threshold L (the work list is
-// longest first; the n_wide widest are the one-warp kernel's).
-int count_coop_items(const pulda_batch *b, int64_t L) {
-    if (L <= 0) return 0;
-    int n = b->bl.n_wide;
-    while (n < static_cast<int>(b->dlen.size()) && b->dlen[n] >= L) ++n;
-    return n - b->bl.n_wide;
+// Sets how many of each form's documents the long-document z-step takes at
+// threshold L (a form's list is longest first; the n_wide widest are the
+// one-warp kernel's).
+void set_coop_items(pulda_batch *b, int64_t L) {
+    for (int f = 0; f < b->bl.n_forms; ++f) {
+        BatchForm &F = b->bl.form[f];
+        int n = F.n_wide;
+        while (L > 0 && n < F.n && b->form_len[F.first + n] >= L) ++n;
+        F.n_coop = n - F.n_wide;
+    }
+}
+
+bool make_side_streams(BatchLaunch &bl) {
+    for (int i = 0; i < 2 * bl.n_forms - 1; ++i)
+        if (cudaStreamCreateWithFlags(&bl.side[i], cudaStreamNonBlocking) != cudaSuccess ||
+            cudaEventCreateWithFlags(&bl.ev_join[i], cudaEventDisableTiming) != cudaSuccess)
+            return false;
+    return true;
 }
 
 // Starts a tuning phase over candidates [first, cand.size()): forward, then backward.
@@ -107,9 +119,10 @@ void schedule_phase(pulda_batch *b, int first) {
 // z-step reads whichever layout its own descriptor names.
 cudaError_t apply_candidate(pulda_batch *b, const pulda_batch::Cand &c) {
     b->bl.z_warps = c.warps;
-    b->bl.z_grid = b->sms * batch_z_blocks_per_sm(b->bl.kmax, c.warps, b->bl.narrow != 0);
+    for (int f = 0; f < b->bl.n_forms; ++f)
+        b->bl.form[f].z_grid = b->sms * batch_z_blocks_per_sm(b->bl.form[f].kmax, c.warps, true);
     b->coop_len = c.coop_len;
-    b->bl.n_coop = count_coop_items(b, c.coop_len);
+    set_coop_items(b, c.coop_len);
     b->one_launch = c.one_launch;
     if (c.packed == b->packed) return cudaSuccess;
     for (size_t i = 0; i < b->ch.size(); ++i) {
@@ -233,7 +246,7 @@ pulda_status pulda_batch_init(pulda_batch **out, const pulda_chain_desc *chains,
     ZArgs *d_z = nullptr;
     cudaError_t ea = cudaSuccess;
     if ((ea = balloc(b, &d_bar, 1)) != cudaSuccess || (ea = balloc(b, &d_sweep, 1)) != cudaSuccess ||
-        (ea = balloc(b, &d_work, 4)) != cudaSuccess ||
+        (ea = balloc(b, &d_work, kBatchCounters)) != cudaSuccess ||
         (ea = balloc(b, &d_phi, n_chains)) != cudaSuccess || (ea = balloc(b, &d_z, n_chains)) != cudaSuccess) {
         b->err = std::string("device allocation of the batch descriptors failed: ") + cudaGetErrorString(ea);
         return bail(ea == cudaErrorMemoryAllocation ? PULDA_ERR_OOM : PULDA_ERR_CUDA);
@@ -279,19 +292,32 @@ pulda_status pulda_batch_init(pulda_batch **out, const pulda_chain_desc *chains,
     };
     std::stable_sort(wi.begin(), wi.end(), heavy_first);
     std::stable_sort(di.begin(), di.end(), heavy_first);
-    std::vector<int2> wlist(wi.size()), dlist(di.size());
+    std::vector<int2> wlist(wi.size());
     for (size_t i = 0; i < wi.size(); ++i) wlist[i] = wi[i].second;
-    for (size_t i = 0; i < di.size(); ++i) dlist[i] = di[i].second;
-    b->dlen.resize(di.size());
     int64_t n_tokens = 0;
-    for (size_t i = 0; i < di.size(); ++i) {
-        b->dlen[i] = di[i].first;
-        n_tokens += di[i].first;
+    for (const auto &x : di) n_tokens += x.first;
+    // the documents form by form: the order is stable, so longest first in each
+    std::vector<int2> flist;
+    for (int nw : {8, 4, 2, 1, 0}) {        // the form of the most work per token first; 0 = above 1,024 topics
+        BatchForm F{};
+        F.first = static_cast<int>(flist.size());
+        for (const auto &x : di) {
+            const int K = b->ch[x.second.x]->K;
+            if ((K <= 1024 ? dense_words(K) : 0) != nw) continue;
+            F.kmax = std::max(F.kmax, K);
+            if (x.first > kNarrowMaxLen) ++F.n_wide;
+            flist.push_back(x.second);
+            b->form_len.push_back(x.first);
+        }
+        F.n = static_cast<int>(flist.size()) - F.first;
+        if (F.n == 0) continue;
+        F.coop_grid = b->sms * batch_coop_blocks_per_sm(F.kmax);
+        b->bl.form[b->bl.n_forms++] = F;
     }
-    while (b->bl.n_wide < static_cast<int>(b->dlen.size()) && b->dlen[b->bl.n_wide] > kNarrowMaxLen) ++b->bl.n_wide;
-    int2 *d_wl = nullptr, *d_dl = nullptr;
+    int2 *d_wl = nullptr, *d_fl = nullptr;
     HeavyChunk *d_heavy = nullptr;
-    if ((ea = balloc(b, &d_wl, wlist.size())) != cudaSuccess || (ea = balloc(b, &d_dl, dlist.size())) != cudaSuccess ||
+    if ((ea = balloc(b, &d_wl, wlist.size())) != cudaSuccess || 
+        (ea = balloc(b, &d_fl, flist.size())) != cudaSuccess ||
         (ea = balloc(b, &d_heavy, heavy.size())) != cudaSuccess) {
         b->err = std::string("device allocation of the work lists failed: ") + cudaGetErrorString(ea);
         return bail(ea == cudaErrorMemoryAllocation ? PULDA_ERR_OOM : PULDA_ERR_CUDA);
@@ -302,7 +328,7 @@ pulda_status pulda_batch_init(pulda_batch **out, const pulda_chain_desc *chains,
     if (cudaMemcpyAsync(d_phi, hp.data(), sizeof(PhiArgs) * n_chains, cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaMemcpyAsync(d_z, hz.data(), sizeof(ZArgs) * n_chains, cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaMemcpyAsync(d_wl, wlist.data(), sizeof(int2) * wlist.size(), cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaMemcpyAsync(d_dl, dlist.data(), sizeof(int2) * dlist.size(), cudaMemcpyHostToDevice, st) != cudaSuccess ||
+        cudaMemcpyAsync(d_fl, flist.data(), sizeof(int2) * flist.size(), cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaMemcpyAsync(d_sweep, &zero, sizeof zero, cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaMemsetAsync(d_bar, 0, sizeof(GridBarrier), st) != cudaSuccess ||
         (!heavy.empty() && cudaMemcpyAsync(d_heavy, heavy.data(), sizeof(HeavyChunk) * heavy.size(),
@@ -319,29 +345,25 @@ pulda_status pulda_batch_init(pulda_batch **out, const pulda_chain_desc *chains,
     bl.n_chains = n_chains;
     bl.phi_items = d_wl;
     bl.n_phi_items = static_cast<int>(wlist.size());
-    bl.z_items = d_dl;
-    bl.n_z_items = static_cast<int>(dlist.size());
+    bl.form_items = d_fl;
     bl.sweep = d_sweep;
     bl.work = d_work;
     bl.kmax = kmax;
     bl.narrow = narrow ? 1 : 0;
     bl.phi_grid = b->sms * batch_phi_blocks_per_sm(kmax);
-    bl.coop_grid = b->sms * batch_coop_blocks_per_sm(kmax);
     bl.bar = d_bar;
     bl.persist_grid = b->sms * batch_persistent_blocks_per_sm(kmax, narrow, &bl.persist_z_warps, &bl.table_stage);
-    // The cooperative threshold: fixed, none, or the automatic rule of the
-    // single-chain z-step over all chains' tokens (documents that would outlast
-    // the pass on one warp).  It is not timed: on the 32-chain workload, timing
-    // thresholds on a few sweeps chose a quarter of the rule's (and once none),
-    // while over the steady sweeps the rule's threshold ran at 42.9 ms per sweep
-    // against 47.2 (a quarter) and 53.0 (none).
+    // The threshold of the documents on CTAs: fixed, none, or the automatic rule
+    // over all chains' tokens (documents that would outlast the pass on one
+    // warp).  It is not timed: a few early sweeps chose worse thresholds than
+    // the steady ones call for.
     int64_t fixed_coop = o.coop_min_len > 0 ? o.coop_min_len : 0;
     if (o.coop_min_len == 0) {
-        const int64_t L = std::max<int64_t>(kCoopAutoMin, n_tokens / kCoopAutoDiv + 1);
-        if (count_coop_items(b, L) > 0) fixed_coop = L;
+        const int64_t L = std::max<int64_t>(kCoopAutoMin, n_tokens / kBatchCoopDiv + 1);
+        if (std::any_of(b->form_len.begin(), b->form_len.end(), [&](int64_t n) { return n >= L && n <= kNarrowMaxLen; })) fixed_coop = L;
     }
-    // Launch forms: six launches per sweep with a CTA size for the z-step, and
-    // (without cooperative CTAs) one persistent launch; tuned forms are timed.
+    // Launch forms: a launch or a few per phase with a CTA size for the z-step, and
+    // (without documents on CTAs) one persistent launch; tuned forms are timed.
     const bool one_ok = bl.persist_grid > 0 && fixed_coop == 0;
     const bool pk = b->packed;
     if (o.batch_form == 2) {
@@ -375,9 +397,8 @@ pulda_status pulda_batch_init(pulda_batch **out, const pulda_chain_desc *chains,
         return bail(PULDA_ERR_CUDA);
     }
     if (cudaEventCreate(&b->ev0) != cudaSuccess || cudaEventCreate(&b->ev1) != cudaSuccess ||
-        cudaStreamCreateWithFlags(&bl.stream2, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&bl.ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&bl.ev_join, cudaEventDisableTiming) != cudaSuccess ||
+        !make_side_streams(bl) ||
         cudaGetLastError() != cudaSuccess) {
         b->err = "CUDA set-up of the batch failed";
         return bail(PULDA_ERR_CUDA);
@@ -489,12 +510,14 @@ void pulda_batch_free(pulda_batch *b) {
     if (b->graph) cudaGraphDestroy(b->graph);
     if (b->ev0) cudaEventDestroy(b->ev0);
     if (b->ev1) cudaEventDestroy(b->ev1);
-    if (b->bl.stream2) {
-        cudaStreamSynchronize(b->bl.stream2);
-        cudaStreamDestroy(b->bl.stream2);
-    }
+    for (cudaStream_t s : b->bl.side)
+        if (s) {
+            cudaStreamSynchronize(s);
+            cudaStreamDestroy(s);
+        }
     if (b->bl.ev_fork) cudaEventDestroy(b->bl.ev_fork);
-    if (b->bl.ev_join) cudaEventDestroy(b->bl.ev_join);
+    for (cudaEvent_t e : b->bl.ev_join)
+        if (e) cudaEventDestroy(e);
     for (pulda_handle *h : b->ch) pulda_free(h);
     if (b->stream) cudaStreamSynchronize(b->stream);
     for (void *p : b->allocs) dev_free(b->opt, b->stream, p, false);

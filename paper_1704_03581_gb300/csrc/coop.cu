@@ -42,10 +42,11 @@ __global__ void __launch_bounds__(kChainThreads, 4) k_z_step_coop(ZArgs a, int n
     if (threadIdx.x < 32) flush_warp_counters(a.stats, ctl.cnt);
 }
 
-// Many chains: the longest documents of every chain; items[0 .. n_items) are
+// Many chains of one form: their longest documents; items[0 .. n_items) are
 // (chain, document) pairs.
+template <int NW>
 __global__ void __launch_bounds__(kChainThreads, 4) k_z_step_coop_multi(const ZArgs *chains, const int2 *items, int n_items,
-                                                                     int *work) {
+                                                                        int *work) {
     extern __shared__ __align__(16) uint8_t csm[];
     ChainCtl &ctl = *reinterpret_cast<ChainCtl *>(csm);
     chain_begin(csm);
@@ -54,17 +55,11 @@ __global__ void __launch_bounds__(kChainThreads, 4) k_z_step_coop_multi(const ZA
         const int item = next_item(ctl, work);
         if (item >= n_items) break;
         const int2 it = items[item];
-        const ZArgs &a = chains[it.x];
+        const ZArgs a = chains[it.x];
         const int64_t s = a.doc_off[it.y];
         const int len = static_cast<int>(a.doc_off[it.y + 1] - s);
         DocRun r{a.w + s, a.z + s, len, a.seed, a.index_base + s, sweep_of(a), 0, len, 1};
-        switch (z_nw(a.K)) {
-            case 1: z_doc_chain<1>(a, csm, r, phases); break;
-            case 2: z_doc_chain<2>(a, csm, r, phases); break;
-            case 4: z_doc_chain<4>(a, csm, r, phases); break;
-            case 8: z_doc_chain<8>(a, csm, r, phases); break;
-            default: z_doc_chain<0>(a, csm, r, phases);
-        }
+        z_doc_chain<NW>(a, csm, r, phases);
         if (threadIdx.x < 32) flush_warp_counters(a.stats, ctl.cnt);
     }
 }
@@ -149,12 +144,25 @@ void launch_z_step_coop(const ZArgs &a, int n_coop, int *work, int grid, cudaStr
     coop_kernel(a.K)<<<std::max(1, std::min(grid, n_coop)), kChainThreads, chain_smem_bytes(a.K), st>>>(a, n_coop, work);
 }
 
-int batch_coop_blocks_per_sm(int kmax) { return blocks_per_sm(k_z_step_coop_multi, chain_smem_bytes_upto(kmax)); }
+using CoopMultiKernel = void (*)(const ZArgs *, const int2 *, int, int *);
+static CoopMultiKernel coop_multi_kernel(int kmax) {
+    switch (z_nw(kmax)) {
+        case 1: return k_z_step_coop_multi<1>;
+        case 2: return k_z_step_coop_multi<2>;
+        case 4: return k_z_step_coop_multi<4>;
+        case 8: return k_z_step_coop_multi<8>;
+        default: return k_z_step_coop_multi<0>;
+    }
+}
+// Chains of one form need the shared memory of that form's largest K.
+static int coop_multi_smem(int kmax) { return z_nw(kmax) > 0 ? chain_smem_bytes(kmax) : chain_smem_bytes_upto(kmax); }
+
+int batch_coop_blocks_per_sm(int kmax) { return blocks_per_sm(coop_multi_kernel(kmax), coop_multi_smem(kmax)); }
 
 void launch_z_step_coop_multi(const ZArgs *chains, const int2 *items, int n_items, int *work, int kmax, int grid,
                               cudaStream_t st) {
     if (n_items <= 0) return;
-    k_z_step_coop_multi<<<std::max(1, std::min(grid, n_items)), kChainThreads, chain_smem_bytes_upto(kmax), st>>>(
+    coop_multi_kernel(kmax)<<<std::max(1, std::min(grid, n_items)), kChainThreads, coop_multi_smem(kmax), st>>>(
         chains, items, n_items, work);
 }
 

@@ -748,27 +748,37 @@ __global__ void k_slice_counts(const int64_t *doc_off, const int32_t *sliced_doc
     }
 }
 
-// Many chains: the work list holds (chain, document) pairs, longest first
-// across all chains; shared memory per warp is sized for the largest K.
-// Chains take the form of their own K.
-__global__ void __launch_bounds__(32 * kMultiWarps, PULDA_MULTI_MINB) k_z_step_multi(const ZArgs *chains, const int2 *items,
-                                                                        int n_items, int *work, int kmax, int narrow) {
-    extern __shared__ __align__(16) uint32_t zsm[];
+// Many chains of one form (NW): items[0 .. n_items) are (chain, document)
+// pairs, longest first, taken one after another by every warp.  m: the warp's
+// area, sized for kmax topics.
+template <int NW>
+__device__ __forceinline__ void z_multi_items(const ZArgs *chains, const int2 *items, int n_items, int *work, uint32_t *m, u64 *wcnt,
+                                              int narrow) {
     const int lane = threadIdx.x & 31;
-    uint32_t *m = zsm + static_cast<size_t>(threadIdx.x >> 5) * z_dense_warp_words(kmax, narrow != 0);
-    u64 *wcnt = z_dense_counters(m, kmax, narrow != 0);     // beyond every chain's counts and token records
-    zero_warp_counters(wcnt);
     for (;;) {
         int item = 0;
         if (lane == 0) item = atomicAdd(work, 1);
         item = __shfl_sync(0xFFFFFFFFu, item, 0);
         if (item >= n_items) break;
         const int2 it = items[item];
-        const ZArgs &a = chains[it.x];
+        ZArgs a = chains[it.x];         // a copy: the token loop's stores would have its fields read again
+        a.narrow = narrow;
         const int64_t s = a.doc_off[it.y];
-        z_doc_any(&a, m, s, static_cast<int>(a.doc_off[it.y + 1] - s), sweep_of(a), wcnt);
+        const int len = static_cast<int>(a.doc_off[it.y + 1] - s);
+        DocRun r{a.w + s, a.z + s, len, a.seed, a.index_base + s, sweep_of(a), 0, len, 1};
+        z_doc<NW>(a, m, r, wcnt, nullptr);
         flush_warp_counters(a.stats, wcnt);
     }
+}
+
+template <int NW>
+__global__ void __launch_bounds__(32 * kMultiWarps, PULDA_MULTI_MINB) k_z_step_multi(const ZArgs *chains, const int2 *items,
+                                                                        int n_items, int *work, int kmax, int narrow) {
+    extern __shared__ __align__(16) uint32_t zsm[];
+    uint32_t *m = zsm + static_cast<size_t>(threadIdx.x >> 5) * z_dense_warp_words(kmax, narrow != 0);
+    u64 *wcnt = z_dense_counters(m, kmax, narrow != 0);     // beyond every chain's counts and token records
+    zero_warp_counters(wcnt);
+    z_multi_items<NW>(chains, items, n_items, work, m, wcnt, narrow);
 }
 
 // ============================================================ batches
@@ -776,7 +786,7 @@ __global__ void __launch_bounds__(32 * kMultiWarps, PULDA_MULTI_MINB) k_z_step_m
 // and clear every chain's row sums, per-sweep counters and the work queues.
 __device__ void batch_begin_sweep(const PhiArgs *chains, int n_chains, uint32_t *sweep, int *work) {
     if (threadIdx.x == 0) *sweep += 1u;
-    if (threadIdx.x < 4) work[threadIdx.x] = 0;
+    if (threadIdx.x < kBatchCounters) work[threadIdx.x] = 0;
     for (int c = 0; c < n_chains; ++c) {
         const PhiArgs &a = chains[c];
         for (int k = threadIdx.x; k < a.K; k += blockDim.x) a.S[k] = 0;
@@ -1012,10 +1022,23 @@ void launch_z_step(const ZArgs &a, int warps_per_block, int grid, cudaStream_t s
     z_step_kernel(a.K)<<<grid, 32 * warps_per_block, z_step_smem(a.K, warps_per_block, a.narrow != 0), st>>>(a);
 }
 
-static void launch_z_step_multi(const BatchLaunch &b, const int2 *items, int n, int *work, cudaStream_t st) {
+using ZMultiKernel = void (*)(const ZArgs *, const int2 *, int, int *, int, int);
+static ZMultiKernel z_multi_kernel(int kmax) {
+    switch (z_nw(kmax)) {
+        case 1: return k_z_step_multi<1>;
+        case 2: return k_z_step_multi<2>;
+        case 4: return k_z_step_multi<4>;
+        case 8: return k_z_step_multi<8>;
+        default: return k_z_step_multi<0>;
+    }
+}
+
+static void launch_z_step_multi(const BatchLaunch &b, const BatchForm &f, const int2 *items, int n, bool narrow, int *work,
+                                cudaStream_t st) {
     if (n <= 0) return;
-    k_z_step_multi<<<b.z_grid, 32 * b.z_warps, z_step_smem(b.kmax, b.z_warps, b.narrow != 0), st>>>(
-        b.z, items, n, work, b.kmax, b.narrow);
+    const int grid = std::min(f.z_grid, (n + b.z_warps - 1) / b.z_warps);
+    z_multi_kernel(f.kmax)<<<grid, 32 * b.z_warps, z_step_smem(f.kmax, b.z_warps, narrow), st>>>(b.z, items, n, work, f.kmax,
+                                                                                                narrow ? 1 : 0);
 }
 
 void launch_batch_sweep(const BatchLaunch &b, cudaStream_t st) {
@@ -1026,18 +1049,37 @@ void launch_batch_sweep(const BatchLaunch &b, cudaStream_t st) {
     k_phi_fixup_multi<<<b.n_chains, kFixBlock, 0, st>>>(b.phi);
     k_colptr_scan_multi<<<b.n_chains, 1024, 0, st>>>(b.phi);
     launch_phi_tables_multi(b.phi, b.phi_items, b.n_phi_items, b.kmax, st);
-    if (b.n_coop > 0) {
-        // the longest documents on CTAs, the rest one per warp beside them
-        const int head = b.n_wide + b.n_coop;
-        cudaEventRecord(b.ev_fork, st);
-        launch_z_step_multi(b, b.z_items, b.n_wide, b.work + 3, st);
-        launch_z_step_coop_multi(b.z, b.z_items + b.n_wide, b.n_coop, b.work + 2, b.kmax, b.coop_grid, st);
-        cudaStreamWaitEvent(b.stream2, b.ev_fork, 0);
-        launch_z_step_multi(b, b.z_items + head, b.n_z_items - head, b.work + 1, b.stream2);
-        cudaEventRecord(b.ev_join, b.stream2);
-        cudaStreamWaitEvent(st, b.ev_join, 0);
-    } else {
-        launch_z_step_multi(b, b.z_items, b.n_z_items, b.work + 1, st);
+    // The chains' documents by form, the longest ones of each on CTAs beside
+    // the others: every launch on a stream of its own (the CTAs first), so that
+    // one's last documents do not hold up the next.
+    cudaEventRecord(b.ev_fork, st);
+    int used = 0;
+    auto branch = [&](auto launch) {
+        cudaStream_t s = used == 0 ? st : b.side[used - 1];
+        if (used > 0) cudaStreamWaitEvent(s, b.ev_fork, 0);
+        launch(s);
+        ++used;
+    };
+    for (int f = 0; f < b.n_forms; ++f) {
+        const BatchForm &F = b.form[f];
+        const int2 *items = b.form_items + F.first;
+        if (F.n_wide + F.n_coop > 0)
+            branch([&](cudaStream_t s) {
+                launch_z_step_multi(b, F, items, F.n_wide, false, b.work + 2 + 3 * f, s);
+                launch_z_step_coop_multi(b.z, items + F.n_wide, F.n_coop, b.work + 3 + 3 * f, F.kmax, F.coop_grid, s);
+            });
+    }
+    for (int f = 0; f < b.n_forms; ++f) {
+        const BatchForm &F = b.form[f];
+        const int head = F.n_wide + F.n_coop;
+        if (F.n > head)
+            branch([&](cudaStream_t s) {
+                launch_z_step_multi(b, F, b.form_items + F.first + head, F.n - head, true, b.work + 4 + 3 * f, s);
+            });
+    }
+    for (int i = 1; i < used; ++i) {
+        cudaEventRecord(b.ev_join[i - 1], b.side[i - 1]);
+        cudaStreamWaitEvent(st, b.ev_join[i - 1], 0);
     }
 }
 
@@ -1051,8 +1093,10 @@ void launch_batch_sweep(const BatchLaunch &b, cudaStream_t st) {
 // the row sums and heavy-word histograms, which are read from L2.
 constexpr int kPersistThreads = 256;
 constexpr int kPersistWarps = kPersistThreads / 32;
+// Two CTAs per SM: five forms of the z-step in one kernel spill at more (99.9M
+// tokens in eight chains: a sweep takes 62 / 47 / 46 ms at 4 / 3 / 2).
 #ifndef PULDA_PERSIST_MINB
-#define PULDA_PERSIST_MINB 4
+#define PULDA_PERSIST_MINB 2
 #endif
 
 // A grid barrier with a bounded wait: thread 0 of each CTA arrives; the last
@@ -1149,23 +1193,24 @@ __global__ void __launch_bounds__(kPersistThreads, PULDA_PERSIST_MINB) k_batch_s
         }
     }
     if (!grid_barrier(b.bar, nb, err)) return;
-    // z-step, one warp per (chain, document), longest first
-    {
-        const int lane = threadIdx.x & 31;
+    // z-step, one warp per (chain, document), form by form (a warp goes on to
+    // the next form's documents as soon as one's are all taken)
+    if (static_cast<int>(threadIdx.x >> 5) < b.persist_z_warps) {
         uint32_t *m = psm + static_cast<size_t>(threadIdx.x >> 5) * z_dense_warp_words(b.kmax, b.narrow != 0);
         u64 *wcnt = z_dense_counters(m, b.kmax, b.narrow != 0);
-        const bool in = static_cast<int>(threadIdx.x >> 5) < b.persist_z_warps;
-        if (in) zero_warp_counters(wcnt);
-        while (in) {
-            int item = 0;
-            if (lane == 0) item = atomicAdd(&b.work[1], 1);
-            item = __shfl_sync(0xFFFFFFFFu, item, 0);
-            if (item >= b.n_z_items) break;
-            const int2 it = b.z_items[item];
-            const ZArgs &a = b.z[it.x];
-            const int64_t s0 = a.doc_off[it.y];
-            z_doc_any(&a, m, s0, static_cast<int>(a.doc_off[it.y + 1] - s0), sweep_of(a), wcnt);
-            flush_warp_counters(a.stats, wcnt);
+        zero_warp_counters(wcnt);
+#pragma unroll 1
+        for (int f = 0; f < b.n_forms; ++f) {
+            const int2 *items = b.form_items + b.form[f].first;
+            const int n = b.form[f].n;
+            int *work = b.work + 4 + 3 * f;
+            switch (z_nw(b.form[f].kmax)) {
+                case 1: z_multi_items<1>(b.z, items, n, work, m, wcnt, b.narrow); break;
+                case 2: z_multi_items<2>(b.z, items, n, work, m, wcnt, b.narrow); break;
+                case 4: z_multi_items<4>(b.z, items, n, work, m, wcnt, b.narrow); break;
+                case 8: z_multi_items<8>(b.z, items, n, work, m, wcnt, b.narrow); break;
+                default: z_multi_items<0>(b.z, items, n, work, m, wcnt, b.narrow);
+            }
         }
     }
 }
@@ -1226,9 +1271,10 @@ int batch_phi_blocks_per_sm(int kmax) {
 }
 
 int batch_z_blocks_per_sm(int kmax, int warps, bool narrow) {
-    allow_dynamic_smem(k_z_step_multi);
+    ZMultiKernel kern = z_multi_kernel(kmax);
+    allow_dynamic_smem(kern);
     int n = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_z_step_multi, 32 * warps, z_step_smem(kmax, warps, narrow));
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, 32 * warps, z_step_smem(kmax, warps, narrow));
     return n > 0 ? n : 1;
 }
 

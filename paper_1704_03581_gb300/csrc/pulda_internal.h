@@ -232,6 +232,10 @@ int z_coop_blocks_per_sm(int K);
 // 1,000 / 2,000 / none: 8.88 / 6.90 / 7.27 / 16.1.
 constexpr int64_t kCoopAutoDiv = 4500;
 constexpr int64_t kCoopAutoMin = 256;
+// The same over a batch's chains, whose passes are of mixed K (eight chains,
+// 6.3M tokens, K 50 to 500: a sweep takes 3.97 ms at N / 8000, 4.35 at N /
+// 4500, 4.68 at N / 2500).
+constexpr int64_t kBatchCoopDiv = 8000;
 // The same beside the grouped z-step, whose pass is faster and whose
 // documents each advance more slowly (four share a warp's issue slots).
 #ifndef PULDA_COOP_DIV_GROUPED
@@ -290,9 +294,20 @@ struct GridBarrier {
     unsigned gen;
 };
 
-// One sweep of many chains: six launches, every kernel over all chains'
-// work items, or one persistent launch doing the same.  Pointers are device
-// memory.
+// The chains of one form of the z-step (dense_words up to 1,024 topics, one
+// form above): their documents, n from `first` on in the form order, the n_wide
+// widest (2^16 tokens or more) one per warp, the next n_coop on CTAs.
+constexpr int kMaxForms = 5;
+struct BatchForm {
+    int kmax, first, n;
+    int n_wide, n_coop;
+    int z_grid, coop_grid;
+};
+constexpr int kBatchCounters = 2 + 3 * kMaxForms;     // work queues of a sweep
+
+// One sweep of many chains: a launch or a few per phase, every kernel over all
+// chains' work items (of a form, in the z-step), or one persistent launch doing
+// the same.  Pointers are device memory.
 struct BatchLaunch {
     const HeavyChunk *heavy;     // heavy-word histogram chunks of every chain
     int n_heavy;
@@ -301,19 +316,18 @@ struct BatchLaunch {
     int n_chains;
     const int2 *phi_items;       // (chain, word), most tokens first
     int n_phi_items;
-    const int2 *z_items;         // (chain, document), longest first
-    int n_z_items;
+    const int2 *form_items;      // (chain, document), form by form, longest first in each
+    BatchForm form[kMaxForms];
+    int n_forms;
     uint32_t *sweep;             // shared sweep counter, advanced by the first launch
-    int *work;                   // [4] dynamic work queues
+    int *work;                   // [kBatchCounters] dynamic work queues
     int kmax;                    // largest K of the chains
     int narrow;                  // 1: every document of every chain has fewer than 2^16 tokens
-    int phi_grid, z_grid, z_warps;
-    // the n_coop z_items after the first n_wide (2^16 tokens or more) go to the
-    // long-document z-step on `st`, the others to the one-warp kernel, the
-    // shorter ones on stream2 (forked and joined with the events)
-    int n_wide, n_coop, coop_grid;
-    cudaStream_t stream2;
-    cudaEvent_t ev_fork, ev_join;
+    int phi_grid, z_warps;
+    // streams beside the batch's for the z-step's launches, forked and joined
+    // with the events
+    cudaStream_t side[2 * kMaxForms - 1];
+    cudaEvent_t ev_fork, ev_join[2 * kMaxForms - 1];
     // the one-launch form: its grid (all CTAs resident) and barrier
     int persist_grid;
     GridBarrier *bar;

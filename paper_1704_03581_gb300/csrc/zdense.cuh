@@ -660,22 +660,4 @@ __device__ __forceinline__ void z_doc(const ZArgs &a, uint32_t *sm, DocRun &r, u
     else z_doc_regs<NW>(a, sm, r, wcnt, m0);
 }
 
-// The same with the form picked at run time (chains of different K in one
-// launch), each form a function of its own so that the largest does not set the
-// registers of all.
-template <int NW>
-__device__ __noinline__ void z_doc_form(const ZArgs *a, uint32_t *sm, int64_t first, int len, uint32_t sweep, u64 *wcnt) {
-    DocRun r{a->w + first, a->z + first, len, a->seed, a->index_base + first, sweep, 0, len, 1};
-    z_doc<NW>(*a, sm, r, wcnt, nullptr);
-}
-__device__ __forceinline__ void z_doc_any(const ZArgs *a, uint32_t *sm, int64_t first, int len, uint32_t sweep, u64 *wcnt) {
-    switch (z_nw(a->K)) {
-        case 1: z_doc_form<1>(a, sm, first, len, sweep, wcnt); break;
-        case 2: z_doc_form<2>(a, sm, first, len, sweep, wcnt); break;
-        case 4: z_doc_form<4>(a, sm, first, len, sweep, wcnt); break;
-        case 8: z_doc_form<8>(a, sm, first, len, sweep, wcnt); break;
-        default: z_doc_form<0>(a, sm, first, len, sweep, wcnt);
-    }
-}
-
 }  // namespace pulda
