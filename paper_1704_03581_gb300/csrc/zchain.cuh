@@ -1,4 +1,4 @@
-// The z-step of one long document by a CTA of three warps, for the least time
+// The z-step of one long document by a CTA of four warps, for the least time
 // per token.
 //
 // A document's tokens are strictly sequential, so a long document is one
@@ -10,17 +10,15 @@
 //     (bulk copies, one group of tokens ahead), so no load on the chain goes
 //     past shared memory;
 //   - warp 2 replays the drawn topics one group behind, on counts of its own,
-//     for the sweep's counters, and writes them out.
-// On the chain itself, the sum q m of token t + 1 is taken while token t is
-// drawn, from the counts without token t; the token's own weight is taken off
-// beforehand, and the one thing missing, the weight of token t's new topic, is
-// added to the scanned prefixes afterwards.  All sums are exact integers, so
-// they are those of the sequential order.  The topic within the found lane
-// comes from masked dp4a, every lane summing the lane's topics up to its own
-// (no scan), and the steps of token t + 1's scan stand between the votes,
-// shuffles and loads of token t's draw: they issue in program order, and each
-// would otherwise be waited for by itself.
-// The warps meet once per group.
+//     for the sweep's counters, and writes them out;
+//   - warp 3 sums q m for token t + 1 and scans it while token t is drawn, from
+//     counts (its own again) that lack token t.  The token's own weight is
+//     taken off beforehand; the one thing missing, the weight of token t's new
+//     topic, warp 0 adds to the scanned prefixes.  All sums are exact integers,
+//     so they are those of the sequential order.
+// Warp 0 finds the topic within the found lane by masked dp4a, every lane
+// summing the lane's topics up to its own, without a scan.  Warps 0 and 3 meet
+// once per token, all four once per group of tokens.
 #pragma once
 #include <cstdint>
 
@@ -30,7 +28,7 @@
 
 namespace pulda {
 
-constexpr int kChainThreads = 96;
+constexpr int kChainThreads = 128;
 
 // Tokens of a group: the ring holds three groups' rows (drawn, landed, on
 // their way), within what leaves room for several CTAs per SM where rows are
@@ -45,36 +43,46 @@ __host__ __device__ __forceinline__ int chain_group(int K) {
 // column's start}.
 constexpr int kChainRecWords = 12;
 
+// Warp 3 has counts of its own up to here; above, where they no longer fit,
+// warp 0 takes the next token's sum itself.
+constexpr int kChainAheadMaxK = 8192;
+__host__ __device__ __forceinline__ int chain_count_sets(int K) { return K <= kChainAheadMaxK ? 3 : 2; }
+
 // Shared memory of a CTA, in bytes: the barriers and counters; the drawn
-// topics of two groups; three blocks of records; two sets of counts (two
-// planes each) and, above 1024 topics, the lanes' bits; the ring.
+// topics of two groups; the coming token's sums; three blocks of records; the
+// sets of counts (two planes each) and, above 1024 topics, the lanes' bits; the
+// ring.
 struct ChainCtl {
     u64 full[3];                // a group's rows have arrived
     u64 cnt[6];                 // the counters
     u64 deadline;
     int item, stop;
-    int stops[2];               // after an even / odd group: a fast warp may already set the next one
+    int after[2];               // after an even / odd group (a fast warp may already set the next one):
+                                // kStop, kMixed: the next group holds a token without a dense row
     uint32_t drawn[16];         // two groups: position | flags
+    int last[2];                // the topic of an even / odd token
+    ulonglong2 ahead[2][32];    // an even / odd token's prefixes, by lane: with and without the lane's own sum
 };
-constexpr int kChainRecOff = 256;
+constexpr int kChainRecOff = 1280;
 static_assert(sizeof(ChainCtl) <= kChainRecOff, "the control block must fit");
 constexpr int kChainCountOff = kChainRecOff + 3 * 32 * 4 * kChainRecWords;
 static_assert(kChainCountOff % 16 == 0, "counts and rows are read 16 bytes at a time");
 __host__ __device__ __forceinline__ int chain_ring_off(int K) {
-    return kChainCountOff + 4 * 128 * dense_words(K) + (K > 1024 ? 16 * dense_words(K) : 0);
+    return kChainCountOff + 2 * chain_count_sets(K) * 128 * dense_words(K) + (K > 1024 ? 16 * dense_words(K) : 0);
 }
 __host__ __device__ __forceinline__ int chain_smem_bytes(int K) { return chain_ring_off(K) + 3 * chain_group(K) * dense_row_bytes(K); }
 // The same for chains of any K up to kmax in one launch (shorter groups can
 // take less room than the longer ones below them).
 __host__ __device__ __forceinline__ int chain_smem_bytes_upto(int kmax) {
     int most = 0;
-    const int edge[4] = {512, 1024, 8192, 16384};
+    const int edge[4] = {512, 1024, kChainAheadMaxK, kMaxK};
     for (int e : edge) {
         const int b = chain_smem_bytes(kmax < e ? kmax : e);
         most = b > most ? b : most;
     }
     return most;
 }
+constexpr int kStop = 1, kMixed = 2;
 // Flags of a drawn topic: taken from the alias table, kept for want of mass.
 constexpr uint32_t kDrawnAlias = 1u << 14, kDrawnZero = 1u << 15;
 static_assert(kMaxK <= (1 << 14), "positions must leave room for the flags");
@@ -167,44 +175,64 @@ struct ChainForm {
         }
         return sum;
     }
-    // Masks of the first `j + 1` of a lane's topics, j = this lane's number
-    // among them.
-    __device__ __forceinline__ static void topic_masks(int lane, uint32_t (&mask)[NW]) {
-        const int j = lane & (G::TPL - 1);
+    // The running sum of q m over lane L's topics up to this lane's: eight
+    // lanes share two words of every plane, each summing them up to its own
+    // topic (mask) with dp4a, and the groups of eight lanes before add their
+    // totals.
+    static constexpr int GW = NW >= 2 ? 2 : 1, GL = 4 * GW, GROUPS = NW / GW;
+    __device__ __forceinline__ static void topic_masks(int lane, uint32_t (&mask)[GW]) {
+        const int j = lane & (GL - 1);
 #pragma unroll
-        for (int x = 0; x < NW; ++x) {
+        for (int x = 0; x < GW; ++x) {
             const int t = j - 4 * x;                // last topic of word x that counts
             mask[x] = t >= 3 ? 0xFFFFFFFFu : t < 0 ? 0u : (1u << (8 * (t & 3) + 8)) - 1u;
         }
     }
-    // the running sum of q m over lane L's topics up to this lane's
     template <int P>
-    __device__ __forceinline__ u64 prefix(int L, const uint8_t *row, const uint8_t *m, const uint32_t (&mask)[NW]) const {
-        uint32_t q[3][NW];
+    __device__ __forceinline__ u64 prefix(int L, const uint8_t *row, const uint8_t *m, const uint32_t (&mask)[GW], int lane) const {
+        const int grp = (lane / GL) & (GROUPS - 1);
+        const int at = G::lane0(GL * grp) + L * G::STRIDE;
+        uint32_t q[3][GW], w[P][GW];
 #pragma unroll
-        for (int p = 0; p < 3; ++p) load_words<NW>(row + p * G::PB, L, q[p]);
+        for (int p = 0; p < 3; ++p) load_group(row + p * G::PB + at, q[p]);
+#pragma unroll
+        for (int p = 0; p < P; ++p) load_group(m + p * G::PB + at, w[p]);
         u64 sum = 0;
 #pragma unroll
         for (int p = 0; p < P; ++p) {
-            uint32_t w[NW];
-            load_words<NW>(m + p * G::PB, L, w);
             uint32_t s0 = 0, s1 = 0, s2 = 0;
 #pragma unroll
-            for (int x = 0; x < NW; ++x) {
-                s0 = __dp4a(w[x] & mask[x], q[0][x], s0);
-                s1 = __dp4a(w[x] & mask[x], q[1][x], s1);
-                s2 = __dp4a(w[x] & mask[x], q[2][x], s2);
+            for (int x = 0; x < GW; ++x) {
+                s0 = __dp4a(w[p][x] & mask[x], q[0][x], s0);
+                s1 = __dp4a(w[p][x] & mask[x], q[1][x], s1);
+                s2 = __dp4a(w[p][x] & mask[x], q[2][x], s2);
             }
             sum += (static_cast<u64>(s0 + (s1 << 8)) + (static_cast<u64>(s2) << 16)) << (8 * p);
         }
+        if constexpr (GROUPS > 1) {
+            u64 t[GROUPS - 1];
+#pragma unroll
+            for (int g = 0; g + 1 < GROUPS; ++g) t[g] = __shfl_sync(0xFFFFFFFFu, sum, GL * g + GL - 1);
+#pragma unroll
+            for (int g = 0; g + 1 < GROUPS; ++g) sum += grp > g ? t[g] : 0ull;
+        }
         return sum;
+    }
+    __device__ __forceinline__ static void load_group(const uint8_t *p, uint32_t (&w)[GW]) {
+        if constexpr (GW == 2) {
+            const uint2 v = *reinterpret_cast<const uint2 *>(p);
+            w[0] = v.x;
+            w[1] = v.y;
+        } else {
+            w[0] = *reinterpret_cast<const uint32_t *>(p);
+        }
     }
     // lane L's topic whose running sum passes res (position, or -1)
     template <int P>
     __device__ __forceinline__ int find(int L, u64 res, const uint8_t *row, const uint8_t *m, int lane) const {
-        uint32_t mask[NW];
+        uint32_t mask[GW];
         topic_masks(lane, mask);
-        const uint32_t f = __ballot_sync(0xFFFFFFFFu, res < prefix<P>(L, row, m, mask));
+        const uint32_t f = __ballot_sync(0xFFFFFFFFu, res < prefix<P>(L, row, m, mask, lane));
         return f ? G::lane0(__ffs(f) - 1) + L * G::STRIDE : -1;
     }
 };
@@ -262,97 +290,151 @@ struct ChainForm<0> {
     }
 };
 
-// What warp 0 carries from token to token.
+__device__ __forceinline__ void pair_barrier() { asm volatile("bar.sync 1, 64;" ::: "memory"); }     // warps 0 and 3
+
+// What warps 0 and 3 each carry from token to token.
 struct ChainState {
-    u64 sum, incl, B;           // the coming token's: this lane's sum, its prefix, the total; all without `prev`
     int prev;                   // the last token's new topic, not in the counts yet (at a document's
                                 // start the first token's topic, taken out of the counts)
     uint32_t top;               // a bound on every count
     uint32_t bad;               // a draw found no topic
+    u64 incl, below;            // without warp 3: the coming token's prefixes, without `prev`
 };
 
-// The lane's sum for the token of record part r1 from the counts at hand, less
-// the token itself.
-template <int NW, int P>
-__device__ __forceinline__ u64 chain_ahead(const ChainForm<NW> &form, const uint8_t *sm, const uint8_t *m, const uint4 r1, int lane) {
-    const uint32_t own = lane == form.owner(static_cast<int>(r1.x & 0xFFFFu)) ? r1.z : 0u;
-    return form.template dot<P>(sm + r1.y, m, lane) - own;
+// The last token's topic into the counts, this one's out.  Every lane stores
+// the same bytes, once every lane has read the old ones.
+template <int P>
+__device__ __forceinline__ void chain_update(uint8_t *m, int PB, int kold, ChainState &st) {
+    const uint32_t c1 = chain_count<P>(m, PB, st.prev) + 1u;
+    const uint32_t c0 = (st.prev == kold ? c1 : chain_count<P>(m, PB, kold)) - 1u;
+    __syncwarp();
+    chain_set<P>(m, PB, st.prev, c1);
+    chain_set<P>(m, PB, kold, c0);
+    st.top = max(st.top, c1);
 }
 
-// Warp 0: tokens [t, t + cnt) of a pass, every one of them and the one after
-// with a dense row (after the last token of a pass a stand-in, whose sums go
-// unused).
+// The lanes' sums, in the counts at hand, for the token of record part r1, less
+// the token itself; prefixes with and without the lane's own.
 template <int NW, int P>
-__device__ __forceinline__ void chain_group_fast(const ChainForm<NW> &form, uint8_t *sm, uint8_t *m, int t, int cnt, uint32_t *drawn,
-                                                 ChainState &st) {
+__device__ __forceinline__ ulonglong2 chain_sums(const ChainForm<NW> &form, const uint8_t *sm, const uint8_t *m, const uint4 r1, int lane) {
+    const u64 sum = form.template dot<P>(sm + r1.y, m, lane) - (lane == form.owner(static_cast<int>(r1.x & 0xFFFFu)) ? r1.z : 0u);
+    const u64 incl = warp_incl_scan<32>(sum);
+    return make_ulonglong2(incl, incl - sum);
+}
+
+// Where a pass stands: n tokens in ng groups of G, group g next.
+struct ChainPass {
+    int n, ng, G, g;
+    int done;                   // tokens drawn
+    int after;                  // what warp 1 said after the last group
+    __device__ __forceinline__ int group_tokens() const { return min(G, n - g * G); }
+    // the end of a group: all four warps
+    __device__ __forceinline__ void meet(const ChainCtl &ctl) {
+        done += group_tokens();
+        __syncthreads();
+        after = ctl.after[g & 1];
+        ++g;
+    }
+    __device__ __forceinline__ bool more() const { return g < ng && !(after & kStop); }
+};
+
+// Warp 3: the sums of the token after each of the coming groups' tokens, while
+// that one is drawn; for as long as counts stay in P planes.
+template <int NW, int P>
+__device__ __forceinline__ void chain_run_ahead(const ChainForm<NW> &form, uint8_t *sm, ChainCtl &ctl, uint8_t *m, ChainPass &ps,
+                                                ChainState &st) {
+    const int lane = threadIdx.x & 31;
+    const int PB = form.plane();
+    const uint4 *recs = reinterpret_cast<const uint4 *>(sm + kChainRecOff), *end = recs + 3 * 96;
+    int t = ps.g * ps.G;
+    const uint4 *rec = recs + 3 * (t % 96);
+    uint4 r1 = rec[1];
+    do {
+        const int cnt = ps.group_tokens();
+#pragma unroll 1
+        for (int u = 0; u < cnt; ++u, ++t) {
+            const int kold = static_cast<int>(r1.x & 0xFFFFu);
+            rec = rec + 3 == end ? recs : rec + 3;
+            const uint4 n1 = rec[1];
+            if (st.prev < 0) st.prev = ctl.last[(t + 1) & 1];           // token t - 1's, drawn meanwhile
+            if (n1.y != 0xFFFFFFFFu) {
+                // from the counts as they were, less this token's and its own
+                // topic (nothing here waits for a draw); then with the new
+                // topic of the token before, in the prefixes
+                const uint8_t *row = sm + n1.y;
+                const u64 sum = form.template dot<P>(row, m, lane) - (lane == form.owner(kold) ? n1.w : 0u) -
+                                (lane == form.owner(static_cast<int>(n1.x & 0xFFFFu)) ? n1.z : 0u);
+                const uint32_t dn = form.weight(row, st.prev);
+                const int ow = form.owner(st.prev);
+                const u64 incl = warp_incl_scan<32>(sum);
+                ctl.ahead[(t + 1) & 1][lane] = make_ulonglong2(incl + (lane >= ow ? dn : 0u), incl - sum + (lane > ow ? dn : 0u));
+            }
+            chain_update<P>(m, PB, kold, st);
+            st.prev = -1;
+            r1 = n1;
+            pair_barrier();
+        }
+        ps.meet(ctl);
+    } while (ps.more() && (P == 2 || st.top + static_cast<uint32_t>(ps.G) <= 255u));
+}
+
+// Warp 0: the coming groups, while every token of theirs has a dense row and
+// counts stay in P planes.
+template <int NW, int P>
+__device__ __forceinline__ void chain_run_fast(const ChainForm<NW> &form, uint8_t *sm, ChainCtl &ctl, uint8_t *m, ChainPass &ps,
+                                               ChainState &st) {
     using G = DenseGeo<NW>;
     const int lane = threadIdx.x & 31;
-    const uint4 *recs = reinterpret_cast<const uint4 *>(sm + kChainRecOff);
-    uint32_t mask[NW];
+    uint32_t mask[ChainForm<NW>::GW];
     form.topic_masks(lane, mask);
-    const uint4 *rec = recs + 3 * (t % 96), *last = recs + 3 * 95;
+    const uint4 *recs = reinterpret_cast<const uint4 *>(sm + kChainRecOff), *end = recs + 3 * 96;
+    int t = ps.g * ps.G;
+    const uint4 *rec = recs + 3 * (t % 96);
     uint4 r1 = rec[1];
+    uint32_t delta = form.weight(sm + r1.y, st.prev);
+    do {
+        const int cnt = ps.group_tokens();
+        uint32_t *drawn = ctl.drawn + 8 * (ps.g & 1);
 #pragma unroll 1
-    for (int u = 0; u < cnt; ++u) {
-        const uint4 r0 = rec[0];
-        rec = rec == last ? recs : rec + 3;
-        const uint4 n1 = rec[1];                // the next token's
-        const u64 At = (static_cast<u64>(r0.y) << 32) | r0.x, U = (static_cast<u64>(r0.w) << 32) | r0.z;
-        const int kold = static_cast<int>(r1.x & 0xFFFFu);
-        const uint8_t *row = sm + r1.y, *nrow = sm + n1.y;
-        const uint32_t delta = form.weight(row, st.prev), dn = form.weight(nrow, st.prev);
-        const int ow = G::owner(st.prev);
-        // the next token's sum: from the counts as they were before this token
-        // (these loads do not wait for the previous draw), less this token's
-        // and its own topic, and with the previous one's new topic
-        const u64 before = form.template dot<P>(nrow, m, lane);
-        // the last token's topic in, this one out: m^{-i}.  Every lane stores
-        // the same bytes
-        const uint32_t c1 = chain_count<P>(m, G::PB, st.prev) + 1u;
-        const uint32_t c0 = (st.prev == kold ? c1 : chain_count<P>(m, G::PB, kold)) - 1u;
-        __syncwarp();                           // every lane has read the old counts
-        chain_set<P>(m, G::PB, st.prev, c1);
-        chain_set<P>(m, G::PB, kold, c0);
-        st.top = max(st.top, c1);
-        const u64 upto = st.incl + (lane >= ow ? delta : 0u), mine = st.sum + (lane == ow ? delta : 0u);
-        st.sum = before + (lane == ow ? dn : 0u) - (lane == G::owner(kold) ? n1.w : 0u) -
-                 (lane == G::owner(static_cast<int>(n1.x & 0xFFFFu)) ? n1.z : 0u);
-        u64 v = st.sum;
-        const u64 T = At + ((st.B + delta) << kFracBits);
-        const u64 rr = __umul64hi(U, T);
-        const u64 rb = (rr - At) >> kFracBits;
-        u64 w = shfl_up64(v, 1);
-        // no lane passes for an alias draw (rr < At wraps round) or without any mass
-        const uint32_t bal = __ballot_sync(0xFFFFFFFFu, rb < upto);
-        v += lane >= 1 ? w : 0u;
-        w = shfl_up64(v, 2);
-        const int L = (__ffs(bal) - 1) & 31;
-        v += lane >= 2 ? w : 0u;
-        w = shfl_up64(v, 4);
-        const u64 res = __shfl_sync(0xFFFFFFFFu, rb - (upto - mine), L);
-        v += lane >= 4 ? w : 0u;
-        w = shfl_up64(v, 8);
-        const u64 pre = form.template prefix<P>(L, row, m, mask);
-        v += lane >= 8 ? w : 0u;
-        w = shfl_up64(v, 16);
-        const uint32_t f = __ballot_sync(0xFFFFFFFFu, res < pre);
-        v += lane >= 16 ? w : 0u;
-        st.incl = v;
-        st.B = __shfl_sync(0xFFFFFFFFu, v, 31);
-        uint32_t knew = static_cast<uint32_t>(G::lane0((__ffs(f) - 1) & 31) + L * G::STRIDE);
-        knew = rr < At ? (r1.x >> 16) | kDrawnAlias : bal ? knew : static_cast<uint32_t>(kold) | kDrawnZero;
-        st.bad |= bal != 0 && f == 0 ? 1u : 0u;
-        drawn[u] = knew;
-        st.prev = static_cast<int>(knew & 0x3FFFu);
-        r1 = n1;
-    }
-    __syncwarp();
+        for (int u = 0; u < cnt; ++u, ++t) {
+            const uint4 r0 = rec[0];
+            rec = rec + 3 == end ? recs : rec + 3;
+            const uint4 n1 = rec[1];
+            const uint8_t *row = sm + r1.y, *nrow = sm + (n1.y == 0xFFFFFFFFu ? r1.y : n1.y);
+            const u64 At = (static_cast<u64>(r0.y) << 32) | r0.x, U = (static_cast<u64>(r0.w) << 32) | r0.z;
+            const int kold = static_cast<int>(r1.x & 0xFFFFu);
+            const ulonglong2 mine = ctl.ahead[t & 1][lane];
+            const u64 all = ctl.ahead[t & 1][31].x;
+            const int ow = G::owner(st.prev);
+            chain_update<P>(m, G::PB, kold, st);
+            const u64 upto = mine.x + (lane >= ow ? delta : 0u), below = mine.y + (lane > ow ? delta : 0u);
+            const u64 T = At + ((all + delta) << kFracBits);
+            const u64 rr = __umul64hi(U, T);
+            const u64 rb = (rr - At) >> kFracBits;
+            // no lane passes for an alias draw (rr < At wraps round) or without any
+            // mass: the outcome then does not wait for the rest
+            const uint32_t bal = __ballot_sync(0xFFFFFFFFu, rb < upto);
+            const uint32_t other = rr < At ? (r1.x >> 16) | kDrawnAlias : static_cast<uint32_t>(kold) | kDrawnZero;
+            const int L = (__ffs(bal) - 1) & 31;
+            const u64 res = __shfl_sync(0xFFFFFFFFu, rb - below, L);
+            const uint32_t f = __ballot_sync(0xFFFFFFFFu, res < form.template prefix<P>(L, row, m, mask, lane));
+            const uint32_t knew = bal ? static_cast<uint32_t>(G::lane0((__ffs(f) - 1) & 31) + L * G::STRIDE) : other;
+            st.prev = static_cast<int>(knew & 0x3FFFu);
+            ctl.last[t & 1] = st.prev;
+            delta = form.weight(nrow, st.prev);         // the next token's, on its way over the barrier
+            drawn[u] = knew;
+            st.bad |= bal != 0 && f == 0 ? 1u : 0u;
+            r1 = n1;
+            pair_barrier();
+        }
+        ps.meet(ctl);
+    } while (ps.more() && !(ps.after & kMixed) && (P == 2 || st.top + static_cast<uint32_t>(ps.G) <= 255u));
 }
 
 // The same for any group: tokens without a dense row among them, or K > 1024.
 template <int NW, int P>
-__device__ __forceinline__ void chain_group_any(const ZArgs &a, const ChainForm<NW> &form, uint8_t *sm, uint8_t *m, int t, int cnt,
-                                                uint32_t *drawn, ChainState &st) {
+__device__ __forceinline__ void chain_group_any(const ZArgs &a, const ChainForm<NW> &form, uint8_t *sm, ChainCtl &ctl, uint8_t *m, int t,
+                                                int cnt, bool paired, uint32_t *drawn, ChainState &st) {
     const int lane = threadIdx.x & 31;
     const int PB = form.plane();
     const uint4 *recs = reinterpret_cast<const uint4 *>(sm + kChainRecOff);
@@ -362,22 +444,22 @@ __device__ __forceinline__ void chain_group_any(const ZArgs &a, const ChainForm<
         const uint4 r0 = rec[0], r1 = rec[1], n1 = recs[3 * ((t + 1) % 96) + 1];
         const u64 At = (static_cast<u64>(r0.y) << 32) | r0.x, U = (static_cast<u64>(r0.w) << 32) | r0.z;
         const int kold = static_cast<int>(r1.x & 0xFFFFu);
-        const bool dense = r1.y != 0xFFFFFFFFu, ahead = n1.y != 0xFFFFFFFFu;
+        const bool dense = r1.y != 0xFFFFFFFFu;
         const uint8_t *row = sm + r1.y;
         const uint32_t delta = dense ? form.weight(row, st.prev) : 0u;
         const int ow = form.owner(st.prev);
-        const uint32_t c1 = chain_count<P>(m, PB, st.prev) + 1u;
-        const uint32_t c0 = (st.prev == kold ? c1 : chain_count<P>(m, PB, kold)) - 1u;
+        const ulonglong2 mine = paired ? ctl.ahead[t & 1][lane] : make_ulonglong2(st.incl, st.below);
+        chain_update<P>(m, PB, kold, st);
         __syncwarp();
-        chain_set<P>(m, PB, st.prev, c1);
-        chain_set<P>(m, PB, kold, c0);
-        __syncwarp();
-        st.top = max(st.top, c1);
-        const u64 upto = st.incl + (lane >= ow ? delta : 0u), mine = st.sum + (lane == ow ? delta : 0u), B = st.B + delta;
-        if (ahead) st.sum = chain_ahead<NW, P>(form, sm, m, n1, lane);
+        const u64 upto = mine.x + (lane >= ow ? delta : 0u), below = mine.y + (lane > ow ? delta : 0u);
         uint32_t knew;
+        if (!paired && n1.y != 0xFFFFFFFFu) {
+            const ulonglong2 x = chain_sums<NW, P>(form, sm, m, n1, lane);
+            st.incl = x.x;
+            st.below = x.y;
+        }
         if (dense) {
-            const u64 rr = __umul64hi(U, At + (B << kFracBits));
+            const u64 rr = __umul64hi(U, At + (__shfl_sync(0xFFFFFFFFu, upto, 31) << kFracBits));
             if (rr < At) {
                 knew = (r1.x >> 16) | kDrawnAlias;
             } else {
@@ -386,7 +468,7 @@ __device__ __forceinline__ void chain_group_any(const ZArgs &a, const ChainForm<
                 knew = static_cast<uint32_t>(kold) | kDrawnZero;
                 if (bal) {
                     const int L = __ffs(bal) - 1;
-                    const u64 res = __shfl_sync(0xFFFFFFFFu, rb - (upto - mine), L);
+                    const u64 res = __shfl_sync(0xFFFFFFFFu, rb - below, L);
                     const int k = form.template find<P>(L, res, row, m, lane);
                     st.bad |= k < 0 ? 1u : 0u;
                     knew = static_cast<uint32_t>(k < 0 ? kold : k);
@@ -401,12 +483,10 @@ __device__ __forceinline__ void chain_group_any(const ZArgs &a, const ChainForm<
                                       [&](int x) { return form.pos(x); });
             knew = static_cast<uint32_t>(k) | (c & (1u << 6) ? kDrawnAlias : 0u) | (c & (1u << 12) ? kDrawnZero : 0u);
         }
-        if (ahead) {
-            st.incl = warp_incl_scan<32>(st.sum);
-            st.B = __shfl_sync(0xFFFFFFFFu, st.incl, 31);
-        }
         drawn[u] = knew;
         st.prev = static_cast<int>(knew & 0x3FFFu);
+        ctl.last[t & 1] = st.prev;
+        if (paired) pair_barrier();
         __syncwarp();
     }
 }
@@ -417,7 +497,7 @@ __device__ __forceinline__ void chain_group_any(const ZArgs &a, const ChainForm<
 template <int NW>
 __device__ __forceinline__ void z_doc_chain(const ZArgs &a, uint8_t *sm, DocRun &r, uint32_t &phases) {
     const int lane = threadIdx.x & 31;
-    const int role = threadIdx.x >> 5;      // 0: the chain, 1: records and rows, 2: counters and topics
+    const int role = threadIdx.x >> 5;      // 0: the chain, 1: records and rows, 2: counters and topics, 3: sums ahead
     const int K = a.K;
     if (r.len == 0 || r.budget <= 0) return;
     ChainCtl &ctl = *reinterpret_cast<ChainCtl *>(sm);
@@ -426,18 +506,20 @@ __device__ __forceinline__ void z_doc_chain(const ZArgs &a, uint8_t *sm, DocRun 
     ChainForm<NW> form(K);
     const int PB = form.plane();
     auto pos = [&](int k) { return form.pos(k); };
-    // warps 0 and 2 each keep the document's counts
-    DocCounts m{sm + kChainCountOff + role * PB, PB, 0};
-    if (role != 1) build_counts(a, m, r, nullptr, 2, pos);
+    // warps 0, 2 and 3 each keep the document's counts
+    const bool paired = K <= kChainAheadMaxK;
+    DocCounts m{sm + kChainCountOff + (role == 0 ? 0 : role == 2 ? 2 * PB : 4 * PB), PB, 0};
+    if (role == 0 || role == 2 || (role == 3 && paired)) build_counts(a, m, r, nullptr, 2, pos);
     ChainState st{};
     st.prev = -1;
+    bool begun = false;
     int kd = 0;
-    if (role == 0) {
+    if (role == 0 || (role == 3 && paired)) {
         uint32_t top = 0;
         for (int p = lane; p < PB; p += 32) top = max(top, m.b[p] | (static_cast<uint32_t>(m.b[p + PB]) << 8));
         st.top = __reduce_max_sync(0xFFFFFFFFu, top);
     } else if (role == 2) {
-        kd = static_cast<int>(__reduce_add_sync(0xFFFFFFFFu, static_cast<unsigned>(form.init_bits(m, sm + kChainCountOff + 4 * PB, lane))));
+        kd = static_cast<int>(__reduce_add_sync(0xFFFFFFFFu, static_cast<unsigned>(form.init_bits(m, sm + kChainCountOff + 2 * chain_count_sets(K) * PB, lane))));
     }
     const int colmax = a.path == 1 ? 0x7FFFFFFF : -1;
     const uint32_t sweep_end = r.sweep + static_cast<uint32_t>(r.max_pass_end);
@@ -447,18 +529,24 @@ __device__ __forceinline__ void z_doc_chain(const ZArgs &a, uint8_t *sm, DocRun 
         const int p0 = r.pos;
         const int n = static_cast<int>(min(static_cast<int64_t>(r.len - p0), r.budget));
         const int ng = (n + G - 1) / G;
-        auto stage = [&](int b) {
-            const int t = 32 * b + lane;
+        StagedToken tok;
+        auto record = [&](int t) {
             uint4 *rec = recs + 3 * (t % 96);
             if (t == n) rec[1] = make_uint4(0u, static_cast<uint32_t>(ring), 0u, 0u);     // the stand-in after the last token
             if (t >= n) return;
-            uint4 x[2];
-            uint32_t d;
-            stage_token(a, r, p0 + t, x, &d, colmax, pos);
-            rec[0] = make_uint4(x[0].z, x[0].w, x[1].y, x[1].x);
-            rec[1] = make_uint4((x[1].w >> 16) | (x[0].y & 0xFFFF0000u),
-                                d == 0xFFFFFFFFu ? d : static_cast<uint32_t>(ring + (t % (3 * G)) * RB), 0u, d);
-            rec[2] = make_uint4(x[0].x, x[0].y & 0xFFFFu, x[1].w & 0xFFFFu, x[1].z);
+            const uint32_t ka = static_cast<uint32_t>(pos(tok.load_alias(a)));
+            rec[0] = make_uint4(static_cast<uint32_t>(tok.A), static_cast<uint32_t>(tok.A >> 32), tok.x.y, tok.x.x);
+            rec[1] = make_uint4(static_cast<uint32_t>(pos(tok.topic)) | (ka << 16),
+                                tok.row == 0xFFFFFFFFu ? tok.row : static_cast<uint32_t>(ring + (t % (3 * G)) * RB), 0u, tok.row);
+            rec[2] = make_uint4(static_cast<uint32_t>(tok.col), static_cast<uint32_t>(static_cast<u64>(tok.col) >> 32),
+                                static_cast<uint32_t>(tok.n_w), static_cast<uint32_t>(tok.word));
+        };
+        // block b, a step at a time (lane l its token l)
+        auto stage = [&](int b, int step) {
+            const int t = 32 * b + lane;
+            if (step == 0 && t < n) tok.load_token(a, r, p0 + t);
+            if (step == 1 && t < n) tok.load_word(a, colmax);
+            if (step == 2) record(t);
         };
         // group g's rows on their way (lane u < G its token u)
         auto fetch = [&](int g) {
@@ -488,7 +576,13 @@ __device__ __forceinline__ void z_doc_chain(const ZArgs &a, uint8_t *sm, DocRun 
                     if (t > 0) r1->w = form.weight(sm + r1->y, static_cast<int>(recs[3 * ((t - 1) % 96) + 1].x & 0xFFFFu));
                 }
             }
+            __syncwarp();
             return ok;
+        };
+        // whether group g holds a token without a row
+        auto mixed = [&](int g) {
+            const int t = g * G + lane;
+            return __any_sync(0xFFFFFFFFu, lane < G && t < n && recs[3 * (t % 96) + 1].y == 0xFFFFFFFFu) != 0;
         };
         // the counters and topics of group g, as drawn
         auto replay = [&](int g) {
@@ -535,7 +629,8 @@ __device__ __forceinline__ void z_doc_chain(const ZArgs &a, uint8_t *sm, DocRun 
             add_block_counts(ctl.cnt, lane, cnt, c_min, c_cnt, c_int);
         };
         __syncthreads();            // the last pass's topics are written and its records done with
-        stage(role);
+        if (role < 3)
+            for (int step = 0; step < 3; ++step) stage(role, step);
         __syncthreads();
         bool ok = true;
         if (role == 1) {
@@ -543,61 +638,74 @@ __device__ __forceinline__ void z_doc_chain(const ZArgs &a, uint8_t *sm, DocRun 
             if (ng > 1) fetch(1);
             ok = landed(0);
             if (ng > 1) ok = landed(1) && ok;
-            if (lane == 0) ctl.stop = ok ? 0 : 1;
+            const bool mix = mixed(0);
+            if (lane == 0) ctl.stop = (ok ? 0 : kStop) | (mix ? kMixed : 0);
         }
         __syncthreads();
-        stop = ctl.stop != 0;
-        int done = 0;
-        if (role == 0 && !stop) {
+        ChainPass ps{n, ng, G, 0, 0, ctl.stop};
+        if ((role == 0 || (role == 3 && paired)) && ps.more()) {
             const uint4 r1 = recs[1];
-            if (st.prev < 0) {
+            if (!begun) {
                 st.prev = static_cast<int>(r1.x & 0xFFFFu);
-                chain_set<2>(m.b, PB, st.prev, chain_count<2>(m.b, PB, st.prev) - 1u);
+                const uint32_t c = chain_count<2>(m.b, PB, st.prev) - 1u;
+                __syncwarp();
+                chain_set<2>(m.b, PB, st.prev, c);
                 __syncwarp();
             }
-            if (r1.y != 0xFFFFFFFFu) {
-                st.sum = chain_ahead<NW, 2>(form, sm, m.b, r1, lane);
-                st.incl = warp_incl_scan<32>(st.sum);
-                st.B = __shfl_sync(0xFFFFFFFFu, st.incl, 31);
+            if (r1.y != 0xFFFFFFFFu && (role == 3) == paired) {
+                const ulonglong2 x = chain_sums<NW, 2>(form, sm, m.b, r1, lane);
+                st.incl = x.x;
+                st.below = x.y;
+                if (paired) ctl.ahead[0][lane] = x;
             }
+            begun = true;
         }
-        for (int g = 0; g < ng && !stop; ++g) {
-            const int t0 = g * G, cnt = min(G, n - t0);
+        __syncthreads();
+        while (ps.more()) {
+            const int g = ps.g, t0 = g * G, cnt = ps.group_tokens();
+            const bool one = st.top + static_cast<uint32_t>(G) <= 255u;      // counts stay in one plane
             if (role == 0) {
                 uint32_t *drawn = ctl.drawn + 8 * (g & 1);
-                const bool one = st.top + static_cast<uint32_t>(G) <= 255u;      // counts stay in one plane
                 if constexpr (NW > 0) {
-                    // every token and the next group's first with a row
-                    const uint32_t y = lane <= cnt ? recs[3 * ((t0 + lane) % 96) + 1].y : 0u;
-                    if (!__any_sync(0xFFFFFFFFu, y == 0xFFFFFFFFu)) {
-                        if (one) chain_group_fast<NW, 1>(form, sm, m.b, t0, cnt, drawn, st);
-                        else chain_group_fast<NW, 2>(form, sm, m.b, t0, cnt, drawn, st);
-                    } else {
-                        chain_group_any<NW, 2>(a, form, sm, m.b, t0, cnt, drawn, st);
+                    if (!(ps.after & kMixed)) {
+                        if (one) chain_run_fast<NW, 1>(form, sm, ctl, m.b, ps, st);
+                        else chain_run_fast<NW, 2>(form, sm, ctl, m.b, ps, st);
+                        continue;
                     }
+                    chain_group_any<NW, 2>(a, form, sm, ctl, m.b, t0, cnt, paired, drawn, st);
                 } else {
-                    if (one) chain_group_any<NW, 1>(a, form, sm, m.b, t0, cnt, drawn, st);
-                    else chain_group_any<NW, 2>(a, form, sm, m.b, t0, cnt, drawn, st);
+                    if (one) chain_group_any<NW, 1>(a, form, sm, ctl, m.b, t0, cnt, paired, drawn, st);
+                    else chain_group_any<NW, 2>(a, form, sm, ctl, m.b, t0, cnt, paired, drawn, st);
+                }
+            } else if (role == 3) {
+                if (paired) {
+                    if (one) chain_run_ahead<NW, 1>(form, sm, ctl, m.b, ps, st);
+                    else chain_run_ahead<NW, 2>(form, sm, ctl, m.b, ps, st);
+                    continue;
                 }
             } else if (role == 1) {
                 if (g + 2 < ng) fetch(g + 2);
-                // block b - 1 was drawn before the last group, and is replayed
-                const int b = (t0 - G) >> 5;
-                if (g > 0 && ((t0 - G) & 31) == 0 && b > 0 && 32 * (b + 2) <= n) {
-                    stage(b + 2);
+                // block b - 1 was drawn before this block's second group, and is
+                // replayed then: block b + 2 takes its place, a step a group, so
+                // that no step's loads are waited for
+                const int b = t0 >> 5, step = (t0 & 31) / G - 1;
+                if (b > 0 && 32 * (b + 2) <= n) {
+                    if (step >= 0 && step < 3) stage(b + 2, step);
                     __syncwarp();
                 }
                 if (g + 2 < ng) ok = landed(g + 2);
                 const bool late = ((t0 + cnt) & 31) == 0 && r.deadline != ~0ull && global_ns() >= r.deadline;
-                if (lane == 0) ctl.stops[g & 1] = late || !ok;
+                const bool mix = g + 1 < ng && mixed(g + 1);
+                if (lane == 0) ctl.after[g & 1] = (late || !ok ? kStop : 0) | (mix ? kMixed : 0);
             } else if (g > 0) {
                 replay(g - 1);
             }
-            done += cnt;
-            __syncthreads();
-            stop = ctl.stops[g & 1] != 0;
+            ps.meet(ctl);
         }
+        const int done = ps.done;
+        stop = (ps.after & kStop) != 0;
         if (role == 2 && done > 0) replay((done - 1) / G);
+        if (role == 3 && done > 0) st.prev = ctl.last[(done - 1) & 1];
         if (role == 0 && lane == 0 && st.bad) atomicOr(&a.stats[ST_ERROR], ERR_INTERNAL);
         r.budget -= done;
         r.pos += done;

@@ -79,32 +79,52 @@ __device__ __forceinline__ int alias_outcome(const ZArgs &a, int64_t e, uint32_t
     return guard_index(u < a.athr[e] ? a.topic[e] : a.atopic[e], a.K, a.stats);
 }
 
-// Stages what depends only on token i of run r: its word, Philox words, alias
-// outcome and column,
+// What depends only on a token, gathered in three steps that each wait for the
+// loads of the one before: its word, topic and Philox words; its word's
+// column, sigma_a and dense row (~0 when it is to be summed over its column: it
+// has at most colmax topics, or no row); its alias outcome.
+struct StagedToken {
+    int word, topic;
+    U4 x;
+    int64_t col;
+    int n_w;
+    u64 A;
+    uint32_t row;
+    __device__ __forceinline__ void load_token(const ZArgs &a, const DocRun &r, int i) {
+        word = r.w[i];
+        topic = guard_index(r.z[i], a.K, a.stats);
+        const uint64_t t = static_cast<uint64_t>(r.index_base + i);
+        x = draw(r.seed, static_cast<uint32_t>(t), static_cast<uint32_t>(t >> 32), r.sweep, TAG_Z, 0);
+    }
+    __device__ __forceinline__ void load_word(const ZArgs &a, int colmax) {
+        col = a.col_ptr[word];
+        n_w = static_cast<int>(a.col_ptr[word + 1] - col);
+        A = a.A[word];
+        const uint32_t d = static_cast<uint32_t>(a.drow[word]);
+        row = n_w > colmax ? d : 0xFFFFFFFFu;
+    }
+    __device__ __forceinline__ int load_alias(const ZArgs &a) const {
+        return n_w > 0 ? alias_outcome(a, col + __umulhi(x.z, static_cast<uint32_t>(n_w)), x.w) : 0;
+    }
+};
+
+// Stages token i of run r for the one-warp kernel,
 //   rec2[0] = {column start (low 32), column start >> 32 | alias outcome << 16, sigma_a (lo, hi)}
 //   rec2[1] = {Philox x0, x1, word, K_v | old topic << 16}
-// and its word's dense row, or ~0 when it is to be summed over its column: it
-// has at most colmax topics, or no row.  Topics are staged as their positions,
-// pos(k) (column starts are below 2^48, K_v <= 16384, positions < 16384).
+// and its dense row.  Topics are staged as their positions, pos(k) (column
+// starts are below 2^48, K_v <= 16384, positions < 16384).
 template <typename Pos>
 __device__ __forceinline__ void stage_token(const ZArgs &a, const DocRun &r, int i, uint4 *rec2, uint32_t *drow, int colmax, Pos pos) {
-    const int wv = r.w[i];
-    const int zo = guard_index(r.z[i], a.K, a.stats);
-    const uint64_t t = static_cast<uint64_t>(r.index_base + i);
-    const U4 x = draw(r.seed, static_cast<uint32_t>(t), static_cast<uint32_t>(t >> 32), r.sweep, TAG_Z, 0);
-    const int64_t cb = a.col_ptr[wv];
-    const int nw = static_cast<int>(a.col_ptr[wv + 1] - cb);
-    const u64 Av = a.A[wv];
-    int ta = 0;
-    if (nw > 0) {
-        const uint32_t sl = __umulhi(x.z, static_cast<uint32_t>(nw));
-        ta = pos(alias_outcome(a, cb + sl, x.w));
-    }
-    rec2[0] = make_uint4(static_cast<uint32_t>(cb),
-                         static_cast<uint32_t>(static_cast<u64>(cb) >> 32) | (static_cast<uint32_t>(ta) << 16),
-                         static_cast<uint32_t>(Av), static_cast<uint32_t>(Av >> 32));
-    rec2[1] = make_uint4(x.x, x.y, static_cast<uint32_t>(wv), static_cast<uint32_t>(nw) | (static_cast<uint32_t>(pos(zo)) << 16));
-    *drow = nw > colmax ? static_cast<uint32_t>(a.drow[wv]) : 0xFFFFFFFFu;
+    StagedToken s;
+    s.load_token(a, r, i);
+    s.load_word(a, colmax);
+    const int ta = pos(s.load_alias(a));
+    rec2[0] = make_uint4(static_cast<uint32_t>(s.col),
+                         static_cast<uint32_t>(static_cast<u64>(s.col) >> 32) | (static_cast<uint32_t>(ta) << 16),
+                         static_cast<uint32_t>(s.A), static_cast<uint32_t>(s.A >> 32));
+    rec2[1] = make_uint4(s.x.x, s.x.y, static_cast<uint32_t>(s.word),
+                         static_cast<uint32_t>(s.n_w) | (static_cast<uint32_t>(pos(s.topic)) << 16));
+    *drow = s.row;
 }
 
 

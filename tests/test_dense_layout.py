@@ -59,7 +59,7 @@ int main() {
         }
         const int G = chain_group(K), ring = chain_ring_off(K);
         CHECK(G >= 1 && G <= 8 && 32 % G == 0, "K=%d: groups of %d", K, G);
-        CHECK(ring % 16 == 0 && kChainCountOff + 4 * pb + (K > 1024 ? 64 * C : 0) <= ring, "K=%d: ring at %d", K, ring);
+        CHECK(ring % 16 == 0 && kChainCountOff + 2 * chain_count_sets(K) * pb + (K > 1024 ? 64 * C : 0) <= ring, "K=%d: ring at %d", K, ring);
         CHECK(chain_smem_bytes(K) == ring + 3 * G * 3 * pb && chain_smem_bytes(K) <= 227 * 1024, "K=%d: %d bytes", K, chain_smem_bytes(K));
     }
     int most = 0;
