@@ -521,7 +521,7 @@ def run_pulda(args, corpus, rank: int, world: int):
         "roofline_issue": issue_roofline(K * corpus.N / (z_ms / 1000.0), (clk or {}).get("sm_mhz")),
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic,
-                     "kernel": "k_z_step" if layout["docs_per_warp"] == 1 else "k_z_step_grouped",
+                     "kernel": {1: "k_z_step", 2: "k_z_step_pairs", 4: "k_z_step_grouped"}[layout["docs_per_warp"]],
                      "peak_kind": f"{peak_kind} HBM copy bandwidth",
                      "algorithmic_bytes_per_launch": zbytes / K,
                      "bytes_model": "12 B per token + 6 B per min(K_d, K_v) element + 8 B per alias draw + "
@@ -531,7 +531,7 @@ def run_pulda(args, corpus, rank: int, world: int):
                                                    "min(K_d, K_v) element + 6 B per alias draw + 8 B per document"},
         "gpu_launches": kernels_per_sweep(corpus.w, args.phi_mode, layout,
                                           int(args.slice_len > 0 and np.diff(corpus.doc_off).max() > args.slice_len)) * K,
-        "z_kernel": (f"{'four documents' if layout['docs_per_warp'] == 4 else 'one document'} per warp; "
+        "z_kernel": (f"{ {1: 'one document', 2: 'two documents', 4: 'four documents'}[layout['docs_per_warp']] } per warp; "
                      f"{layout['coop_docs']} longest documents on one CTA each"),
         "clocks": clk,
         "cpu_baseline": cpu,

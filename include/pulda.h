@@ -58,12 +58,11 @@ typedef struct {
                                results are identical */
     int32_t warps_per_block;/* warp-per-document z-step: warps per CTA, 1..4; 0 = 4, halved
                                while the CTA's shared memory would pass 160 KB */
-    int32_t docs_per_warp;  /* z-step documents per warp: 0 = auto (one: measured faster at
-                               every K), 1 = one, 4 = four (needs K <= 1024; falls back to
-                               one when V K 4-byte weights do not fit 2 GB;
-                               documents longer than 65,535 tokens still go one per warp,
-                               the longest to CTAs as coop_min_len says); results are
-                               identical */
+    int32_t docs_per_warp;  /* z-step documents per warp: 0 = auto (two at K <= 1024 in passes
+                               over many documents, else one), 1 = one, 4 = four (needs
+                               K <= 1024; falls back to one when V K 4-byte weights do not fit
+                               2 GB); documents longer than 65,535 tokens still go one per warp,
+                               the longest to CTAs as coop_min_len says; results are identical */
     int32_t phi_mode;       /* 0 = Poisson Polya urn (Algorithm 2), 1 = Dirichlet (Algorithm 1:
                                phi_k ~ Dir(n_k + beta) through Gamma draws, entries below 2^-24
                                of their column's maximum dropped); the batched form takes 0 only */
@@ -81,7 +80,7 @@ typedef struct {
                                time per token -- concurrently with the other documents' one-warp
                                kernel; results are identical.
                                0 = auto (documents longer than max(256, N / 4500) tokens,
-                               N / 16000 beside four documents per warp: those that would
+                               N / 9000 or N / 16000 beside two or four documents per warp: those that would
                                outlast the rest of the pass; where a pass has at most two
                                documents for every such CTA the GPU holds, all of them run in
                                that form), -1 = never, > 0 = this length.
@@ -403,9 +402,10 @@ pulda_status pulda_serve_close(pulda_server *s);
 
 /* pulda_z_layout -- how the handle's corpus z-step is laid out (launch shape
  * only: results never depend on it): documents per warp of the main z-step
- * kernel (1 or 4), the number of (longest) documents that coop_min_len puts on
- * CTAs of their own, and, beside four per warp, the documents too long for it that run one
- * per warp (otherwise every document not on a CTA).  Any pointer may be NULL.
+ * kernel (1, 2 or 4), the number of (longest) documents that coop_min_len
+ * puts on CTAs of their own, and, beside four per warp, the documents too long
+ * for it that run one per warp (otherwise every document not on a CTA).  Any
+ * pointer may be NULL.
  * Errors: PULDA_ERR_INVALID (NULL handle). */
 pulda_status pulda_z_layout(pulda_handle *h, int32_t *docs_per_warp, int64_t *coop_docs, int64_t *one_warp_docs);
 

@@ -146,7 +146,7 @@ int64_t count_wide(const int64_t *off, const std::vector<int32_t> &order) {
 // Number of documents, after the n_wide widest of a length-ordered schedule,
 // that the long-document z-step takes.
 int64_t count_coop(const pulda_handle *h, const int64_t *off, const std::vector<int32_t> &order, int64_t n_wide, int64_t N) {
-    const int64_t L = long_document_tokens(h, N);
+    const int64_t L = long_document_tokens(h, static_cast<int64_t>(order.size()), N);
     int64_t n = n_wide;
     while (n < static_cast<int64_t>(order.size()) && off[order[n] + 1] - off[order[n]] >= L) ++n;
     return n - n_wide;
@@ -207,12 +207,23 @@ ZArgs z_args(pulda_handle *h, const int64_t *doc_off, const int32_t *doc_order, 
 }
 
 
+// Two documents per warp pay once every warp takes many pairs: a document's
+// tokens advance half as fast, so short passes end on their last documents
+// (z-step ms at K = 1000, one per warp / two: D = 300,000 32.2 / 27.8,
+// D = 37,500 4.01 / 3.97 at best).
+bool pairs_of_documents(const pulda_handle *h, int64_t D) {
+    return h->opt.docs_per_warp == 0 && h->opt.slice_len == 0 && h->pair_grid > 0 &&
+           D >= 8 * 2 * static_cast<int64_t>(h->z_warps) * h->pair_grid;
+}
+
 // At least coop_min_len tokens (0 = automatic: longer than max(256, N / 4500),
-// or N / 16000 beside the grouped z-step); none with coop_min_len < 0 or slices.
-int64_t long_document_tokens(const pulda_handle *h, int64_t N) {
+// N / 9000 where the others go two per warp, or N / 16000 beside the grouped
+// z-step); none with coop_min_len < 0 or slices.
+int64_t long_document_tokens(const pulda_handle *h, int64_t D, int64_t N) {
     if (h->opt.coop_min_len < 0 || h->opt.slice_len > 0) return INT64_MAX;
     if (h->opt.coop_min_len > 0) return h->opt.coop_min_len;
-    return std::max<int64_t>(kCoopAutoMin, N / (h->z_groups ? kCoopAutoDivGrouped : kCoopAutoDiv) + 1);
+    const int64_t div = h->z_groups ? kCoopAutoDivGrouped : pairs_of_documents(h, D) ? kCoopAutoDivPairs : kCoopAutoDiv;
+    return std::max<int64_t>(kCoopAutoMin, N / div + 1);
 }
 
 // The n_wide widest documents one per warp, the next n_coop on a CTA each,
@@ -228,6 +239,7 @@ cudaError_t run_z(pulda_handle *h, ZArgs a, int64_t n_wide, int64_t n_coop, int 
     if (h->opt.coop_min_len == 0 && h->opt.slice_len == 0 && !h->z_groups && D - n_wide <= 2 * static_cast<int64_t>(h->coop_grid))
         n_coop = D - n_wide;
     const int64_t n_head = n_wide + n_coop;
+    const bool pairs = pairs_of_documents(h, D);
     const int32_t *order = a.doc_order;
     auto launch_rest = [&](cudaStream_t st) {
         if (D <= n_head) return;
@@ -237,6 +249,7 @@ cudaError_t run_z(pulda_handle *h, ZArgs a, int64_t n_wide, int64_t n_coop, int 
         ar.narrow = 1;
         ar.work = work + (h->z_groups ? 1 : 0);
         if (h->z_groups) launch_z_step_groups(ar, h->zg_grid, st);
+        else if (pairs) launch_z_step_pairs(ar, h->z_warps, h->pair_grid, st);
         else launch_z_step(ar, h->z_warps, h->z_grid, st);
     };
     auto launch_head = [&](cudaStream_t st) {
@@ -500,11 +513,12 @@ pulda_status pulda_init(pulda_handle **out, const int32_t *word_ids, const int64
     while (wpb > 1 && z_step_smem(K, wpb) > 160 * 1024) wpb >>= 1;
     h->z_warps = wpb;
     CUI(cudaGetLastError());
-    h->n_wide = count_wide(doc_offsets, dord);
-    h->n_coop = count_coop(h, doc_offsets, dord, h->n_wide, N);
     // as many one-warp CTAs as fit with two count planes; a launch with three
     // queues the CTAs that do not fit, each taking documents from the same counter
     h->z_grid = sms * z_step_blocks_per_sm(K, wpb, true);
+    h->pair_grid = sms * z_pair_blocks_per_sm(K, wpb);
+    h->n_wide = count_wide(doc_offsets, dord);
+    h->n_coop = count_coop(h, doc_offsets, dord, h->n_wide, N);
     CUI(cudaGetLastError());
     h->coop_grid = sms * z_coop_blocks_per_sm(K);
     CUI(cudaGetLastError());
@@ -778,7 +792,7 @@ pulda_status pulda_infer(pulda_handle *h, const int32_t *word_ids, const int64_t
 
 pulda_status pulda_z_layout(pulda_handle *h, int32_t *docs_per_warp, int64_t *coop_docs, int64_t *one_warp_docs) {
     if (!h) return PULDA_ERR_INVALID;
-    if (docs_per_warp) *docs_per_warp = h->z_groups ? 4 : 1;
+    if (docs_per_warp) *docs_per_warp = h->z_groups ? 4 : pairs_of_documents(h, h->D) ? 2 : 1;
     if (coop_docs) *coop_docs = h->n_coop;
     if (one_warp_docs) *one_warp_docs = h->z_groups ? h->n_wide : h->D - h->n_coop;
     return PULDA_OK;

@@ -23,6 +23,7 @@ struct pulda_handle {
     float beta = 0;
     double alpha_sum = 0;       // sum_k alpha_k in double, index order
     int z_warps = 8, z_grid = 0, phi_grid = 0;
+    int pair_grid = 0;          // the z-step with two documents per warp (0: K > 1024)
     bool z_groups = false;      // grouped z-step (four documents per warp) in use
     int zg_grid = 0;
     int64_t n_wide = 0;         // documents of 2^16 tokens or more (first in doc_order)
@@ -96,9 +97,11 @@ struct DevTemp {
         return e;
     }
 };
-// Tokens from which a document of an N-token pass goes to a CTA of its own
-// (INT64_MAX: none do).
-int64_t long_document_tokens(const pulda_handle *h, int64_t N);
+// Tokens from which a document of a pass over D documents and N tokens goes to
+// a CTA of its own (INT64_MAX: none do).
+int64_t long_document_tokens(const pulda_handle *h, int64_t D, int64_t N);
+// Whether a pass over D documents takes them two per warp.
+bool pairs_of_documents(const pulda_handle *h, int64_t D);
 // One z-step over a's documents doc_order[0 .. D) on the handle's streams: the
 // first n_wide have 2^16 tokens or more, the next n_coop go to a CTA each, and
 // so do the others when they are few.  work: five counters.

@@ -29,6 +29,7 @@
 #include "device_rng.cuh"
 #include "pulda_internal.h"
 #include "zdense.cuh"
+#include "zpair.cuh"
 #include "zstep.cuh"
 #include "checks.cuh"
 
@@ -732,6 +733,38 @@ __global__ void __launch_bounds__(32 * kZWarps, PULDA_ZMINBLOCKS) k_z_step(ZArgs
     flush_warp_counters(a.stats, wcnt);
 }
 
+#ifndef PULDA_PAIR_MINB
+#define PULDA_PAIR_MINB 8
+#endif
+// The same with two documents per warp, of at most kNarrowMaxLen tokens each
+// (neighbours of the length order, so their lengths are near); no slices.
+template <int NW>
+__global__ void __launch_bounds__(32 * kZWarps, PULDA_PAIR_MINB) k_z_step_pairs(ZArgs a) {
+    extern __shared__ __align__(16) uint32_t zsm[];
+    const int lane = threadIdx.x & 31;
+    uint32_t *m = zsm + static_cast<size_t>(threadIdx.x >> 5) * z_pair_words(a.K);
+    u64 *wcnt = reinterpret_cast<u64 *>(m + 2 * 2 * 32 * NW + 32 * kTokRecWords);
+    zero_warp_counters(wcnt);
+    const uint32_t sweep = sweep_of(a);
+    for (;;) {
+        int item = 0;
+        if (lane == 0) item = atomicAdd(a.work, 1);
+        item = __shfl_sync(0xFFFFFFFFu, item, 0);
+        if (2 * static_cast<int64_t>(item) >= a.D) break;
+        const int64_t di = 2 * static_cast<int64_t>(item) + (lane >> 4);
+        int64_t s = 0;
+        int len = 0;
+        if (di < a.D) {
+            const int d = a.doc_order[di];
+            s = a.doc_off[d];
+            len = static_cast<int>(a.doc_off[d + 1] - s);
+        }
+        const DocRun r{a.w + s, a.z + s, len, a.seed, a.index_base + s, sweep, 0, len, 1};
+        z_pair<NW>(a, m, r, wcnt);
+    }
+    flush_warp_counters(a.stats, wcnt);
+}
+
 // m0[j * K + k] = the topic-k count of document sliced_docs[j] (one warp per
 // document): the pass-start counts its slices start from.
 __global__ void k_slice_counts(const int64_t *doc_off, const int32_t *sliced_docs, int n, const int16_t *z, int K,
@@ -1000,6 +1033,29 @@ static ZStepKernel z_step_kernel(int K) {
         case 8: return k_z_step<8>;
         default: return k_z_step<0>;
     }
+}
+
+static ZStepKernel z_pair_kernel(int K) {
+    switch (z_nw(K)) {
+        case 1: return k_z_step_pairs<1>;
+        case 2: return k_z_step_pairs<2>;
+        case 4: return k_z_step_pairs<4>;
+        case 8: return k_z_step_pairs<8>;
+        default: return nullptr;
+    }
+}
+
+int z_pair_blocks_per_sm(int K, int warps_per_block) {
+    ZStepKernel kern = z_pair_kernel(K);
+    if (!kern) return 0;
+    allow_dynamic_smem(kern);
+    int b = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kern, 32 * warps_per_block, sizeof(uint32_t) * z_pair_words(K) * warps_per_block);
+    return b;
+}
+
+void launch_z_step_pairs(const ZArgs &a, int warps_per_block, int grid, cudaStream_t st) {
+    z_pair_kernel(a.K)<<<grid, 32 * warps_per_block, sizeof(uint32_t) * z_pair_words(a.K) * warps_per_block, st>>>(a);
 }
 
 int z_step_blocks_per_sm(int K, int warps_per_block, bool narrow) {

@@ -136,7 +136,7 @@ extern "C" pulda_status pulda_infer_noalloc(pulda_handle *h, const int32_t *word
     auto *first = reinterpret_cast<unsigned long long *>(scratch + kOffFlag);
     auto *order = reinterpret_cast<int32_t *>(scratch + kOffOrder);
     auto *count = reinterpret_cast<int *>(scratch + kOffCount);
-    const int64_t coop_len = long_document_tokens(h, N_new);
+    const int64_t coop_len = long_document_tokens(h, D_new, N_new);
     // the array keeps the previous call's contents: clear what counts from
     // zero, and set the input check's "first bad index" slots to ~0 (none)
     e = cudaMemsetAsync(scratch, 0, kOffFlag, st);

@@ -219,6 +219,10 @@ void launch_phi_fixup(const PhiArgs &a, cudaStream_t st);
 void launch_colptr_scan(const PhiArgs &a, cudaStream_t st);
 void launch_phi_tables(const PhiArgs &a, cudaStream_t st);
 void launch_z_step(const ZArgs &a, int warps_per_block, int grid, cudaStream_t st);
+// The same with two documents per warp (zpair.cuh): K <= 1024 (else no CTA
+// fits), documents of at most kNarrowMaxLen tokens, no slices.
+void launch_z_step_pairs(const ZArgs &a, int warps_per_block, int grid, cudaStream_t st);
+int z_pair_blocks_per_sm(int K, int warps_per_block);
 // The documents doc_order[0 .. n_coop), of at most kNarrowMaxLen tokens, one
 // CTA each (zchain.cuh); `work` is a counter zeroed before the launch.
 void launch_z_step_coop(const ZArgs &a, int n_coop, int *work, int grid, cudaStream_t st);
@@ -231,6 +235,7 @@ int z_coop_blocks_per_sm(int K);
 // N = 9.9M 4.04 / 3.85 / 3.48 / 6.02; K = 3000, N = 6.5M, threshold 500 /
 // 1,000 / 2,000 / none: 8.88 / 6.90 / 7.27 / 16.1.
 constexpr int64_t kCoopAutoDiv = 4500;
+constexpr int64_t kCoopAutoDivPairs = 9000;     // two documents per warp: each takes twice as long
 constexpr int64_t kCoopAutoMin = 256;
 // The same over a batch's chains, whose passes are of mixed K (eight chains,
 // 6.3M tokens, K 50 to 500: a sweep takes 3.97 ms at N / 8000, 4.35 at N /

@@ -112,3 +112,20 @@ def test_noalloc_schedules_every_length_class():
     P.pulda_infer_noalloc(s.h, torch.from_numpy(nw).cuda(), torch.from_numpy(noff).cuda(), 2, 77, z)
     assert np.array_equal(z.cpu().numpy(), s.infer(nw, noff, 2, seed=77))
     s.close()
+
+
+@pytest.mark.parametrize("K", [3, 128, 129, 257, 512, 513, 1000, 1024])
+def test_two_documents_per_warp(K):
+    """A pass over enough documents to go two per warp: uneven neighbours, empty
+    documents, lengths around the 16-token blocks, counts past one plane."""
+    rng = np.random.default_rng(K)
+    lengths = rng.integers(0, 24, size=90001)
+    lengths[:9] = [15, 16, 17, 31, 33, 255, 400, 2600, 2601]
+    w, off = corpus(rng, lengths, 700)
+    heavy = slice(int(off[7]), int(off[9]))
+    w[heavy] = rng.integers(0, 4, size=heavy.stop - heavy.start)
+    alpha = np.full(K, 0.05, np.float32)
+    alpha[0] = 5.0
+    s, _ = lockstep(w, off, K, 700, alpha, 0.01, seed=K, sweeps=2, check_tables=False, coop_min_len=-1)
+    assert s.z_layout()["docs_per_warp"] == 2
+    s.close()
