@@ -48,7 +48,7 @@ def kernels_per_sweep(w: np.ndarray, phi_mode: int, layout: dict | None = None, 
     cooperative kernel when some document is on CTAs, the one-warp kernel for
     documents too long for four per warp, or the pass-start counts before a
     z-step in slices."""
-    heavy = 1 if np.bincount(w).max(initial=0) > (1 << 17) else 0
+    heavy = 1 if np.bincount(w).max(initial=0) > min(max(len(w) // 1024, 4096), 1 << 17) else 0
     extra = 1 if slice_docs > 0 else 0
     if layout is not None:
         extra += (1 if layout["coop_docs"] > 0 else 0)

@@ -113,8 +113,6 @@ pulda_status check_corpus(pulda_handle *h, const int32_t *w, const int64_t *off,
 // Topic histograms of the most frequent words, before the per-word pass.
 cudaError_t run_heavy(pulda_handle *h) {
     if (h->n_heavy == 0) return cudaSuccess;
-    cudaError_t e = cudaMemsetAsync(h->heavy_hist, 0, sizeof(uint32_t) * static_cast<size_t>(h->n_heavy) * h->K, h->stream);
-    if (e != cudaSuccess) return e;
     launch_heavy_hist(h->d_self, h->d_heavy_chunks, static_cast<int>(h->heavy_chunks.size()), h->K, h->stream);
     return cudaGetLastError();
 }
@@ -188,7 +186,7 @@ PhiArgs phi_args(pulda_handle *h) {
     a.topic = h->topic; a.c = h->c; a.q = h->q; a.athr = h->athr; a.atopic = h->atopic; a.apack = h->apack;
     a.A = h->A; a.vose_p = h->vose_p; a.vose_stack = h->vose_stack; a.bits = h->bits; a.KW = h->KW; a.KWp = h->KWp;
     a.qrow = h->qrow; a.row_slot = h->row_slot; a.drow = h->drow; a.qdense = h->qdense;
-    a.alpha = h->alpha; a.work = h->work; a.stats = h->stats;
+    a.alpha = h->alpha; a.work = h->work; a.work_warp = h->work + 6; a.n_big = h->n_big; a.stats = h->stats;
     a.heavy_row = h->heavy_row; a.heavy_hist = h->heavy_hist; a.n_heavy = h->n_heavy;
     a.gam = h->gam; a.Sd = h->Sd; a.invS = h->invS; a.invSf = h->invSf; a.dpart = h->dpart;
     return a;
@@ -399,7 +397,7 @@ pulda_status pulda_init(pulda_handle **out, const int32_t *word_ids, const int64
         ALLOC(h->gam, h->cap); ALLOC(h->Sd, K); ALLOC(h->invS, K); ALLOC(h->invSf, K);
         ALLOC(h->dpart, dir_part_count(V, K));
     }
-    ALLOC(h->work, 6); ALLOC(h->stats, ST_TOTAL_SLOTS);
+    ALLOC(h->work, 7); ALLOC(h->stats, ST_TOTAL_SLOTS);     // words by CTAs, the five of a z-step, words by warps
     if (h->opt.count_path == 1) ALLOC(h->sort_scratch, count_sort_scratch_words(N));
     cudaStream_t st = h->stream;
     CUI(cudaMemcpyAsync(h->w, word_ids, sizeof(int32_t) * N, cudaMemcpyHostToDevice, st));
@@ -482,16 +480,17 @@ pulda_status pulda_init(pulda_handle **out, const int32_t *word_ids, const int64
         std::vector<int32_t> row(V, -1);
         for (int32_t v : word_order) {
             const int64_t cnt = woff[v + 1] - woff[v];
-            if (cnt <= kHeavyWord) break;
+            if (cnt <= heavy_word(N)) break;
             row[v] = h->n_heavy;
-            for (int64_t b = woff[v]; b < woff[v + 1]; b += kHeavyChunk)
-                h->heavy_chunks.push_back(HeavyChunk{0, h->n_heavy, v, 0, b, std::min(woff[v + 1], b + kHeavyChunk)});
+            for (int64_t b = woff[v]; b < woff[v + 1]; b += heavy_chunk_tokens(N))
+                h->heavy_chunks.push_back(HeavyChunk{0, h->n_heavy, v, 0, b, std::min(woff[v + 1], b + heavy_chunk_tokens(N))});
             ++h->n_heavy;
         }
         ALLOC(h->heavy_row, V);
         ALLOC(h->d_self, 1);
         if (h->n_heavy > 0) {
             ALLOC(h->heavy_hist, static_cast<size_t>(h->n_heavy) * K);
+            CUI(cudaMemsetAsync(h->heavy_hist, 0, sizeof(uint32_t) * static_cast<size_t>(h->n_heavy) * K, st));
             ALLOC(h->d_heavy_chunks, h->heavy_chunks.size());
             CUI(cudaMemcpyAsync(h->d_heavy_chunks, h->heavy_chunks.data(), sizeof(HeavyChunk) * h->heavy_chunks.size(),
                                 cudaMemcpyHostToDevice, st));
@@ -530,6 +529,9 @@ pulda_status pulda_init(pulda_handle **out, const int32_t *word_ids, const int64
         CUI(cudaGetLastError());
     }
     h->phi_grid = sms * phi_counts_blocks_per_sm(K);
+    const auto rare = std::partition_point(word_order.begin(), word_order.end(),
+                                           [&](int32_t v) { return woff[v + 1] - woff[v] > phi_warp_word_tokens(); });
+    h->n_big = phi_big_words(K, V, rare - word_order.begin(), h->phi_grid);
     CUI(cudaGetLastError());
     CUI(cudaStreamSynchronize(st));
     *out = h;
@@ -542,7 +544,7 @@ pulda_status pulda_phi_step(pulda_handle *h) {
     h->sweep += 1;
     cudaStream_t st = h->stream;
     CU(h, cudaMemsetAsync(h->stats, 0, sizeof(unsigned long long) * ST_COUNT, st));
-    CU(h, cudaMemsetAsync(h->work, 0, sizeof(int), st));
+    CU(h, cudaMemsetAsync(h->work, 0, 7 * sizeof(int), st));
     CU(h, cudaMemsetAsync(h->S, 0, sizeof(unsigned long long) * h->K, st));
     PhiArgs a = phi_args(h);
     if (h->opt.count_path == 1) {
@@ -664,7 +666,7 @@ pulda_status pulda_get_counts(pulda_handle *h, int32_t *n_kv, int32_t *m_dk) {
     if (n_kv) {
         // rebuild n from the current z (counts only, no draws)
         PhiArgs a = phi_args(h);
-        CU(h, cudaMemsetAsync(h->work, 0, sizeof(int), st));
+        CU(h, cudaMemsetAsync(h->work, 0, 7 * sizeof(int), st));
         CU(h, run_heavy(h));
         launch_phi_counts(a, false, h->phi_grid, st);
         int32_t *dn = nullptr;
@@ -691,7 +693,7 @@ pulda_status pulda_log_posterior(pulda_handle *h, double *out) {
     cudaStream_t st = h->stream;
     // n from the current z (counts only, no draws), then the three reductions
     PhiArgs a = phi_args(h);
-    CU(h, cudaMemsetAsync(h->work, 0, sizeof(int), st));
+    CU(h, cudaMemsetAsync(h->work, 0, 7 * sizeof(int), st));
     CU(h, run_heavy(h));
     launch_phi_counts(a, false, h->phi_grid, st);
     unsigned char *scratch = nullptr;

@@ -351,6 +351,9 @@ pulda_status pulda_batch_init(pulda_batch **out, const pulda_chain_desc *chains,
     bl.kmax = kmax;
     bl.narrow = narrow ? 1 : 0;
     bl.phi_grid = b->sms * batch_phi_blocks_per_sm(kmax);
+    const auto rare = std::partition_point(wi.begin(), wi.end(), [](const std::pair<int64_t, int2> &x) { return x.first > phi_warp_word_tokens(); });
+    bl.n_big = phi_big_words(kmax, static_cast<int64_t>(wi.size()), rare - wi.begin(), bl.phi_grid);
+    for (const pulda_handle *h : b->ch) bl.vmax = std::max(bl.vmax, h->V);
     bl.bar = d_bar;
     bl.persist_grid = b->sms * batch_persistent_blocks_per_sm(kmax, narrow, &bl.persist_z_warps, &bl.table_stage);
     // The threshold of the documents on CTAs: fixed, none, or the automatic rule

@@ -61,8 +61,9 @@ struct pulda_handle {
     int *work = nullptr;
     unsigned long long *stats = nullptr;
     uint32_t *sort_scratch = nullptr;   // count_path 1: keys, run ids, scan sums
+    int n_big = 0;                      // words counted by a CTA each
     int64_t cap = 0;   // capacity of the per-word tables: K * V entries
-    // words histogrammed by several CTAs (more than kHeavyWord tokens)
+    // words histogrammed by several CTAs (more than heavy_word(N) tokens)
     int32_t *heavy_row = nullptr;
     uint32_t *heavy_hist = nullptr;
     int n_heavy = 0;

@@ -9,7 +9,7 @@
 //                            "Efficient sampling of Phi"), accumulate S_k.
 //             k_phi_fixup    rows with S_k = 0 are redrawn until nonzero
 //                            (Definition "Poisson Polya Urn").
-//             k_scan_single  column offsets of the sparse Phi.
+//             k_scan         column offsets of the sparse Phi.
 //             k_phi_tables   phi = c/S, fixed-point weights, sigma_a, the
 //                            per-word alias table, bitmaps and dense q rows
 //                            ("Efficient sampling of z").
@@ -117,26 +117,74 @@ __global__ void k_word_hist(int64_t N, const int32_t *w, int32_t *cnt) {
         atomicAdd(&cnt[w[i]], 1);
 }
 
-// Exclusive scan of cnt[0..n) into out[0..n] (out[n] = total), one block.
-template <typename TIn>
-__global__ void k_scan_single(const TIn *cnt, int64_t n, int64_t *out, unsigned long long *total_slot) {
-    __shared__ int64_t part[1024];
-    const int t = threadIdx.x;
-    const int64_t per = (n + blockDim.x - 1) / blockDim.x;
-    const int64_t a = t * per, b = min(n, a + per);
-    int64_t s = 0;
-    for (int64_t i = a; i < b; ++i) s += cnt[i];
-    part[t] = s;
+// Exclusive scan of cnt[0..n) into out[0..n] (out[n] = total), chunk by chunk
+// of the entries: a CTA adds up everything before its chunk itself, so the
+// chunks wait neither for each other nor for a second launch.  The repeated
+// reads come from L2 (400 KB for 100,000 words); one CTA over all the entries,
+// each thread over a stretch of its own, was bound by its uncoalesced loads:
+// 106 us for 100,000 words, the chunks take 12.
+constexpr int kScanChunk = 2048;
+__host__ __device__ __forceinline__ int64_t scan_chunk(int64_t n) {     // entries per CTA: at most 256 CTAs
+    const int64_t c = (n + 255) / 256;
+    return c <= kScanChunk ? kScanChunk : (c + 3) / 4 * 4;
+}
+__host__ __device__ __forceinline__ int scan_chunks(int64_t n) { return static_cast<int>(n > 0 ? (n + scan_chunk(n) - 1) / scan_chunk(n) : 1); }
+
+template <int BLOCK>
+__device__ void scan_one_chunk(const int32_t *cnt, int64_t n, int64_t *out, unsigned long long *total_slot, int c, int *tmp,
+                               u64 *red) {
+    const int64_t size = scan_chunk(n), lo = c * size, hi = min(n, lo + size);
+    const int4 *c4 = reinterpret_cast<const int4 *>(cnt);
+    u64 before = 0;
+#pragma unroll 4
+    for (int64_t i = threadIdx.x; i < lo / 4; i += BLOCK) {
+        const int4 x = __ldcg(&c4[i]);
+        before += static_cast<u64>(x.x) + static_cast<u64>(x.y) + static_cast<u64>(x.z) + static_cast<u64>(x.w);
+    }
+    before = warp_sum64(before);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = before;
     __syncthreads();
-    if (t == 0) {
-        int64_t run = 0;
-        for (int i = 0; i < static_cast<int>(blockDim.x); ++i) { const int64_t v = part[i]; part[i] = run; run += v; }
+    int64_t run = 0;
+    for (int i = 0; i < BLOCK / 32; ++i) run += static_cast<int64_t>(red[i]);
+    for (int64_t t0 = lo; t0 < hi; t0 += 4 * BLOCK) {
+        const int64_t t = t0 + 4 * threadIdx.x;
+        int x[4] = {0, 0, 0, 0};
+        if (t + 3 < hi) {
+            const int4 y = __ldcg(&c4[t / 4]);
+            x[0] = y.x; x[1] = y.y; x[2] = y.z; x[3] = y.w;
+        } else {
+            for (int j = 0; j < 4 && t + j < hi; ++j) x[j] = __ldcg(&cnt[t + j]);
+        }
+        int total;
+        int64_t o = run + block_excl_scan<BLOCK>(x[0] + x[1] + x[2] + x[3], tmp, total);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (t + j < hi) out[t + j] = o;
+            o += x[j];
+        }
+        run += total;
+    }
+    if (hi == n && threadIdx.x == 0) {
         out[n] = run;
         if (total_slot) *total_slot = static_cast<unsigned long long>(run);
     }
     __syncthreads();
-    int64_t run = part[t];
-    for (int64_t i = a; i < b; ++i) { out[i] = run; run += cnt[i]; }
+}
+
+constexpr int kScanBlock = 512;
+__global__ void __launch_bounds__(kScanBlock) k_scan(const int32_t *cnt, int64_t n, int64_t *out, unsigned long long *total_slot) {
+    __shared__ int tmp[kScanBlock / 32 + 1];
+    __shared__ u64 red[kScanBlock / 32];
+    scan_one_chunk<kScanBlock>(cnt, n, out, total_slot, blockIdx.x, tmp, red);
+}
+
+// Column offsets of every chain's Phi: chunk blockIdx.y of chain blockIdx.x.
+__global__ void __launch_bounds__(kScanBlock) k_colptr_scan_multi(const PhiArgs *chains) {
+    __shared__ int tmp[kScanBlock / 32 + 1];
+    __shared__ u64 red[kScanBlock / 32];
+    const PhiArgs &a = chains[blockIdx.x];
+    if (static_cast<int>(blockIdx.y) >= scan_chunks(a.V)) return;
+    scan_one_chunk<kScanBlock>(a.nnz_c, a.V, a.col_ptr, &a.stats[ST_NNZPHI], blockIdx.y, tmp, red);
 }
 
 __global__ void k_word_scatter(int64_t N, const int32_t *w, const int64_t *word_off, int32_t *fill, int32_t *perm) {
@@ -208,8 +256,9 @@ __device__ void phi_word(const PhiArgs &a, int v, bool do_draw, uint32_t *hist, 
             hist[guard_index(a.nst_k[wbeg + j], K, a.stats)] = a.nst_n[wbeg + j];
         __syncthreads();
     } else if (hrow >= 0) {
-        const uint32_t *hh = a.heavy_hist + static_cast<int64_t>(hrow) * K;   // from L2: just summed by other CTAs
-        for (int k = threadIdx.x; k < K; k += BLOCK) { hist[k] = __ldcg(&hh[k]); cbin[k] = 0; }
+        // from L2: just summed by other CTAs; left zero for the next time
+        uint32_t *hh = a.heavy_hist + static_cast<int64_t>(hrow) * K;
+        for (int k = threadIdx.x; k < K; k += BLOCK) { hist[k] = __ldcg(&hh[k]); hh[k] = 0; cbin[k] = 0; }
         __syncthreads();
     } else {
         for (int k = threadIdx.x; k < K; k += BLOCK) { hist[k] = 0; cbin[k] = 0; }
@@ -286,11 +335,158 @@ __device__ void phi_word(const PhiArgs &a, int v, bool do_draw, uint32_t *hist, 
     __syncthreads();
 }
 
-// One chain's words, dynamically scheduled, most frequent first; CTAs of
-// kPhiCountBlock threads (more words in flight per SM than 256-thread CTAs;
-// a word's barriers then wait on fewer warps).
-__global__ void __launch_bounds__(kPhiCountBlock) k_phi_counts(PhiArgs a, bool do_draw) {
-    extern __shared__ uint32_t sm[];
+// A word of at most kWarpWord tokens, by one warp.  Most words are rare: a pass
+// of a CTA over all K topics, several times with barriers in between, costs
+// far more than the word's few entries.  pk[k] holds n_{k,v} in the low and
+// c_{k,v} in the high 16 bits (n <= 256, so c ~ Pois(beta + n) stays far
+// below 2^16), with bitmaps of the topics that have either.  A lane lists the
+// topics of its bitmap words in ascending order, then the lanes share out the
+// list, so the draws and the stores do not wait on the lane of the most topics.
+// pk and the bitmaps are zero between words; kmax lays them out, the same for
+// every word of a launch.
+#ifndef PULDA_WARP_WORD
+#define PULDA_WARP_WORD 256
+#endif
+#ifndef PULDA_WARP_MAXK
+#define PULDA_WARP_MAXK 4096
+#endif
+constexpr int64_t kWarpWord = PULDA_WARP_WORD;
+constexpr int kWarpWordMaxK = PULDA_WARP_MAXK;
+__host__ __device__ __forceinline__ int warp_word_words(int K) {
+    return ((K + 3) & ~3) + 2 * (((K + 31) / 32 + 3) & ~3) + (((K + 1) / 2 + 3) & ~3);
+}
+
+// The topics of a bitmap of KW words as a list, by one warp; returns how many.
+__device__ __forceinline__ int list_topics(const uint32_t *bitmap, int KW, uint16_t *list) {
+    const int lane = threadIdx.x & 31;
+    int base = 0;
+    for (int w0 = 0; w0 < KW; w0 += 32) {
+        const int w = w0 + lane;
+        uint32_t bits = w < KW ? bitmap[w] : 0u;
+        int x = __popc(bits);
+        const int own = x;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+            if (lane >= o) x += y;
+        }
+        uint16_t *o = list + base + x - own;
+        for (; bits; bits &= bits - 1u) *o++ = static_cast<uint16_t>(32 * w + __ffs(bits) - 1);
+        base += __shfl_sync(0xFFFFFFFFu, x, 31);
+    }
+    __syncwarp();
+    return base;
+}
+
+__device__ void phi_word_warp(const PhiArgs &a, int v, bool do_draw, uint32_t *pk, int kmax, const uint32_t *geo) {
+    const int lane = threadIdx.x & 31;
+    const int K = a.K, KW = (K + 31) >> 5;
+    const int kw_max = ((kmax + 31) / 32 + 3) & ~3;
+    uint32_t *nb = pk + ((kmax + 3) & ~3), *cb = nb + kw_max;
+    uint16_t *list = reinterpret_cast<uint16_t *>(cb + kw_max);
+    const uint32_t sweep = sweep_of(a);
+    const int64_t wbeg = a.word_off[v], wend = a.word_off[v + 1];
+    auto add = [&](int k) {
+        if (atomicAdd(&pk[k], 1u) == 0) atomicOr(&nb[k >> 5], 1u << (k & 31));
+    };
+    int64_t t = wbeg + lane;
+    for (; t + 3 * 32 < wend; t += 4 * 32) {
+        int p[4], zz[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) p[u] = a.perm[t + 32 * u];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) zz[u] = a.z[p[u]];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) add(guard_index(zz[u], K, a.stats));
+    }
+    for (; t < wend; t += 32) add(guard_index(a.z[a.perm[t]], K, a.stats));
+    __syncwarp();
+    // the n column, and c ~ Pois(beta + n) for its entries
+    const int nn = list_topics(nb, KW, list);
+    for (int i = lane; i < nn; i += 32) {
+        const int k = list[i];
+        const uint32_t l = pk[k];
+        a.nst_k[wbeg + i] = static_cast<uint16_t>(k);
+        a.nst_n[wbeg + i] = l;
+        if (do_draw) {
+            const U4 x = draw(a.seed, static_cast<uint32_t>(v), static_cast<uint32_t>(k), sweep, TAG_POIS, 0);
+            const uint32_t c = draw_entry(a.tab, l, x.x, x.y);
+            if (c) {
+                pk[k] = l | (c << 16);
+                atomicOr(&cb[k >> 5], 1u << (k & 31));
+            }
+        } else {
+            pk[k] = 0;
+        }
+    }
+    if (lane == 0) a.nnz_n[v] = nn;
+    if (!do_draw) {
+        for (int w = lane; w < KW; w += 32) nb[w] = 0;
+        __syncwarp();
+        return;
+    }
+    __syncwarp();
+    // entries with n = 0: Pois(beta) by geometric skip-ahead (see phi_word)
+    int pos = -1;
+    for (uint32_t h0 = 0;; h0 += 32) {
+        const U4 x = draw(a.seed, static_cast<uint32_t>(v), h0 + lane, sweep, TAG_BETA, 0);
+        const int g = geo_gap(geo, x.x);
+        const int step = g < 0 ? kGeoLen : g + 1;
+        int incl = step;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        const int p = pos + incl;
+        const bool stop = g < 0 ? p >= K - 1 : p >= K;
+        const uint32_t bal = __ballot_sync(0xFFFFFFFFu, stop);
+        const int first_stop = bal ? __ffs(bal) - 1 : 32;
+        if (lane < first_stop && g >= 0 && pk[p] == 0) {
+            const uint32_t c = table_draw(a.tab, 0, x.y, x.z);
+            if (c) {
+                pk[p] = c << 16;
+                atomicOr(&cb[p >> 5], 1u << (p & 31));
+            }
+        }
+        if (bal) break;
+        pos = __shfl_sync(0xFFFFFFFFu, p, 31);
+    }
+    __syncwarp();
+    // entries of n without a draw are cleared off the list of n, then the c column
+    for (int i = lane; i < nn; i += 32) {
+        const int k = list[i];
+        if (pk[k] < 0x10000u) pk[k] = 0;
+    }
+    __syncwarp();
+    const int nc = list_topics(cb, KW, list);
+    for (int i = lane; i < nc; i += 32) {
+        const int k = list[i];
+        const uint32_t c = pk[k] >> 16;
+        const int64_t o = static_cast<int64_t>(v) * K + i;
+        pk[k] = 0;
+        a.cst_k[o] = static_cast<uint16_t>(k);
+        a.cst_c[o] = c;
+        atomicAdd(&a.S[k], static_cast<u64>(c));
+    }
+    for (int w = lane; w < KW; w += 32) nb[w] = cb[w] = 0;
+    if (lane == 0) a.nnz_c[v] = nc;
+    __syncwarp();
+}
+
+// Shared memory of the count pass: a CTA's two K-entry arrays, or its warps'.
+__host__ __device__ __forceinline__ int phi_count_words(int K) {
+    const int w = K <= kWarpWordMaxK ? (kPhiCountBlock / 32) * warp_word_words(K) : 0;
+    return w > 2 * K ? w : 2 * K;
+}
+
+// One chain's words, dynamically scheduled, most frequent first: the first
+// n_big by the CTA (kPhiCountBlock threads: more words in flight per SM than
+// with 256; a word's barriers then wait on fewer warps), the others by a warp
+// each, kWarpWordBatch at a time.
+constexpr int kWarpWordBatch = 4;
+__global__ void __launch_bounds__(kPhiCountBlock) k_phi_counts(PhiArgs a, bool do_draw, int n_big) {
+    extern __shared__ __align__(16) uint32_t sm[];
     __shared__ int scan_tmp[kPhiCountBlock / 32 + 1];
     __shared__ int s_item;
     __shared__ uint32_t geo[kGeoLen];
@@ -299,17 +495,30 @@ __global__ void __launch_bounds__(kPhiCountBlock) k_phi_counts(PhiArgs a, bool d
     __syncthreads();
     for (;;) {
         const int item = s_item;      // published by the barrier above, then by phi_word's last one
-        if (item >= a.V) break;
+        if (item >= n_big) break;
         phi_word<kPhiCountBlock>(a, a.word_order[item], do_draw, sm, sm + a.K, scan_tmp, geo, &s_item, a.work);
+    }
+    if (n_big >= a.V) return;
+    const int lane = threadIdx.x & 31;
+    uint32_t *pk = sm + static_cast<size_t>(threadIdx.x >> 5) * warp_word_words(a.K);
+    __syncthreads();
+    for (int i = lane; i < warp_word_words(a.K); i += 32) pk[i] = 0;
+    __syncwarp();
+    for (;;) {
+        int first = 0;
+        if (lane == 0) first = n_big + atomicAdd(a.work_warp, kWarpWordBatch);
+        first = __shfl_sync(0xFFFFFFFFu, first, 0);
+        if (first >= a.V) break;
+        for (int i = first; i < min(first + kWarpWordBatch, a.V); ++i) phi_word_warp(a, a.word_order[i], do_draw, pk, a.K, geo);
     }
 }
 
 // Many chains: the work list holds (chain, word) pairs, most frequent first
 // across all chains; shared memory is sized for the largest K.
-__global__ void __launch_bounds__(kPhiBlock) k_phi_counts_multi(const PhiArgs *chains, const int2 *items,
-                                                                 int n_items, int *work, int kmax, bool do_draw) {
-    extern __shared__ uint32_t sm[];
-    __shared__ int scan_tmp[kPhiBlock / 32 + 1];
+__global__ void __launch_bounds__(kPhiCountBlock) k_phi_counts_multi(const PhiArgs *chains, const int2 *items, int n_items, int n_big,
+                                                                 int *work, int *work_warp, int kmax, bool do_draw) {
+    extern __shared__ __align__(16) uint32_t sm[];
+    __shared__ int scan_tmp[kPhiCountBlock / 32 + 1];
     __shared__ int s_item;
     __shared__ uint32_t geo[kGeoLen];
     int geo_chain = -1;
@@ -318,19 +527,35 @@ __global__ void __launch_bounds__(kPhiBlock) k_phi_counts_multi(const PhiArgs *c
         __syncthreads();
         const int item = s_item;
         __syncthreads();
-        if (item >= n_items) break;
+        if (item >= n_big) break;
         const int2 it = items[item];
         if (it.x != geo_chain) {          // the geometric table depends on the chain's beta
-            for (int i = threadIdx.x; i < kGeoLen; i += kPhiBlock) geo[i] = chains[it.x].tab.geo[i];
+            for (int i = threadIdx.x; i < kGeoLen; i += kPhiCountBlock) geo[i] = chains[it.x].tab.geo[i];
             geo_chain = it.x;
             __syncthreads();
         }
-        phi_word<kPhiBlock>(chains[it.x], it.y, do_draw, sm, sm + kmax, scan_tmp, geo);
+        phi_word<kPhiCountBlock>(chains[it.x], it.y, do_draw, sm, sm + kmax, scan_tmp, geo);
+    }
+    if (n_big >= n_items) return;
+    const int lane = threadIdx.x & 31;
+    uint32_t *pk = sm + static_cast<size_t>(threadIdx.x >> 5) * warp_word_words(kmax);
+    for (int i = lane; i < warp_word_words(kmax); i += 32) pk[i] = 0;
+    __syncwarp();
+    for (;;) {
+        int first = 0;
+        if (lane == 0) first = n_big + atomicAdd(work_warp, kWarpWordBatch);
+        first = __shfl_sync(0xFFFFFFFFu, first, 0);
+        if (first >= n_items) break;
+        for (int i = first; i < min(first + kWarpWordBatch, n_items); ++i) {
+            const PhiArgs &a = chains[items[i].x];
+            phi_word_warp(a, items[i].y, do_draw, pk, kmax, a.tab.geo);
+        }
     }
 }
 
 // Topic histograms of the most frequent words, one chunk of a word's tokens
-// per CTA, added into the word's row of heavy_hist (zeroed before).
+// per CTA, added into the word's row of heavy_hist (zero before: the count pass
+// clears what it has read).
 __device__ void heavy_chunk(const PhiArgs *chains, const HeavyChunk &c, uint32_t *hs) {
     const PhiArgs &a = chains[c.chain];
     const int K = a.K;
@@ -462,34 +687,6 @@ __global__ void __launch_bounds__(kFixBlock) k_phi_fixup_multi(const PhiArgs *ch
     __shared__ u64 red[kFixBlock / 32];
     __shared__ u64 s_sum;
     phi_fixup_chain<kFixBlock>(chains[blockIdx.x], red, &s_sum);
-}
-
-// Column offsets of one chain's Phi by one CTA (part: blockDim entries).
-__device__ void colptr_chain(const PhiArgs &a, int64_t *part) {
-    const int t = threadIdx.x;
-    const int64_t n = a.V;
-    const int64_t per = (n + blockDim.x - 1) / blockDim.x;
-    const int64_t lo = t * per, hi = min(n, lo + per);
-    int64_t sum = 0;
-    for (int64_t i = lo; i < hi; ++i) sum += a.nnz_c[i];
-    part[t] = sum;
-    __syncthreads();
-    if (t == 0) {
-        int64_t run = 0;
-        for (int i = 0; i < static_cast<int>(blockDim.x); ++i) { const int64_t v = part[i]; part[i] = run; run += v; }
-        a.col_ptr[n] = run;
-        a.stats[ST_NNZPHI] = static_cast<unsigned long long>(run);
-    }
-    __syncthreads();
-    int64_t run = part[t];
-    for (int64_t i = lo; i < hi; ++i) { a.col_ptr[i] = run; run += a.nnz_c[i]; }
-    __syncthreads();
-}
-
-// Column offsets of every chain's Phi: one CTA per chain.
-__global__ void k_colptr_scan_multi(const PhiArgs *chains) {
-    __shared__ int64_t part[1024];
-    colptr_chain(chains[blockIdx.x], part);
 }
 
 // =================================================== Phi-step: tables
@@ -824,8 +1021,6 @@ __device__ void batch_begin_sweep(const PhiArgs *chains, int n_chains, uint32_t 
         const PhiArgs &a = chains[c];
         for (int k = threadIdx.x; k < a.K; k += blockDim.x) a.S[k] = 0;
         for (int i = threadIdx.x; i < ST_COUNT; i += blockDim.x) a.stats[i] = 0;
-        if (a.heavy_hist)
-            for (int64_t i = threadIdx.x; i < static_cast<int64_t>(a.n_heavy) * a.K; i += blockDim.x) a.heavy_hist[i] = 0;
     }
 }
 
@@ -944,12 +1139,21 @@ void launch_word_perm(int64_t N, int V, const int32_t *w, int64_t *word_off, int
     cudaMemsetAsync(fill, 0, sizeof(int32_t) * V, st);
     const int grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>((N + 255) / 256, 8LL * sm_count() * 8)));
     if (N > 0) k_word_hist<<<grid, 256, 0, st>>>(N, w, fill);
-    k_scan_single<int32_t><<<1, 1024, 0, st>>>(fill, V, word_off, nullptr);
+    k_scan<<<scan_chunks(V), kScanBlock, 0, st>>>(fill, V, word_off, nullptr);
     cudaMemsetAsync(fill, 0, sizeof(int32_t) * V, st);
     if (N > 0) k_word_scatter<<<grid, 256, 0, st>>>(N, w, word_off, fill, perm);
 }
 
 size_t phi_counts_smem(int K) { return sizeof(uint32_t) * 2 * static_cast<size_t>(K); }
+
+// The words that a CTA counts each, of n of which n_over have more than
+// phi_warp_word_tokens() tokens: those, or all where a warp's counts do not fit
+// or one wave of the grid's CTAs has them all (a warp takes longer over a word,
+// and nothing waits for the CTA then).
+int phi_big_words(int K, int64_t n, int64_t n_over, int grid) {
+    return static_cast<int>(K <= kWarpWordMaxK && n > grid ? n_over : n);
+}
+int64_t phi_warp_word_tokens() { return kWarpWord; }
 
 // The dynamic shared-memory opt-in is a per-kernel attribute shared by every
 // handle in the process, so it is set once to the device maximum.
@@ -965,7 +1169,7 @@ int smem_optin() {
 }
 
 int phi_counts_blocks_per_sm(int K) {
-    const size_t smem = phi_counts_smem(K);
+    const size_t smem = sizeof(uint32_t) * phi_count_words(K);
     allow_dynamic_smem(k_phi_counts);
     int b = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_phi_counts, kPhiCountBlock, smem);
@@ -973,14 +1177,15 @@ int phi_counts_blocks_per_sm(int K) {
 }
 
 void launch_phi_counts(const PhiArgs &a, bool draw, int grid, cudaStream_t st) {
-    const size_t smem = phi_counts_smem(a.K);
-    k_phi_counts<<<grid, kPhiCountBlock, smem, st>>>(a, draw);
+    // columns built by the sort path are the CTA's to read
+    const int n_big = a.counted ? a.V : std::min(a.n_big, a.V);
+    k_phi_counts<<<grid, kPhiCountBlock, sizeof(uint32_t) * phi_count_words(a.K), st>>>(a, draw, n_big);
 }
 
 void launch_phi_fixup(const PhiArgs &a, cudaStream_t st) { k_phi_fixup<<<1, kFixBlock, 0, st>>>(a); }
 
 void launch_colptr_scan(const PhiArgs &a, cudaStream_t st) {
-    k_scan_single<int32_t><<<1, 1024, 0, st>>>(a.nnz_c, a.V, a.col_ptr, &a.stats[ST_NNZPHI]);
+    k_scan<<<scan_chunks(a.V), kScanBlock, 0, st>>>(a.nnz_c, a.V, a.col_ptr, &a.stats[ST_NNZPHI]);
 }
 
 // Warps per CTA and stage bytes per warp of the table pass: eight warps while
@@ -1100,10 +1305,10 @@ static void launch_z_step_multi(const BatchLaunch &b, const BatchForm &f, const 
 void launch_batch_sweep(const BatchLaunch &b, cudaStream_t st) {
     k_batch_begin_sweep<<<1, 256, 0, st>>>(b.phi, b.n_chains, b.sweep, b.work);
     launch_heavy_hist(b.phi, b.heavy, b.n_heavy, b.kmax, st);
-    k_phi_counts_multi<<<b.phi_grid, kPhiBlock, phi_counts_smem(b.kmax), st>>>(b.phi, b.phi_items, b.n_phi_items,
-                                                                                b.work, b.kmax, true);
+    k_phi_counts_multi<<<b.phi_grid, kPhiCountBlock, sizeof(uint32_t) * phi_count_words(b.kmax), st>>>(
+        b.phi, b.phi_items, b.n_phi_items, std::min(b.n_big, b.n_phi_items), b.work, b.work + 1, b.kmax, true);
     k_phi_fixup_multi<<<b.n_chains, kFixBlock, 0, st>>>(b.phi);
-    k_colptr_scan_multi<<<b.n_chains, 1024, 0, st>>>(b.phi);
+    k_colptr_scan_multi<<<dim3(b.n_chains, scan_chunks(b.vmax)), kScanBlock, 0, st>>>(b.phi);
     launch_phi_tables_multi(b.phi, b.phi_items, b.n_phi_items, b.kmax, st);
     // The chains' documents by form, the longest ones of each on CTAs beside
     // the others: every launch on a stream of its own (the CTAs first), so that
@@ -1205,7 +1410,6 @@ __global__ void __launch_bounds__(kPersistThreads, PULDA_PERSIST_MINB) k_batch_s
     __shared__ uint32_t geo[kGeoLen];
     __shared__ u64 red[kPersistThreads / 32];
     __shared__ u64 s_sum;
-    __shared__ int64_t part[kPersistThreads];
     const unsigned nb = gridDim.x;
     unsigned long long *err = b.phi[0].stats + ST_ERROR;
     // counters of the sweep
@@ -1236,7 +1440,12 @@ __global__ void __launch_bounds__(kPersistThreads, PULDA_PERSIST_MINB) k_batch_s
     // rows whose draws summed to zero, one CTA per chain
     for (int c = blockIdx.x; c < b.n_chains; c += nb) phi_fixup_chain<kPersistThreads>(b.phi[c], red, &s_sum);
     if (!grid_barrier(b.bar, nb, err)) return;
-    for (int c = blockIdx.x; c < b.n_chains; c += nb) colptr_chain(b.phi[c], part);
+    const int per_chain = scan_chunks(b.vmax);
+    for (int c = blockIdx.x; c < b.n_chains * per_chain; c += nb) {
+        const PhiArgs &a = b.phi[c / per_chain];
+        if (c % per_chain < scan_chunks(a.V))
+            scan_one_chunk<kPersistThreads>(a.nnz_c, a.V, a.col_ptr, &a.stats[ST_NNZPHI], c % per_chain, scan_tmp, red);
+    }
     if (!grid_barrier(b.bar, nb, err)) return;
     // per-word tables, one warp per (chain, word)
     {
@@ -1322,7 +1531,7 @@ cudaError_t launch_batch_sweep_persistent(const BatchLaunch &b, cudaStream_t st)
 int batch_phi_blocks_per_sm(int kmax) {
     allow_dynamic_smem(k_phi_counts_multi);
     int n = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_phi_counts_multi, kPhiBlock, phi_counts_smem(kmax));
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_phi_counts_multi, kPhiCountBlock, sizeof(uint32_t) * phi_count_words(kmax));
     return n > 0 ? n : 1;
 }
 

@@ -149,9 +149,10 @@ struct PhiArgs {
     int32_t *drow;              // [V] the same as the current Phi has it: -1 too where a q is 2^24 (25 bits)
     uint32_t *qdense;           // [V * K] q by topic (0 off the column): four documents per warp only, else null
     const float *alpha;         // [K]
-    int *work;                  // dynamic word counter
+    int *work, *work_warp;      // dynamic word counters: CTAs', warps'
+    int n_big;                  // words (the first of word_order) that a CTA counts; the others a warp each
     unsigned long long *stats;  // [ST_COUNT]
-    // words with more than kHeavyWord tokens get their topic histogram from a
+    // words with more than heavy_word(N) tokens get their topic histogram from a
     // separate pass split over many CTAs
     const int32_t *heavy_row;   // [V] row of the word in heavy_hist, or -1
     uint32_t *heavy_hist;       // [n_heavy * K]
@@ -165,10 +166,15 @@ struct PhiArgs {
     int counted;                // the n columns are already built (sort path): read them, do not histogram
 };
 
-// A word with more tokens than this is histogrammed in chunks of kHeavyChunk
-// tokens by several CTAs before the per-word Phi-step pass.
-constexpr int64_t kHeavyWord = int64_t(1) << 17;
-constexpr int64_t kHeavyChunk = int64_t(1) << 16;
+// A word of a chain of N tokens with more tokens than heavy_word(N) is
+// histogrammed in chunks of heavy_chunk(N) tokens by several CTAs before the
+// per-word Phi-step pass.  The limit follows N: with 2^17 tokens for every N
+// the largest words just below it were a tail that one CTA worked through
+// alone (200 of the pass's 375 us with 12.4 M tokens).  At most 1,024 words
+// are above it while N < 2^27, and fewer than N / 2^17 past that.
+constexpr int64_t heavy_clamp(int64_t x, int64_t hi) { return x < 4096 ? 4096 : x > hi ? hi : x; }
+constexpr int64_t heavy_word(int64_t N) { return heavy_clamp(N / 1024, int64_t(1) << 17); }
+constexpr int64_t heavy_chunk_tokens(int64_t N) { return heavy_clamp(N / 2048, int64_t(1) << 16); }
 // One chunk of a heavy word: chain, row in heavy_hist, word, token range.
 struct HeavyChunk {
     int32_t chain, row, v, pad;
@@ -254,6 +260,8 @@ void launch_slice_counts(const int64_t *doc_off, const int32_t *sliced_docs, int
 int smem_optin();
 size_t z_step_smem(int K, int warps_per_block, bool narrow = false);
 size_t phi_counts_smem(int K);
+int64_t phi_warp_word_tokens();
+int phi_big_words(int K, int64_t n, int64_t n_over, int grid);
 void launch_doc_topic(const int64_t *doc_off, int64_t D, const int16_t *z, int K, int32_t *m_dk, cudaStream_t st);
 void launch_n_dense(const PhiArgs &a, int32_t *n_kv, cudaStream_t st);
 void launch_phi_values(const PhiArgs &a, float *phi, cudaStream_t st);
@@ -320,7 +328,8 @@ struct BatchLaunch {
     const ZArgs *z;              // [n_chains], sweep_ptr = sweep
     int n_chains;
     const int2 *phi_items;       // (chain, word), most tokens first
-    int n_phi_items;
+    int n_phi_items, n_big;      // n_big: those counted by a CTA each
+    int vmax;
     const int2 *form_items;      // (chain, document), form by form, longest first in each
     BatchForm form[kMaxForms];
     int n_forms;
