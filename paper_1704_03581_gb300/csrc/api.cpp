@@ -186,7 +186,7 @@ PhiArgs phi_args(pulda_handle *h) {
     a.topic = h->topic; a.c = h->c; a.q = h->q; a.athr = h->athr; a.atopic = h->atopic; a.apack = h->apack;
     a.A = h->A; a.vose_p = h->vose_p; a.vose_stack = h->vose_stack; a.bits = h->bits; a.KW = h->KW; a.KWp = h->KWp;
     a.qrow = h->qrow; a.row_slot = h->row_slot; a.drow = h->drow; a.qdense = h->qdense;
-    a.alpha = h->alpha; a.work = h->work; a.work_warp = h->work + 6; a.n_big = h->n_big; a.stats = h->stats;
+    a.alpha = h->alpha; a.rcp = h->rcp; a.work = h->work; a.work_warp = h->work + 6; a.n_big = h->n_big; a.stats = h->stats;
     a.heavy_row = h->heavy_row; a.heavy_hist = h->heavy_hist; a.n_heavy = h->n_heavy;
     a.gam = h->gam; a.Sd = h->Sd; a.invS = h->invS; a.invSf = h->invSf; a.dpart = h->dpart;
     return a;
@@ -391,7 +391,7 @@ pulda_status pulda_init(pulda_handle **out, const int32_t *word_ids, const int64
     ALLOC(h->S, K); ALLOC(h->rowbuf, V); ALLOC(h->col_ptr, V + 1);
     ALLOC(h->topic, h->cap); ALLOC(h->c, h->cap); ALLOC(h->q, h->cap); ALLOC(h->athr, h->cap); ALLOC(h->atopic, h->cap);
     if (h->opt.alias_layout == 2) ALLOC(h->apack, h->cap);
-    ALLOC(h->A, V); ALLOC(h->vose_p, h->cap); ALLOC(h->vose_stack, h->cap);
+    ALLOC(h->rcp, K); ALLOC(h->A, V); ALLOC(h->vose_p, h->cap); ALLOC(h->vose_stack, h->cap);
     ALLOC(h->bits, static_cast<size_t>(V) * h->KWp);
     if (h->opt.phi_mode == 1) {
         ALLOC(h->gam, h->cap); ALLOC(h->Sd, K); ALLOC(h->invS, K); ALLOC(h->invSf, K);

@@ -596,7 +596,7 @@ constexpr int kFixBlock = 1024;
 // exits.  S is read from L2 (other CTAs of the same launch may have just
 // summed it).
 template <int BLOCK>
-__device__ void phi_fixup_chain(const PhiArgs &a, u64 *red, u64 *s_sum_p) {
+__device__ void phi_redraw_dead_rows(const PhiArgs &a, u64 *red, u64 *s_sum_p) {
     u64 &s_sum = *s_sum_p;
     const uint32_t sweep = sweep_of(a);
     // almost always no row is dead: one parallel look at S first
@@ -676,6 +676,17 @@ __device__ void phi_fixup_chain(const PhiArgs &a, u64 *red, u64 *s_sum_p) {
     }
 }
 
+// The dead rows, then every row's reciprocal for the tables.
+template <int BLOCK>
+__device__ void phi_fixup_chain(const PhiArgs &a, u64 *red, u64 *s_sum_p) {
+    phi_redraw_dead_rows<BLOCK>(a, red, s_sum_p);
+    __syncthreads();
+    for (int k = threadIdx.x; k < a.K; k += BLOCK) {
+        const u64 S = __ldcg(&a.S[k]);
+        a.rcp[k] = S ? static_cast<u64>(((static_cast<unsigned __int128>(1) << 127) - 1) / (S << __clzll(static_cast<long long>(S)))) : 0;
+    }
+}
+
 __global__ void __launch_bounds__(kFixBlock) k_phi_fixup(PhiArgs a) {
     __shared__ u64 red[kFixBlock / 32];
     __shared__ u64 s_sum;
@@ -695,9 +706,91 @@ __global__ void __launch_bounds__(kFixBlock) k_phi_fixup_multi(const PhiArgs *ch
 // 24 bits relative to the column maximum (q >= 1); alpha-part masses
 // a = round(q alpha 2^16), A = sigma_a; Vose alias table over a; bitmap of
 // the word's nonzero topics.
-// The same per-word tables, one warp per word: the per-entry arithmetic in
-// parallel, the Vose pairing (sequential by definition) in lane 0.
-__device__ void phi_tables_word_warp(const PhiArgs &a, int v, uint8_t *stage) {
+// One warp per word, the pairing included.  Vose's loop takes the small slots
+// (mass below A) and the large ones each in descending slot order; a large
+// slot whose mass falls below A is the next small one.  So the pairing is a
+// merge of two running sums, the smalls' deficits D_i and the larges'
+// excesses E_j:
+//   small i goes to the first large j with E_j >= D_{i-1};
+//   large j becomes small at the first i with D_i > E_j, with A + E_j - D_i
+//   left, and goes to large j + 1;
+// which one warp scan and a binary search per slot give, in exact integers.
+// (In one lane, a step's loads in turn, it took 0.45 us per slot, and the
+// longest columns were the whole pass: 455 us with K = 1000, 39 us with
+// K = 100.)
+constexpr int kTabSlots = 256;                                     // columns up to this long pair in shared memory
+constexpr int kTabScratch = kTabSlots * (8 + 2);                   // bytes per warp
+static_assert(kTabSlots * 8 >= 16384 / 8, "a word's bitmap is put together there too");
+
+// The FP64 units are few (1.25 TFLOP/s), and some 45 FP64 instructions per
+// entry bounded the pass (370 us for 100,000 words); the same values come
+// from integers, with FP64 for one entry in 2^26.
+
+// Mass of an entry of the alpha part: round(q alpha 2^16) in double, where
+// every step is exact: q alpha has 49 bits, and so has the sum with 1/2.
+__device__ __forceinline__ u64 alpha_mass(uint32_t q, float alpha) {
+    const uint32_t b = __float_as_uint(alpha);
+    const uint32_t ex = b >> 23;                              // alpha > 0
+    const uint32_t ma = ex ? (b & 0x7FFFFFu) | 0x800000u : b;
+    const int s = static_cast<int>(ex ? ex : 1) - 150 + 16;   // q alpha 2^16 = q ma 2^s
+    const u64 x = static_cast<u64>(q) * ma;
+    if (s >= 0) return x << s;
+    return s > -64 ? (x + (1ull << (-s - 1))) >> -s : 0;
+}
+
+// p = c / S as (u / 2^63) 2^x, u in [2^62, 2^64) up to 3 below the exact value,
+// and the exponent e of p = f 2^e, f in [1/2, 1).
+struct Ratio { int x, e; };
+__device__ __forceinline__ Ratio ratio_exponent(uint32_t c, u64 S) {
+    const int zc = __clz(static_cast<int>(c)) + 32, zs = __clzll(static_cast<long long>(S));
+    const int x = zs - zc;
+    return {x, x + ((static_cast<u64>(c) << zc) >= (S << zs) ? 1 : 0)};
+}
+
+// max(1, floor(RN(c / S) 2^(24 - e) + 1/2)), the double expression's value.
+// Double rounding and u move the product by less than 2^12 units of u, so
+// integers decide unless the fraction is that close to 1/2.
+__device__ __forceinline__ uint32_t fixed_weight(uint32_t c, u64 S, u64 rcp, int e) {
+    const int zc = __clz(static_cast<int>(c)) + 32, zs = __clzll(static_cast<long long>(S));
+    const u64 u = __umul64hi(static_cast<u64>(c) << zc, rcp);
+    const int t = 39 + e - (zs - zc);                         // at least 39
+    if (t > 63) return 1u;                                    // below 2^(24 - 24)
+    const u64 half = 1ull << (t - 1), low = u & (2 * half - 1);
+    u64 q = (u >> t) + (low >= half ? 1 : 0);
+    if (low - half + 4096 < 8192) {
+        const double scale = __longlong_as_double(static_cast<long long>(1023 + 24 - e) << 52);
+        const double p = __ddiv_rn(static_cast<double>(c), static_cast<double>(S));
+        q = static_cast<u64>(floor(__dadd_rn(__dmul_rn(p, scale), 0.5)));
+    }
+    return q < 1 ? 1u : static_cast<uint32_t>(q);
+}
+
+// The same for p given as a double > 0 (exact: p has 53 bits).
+__device__ __forceinline__ uint32_t fixed_weight(long long pbits, int e) {
+    const int ep = static_cast<int>(pbits >> 52);
+    if (ep == 0) {                                            // subnormal p
+        const double scale = __longlong_as_double(static_cast<long long>(1023 + 24 - e) << 52);
+        const double q = floor(__dadd_rn(__dmul_rn(__longlong_as_double(pbits), scale), 0.5));
+        return q < 1.0 ? 1u : static_cast<uint32_t>(q);
+    }
+    const u64 m = (static_cast<u64>(pbits) & ((1ull << 52) - 1)) | (1ull << 52);
+    const int t = 1075 - ep - 24 + e;                         // p 2^(24 - e) = m 2^-t
+    if (t > 62) return 1u;
+    const u64 q = (m + (1ull << (t - 1))) >> t;
+    return q < 1 ? 1u : static_cast<uint32_t>(q);
+}
+
+__device__ __forceinline__ u64 warp_incl_scan64(u64 x) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const u64 y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+        if (lane >= o) x += y;
+    }
+    return x;
+}
+
+__device__ void phi_tables_word_warp(const PhiArgs &a, int v, uint8_t *stage, uint8_t *scratch) {
     const int lane = threadIdx.x & 31;
     const int n = a.nnz_c[v];
     const int64_t src = static_cast<int64_t>(v) * a.K;
@@ -705,13 +798,16 @@ __device__ void phi_tables_word_warp(const PhiArgs &a, int v, uint8_t *stage) {
     if (a.bits) {
         // a row of KWp words (KW rounded up; the words past KW stay zero)
         uint32_t *bm = a.bits + static_cast<int64_t>(v) * a.KWp;
-        for (int wi = lane; wi < a.KWp; wi += 32) {
-            int lo = 0, hi = n;                       // first entry with topic >= 32 wi
-            while (lo < hi) { const int mid = (lo + hi) >> 1; if (a.cst_k[src + mid] < 32 * wi) lo = mid + 1; else hi = mid; }
-            uint32_t bits = 0;
-            for (int j = lo; j < n && (a.cst_k[src + j] >> 5) == wi; ++j) bits |= 1u << (a.cst_k[src + j] & 31);
-            bm[wi] = bits;
+        uint32_t *sb = reinterpret_cast<uint32_t *>(scratch);
+        for (int wi = lane; wi < a.KWp; wi += 32) sb[wi] = 0;
+        __syncwarp();
+        for (int j = lane; j < n; j += 32) {
+            const int k = a.cst_k[src + j];
+            atomicOr(&sb[k >> 5], 1u << (k & 31));
         }
+        __syncwarp();
+        for (int wi = lane; wi < a.KWp; wi += 32) bm[wi] = sb[wi];
+        __syncwarp();
     }
     uint32_t *q32 = a.qdense ? a.qdense + static_cast<int64_t>(v) * a.K : nullptr;
     if (q32) {
@@ -733,34 +829,30 @@ __device__ void phi_tables_word_warp(const PhiArgs &a, int v, uint8_t *stage) {
         if (lane == 0) a.A[v] = 0;
         return;
     }
-    double phimax = 0.0;
+    // the column's phi, then the running sums of the pairing; the slots by rank
+    u64 *X = n <= kTabSlots ? reinterpret_cast<u64 *>(scratch) : a.vose_p + out;
+    uint16_t *stk = n <= kTabSlots ? reinterpret_cast<uint16_t *>(scratch + 8 * kTabSlots) : a.vose_stack + out;
+    // the column's largest phi is f 2^e, f in [1/2, 1)
+    int e = -100000;
     for (int j = lane; j < n; j += 32) {
         const int k = a.cst_k[src + j];
-        // Polya urn: c / S_k; Dirichlet: gamma (1 / S_k), gamma's float bits staged in cst_c
-        const double p = a.gam ? __dmul_rn(static_cast<double>(__uint_as_float(a.cst_c[src + j])), a.invS[k])
-                               : __ddiv_rn(static_cast<double>(a.cst_c[src + j]), static_cast<double>(__ldcg(&a.S[k])));
-        a.vose_p[out + j] = static_cast<u64>(__double_as_longlong(p));    // phi, kept for the second pass
-        phimax = p > phimax ? p : phimax;
+        if (a.gam) {
+            // gamma (1 / S_k), gamma's float bits staged in cst_c
+            const long long p = __double_as_longlong(__dmul_rn(static_cast<double>(__uint_as_float(a.cst_c[src + j])), a.invS[k]));
+            X[j] = static_cast<u64>(p);
+            e = max(e, static_cast<int>(p >> 52) - 1022);
+        } else {
+            e = max(e, ratio_exponent(a.cst_c[src + j], __ldcg(&a.S[k])).e);
+        }
     }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        const double y = __shfl_xor_sync(0xFFFFFFFFu, phimax, o);
-        phimax = y > phimax ? y : phimax;
-    }
-    // phimax = f 2^e with f in [1/2, 1); scale = 2^(24 - e) (exact)
-    const long long bits = __double_as_longlong(phimax);
-    const int e = static_cast<int>((bits >> 52) & 0x7FF) - 1022;
-    const double scale = __longlong_as_double(static_cast<long long>(1023 + 24 - e) << 52);
+    e = __reduce_max_sync(0xFFFFFFFFu, e);
     u64 asum = 0;
     uint32_t qtop = 0;                  // a q of 2^24 does not fit a row's three bytes
     for (int j = lane; j < n; j += 32) {
         const int k = a.cst_k[src + j];
         const uint32_t c = a.cst_c[src + j];
-        const double p = __longlong_as_double(static_cast<long long>(a.vose_p[out + j]));
-        const double qq = floor(__dadd_rn(__dmul_rn(p, scale), 0.5));
-        const uint32_t qv = qq < 1.0 ? 1u : static_cast<uint32_t>(qq);
-        const double at = __dmul_rn(__dmul_rn(static_cast<double>(qv), static_cast<double>(a.alpha[k])), 65536.0);
-        const u64 am = static_cast<u64>(floor(__dadd_rn(at, 0.5)));
+        const uint32_t qv = a.gam ? fixed_weight(static_cast<long long>(X[j]), e) : fixed_weight(c, __ldcg(&a.S[k]), a.rcp[k], e);
+        const u64 am = alpha_mass(qv, a.alpha[k]);
         a.topic[out + j] = static_cast<uint16_t>(k);
         a.c[out + j] = c;
         a.q[out + j] = qv;
@@ -772,10 +864,6 @@ __device__ void phi_tables_word_warp(const PhiArgs &a, int v, uint8_t *stage) {
             rw[at + 2 * PB] = static_cast<uint8_t>(qv >> 16);
         }
         qtop |= qv >> 24;
-        a.vose_p[out + j] = am * static_cast<u64>(n);   // scaled so each slot holds A units
-        a.athr[out + j] = 0xFFFFFFFFu;
-        a.atopic[out + j] = static_cast<uint16_t>(k);
-        if (a.apack) a.apack[out + j] = make_uint2(0xFFFFFFFFu, static_cast<uint32_t>(k) * 0x10001u);
         asum += am;
     }
     asum = warp_sum64(asum);
@@ -792,99 +880,158 @@ __device__ void phi_tables_word_warp(const PhiArgs &a, int v, uint8_t *stage) {
         }
         __syncwarp();
     }
-    if (asum == 0) return;
-    // Vose: small stack grows up from 0, large stack down from n-1, each in
-    // ascending slot order.  The warp builds the two stacks with a ballot per
-    // 32 slots; lane 0 pairs (sequential by definition); then every lane
-    // computes the thresholds of its paired slots.
     // Thresholds floor(P 2^32 / A) divide by the word's invariant A:
     // Moller and Granlund's 2/1 division with a reciprocal of the normalised
     // divisor, one 128-bit division per word instead of one per slot (exact).
-    const int sh = __clzll(static_cast<long long>(asum));
+    const int sh = asum ? __clzll(static_cast<long long>(asum)) : 0;
     const u64 dn = asum << sh;
-    const u64 vinv = static_cast<u64>((~static_cast<unsigned __int128>(0)) / dn);   // floor((2^128-1)/dn) - 2^64
+    const u64 vinv = asum ? static_cast<u64>((~static_cast<unsigned __int128>(0)) / dn) : 0;   // floor((2^128-1)/dn) - 2^64
+    auto store = [&](int j, int k, bool paired, int alias, u64 ps) {       // a slot that is not paired keeps its own topic
+        u64 q1 = 0xFFFFFFFFu;
+        if (paired) {
+            // (u1, u0) = ps 2^32 2^sh, u1 < dn since ps < asum
+            const u64 hi = ps >> 32, lo = ps << 32;
+            const u64 u1 = sh ? (hi << sh) | (lo >> (64 - sh)) : hi;
+            const u64 u0 = lo << sh;
+            u64 q0 = vinv * u1;
+            q1 = __umul64hi(vinv, u1);
+            const u64 t = q0 + u0;
+            q1 += u1 + (t < q0 ? 1ull : 0ull);
+            q0 = t;
+            q1 += 1;
+            u64 r = u0 - q1 * dn;
+            if (r > q0) { q1 -= 1; r += dn; }
+            if (r >= dn) q1 += 1;
+        }
+        a.athr[out + j] = static_cast<uint32_t>(q1);
+        a.atopic[out + j] = static_cast<uint16_t>(alias);
+        if (a.apack) a.apack[out + j] = make_uint2(static_cast<uint32_t>(q1), static_cast<uint32_t>(k) | (static_cast<uint32_t>(alias) << 16));
+    };
+    const uint16_t *topic = a.topic + out;
+    if (asum == 0) {
+        for (int j = lane; j < n; j += 32) store(j, topic[j], false, topic[j], 0);
+        return;
+    }
+    const u64 un = static_cast<u64>(n);                      // masses are scaled by n, so each slot holds A units
+    if (__umul64hi(un, asum) == 0) {
+        // X, stk: smalls from 0 up, larges from n - 1 down
+        int ns = 0, nl = 0;
+        u64 D = 0, E = 0;
+        for (int j0 = 0; j0 < n; j0 += 32) {
+            const int j = n - 1 - j0 - lane;
+            const bool in = j >= 0;
+            const u64 P = in ? alpha_mass(a.q[out + j], a.alpha[topic[j]]) * un : 0;
+            const bool small = in && P < asum, large = in && !small;
+            const uint32_t bs = __ballot_sync(0xFFFFFFFFu, small), bl = __ballot_sync(0xFFFFFFFFu, large);
+            const uint32_t below = (1u << lane) - 1u;
+            const u64 d = D + warp_incl_scan64(small ? asum - P : 0), e = E + warp_incl_scan64(large ? P - asum : 0);
+            if (in) {
+                const int at = small ? ns + __popc(bs & below) : n - 1 - (nl + __popc(bl & below));
+                X[at] = small ? d : e;
+                stk[at] = static_cast<uint16_t>(j);
+            }
+            D = __shfl_sync(0xFFFFFFFFu, d, 31);
+            E = __shfl_sync(0xFFFFFFFFu, e, 31);
+            ns += __popc(bs);
+            nl += __popc(bl);
+        }
+        __syncwarp();
+        for (int i = lane; i < n; i += 32) {
+            const int j = stk[i], k = topic[j];
+            const u64 x = X[i];
+            bool paired;
+            int to = i;                                      // whose topic is the alias
+            u64 ps = 0;
+            if (i < ns) {
+                const u64 before = i ? X[i - 1] : 0;
+                int lo = 0, hi = nl;
+                while (lo < hi) {
+                    const int mid = (lo + hi) >> 1;
+                    if (X[n - 1 - mid] < before) lo = mid + 1; else hi = mid;
+                }
+                paired = lo < nl;
+                if (paired) { to = n - 1 - lo; ps = asum - (x - before); }
+            } else {
+                int lo = 0, hi = ns;
+                while (lo < hi) {
+                    const int mid = (lo + hi) >> 1;
+                    if (X[mid] <= x) lo = mid + 1; else hi = mid;
+                }
+                paired = lo < ns && i > ns;                  // a next large one exists
+                if (paired) { to = i - 1; ps = asum + x - X[lo]; }
+            }
+            store(j, k, paired, topic[stk[to]], ps);
+        }
+        __syncwarp();
+        return;
+    }
+    // the sums do not fit 64 bits (long columns with large alpha): Vose's loop in lane 0
     u64 *P = a.vose_p + out;
-    uint16_t *stk = a.vose_stack + out;
+    uint16_t *st = a.vose_stack + out;
     int ns = 0, nl = 0;
     for (int j0 = 0; j0 < n; j0 += 32) {
         const int j = j0 + lane;
         const bool in = j < n;
-        const bool small = in && P[j] < asum;
+        const u64 p = in ? alpha_mass(a.q[out + j], a.alpha[topic[j]]) * un : 0;
+        const bool small = in && p < asum;
         const uint32_t bs = __ballot_sync(0xFFFFFFFFu, small), bl = __ballot_sync(0xFFFFFFFFu, in && !small);
         const uint32_t below = (1u << lane) - 1u;
-        if (small) stk[ns + __popc(bs & below)] = static_cast<uint16_t>(j);
-        else if (in) stk[n - 1 - (nl + __popc(bl & below))] = static_cast<uint16_t>(j);
+        if (in) {
+            P[j] = p;
+            a.atopic[out + j] = topic[j];
+            st[small ? ns + __popc(bs & below) : n - 1 - (nl + __popc(bl & below))] = static_cast<uint16_t>(j);
+        }
         ns += __popc(bs);
         nl += __popc(bl);
     }
     __syncwarp();
     if (lane == 0) {
         while (ns > 0 && nl > 0) {
-            const int s = stk[--ns];
+            const int s = st[--ns];
             --nl;
-            const int l = stk[n - 1 - nl];
+            const int l = st[n - 1 - nl];
             const u64 ps = P[s];             // final: s is not pushed again
-            a.atopic[out + s] = a.topic[out + l];
+            a.atopic[out + s] = topic[l];
             const u64 pl = P[l] - (asum - ps);
             P[l] = pl;
-            if (pl < asum) stk[ns++] = static_cast<uint16_t>(l);
-            else { stk[n - 1 - nl] = static_cast<uint16_t>(l); ++nl; }
+            if (pl < asum) st[ns++] = static_cast<uint16_t>(l);
+            else { st[n - 1 - nl] = static_cast<uint16_t>(l); ++nl; }
         }
     }
     __syncwarp();
-    // a paired slot's alias is another topic of the column; the rest keep
-    // their own topic and threshold 2^32 - 1
-    for (int j = lane; j < n; j += 32) {
-        if (a.atopic[out + j] == a.topic[out + j]) continue;
-        const u64 ps = P[j];
-        // (u1, u0) = ps 2^32 2^sh, u1 < dn since ps < asum
-        const u64 hi = ps >> 32, lo = ps << 32;
-        const u64 u1 = sh ? (hi << sh) | (lo >> (64 - sh)) : hi;
-        const u64 u0 = lo << sh;
-        u64 q0 = vinv * u1;
-        u64 q1 = __umul64hi(vinv, u1);
-        const u64 t = q0 + u0;
-        q1 += u1 + (t < q0 ? 1ull : 0ull);
-        q0 = t;
-        q1 += 1;
-        u64 r = u0 - q1 * dn;
-        if (r > q0) { q1 -= 1; r += dn; }
-        if (r >= dn) q1 += 1;
-        a.athr[out + j] = static_cast<uint32_t>(q1);
-        if (a.apack)
-            a.apack[out + j] = make_uint2(static_cast<uint32_t>(q1),
-                                          a.topic[out + j] | (static_cast<uint32_t>(a.atopic[out + j]) << 16));
-    }
+    for (int j = lane; j < n; j += 32) store(j, topic[j], a.atopic[out + j] != topic[j], a.atopic[out + j], P[j]);
+    __syncwarp();
 }
 
-// A warp's stage of the dense row it puts together: RB bytes each, zeroed;
-// null when the CTA has no room (bytes = 0).
-__device__ __forceinline__ uint8_t *table_stage(uint32_t *sm, int stage_bytes) {
-    if (stage_bytes == 0) return nullptr;
-    const int lane = threadIdx.x & 31;
-    uint8_t *st = reinterpret_cast<uint8_t *>(sm) + static_cast<size_t>(threadIdx.x >> 5) * stage_bytes;
-    for (int i = lane; i < stage_bytes / 16; i += 32) reinterpret_cast<uint4 *>(st)[i] = make_uint4(0u, 0u, 0u, 0u);
+// A warp's part of the shared memory: kTabScratch bytes, and where the CTA has
+// the room the stage of the dense row it puts together (stage_bytes, zeroed;
+// else null).
+struct TableMem { uint8_t *stage, *scratch; };
+__device__ __forceinline__ TableMem table_mem(uint32_t *sm, int stage_bytes) {
+    uint8_t *base = reinterpret_cast<uint8_t *>(sm) + static_cast<size_t>(threadIdx.x >> 5) * (stage_bytes + kTabScratch);
+    TableMem t{stage_bytes ? base + kTabScratch : nullptr, base};
+    for (int i = threadIdx.x & 31; i < stage_bytes / 16; i += 32) reinterpret_cast<uint4 *>(t.stage)[i] = make_uint4(0u, 0u, 0u, 0u);
     __syncwarp();
-    return st;
+    return t;
 }
 
 // One warp per word, most frequent first (their columns are the longest).
 __global__ void k_phi_tables(PhiArgs a, int stage_bytes) {
     extern __shared__ __align__(16) uint32_t tsm[];
-    uint8_t *stage = table_stage(tsm, stage_bytes);
+    const TableMem t = table_mem(tsm, stage_bytes);
     const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    for (int i = wid; i < a.V; i += nwarps) phi_tables_word_warp(a, a.word_order[i], stage);
+    for (int i = wid; i < a.V; i += nwarps) phi_tables_word_warp(a, a.word_order[i], t.stage, t.scratch);
 }
 
 __global__ void k_phi_tables_multi(const PhiArgs *chains, const int2 *items, int n_items, int stage_bytes) {
     extern __shared__ __align__(16) uint32_t tsm[];
-    uint8_t *stage = table_stage(tsm, stage_bytes);
+    const TableMem t = table_mem(tsm, stage_bytes);
     const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     for (int i = wid; i < n_items; i += nwarps) {
         const int2 it = items[i];
-        phi_tables_word_warp(chains[it.x], it.y, stage);
+        phi_tables_word_warp(chains[it.x], it.y, t.stage, t.scratch);
     }
 }
 
@@ -1208,14 +1355,14 @@ void launch_phi_tables(const PhiArgs &a, cudaStream_t st) {
     opt_in_tables();
     const int w = table_warps(a.K), rb = dense_row_bytes(a.K);
     const int grid = static_cast<int>(std::min<int64_t>((a.V + w - 1) / w, 128LL / w * sm_count()));
-    k_phi_tables<<<std::max(grid, 1), 32 * w, static_cast<size_t>(w) * rb, st>>>(a, rb);
+    k_phi_tables<<<std::max(grid, 1), 32 * w, static_cast<size_t>(w) * (rb + kTabScratch), st>>>(a, rb);
 }
 
 void launch_phi_tables_multi(const PhiArgs *chains, const int2 *items, int n_items, int kmax, cudaStream_t st) {
     opt_in_tables();
     const int w = table_warps(kmax), rb = dense_row_bytes(kmax);
     const int grid = static_cast<int>(std::min<int64_t>((n_items + w - 1) / w, 128LL / w * sm_count()));
-    k_phi_tables_multi<<<std::max(grid, 1), 32 * w, static_cast<size_t>(w) * rb, st>>>(chains, items, n_items, rb);
+    k_phi_tables_multi<<<std::max(grid, 1), 32 * w, static_cast<size_t>(w) * (rb + kTabScratch), st>>>(chains, items, n_items, rb);
 }
 
 void launch_heavy_hist(const PhiArgs *chains, const HeavyChunk *chunks, int n_chunks, int kmax, cudaStream_t st) {
@@ -1451,10 +1598,10 @@ __global__ void __launch_bounds__(kPersistThreads, PULDA_PERSIST_MINB) k_batch_s
     {
         const int wid = static_cast<int>(blockIdx.x) * kPersistWarps + (threadIdx.x >> 5);
         const int nw = static_cast<int>(nb) * kPersistWarps;
-        uint8_t *stage = table_stage(psm, b.table_stage);
+        const TableMem t = table_mem(psm, b.table_stage);
         for (int i = wid; i < b.n_phi_items; i += nw) {
             const int2 it = b.phi_items[i];
-            phi_tables_word_warp(b.phi[it.x], it.y, stage);
+            phi_tables_word_warp(b.phi[it.x], it.y, t.stage, t.scratch);
         }
     }
     if (!grid_barrier(b.bar, nb, err)) return;
@@ -1498,7 +1645,7 @@ cudaError_t launch_barrier_selftest(GridBarrier *bar, int blocks, int missing, i
 // The z-step phase runs on all of a CTA's warps, or on one fewer where eight
 // warps' counts just do not fit.
 static size_t batch_persistent_smem(int kmax, int z_warps, bool narrow) {
-    return std::max({phi_counts_smem(kmax), sizeof(uint32_t) * static_cast<size_t>(kmax),
+    return std::max({phi_counts_smem(kmax), static_cast<size_t>(kPersistWarps * kTabScratch),
                      z_step_smem(kmax, z_warps, narrow)});
 }
 
@@ -1509,7 +1656,7 @@ int batch_persistent_blocks_per_sm(int kmax, bool narrow, int *z_warps, int *tab
         const size_t smem = batch_persistent_smem(kmax, w, narrow);
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_batch_sweep_persistent, kPersistThreads, smem) != cudaSuccess) n = 0;
         *z_warps = w;
-        *table_stage = static_cast<size_t>(kPersistWarps) * dense_row_bytes(kmax) <= smem ? dense_row_bytes(kmax) : 0;
+        *table_stage = static_cast<size_t>(kPersistWarps) * (dense_row_bytes(kmax) + kTabScratch) <= smem ? dense_row_bytes(kmax) : 0;
     }
     return n;
 }

@@ -149,6 +149,7 @@ struct PhiArgs {
     int32_t *drow;              // [V] the same as the current Phi has it: -1 too where a q is 2^24 (25 bits)
     uint32_t *qdense;           // [V * K] q by topic (0 off the column): four documents per warp only, else null
     const float *alpha;         // [K]
+    unsigned long long *rcp;    // [K] floor((2^127 - 1) / S_k), S_k shifted up to 64 bits (Polya urn)
     int *work, *work_warp;      // dynamic word counters: CTAs', warps'
     int n_big;                  // words (the first of word_order) that a CTA counts; the others a warp each
     unsigned long long *stats;  // [ST_COUNT]

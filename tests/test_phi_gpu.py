@@ -80,3 +80,27 @@ def test_batch_counts_of_mixed_chains():
         assert np.array_equal(b.z(i), s.z()), f"chain {i} differs from its single-chain run"
         s.close()
     b.close()
+
+
+@pytest.mark.parametrize("K", [1, 2, 33, 255, 257, 600])
+def test_alias_pairing(K):
+    """Full and sparse columns around the 256 slots that pair in shared memory."""
+    rng = np.random.default_rng(K)
+    sizes = np.concatenate([np.full(8, 4 * K), rng.integers(0, 60, 60)])
+    w, off = corpus_of(rng, sizes, 30)
+    s, _ = lockstep(w, off, K, sizes.size, rng.uniform(0.001, 5.0, K).astype(np.float32), 0.3, seed=K, sweeps=2)
+    s.close()
+
+
+@pytest.mark.parametrize("K,alpha", [(900, 256.0), (1100, 256.0), (1500, 100.0), (4200, 256.0)])
+def test_alias_pairing_past_64_bits(K, alpha):
+    """Long columns of even counts under a large alpha: n A passes 2^64 for the
+    frequent words, not for the rare ones."""
+    rng = np.random.default_rng(K)
+    sizes = np.concatenate([np.full(4, 3 * K), rng.integers(0, 9, 40)])
+    w, off = corpus_of(rng, sizes, 30)
+    s, ch = lockstep(w, off, K, sizes.size, np.full(K, alpha, np.float32), 40.0, seed=K, sweeps=2)
+    t = s.word_tables()
+    n = np.diff(t["col_ptr"])
+    assert any(int(a) * int(c) >= 1 << 64 for a, c in zip(t["A"].view(np.uint64), n))
+    s.close()
