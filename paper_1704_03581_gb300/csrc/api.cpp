@@ -1,6 +1,7 @@
 // C ABI of the pulda sampler: argument validation, device buffers, and the
 // order of kernel launches that makes one sweep (Algorithm 2, Section 3).
 #include <algorithm>
+#include <cmath>
 #include <chrono>
 #include <cstdarg>
 #include <cstdio>
@@ -179,7 +180,8 @@ PhiArgs phi_args(pulda_handle *h) {
     PhiArgs a{};
     a.K = h->K; a.V = h->V; a.seed = h->seed; a.sweep = static_cast<uint32_t>(h->sweep);
     a.perm = h->perm; a.word_off = h->word_off; a.word_order = h->word_order; a.z = h->z;
-    a.tab = DevTables{h->t_thr, h->t_alias, h->t_off, h->t_lo, h->t_n, h->t_geo, h->t_gauss, static_cast<double>(h->beta)};
+    a.tab = DevTables{h->t_thr, h->t_alias, h->t_off, h->t_lo, h->t_n, h->t_geo, h->t_gauss, static_cast<double>(h->beta),
+                      h->t_gauss_fix};
     a.nst_k = h->nst_k; a.nst_n = h->nst_n; a.nnz_n = h->nnz_n;
     a.cst_k = h->cst_k; a.cst_c = h->cst_c; a.nnz_c = h->nnz_c;
     a.S = h->S; a.rowbuf = h->rowbuf; a.col_ptr = h->col_ptr;
@@ -395,7 +397,7 @@ pulda_status pulda_init(pulda_handle **out, const int32_t *word_ids, const int64
     ALLOC(h->bits, static_cast<size_t>(V) * h->KWp);
     if (h->opt.phi_mode == 1) {
         ALLOC(h->gam, h->cap); ALLOC(h->Sd, K); ALLOC(h->invS, K); ALLOC(h->invSf, K);
-        ALLOC(h->dpart, dir_part_count(V, K));
+        ALLOC(h->dpart, dir_part_count(V, K)); ALLOC(h->t_gauss_fix, kGaussCells);
     }
     ALLOC(h->work, 7); ALLOC(h->stats, ST_TOTAL_SLOTS);     // words by CTAs, the five of a z-step, words by warps
     if (h->opt.count_path == 1) ALLOC(h->sort_scratch, count_sort_scratch_words(N));
@@ -447,6 +449,12 @@ pulda_status pulda_init(pulda_handle **out, const int32_t *word_ids, const int64
     CUI(cudaMemcpyAsync(h->t_n, tab.n.data(), sizeof(int32_t) * (kL + 1), cudaMemcpyHostToDevice, st));
     CUI(cudaMemcpyAsync(h->t_geo, tab.geo.data(), sizeof(uint32_t) * kGeoLen, cudaMemcpyHostToDevice, st));
     CUI(cudaMemcpyAsync(h->t_gauss, tab.gauss.data(), sizeof(double) * (kGaussCells + 1), cudaMemcpyHostToDevice, st));
+    std::vector<longlong2> gauss_fix;
+    if (h->t_gauss_fix) {
+        auto fix = [&](int i) { return std::llrint(std::ldexp(tab.gauss[i], 58)); };
+        for (int i = 0; i < kGaussCells; ++i) gauss_fix.push_back(make_longlong2(fix(i), fix(i + 1) - fix(i)));
+        CUI(cudaMemcpyAsync(h->t_gauss_fix, gauss_fix.data(), sizeof(longlong2) * gauss_fix.size(), cudaMemcpyHostToDevice, st));
+    }
     // word-major permutation and the word schedule (most tokens first)
     CUI(cudaGetLastError());            // nothing pending before the first launch
     launch_word_perm(N, V, h->w, h->word_off, h->fill, h->perm, st);

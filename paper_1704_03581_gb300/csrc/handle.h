@@ -38,7 +38,7 @@ struct pulda_handle {
     float *alpha = nullptr;
     // fixed tables
     uint32_t *t_thr = nullptr; uint16_t *t_alias = nullptr; int32_t *t_off = nullptr, *t_lo = nullptr, *t_n = nullptr;
-    uint32_t *t_geo = nullptr; double *t_gauss = nullptr;
+    uint32_t *t_geo = nullptr; double *t_gauss = nullptr; longlong2 *t_gauss_fix = nullptr;
     // Phi-step buffers
     uint16_t *nst_k = nullptr; uint32_t *nst_n = nullptr; int32_t *nnz_n = nullptr;
     uint16_t *cst_k = nullptr; uint32_t *cst_c = nullptr; int32_t *nnz_c = nullptr;

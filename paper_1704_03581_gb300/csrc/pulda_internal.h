@@ -114,6 +114,7 @@ struct DevTables {
     const uint32_t *geo;
     const double *gauss;
     double beta;
+    const longlong2 *gauss_fix;    // [kGaussCells] lower node and width of the cells in units of 2^-58 (Dirichlet mode)
 };
 
 // Everything the Phi-step kernels read and write.

@@ -104,3 +104,13 @@ def test_alias_pairing_past_64_bits(K, alpha):
     n = np.diff(t["col_ptr"])
     assert any(int(a) * int(c) >= 1 << 64 for a, c in zip(t["A"].view(np.uint64), n))
     s.close()
+
+
+@pytest.mark.parametrize("K,V", [(1, 1), (31, 255), (256, 256), (257, 257), (512, 272), (513, 40), (1024, 60), (1025, 33), (7, 4400)])
+def test_dirichlet_passes(K, V):
+    """Row sums across chunks of 256 words and batches of 16, and the
+    selection's registers (256, 512, 1,024 topics) and memory form."""
+    rng = np.random.default_rng(K + V)
+    w, off = corpus_of(rng, rng.poisson(4, V) + (np.arange(V) < 3) * 200, 20)
+    s, _ = lockstep(w, off, K, V, rng.uniform(0.05, 0.5, K).astype(np.float32), 0.02, seed=V, sweeps=2, phi_mode=1)
+    s.close()
