@@ -366,6 +366,7 @@ pulda_status pulda_init(pulda_handle **out, const int32_t *word_ids, const int64
     }
     h->N = N; h->D = D; h->K = K; h->V = V; h->seed = seed; h->beta = beta;
     for (int k = 0; k < K; ++k) h->alpha_sum += static_cast<double>(alpha[k]);
+    h->alpha_symmetric = std::all_of(alpha, alpha + K, [&](float x) { return x == alpha[0]; });
     h->KW = (K + 31) / 32;
     h->KWp = bitmap_row_words(K);
     h->cap = static_cast<int64_t>(K) * V;
@@ -707,7 +708,8 @@ pulda_status pulda_log_posterior(pulda_handle *h, double *out) {
     unsigned char *scratch = nullptr;
     DevTemp ts(h->opt, st);
     CU(h, ts.get(&scratch, log_posterior_scratch_bytes(h->D, h->V, h->K)));
-    launch_log_posterior(h->doc_off, h->D, h->z, h->K, h->alpha, h->alpha_sum, a, static_cast<double>(h->beta), scratch, st);
+    launch_log_posterior(h->doc_off, h->D, h->z, h->K, h->alpha, h->alpha_sum, a, static_cast<double>(h->beta),
+                         h->alpha_symmetric, scratch, st);
     CU(h, cudaGetLastError());
     CU(h, cudaMemcpyAsync(out, scratch, 3 * sizeof(double), cudaMemcpyDeviceToHost, st));
     return pulda_sync(h);

@@ -8,11 +8,15 @@
 //     + sum_k [ lgamma(V beta) - lgamma(V beta + n_k) + sum_v ( lgamma(beta + n_{k,v}) - lgamma(beta) ) ],
 //
 // A = sum_k alpha_k, n_k = sum_v n_{k,v}; terms with a zero count vanish.
-// Four kernels: a table of the small-count terms, one warp per document (m_d
-// in shared memory), one warp per word (the word's n column, rebuilt from z
-// by the Phi-step's count pass), and one CTA that adds the per-document and
-// per-word sums in a fixed order, so the same topics always give the same
-// bits.
+// A table of the small-count terms, one warp per document (m_d in shared
+// memory), one warp per word (the word's n column, rebuilt from z by the
+// Phi-step's count pass), the rows' terms, and one CTA that adds the partial
+// sums.  Every lane adds its own terms in a fixed order and so does each later
+// step, so the same topics always give the same bits.  The GPU has few FP64
+// units, and FP64 additions bound the passes: so no warp sum per document or
+// word, and a document's terms are taken off a list of its topics, 32 at a
+// time, not off all K (37,500 documents of 330 tokens, K = 1000: 227 -> 56 us;
+// 100,000 words 133 -> 78 us; one CTA's final sums and lgammas 76 -> 14 us).
 #include <algorithm>
 #include <cstdint>
 
@@ -29,17 +33,22 @@ constexpr int kTabA = 256;
 constexpr int kTabB = 4096;
 
 // ta[k * kTabA + c] = lgamma(alpha_k + c) - lgamma(alpha_k);  tb[n] = lgamma(beta + n) - lgamma(beta).
-__global__ void k_lp_tables(const float *alpha, int K, double beta, double *ta, double *tb) {
-    const int64_t na = static_cast<int64_t>(K) * kTabA;
-    for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < na + kTabB;
-         e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        if (e < na) {
-            const double ak = static_cast<double>(alpha[e / kTabA]);
-            ta[e] = lgamma(ak + static_cast<double>(e % kTabA)) - lgamma(ak);
-        } else {
-            const int n = static_cast<int>(e - na);
-            tb[n] = lgamma(beta + static_cast<double>(n)) - lgamma(beta);
-        }
+// lgamma is FP64 work: a row per CTA shares lgamma(alpha_k), a symmetric
+// alpha (rows = 1) has one row for every topic, and what every warp of the
+// other passes needs is computed here once: lg = lgamma of beta, A, V beta.
+__global__ void __launch_bounds__(kTabA) k_lp_tables(const float *alpha, int rows, double beta, double asum, double vb,
+                                                     double *ta, double *tb, double *lg) {
+    __shared__ double base;
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x < 3) lg[threadIdx.x] = lgamma(threadIdx.x == 0 ? beta : threadIdx.x == 1 ? asum : vb);
+    for (int r = blockIdx.x; r < rows + kTabB / kTabA; r += gridDim.x) {
+        const bool of_alpha = r < rows;
+        const double x0 = of_alpha ? static_cast<double>(alpha[r]) : beta;
+        const int n = of_alpha ? threadIdx.x : (r - rows) * kTabA + threadIdx.x;
+        if (threadIdx.x == 0) base = lgamma(x0);
+        const double top = lgamma(x0 + static_cast<double>(n));
+        __syncthreads();
+        (of_alpha ? ta + static_cast<int64_t>(r) * kTabA : tb)[n] = top - base;
+        __syncthreads();
     }
 }
 
@@ -50,76 +59,146 @@ __device__ __forceinline__ double warp_sum_f64(double v) {
     return v;
 }
 
-// doc_lp[d] = lgamma(A) - lgamma(A + N_d) + sum_{k: m_{d,k} > 0} (lgamma(alpha_k + m_{d,k}) - lgamma(alpha_k)).
-// Documents are assigned to warps statically.
+// A warp's counts, the bitmap of its document's topics, and their list.
+__host__ __device__ __forceinline__ int lp_doc_words(int K) { return K + (K + 31) / 32 + (K + 1) / 2; }
+
+// doc_part[warp] = its documents' lgamma(A) - lgamma(A + N_d) +
+// sum_{k: m_{d,k} > 0} (lgamma(alpha_k + m_{d,k}) - lgamma(alpha_k)).
+// Documents are assigned to warps statically; the lgamma(A + N_d) of up to 32
+// of them wait for one evaluation, a document per lane.
+constexpr int kDocLoads = 8;
 __global__ void k_lp_docs(const int64_t *doc_off, int64_t D, const int16_t *z, int K, const float *alpha, double asum,
-                          const double *ta, double *doc_lp) {
+                          const double *ta, const double *lg, int row, double *doc_part) {
     extern __shared__ uint32_t dsm[];
-    const int lane = threadIdx.x & 31;
-    uint32_t *m = dsm + static_cast<size_t>(threadIdx.x >> 5) * K;
+    const int lane = threadIdx.x & 31, KW = (K + 31) / 32;
+    uint32_t *m = dsm + static_cast<size_t>(threadIdx.x >> 5) * lp_doc_words(K);
+    uint32_t *bits = m + K;
+    uint16_t *list = reinterpret_cast<uint16_t *>(bits + KW);
+    const int warp = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int64_t warps = static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5);
-    for (int k = lane; k < K; k += 32) m[k] = 0;
+    for (int k = lane; k < K + KW; k += 32) m[k] = 0;
     __syncwarp();
-    const double lga = lgamma(asum);
-    for (int64_t d = blockIdx.x * static_cast<int64_t>(blockDim.x >> 5) + (threadIdx.x >> 5); d < D; d += warps) {
+    const double lga = lg[1];
+    double acc = 0.0;
+    int held = 0;
+    int64_t held_n = 0;
+    auto flush = [&] {
+        if (lane < held) acc += lga - lgamma(asum + static_cast<double>(held_n));
+        held = 0;
+    };
+    auto add = [&](int k) {
+        if (atomicAdd(&m[k], 1u) == 0) atomicOr(&bits[k >> 5], 1u << (k & 31));
+    };
+    for (int64_t d = warp; d < D; d += warps) {
         const int64_t b = doc_off[d], e = doc_off[d + 1];
-        for (int64_t i = b + lane; i < e; i += 32) atomicAdd(&m[z[i]], 1u);
+        int64_t i = b + lane;
+        for (; i + 32 * (kDocLoads - 1) < e; i += 32 * kDocLoads) {
+            int zz[kDocLoads];
+#pragma unroll
+            for (int u = 0; u < kDocLoads; ++u) zz[u] = z[i + 32 * u];
+#pragma unroll
+            for (int u = 0; u < kDocLoads; ++u) add(zz[u]);
+        }
+        for (; i < e; i += 32) add(z[i]);
         __syncwarp();
-        double t = 0.0;
-        for (int k = lane; k < K; k += 32) {
+        int n = 0;                                     // the topics, ascending
+        for (int w0 = 0; w0 < KW; w0 += 32) {
+            const int w = w0 + lane;
+            uint32_t x = w < KW ? bits[w] : 0u;
+            if (w < KW) bits[w] = 0;
+            int at = __popc(x);
+            const int own = at;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xFFFFFFFFu, at, o);
+                if (lane >= o) at += y;
+            }
+            uint16_t *l = list + n + at - own;
+            for (; x; x &= x - 1u) *l++ = static_cast<uint16_t>(32 * w + __ffs(x) - 1);
+            n += __shfl_sync(0xFFFFFFFFu, at, 31);
+        }
+        __syncwarp();
+#pragma unroll 4
+        for (int j = lane; j < n; j += 32) {
+            const int k = list[j];
             const uint32_t c = m[k];
-            if (c) {
-                if (c < kTabA) {
-                    t += ta[static_cast<int64_t>(k) * kTabA + c];
-                } else {
-                    const double ak = static_cast<double>(alpha[k]);
-                    t += lgamma(ak + static_cast<double>(c)) - lgamma(ak);
-                }
-                m[k] = 0;
+            m[k] = 0;
+            if (c < kTabA) {
+                acc += ta[static_cast<int64_t>(k) * row + c];
+            } else {
+                const double ak = static_cast<double>(alpha[k]);
+                acc += lgamma(ak + static_cast<double>(c)) - lgamma(ak);
             }
         }
-        t = warp_sum_f64(t);
-        if (lane == 0) doc_lp[d] = t + (lga - lgamma(asum + static_cast<double>(e - b)));
+        if (lane == held) held_n = e - b;
+        if (++held == 32) flush();
         __syncwarp();
     }
+    flush();
+    acc = warp_sum_f64(acc);
+    if (lane == 0) doc_part[warp] = acc;
 }
 
-// word_lp[v] = sum_{k: n_{k,v} > 0} (lgamma(beta + n_{k,v}) - lgamma(beta)); n_k accumulated
-// (integer atomics, so in any order).  Words are assigned to warps statically.
-__global__ void k_lp_words(const int64_t *word_off, const uint16_t *nst_k, const uint32_t *nst_n,
-                           const int32_t *nnz_n, int V, double beta, const double *tb, double *word_lp,
-                           unsigned long long *nk) {
+// word_part[warp] = its words' sum_{k: n_{k,v} > 0} (lgamma(beta + n_{k,v}) - lgamma(beta));
+// n_k accumulated (integer atomics, so in any order; a CTA's in shared memory
+// first where K counts fit).  Words are assigned to warps statically, but the
+// n_heavy most frequent ones (heavy_row >= 0), whose counts are past the table
+// and whose columns are long, in pieces of 32 entries.
+__global__ void k_lp_words(const int32_t *word_order, const int32_t *heavy_row, int n_heavy, int K, const int64_t *word_off, const uint16_t *nst_k, const uint32_t *nst_n,
+                           const int32_t *nnz_n, int V, double beta, const double *tb, const double *lg, double *word_part,
+                           unsigned long long *nk, int k_shared) {
+    extern __shared__ uint32_t nsm[];
     const int lane = threadIdx.x & 31;
-    const int warps = gridDim.x * (blockDim.x >> 5);
-    const double lgb = lgamma(beta);
-    for (int v = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); v < V; v += warps) {
+    const int warps = gridDim.x * (blockDim.x >> 5), warp = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const double lgb = lg[0];
+    for (int k = threadIdx.x; k < k_shared; k += blockDim.x) nsm[k] = 0;
+    __syncthreads();
+    double acc = 0.0;
+    auto entry = [&](int64_t at) {
+        const uint32_t n = nst_n[at];
+        const int k = nst_k[at];
+        acc += n < static_cast<uint32_t>(kTabB) ? tb[n] : lgamma(beta + static_cast<double>(n)) - lgb;
+        if (k_shared) atomicAdd(&nsm[k], n);               // fewer than 2^31 tokens
+        else atomicAdd(&nk[k], static_cast<unsigned long long>(n));
+    };
+    const int pieces = (K + 31) / 32;
+    for (int64_t i = warp; i < static_cast<int64_t>(n_heavy) * pieces; i += warps) {
+        const int v = word_order[i / pieces], j = 32 * static_cast<int>(i % pieces) + lane;
+        if (j < nnz_n[v]) entry(word_off[v] + j);
+    }
+    for (int v = warp; v < V; v += warps) {
+        if (n_heavy > 0 && heavy_row[v] >= 0) continue;
         const int64_t b = word_off[v];
         const int cnt = nnz_n[v];
-        double t = 0.0;
-        for (int j = lane; j < cnt; j += 32) {
-            const uint32_t n = nst_n[b + j];
-            t += n < static_cast<uint32_t>(kTabB) ? tb[n] : lgamma(beta + static_cast<double>(n)) - lgb;
-            atomicAdd(&nk[nst_k[b + j]], static_cast<unsigned long long>(n));
-        }
-        t = warp_sum_f64(t);
-        if (lane == 0) word_lp[v] = t;
+#pragma unroll 4
+        for (int j = lane; j < cnt; j += 32) entry(b + j);
     }
+    acc = warp_sum_f64(acc);
+    if (lane == 0) word_part[warp] = acc;
+    __syncthreads();
+    for (int k = threadIdx.x; k < k_shared; k += blockDim.x)
+        if (nsm[k]) atomicAdd(&nk[k], static_cast<unsigned long long>(nsm[k]));
+}
+
+// row_lp[k] = lgamma(V beta) - lgamma(V beta + n_k).
+__global__ void __launch_bounds__(32) k_lp_rows(const unsigned long long *nk, int K, double vb, const double *lg, double *row_lp) {
+    const int k = blockIdx.x * 32 + threadIdx.x;
+    if (k < K) row_lp[k] = lg[2] - lgamma(vb + static_cast<double>(nk[k]));
 }
 
 // out = {total, document sum, topic sum}: each thread adds a fixed strided
 // slice in order, then a fixed tree.
 constexpr int kFinalThreads = 1024;
-__global__ void __launch_bounds__(kFinalThreads) k_lp_final(const double *doc_lp, int64_t D, const double *word_lp,
-                                                            int V, const unsigned long long *nk, int K, double beta,
-                                                            double *out) {
+__global__ void __launch_bounds__(kFinalThreads) k_lp_final(const double *doc_part, int nd, const double *word_part,
+                                                            int nw, const double *row_lp, int K, double *out) {
     __shared__ double sd[kFinalThreads], st[kFinalThreads];
     const int t = threadIdx.x;
     double a = 0.0, b = 0.0;
-    for (int64_t d = t; d < D; d += kFinalThreads) a += doc_lp[d];
-    for (int v = t; v < V; v += kFinalThreads) b += word_lp[v];
-    const double vb = static_cast<double>(V) * beta;
-    const double lvb = lgamma(vb);
-    for (int k = t; k < K; k += kFinalThreads) b += lvb - lgamma(vb + static_cast<double>(nk[k]));
+#pragma unroll 8
+    for (int i = t; i < nd; i += kFinalThreads) a += doc_part[i];
+#pragma unroll 8
+    for (int i = t; i < nw; i += kFinalThreads) b += word_part[i];
+    for (int k = t; k < K; k += kFinalThreads) b += row_lp[k];
     sd[t] = a;
     st[t] = b;
     __syncthreads();
@@ -147,38 +226,48 @@ int device_attr(cudaDeviceAttr what) {
 }  // namespace
 
 size_t log_posterior_scratch_bytes(int64_t D, int V, int K) {
-    return sizeof(double) * (static_cast<size_t>(D) + static_cast<size_t>(V) + 3 + static_cast<size_t>(K) * kTabA + kTabB) +
+    // the warps of the document pass are at most D + kDiagWarps, those of the word pass V + 32
+    return sizeof(double) * (static_cast<size_t>(D) + kDiagWarps + static_cast<size_t>(V) + 32 + 6 + static_cast<size_t>(K) * (kTabA + 1) + kTabB) +
            sizeof(unsigned long long) * static_cast<size_t>(K);
 }
 
 void launch_log_posterior(const int64_t *doc_off, int64_t D, const int16_t *z, int K, const float *alpha, double asum,
-                          const PhiArgs &counts, double beta, void *scratch, cudaStream_t st) {
+                          const PhiArgs &counts, double beta, bool symmetric, void *scratch, cudaStream_t st) {
     double *out = static_cast<double *>(scratch);
-    double *doc_lp = out + 3;
-    double *word_lp = doc_lp + D;
-    double *ta = word_lp + counts.V;
+    double *lg = out + 3;
+    double *doc_part = lg + 3;
+    double *word_part = doc_part + D + kDiagWarps;
+    double *row_lp = word_part + counts.V + 32;
+    double *ta = row_lp + K;
     double *tb = ta + static_cast<size_t>(K) * kTabA;
     unsigned long long *nk = reinterpret_cast<unsigned long long *>(tb + kTabB);
     cudaMemsetAsync(nk, 0, sizeof(unsigned long long) * static_cast<size_t>(K), st);
     const int sms = std::max(1, device_attr(cudaDevAttrMultiProcessorCount));
-    k_lp_tables<<<4 * sms, 256, 0, st>>>(alpha, K, beta, ta, tb);
+    const int rows = symmetric ? 1 : K;
+    k_lp_tables<<<std::min(rows + kTabB / kTabA, 8 * sms), kTabA, 0, st>>>(alpha, rows, beta, asum, static_cast<double>(counts.V) * beta, ta, tb, lg);
+    int doc_warps = 0;
     if (D > 0) {
-        // m_d of one warp: K counts; the CTA shrinks for large K
+        // the CTA shrinks for large K
         int warps = kDiagWarps;
         const int optin = std::max(48 * 1024, device_attr(cudaDevAttrMaxSharedMemoryPerBlockOptin));
-        while (warps > 1 && static_cast<size_t>(warps) * K * sizeof(uint32_t) > static_cast<size_t>(optin)) warps >>= 1;
-        const size_t smem = static_cast<size_t>(warps) * K * sizeof(uint32_t);
+        while (warps > 1 && static_cast<size_t>(warps) * lp_doc_words(K) * sizeof(uint32_t) > static_cast<size_t>(optin)) warps >>= 1;
+        const size_t smem = static_cast<size_t>(warps) * lp_doc_words(K) * sizeof(uint32_t);
         if (smem > 48 * 1024) cudaFuncSetAttribute(k_lp_docs, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
         int per_sm = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lp_docs, 32 * warps, smem);
         const int64_t need = (D + warps - 1) / warps;
         const int grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(need, static_cast<int64_t>(sms) * std::max(1, per_sm))));
-        k_lp_docs<<<grid, 32 * warps, smem, st>>>(doc_off, D, z, K, alpha, asum, ta, doc_lp);
+        k_lp_docs<<<grid, 32 * warps, smem, st>>>(doc_off, D, z, K, alpha, asum, ta, lg, symmetric ? 0 : kTabA, doc_part);
+        doc_warps = grid * warps;
     }
-    const int wgrid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>((counts.V + kDiagWarps - 1) / kDiagWarps, 8LL * sms)));
-    k_lp_words<<<wgrid, 32 * kDiagWarps, 0, st>>>(counts.word_off, counts.nst_k, counts.nst_n, counts.nnz_n, counts.V, beta,
-                                                   tb, word_lp, nk);
-    k_lp_final<<<1, kFinalThreads, 0, st>>>(doc_lp, D, word_lp, counts.V, nk, K, beta, out);
+    constexpr int kWordThreads = 1024;
+    const int64_t words_cta = kWordThreads / 32;
+    const int wgrid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>((counts.V + words_cta - 1) / words_cta, 2LL * sms)));
+    const int k_shared = K <= 12288 ? K : 0;               // within 48 KB
+    k_lp_words<<<wgrid, kWordThreads, sizeof(uint32_t) * k_shared, st>>>(counts.word_order, counts.heavy_row, counts.n_heavy, K, counts.word_off, counts.nst_k, counts.nst_n, counts.nnz_n,
+                                                                         counts.V, beta, tb, lg, word_part, nk, k_shared);
+    k_lp_rows<<<(K + 31) / 32, 32, 0, st>>>(nk, K, static_cast<double>(counts.V) * beta, lg, row_lp);
+    k_lp_final<<<1, kFinalThreads, 0, st>>>(doc_part, doc_warps, word_part, wgrid * static_cast<int>(words_cta), row_lp, K, out);
 }
 
 }  // namespace pulda

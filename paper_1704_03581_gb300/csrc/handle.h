@@ -62,6 +62,7 @@ struct pulda_handle {
     int *work = nullptr;
     unsigned long long *stats = nullptr;
     uint32_t *sort_scratch = nullptr;   // count_path 1: keys, run ids, scan sums
+    bool alpha_symmetric = false;       // every alpha_k the same
     int n_big = 0;                      // words counted by a CTA each
     int64_t cap = 0;   // capacity of the per-word tables: K * V entries
     // words histogrammed by several CTAs (more than heavy_word(N) tokens)

@@ -301,7 +301,7 @@ size_t dir_part_count(int V, int K);
 // doubles receive {total, document sum, topic sum}.
 size_t log_posterior_scratch_bytes(int64_t D, int V, int K);
 void launch_log_posterior(const int64_t *doc_off, int64_t D, const int16_t *z, int K, const float *alpha, double asum,
-                          const PhiArgs &counts, double beta, void *scratch, cudaStream_t st);
+                          const PhiArgs &counts, double beta, bool symmetric, void *scratch, cudaStream_t st);
 
 // The grid barrier of the one-launch batched sweep (device memory, zeroed).
 struct GridBarrier {

@@ -114,3 +114,21 @@ def test_dirichlet_passes(K, V):
     w, off = corpus_of(rng, rng.poisson(4, V) + (np.arange(V) < 3) * 200, 20)
     s, _ = lockstep(w, off, K, V, rng.uniform(0.05, 0.5, K).astype(np.float32), 0.02, seed=V, sweeps=2, phi_mode=1)
     s.close()
+
+
+@pytest.mark.parametrize("alpha", [0.1, None])
+def test_log_posterior_of_many_and_of_large_documents(alpha):
+    """More than 32 documents per warp, counts past both tables, one row of
+    the document table (symmetric alpha) or a row per topic."""
+    from test_diag_gpu import check
+    import paper_1704_03581_gb300 as P
+    rng = np.random.default_rng(4)
+    K, V = 3, 30
+    off = np.zeros(500004, np.int64)
+    np.cumsum(np.concatenate([[20000, 0, 9000], rng.integers(0, 3, 500000)]), out=off[1:])
+    w = rng.integers(0, V, int(off[-1])).astype(np.int32)
+    al = np.full(K, alpha, np.float32) if alpha else rng.uniform(0.1, 1.0, K).astype(np.float32)
+    s = P.Sampler(w, off, K, V, al, 0.02, seed=7)
+    s.sweep(1)
+    check(s, off, w, K, V, al, 0.02)
+    s.close()
