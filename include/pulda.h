@@ -257,7 +257,7 @@ pulda_status pulda_infer(pulda_handle *h, const int32_t *word_ids_host, const in
  *   also its working state).
  * The results equal pulda_infer's with the same seed and n_sweeps.
  * The few bytes of scratch the z-step needs live in a fixed array of static
- * device memory (262,912 bytes, held by every GPU that loads the library until
+ * device memory (263,680 bytes, held by every GPU that loads the library until
  * the process exits), so D_new is limited to 65,536 documents per call; larger
  * D_new returns PULDA_ERR_INVALID.  The first call on each device looks up
  * that array's device address once; make that first call before any stream

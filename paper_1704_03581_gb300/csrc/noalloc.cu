@@ -28,16 +28,24 @@ namespace {
 // Largest number of documents one call may carry.
 constexpr int64_t kNoAllocMaxDocs = 65536;
 
-// Layout of the scratch array (bytes, each part 256-byte aligned).
+// Length classes of documents, eight to an octave and the longest first: those
+// of 2^16 tokens or more (one warp each), then those of at least coop_len (a
+// CTA each), then the rest.  So the schedule is longest first, but for lengths
+// within an eighth of each other; in any order within the three groups, a long
+// document taken up late was the end of the pass (4,096 documents: 2.10 ms).
+constexpr int kLengthKeys = 112;
+constexpr int kClasses = 1 + 2 * kLengthKeys;
+
+// Layout of the scratch array (bytes).
 constexpr size_t kOffStats = 0;                                       // u64[ST_TOTAL_SLOTS]
 constexpr size_t kOffWork = 256;                                      // int[5]: z-step work counters
-constexpr size_t kOffCount = 320;                                     // int[4]: documents by length class
-constexpr size_t kOffFlag = 512;                                      // u64[2]: first bad token, first bad document
-constexpr size_t kOffOrder = 768;                                     // int32[kNoAllocMaxDocs]
-constexpr size_t kScratchBytes = kOffOrder + sizeof(int32_t) * kNoAllocMaxDocs;   // 262,912 bytes
+constexpr size_t kOffCount = 320;                                     // int[kClasses]: documents by length class
+constexpr size_t kOffFlag = 1280;                                     // u64[2]: first bad token, first bad document
+constexpr size_t kOffOrder = 1536;                                    // int32[kNoAllocMaxDocs]
+constexpr size_t kScratchBytes = kOffOrder + sizeof(int32_t) * kNoAllocMaxDocs;   // 263,680 bytes
 static_assert(ST_TOTAL_SLOTS * sizeof(unsigned long long) <= kOffWork, "the counters overlap the work counter");
 static_assert(5 * sizeof(int) <= kOffCount - kOffWork, "the work counters overlap the class counts");
-static_assert(4 * sizeof(int) <= kOffFlag - kOffCount, "the class counts overlap the input check");
+static_assert(kClasses * sizeof(int) <= kOffFlag - kOffCount, "the class counts overlap the input check");
 static_assert(2 * sizeof(unsigned long long) <= kOffOrder - kOffFlag, "the input check overlaps the schedule");
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
@@ -65,10 +73,11 @@ cudaError_t scratch_on_device(int dev, unsigned char **out) {
     return cudaSuccess;
 }
 
-// A document's class: 0 with 2^16 tokens or more (one warp), 1 at least coop_len
-// (a CTA each), 2 the rest.
 __device__ __forceinline__ int length_class(int64_t len, int64_t coop_len) {
-    return len > kNarrowMaxLen ? 0 : len >= coop_len ? 1 : 2;
+    if (len > kNarrowMaxLen) return 0;
+    const int n = static_cast<int>(len), e = 31 - __clz(n | 1);
+    const int key = n < 8 ? n : 8 * (e - 2) + ((n >> (e - 3)) & 7);       // at most 111
+    return (len >= coop_len ? 1 : 1 + kLengthKeys) + kLengthKeys - 1 - key;
 }
 
 // Checks the caller's device inputs (ids in [0, V), offsets nondecreasing from
@@ -145,7 +154,7 @@ extern "C" pulda_status pulda_infer_noalloc(pulda_handle *h, const int32_t *word
         k_noalloc_check<<<64, 256, 0, st>>>(word_ids_dev, N_new, doc_offsets_dev, D_new, hv.V, first, count, coop_len);
         e = cudaGetLastError();
     }
-    int hcount[3] = {0, 0, 0};
+    int hcount[kClasses] = {};
     if (e == cudaSuccess) e = cudaMemcpyAsync(hcount, count, sizeof hcount, cudaMemcpyDeviceToHost, st);
     unsigned long long hfirst[2] = {~0ull, ~0ull};
     if (e == cudaSuccess) e = cudaMemcpyAsync(hfirst, first, sizeof hfirst, cudaMemcpyDeviceToHost, st);
@@ -162,7 +171,13 @@ extern "C" pulda_status pulda_infer_noalloc(pulda_handle *h, const int32_t *word
         snprintf(msg, sizeof msg, "the word id at token %llu is outside [0, %d)", hfirst[0], hv.V);
         return static_cast<pulda_status>(handle_fail(h, PULDA_ERR_INVALID, msg));
     }
-    const int cursor[3] = {0, hcount[0], hcount[0] + hcount[1]};
+    const int n_wide = hcount[0];
+    int n_coop = 0, cursor[kClasses], run = 0;
+    for (int c = 0; c < kClasses; ++c) {
+        cursor[c] = run;
+        run += hcount[c];
+        if (c >= 1 && c <= kLengthKeys) n_coop += hcount[c];
+    }
     e = cudaMemcpyAsync(count, cursor, sizeof cursor, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) {
         k_noalloc_order<<<64, 256, 0, st>>>(doc_offsets_dev, D_new, coop_len, count, order);
@@ -180,7 +195,7 @@ extern "C" pulda_status pulda_infer_noalloc(pulda_handle *h, const int32_t *word
     a.stats = stats;
     for (int32_t sw = 1; sw <= n_sweeps && e == cudaSuccess; ++sw) {
         a.sweep = static_cast<uint32_t>(sw);
-        e = run_z(h, a, hcount[0], hcount[1], work);
+        e = run_z(h, a, n_wide, n_coop, work);
     }
     unsigned long long err = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&err, stats + ST_ERROR, sizeof err, cudaMemcpyDeviceToHost, st);
