@@ -16,7 +16,7 @@
 // units, and FP64 additions bound the passes: so no warp sum per document or
 // word, and a document's terms are taken off a list of its topics, 32 at a
 // time, not off all K (37,500 documents of 330 tokens, K = 1000: 227 -> 56 us;
-// 100,000 words 133 -> 78 us; one CTA's final sums and lgammas 76 -> 14 us).
+// 100,000 words 133 -> 78 us; one CTA's final sums and lgammas 76 -> 20 us).
 #include <algorithm>
 #include <cstdint>
 
@@ -186,33 +186,50 @@ __global__ void __launch_bounds__(32) k_lp_rows(const unsigned long long *nk, in
     if (k < K) row_lp[k] = lg[2] - lgamma(vb + static_cast<double>(nk[k]));
 }
 
+// A sum with the rounding errors of its additions kept beside it (Knuth's
+// two-sum): the last, largest additions would otherwise decide the error.
+struct Sum2 {
+    double s, e;
+    __device__ __forceinline__ void add(double x) {
+        const double t = s + x, y = t - s;
+        e += (s - (t - y)) + (x - y);
+        s = t;
+    }
+    __device__ __forceinline__ void add(const Sum2 &o) {
+        add(o.s);
+        e += o.e;
+    }
+    __device__ __forceinline__ double value() const { return s + e; }
+};
+
 // out = {total, document sum, topic sum}: each thread adds a fixed strided
 // slice in order, then a fixed tree.
-constexpr int kFinalThreads = 1024;
+constexpr int kFinalThreads = 512;
 __global__ void __launch_bounds__(kFinalThreads) k_lp_final(const double *doc_part, int nd, const double *word_part,
                                                             int nw, const double *row_lp, int K, double *out) {
-    __shared__ double sd[kFinalThreads], st[kFinalThreads];
+    __shared__ Sum2 sd[kFinalThreads], st[kFinalThreads];
     const int t = threadIdx.x;
-    double a = 0.0, b = 0.0;
+    Sum2 a{0.0, 0.0}, b{0.0, 0.0};
 #pragma unroll 8
-    for (int i = t; i < nd; i += kFinalThreads) a += doc_part[i];
+    for (int i = t; i < nd; i += kFinalThreads) a.add(doc_part[i]);
 #pragma unroll 8
-    for (int i = t; i < nw; i += kFinalThreads) b += word_part[i];
-    for (int k = t; k < K; k += kFinalThreads) b += row_lp[k];
+    for (int i = t; i < nw; i += kFinalThreads) b.add(word_part[i]);
+    for (int k = t; k < K; k += kFinalThreads) b.add(row_lp[k]);
     sd[t] = a;
     st[t] = b;
     __syncthreads();
     for (int s = kFinalThreads / 2; s > 0; s >>= 1) {
         if (t < s) {
-            sd[t] += sd[t + s];
-            st[t] += st[t + s];
+            sd[t].add(sd[t + s]);
+            st[t].add(st[t + s]);
         }
         __syncthreads();
     }
     if (t == 0) {
-        out[0] = sd[0] + st[0];
-        out[1] = sd[0];
-        out[2] = st[0];
+        out[1] = sd[0].value();
+        out[2] = st[0].value();
+        sd[0].add(st[0]);
+        out[0] = sd[0].value();
     }
 }
 
