@@ -93,9 +93,10 @@ typedef struct {
                                batched form takes 0); the counts are identical */
     int32_t batch_form;     /* batched form only: how a sweep is launched -- 0 = tuned (timed on
                                the first sweeps with the CTA sizes), 1 = six launches (a CUDA
-                               graph), 2 = one persistent cooperative launch whose phases are
-                               separated by grid barriers (every document one per warp; not
-                               with coop_min_len > 0); the chains' results are identical */
+                               graph), 2 = the Phi-step as one persistent cooperative launch
+                               whose phases are separated by grid barriers (every document
+                               one per warp; not with coop_min_len > 0); the chains' results
+                               are identical */
     int32_t alias_layout;   /* how the per-word alias tables of the a part ("Efficient sampling
                                of z") are laid out for the z-step: 1 = a threshold array and an
                                alias-topic array beside the column's topics (two loads per

@@ -355,7 +355,7 @@ pulda_status pulda_batch_init(pulda_batch **out, const pulda_chain_desc *chains,
     bl.n_big = phi_big_words(kmax, static_cast<int64_t>(wi.size()), rare - wi.begin(), bl.phi_grid);
     for (const pulda_handle *h : b->ch) bl.vmax = std::max(bl.vmax, h->V);
     bl.bar = d_bar;
-    bl.persist_grid = b->sms * batch_persistent_blocks_per_sm(kmax, narrow, &bl.persist_z_warps, &bl.table_stage);
+    bl.persist_grid = b->sms * batch_persistent_blocks_per_sm(kmax, narrow, &bl.table_stage);
     // The threshold of the documents on CTAs: fixed, none, or the automatic rule
     // over all chains' tokens (documents that would outlast the pass on one
     // warp).  It is not timed: a few early sweeps chose worse thresholds than
@@ -368,13 +368,15 @@ pulda_status pulda_batch_init(pulda_batch **out, const pulda_chain_desc *chains,
     // Launch forms: a launch or a few per phase with a CTA size for the z-step, and
     // (without documents on CTAs) one persistent launch; tuned forms are timed.
     const bool one_ok = bl.persist_grid > 0 && fixed_coop == 0;
+    int one_warps = kMultiWarps;
+    while (one_warps > 1 && z_step_smem(kmax, one_warps, narrow) > 160 * 1024) one_warps >>= 1;
     const bool pk = b->packed;
     if (o.batch_form == 2) {
         if (!one_ok) {
             b->err = "the one-launch form needs no document on cooperative CTAs and a resident grid";
             return bail(PULDA_ERR_INVALID);
         }
-        b->cand.push_back({kMultiWarps, 0, true, pk});
+        b->cand.push_back({one_warps, 0, true, pk});
     } else if (o.warps_per_block > 0) {
         int w = o.warps_per_block;
         while (w > 1 && z_step_smem(kmax, w, narrow) > static_cast<size_t>(smem_optin())) --w;
@@ -384,7 +386,7 @@ pulda_status pulda_batch_init(pulda_batch **out, const pulda_chain_desc *chains,
             if (w <= kMultiWarps && z_step_smem(kmax, w) <= 160 * 1024) b->cand.push_back({w, fixed_coop, false, pk});
         if (b->cand.empty()) b->cand.push_back({1, fixed_coop, false, pk});
     }
-    if (o.batch_form == 0 && o.warps_per_block == 0 && one_ok) b->cand.push_back({kMultiWarps, 0, true, pk});
+    if (o.batch_form == 0 && o.warps_per_block == 0 && one_ok) b->cand.push_back({one_warps, 0, true, pk});
     b->tune_layout = o.alias_layout == 0;
     if (b->cand.size() == 1 && b->tune_layout) {
         // one launch form: time the two layouts only

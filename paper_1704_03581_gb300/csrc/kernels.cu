@@ -1449,17 +1449,10 @@ static void launch_z_step_multi(const BatchLaunch &b, const BatchForm &f, const 
                                                                                                 narrow ? 1 : 0);
 }
 
-void launch_batch_sweep(const BatchLaunch &b, cudaStream_t st) {
-    k_batch_begin_sweep<<<1, 256, 0, st>>>(b.phi, b.n_chains, b.sweep, b.work);
-    launch_heavy_hist(b.phi, b.heavy, b.n_heavy, b.kmax, st);
-    k_phi_counts_multi<<<b.phi_grid, kPhiCountBlock, sizeof(uint32_t) * phi_count_words(b.kmax), st>>>(
-        b.phi, b.phi_items, b.n_phi_items, std::min(b.n_big, b.n_phi_items), b.work, b.work + 1, b.kmax, true);
-    k_phi_fixup_multi<<<b.n_chains, kFixBlock, 0, st>>>(b.phi);
-    k_colptr_scan_multi<<<dim3(b.n_chains, scan_chunks(b.vmax)), kScanBlock, 0, st>>>(b.phi);
-    launch_phi_tables_multi(b.phi, b.phi_items, b.n_phi_items, b.kmax, st);
-    // The chains' documents by form, the longest ones of each on CTAs beside
-    // the others: every launch on a stream of its own (the CTAs first), so that
-    // one's last documents do not hold up the next.
+// The chains' documents by form, the longest ones of each on CTAs beside the
+// others: every launch on a stream of its own (the CTAs first), so that one's
+// last documents do not hold up the next.
+static void launch_batch_z(const BatchLaunch &b, cudaStream_t st) {
     cudaEventRecord(b.ev_fork, st);
     int used = 0;
     auto branch = [&](auto launch) {
@@ -1491,22 +1484,29 @@ void launch_batch_sweep(const BatchLaunch &b, cudaStream_t st) {
     }
 }
 
-// ---------------------------------------------------------- one persistent launch per sweep
-// The same sweep of many chains as launch_batch_sweep, in one cooperative
+void launch_batch_sweep(const BatchLaunch &b, cudaStream_t st) {
+    k_batch_begin_sweep<<<1, 256, 0, st>>>(b.phi, b.n_chains, b.sweep, b.work);
+    launch_heavy_hist(b.phi, b.heavy, b.n_heavy, b.kmax, st);
+    k_phi_counts_multi<<<b.phi_grid, kPhiCountBlock, sizeof(uint32_t) * phi_count_words(b.kmax), st>>>(
+        b.phi, b.phi_items, b.n_phi_items, std::min(b.n_big, b.n_phi_items), b.work, b.work + 1, b.kmax, true);
+    k_phi_fixup_multi<<<b.n_chains, kFixBlock, 0, st>>>(b.phi);
+    k_colptr_scan_multi<<<dim3(b.n_chains, scan_chunks(b.vmax)), kScanBlock, 0, st>>>(b.phi);
+    launch_phi_tables_multi(b.phi, b.phi_items, b.n_phi_items, b.kmax, st);
+    launch_batch_z(b, st);
+}
+
+// ---------------------------------------------------------- one persistent launch per Phi-step
+// The same Phi-step of many chains as launch_batch_sweep's, in one cooperative
 // launch whose CTAs are all resident: the phases (counter reset, heavy-word
 // histograms, counts and draws, dead-row redraws, column offsets, per-word
-// tables, z-step) run one after another, each over the whole grid, separated
-// by a grid barrier.  Nothing a phase reads was read earlier in the launch by
+// tables) run one after another, each over the whole grid, separated by a grid
+// barrier.  The z-step follows in its own launches: five forms of it in this
+// kernel took 128 registers, so 16 warps per SM against their 28 (99.9M tokens
+// in eight chains: a sweep took 46 ms).  Nothing a phase reads was read earlier in the launch by
 // another SM before its writers finished (so no stale L1 line is read), except
 // the row sums and heavy-word histograms, which are read from L2.
 constexpr int kPersistThreads = 256;
 constexpr int kPersistWarps = kPersistThreads / 32;
-// Two CTAs per SM: five forms of the z-step in one kernel spill at more (99.9M
-// tokens in eight chains: a sweep takes 62 / 47 / 46 ms at 4 / 3 / 2).
-#ifndef PULDA_PERSIST_MINB
-#define PULDA_PERSIST_MINB 2
-#endif
-
 // A grid barrier with a bounded wait: thread 0 of each CTA arrives; the last
 // to arrive opens the next generation.  A CTA that has waited 2 s sets
 // ERR_BARRIER in err and returns false (the launch then ends with an error
@@ -1550,7 +1550,7 @@ __global__ void k_barrier_selftest(GridBarrier *bar, unsigned expect, int rounds
     }
 }
 
-__global__ void __launch_bounds__(kPersistThreads, PULDA_PERSIST_MINB) k_batch_sweep_persistent(BatchLaunch b) {
+__global__ void __launch_bounds__(kPersistThreads, 4) k_batch_sweep_persistent(BatchLaunch b) {
     extern __shared__ __align__(16) uint32_t psm[];
     __shared__ int scan_tmp[kPersistThreads / 32 + 1];
     __shared__ int s_item;
@@ -1604,27 +1604,6 @@ __global__ void __launch_bounds__(kPersistThreads, PULDA_PERSIST_MINB) k_batch_s
             phi_tables_word_warp(b.phi[it.x], it.y, t.stage, t.scratch);
         }
     }
-    if (!grid_barrier(b.bar, nb, err)) return;
-    // z-step, one warp per (chain, document), form by form (a warp goes on to
-    // the next form's documents as soon as one's are all taken)
-    if (static_cast<int>(threadIdx.x >> 5) < b.persist_z_warps) {
-        uint32_t *m = psm + static_cast<size_t>(threadIdx.x >> 5) * z_dense_warp_words(b.kmax, b.narrow != 0);
-        u64 *wcnt = z_dense_counters(m, b.kmax, b.narrow != 0);
-        zero_warp_counters(wcnt);
-#pragma unroll 1
-        for (int f = 0; f < b.n_forms; ++f) {
-            const int2 *items = b.form_items + b.form[f].first;
-            const int n = b.form[f].n;
-            int *work = b.work + 4 + 3 * f;
-            switch (z_nw(b.form[f].kmax)) {
-                case 1: z_multi_items<1>(b.z, items, n, work, m, wcnt, b.narrow); break;
-                case 2: z_multi_items<2>(b.z, items, n, work, m, wcnt, b.narrow); break;
-                case 4: z_multi_items<4>(b.z, items, n, work, m, wcnt, b.narrow); break;
-                case 8: z_multi_items<8>(b.z, items, n, work, m, wcnt, b.narrow); break;
-                default: z_multi_items<0>(b.z, items, n, work, m, wcnt, b.narrow);
-            }
-        }
-    }
 }
 
 cudaError_t launch_barrier_selftest(GridBarrier *bar, int blocks, int missing, int rounds, unsigned long long *err,
@@ -1642,22 +1621,20 @@ cudaError_t launch_barrier_selftest(GridBarrier *bar, int blocks, int missing, i
                               passed);
 }
 
-// The z-step phase runs on all of a CTA's warps, or on one fewer where eight
-// warps' counts just do not fit.
-static size_t batch_persistent_smem(int kmax, int z_warps, bool narrow) {
-    return std::max({phi_counts_smem(kmax), static_cast<size_t>(kPersistWarps * kTabScratch),
-                     z_step_smem(kmax, z_warps, narrow)});
+static size_t batch_persistent_smem(int kmax, int stage) {
+    return std::max(phi_counts_smem(kmax), static_cast<size_t>(kPersistWarps) * (stage + kTabScratch));
 }
 
-int batch_persistent_blocks_per_sm(int kmax, bool narrow, int *z_warps, int *table_stage) {
+// 0 where the form is not offered: no room for a CTA, or K so large that the
+// counts of seven documents do not fit a CTA.
+int batch_persistent_blocks_per_sm(int kmax, bool narrow, int *table_stage) {
     allow_dynamic_smem(k_batch_sweep_persistent);
+    if (z_step_smem(kmax, kPersistWarps - 1, narrow) > static_cast<size_t>(smem_optin())) return 0;
+    const size_t rows = static_cast<size_t>(kPersistWarps) * (dense_row_bytes(kmax) + kTabScratch);
+    *table_stage = rows <= 56 * 1024 ? dense_row_bytes(kmax) : 0;       // four CTAs per SM
     int n = 0;
-    for (int w = kPersistWarps; w >= kPersistWarps - 1 && n <= 0; --w) {
-        const size_t smem = batch_persistent_smem(kmax, w, narrow);
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_batch_sweep_persistent, kPersistThreads, smem) != cudaSuccess) n = 0;
-        *z_warps = w;
-        *table_stage = static_cast<size_t>(kPersistWarps) * (dense_row_bytes(kmax) + kTabScratch) <= smem ? dense_row_bytes(kmax) : 0;
-    }
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_batch_sweep_persistent, kPersistThreads,
+                                                      batch_persistent_smem(kmax, *table_stage)) != cudaSuccess) n = 0;
     return n;
 }
 
@@ -1665,14 +1642,17 @@ cudaError_t launch_batch_sweep_persistent(const BatchLaunch &b, cudaStream_t st)
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(b.persist_grid));
     cfg.blockDim = dim3(kPersistThreads);
-    cfg.dynamicSmemBytes = batch_persistent_smem(b.kmax, b.persist_z_warps, b.narrow != 0);
+    cfg.dynamicSmemBytes = batch_persistent_smem(b.kmax, b.table_stage);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_batch_sweep_persistent, b);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_batch_sweep_persistent, b);
+    if (e != cudaSuccess) return e;
+    launch_batch_z(b, st);
+    return cudaGetLastError();
 }
 
 int batch_phi_blocks_per_sm(int kmax) {

@@ -321,8 +321,8 @@ struct BatchForm {
 constexpr int kBatchCounters = 2 + 3 * kMaxForms;     // work queues of a sweep
 
 // One sweep of many chains: a launch or a few per phase, every kernel over all
-// chains' work items (of a form, in the z-step), or one persistent launch doing
-// the same.  Pointers are device memory.
+// chains' work items (of a form, in the z-step), or one persistent launch for
+// the Phi-step.  Pointers are device memory.
 struct BatchLaunch {
     const HeavyChunk *heavy;     // heavy-word histogram chunks of every chain
     int n_heavy;
@@ -347,15 +347,13 @@ struct BatchLaunch {
     // the one-launch form: its grid (all CTAs resident) and barrier
     int persist_grid;
     GridBarrier *bar;
-    int persist_z_warps;         // warps of a CTA in its z-step phase
     int table_stage;             // bytes of a warp's stage in its table phase (0: rows are written in place)
 };
 void launch_batch_sweep(const BatchLaunch &b, cudaStream_t st);
-// The same sweep as one cooperative launch (no cooperative z-step: every
-// document one per warp); needs persist_grid <= SMs x
+// The same sweep with the Phi-step as one cooperative launch; needs persist_grid <= SMs x
 // batch_persistent_blocks_per_sm(kmax).
 cudaError_t launch_batch_sweep_persistent(const BatchLaunch &b, cudaStream_t st);
-int batch_persistent_blocks_per_sm(int kmax, bool narrow, int *z_warps, int *table_stage);
+int batch_persistent_blocks_per_sm(int kmax, bool narrow, int *table_stage);
 // The grid barrier's self-test: `blocks` resident CTAs pass `rounds`
 // barriers that expect blocks + missing arrivals.
 cudaError_t launch_barrier_selftest(GridBarrier *bar, int blocks, int missing, int rounds, unsigned long long *err,
