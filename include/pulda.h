@@ -53,9 +53,9 @@ typedef struct pulda_handle pulda_handle;
 typedef struct {
     void *stream;           /* cudaStream_t to run on; NULL = a stream the handle creates */
     int32_t zstep_path;     /* 0 = auto (a word with few nonzero topics is summed over its Phi
-                               column, the others over a dense row of its weights), 1 = always
-                               over the column, 2 = over the dense row wherever there is one;
-                               results are identical */
+                               column, the others over a dense row of its weights), 1 = the
+                               column for words of up to twice as many topics, 2 = the dense row
+                               wherever there is one; results are identical */
     int32_t warps_per_block;/* warp-per-document z-step: warps per CTA, 1..4; 0 = 4, halved
                                while the CTA's shared memory would pass 160 KB */
     int32_t docs_per_warp;  /* z-step documents per warp: 0 = auto (two at K <= 1024 in passes

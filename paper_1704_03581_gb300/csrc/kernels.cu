@@ -1045,7 +1045,7 @@ __global__ void k_phi_tables_multi(const PhiArgs *chains, const int2 *items, int
 // one pass.
 // NW = z_nw(K) words per lane and plane, one instantiation per kernel.
 template <int NW>
-__global__ void __launch_bounds__(32 * kZWarps, PULDA_ZMINBLOCKS) k_z_step(ZArgs a) {
+__global__ void __launch_bounds__(32 * kZWarps, NW < 0 ? 2 : PULDA_ZMINBLOCKS) k_z_step(ZArgs a) {
     extern __shared__ __align__(16) uint32_t zsm[];
     const int lane = threadIdx.x & 31;
     uint32_t *m = zsm + static_cast<size_t>(threadIdx.x >> 5) * z_dense_warp_words(a.K, a.narrow != 0);
@@ -1427,7 +1427,13 @@ void launch_slice_counts(const int64_t *doc_off, const int32_t *sliced_docs, int
 }
 
 void launch_z_step(const ZArgs &a, int warps_per_block, int grid, cudaStream_t st) {
-    z_step_kernel(a.K)<<<grid, 32 * warps_per_block, z_step_smem(a.K, warps_per_block, a.narrow != 0), st>>>(a);
+    // documents of 2^16 tokens or more are few, and each is bound by its loads'
+    // latency: above 1,024 topics they take the form that has more of them in
+    // flight
+    const bool few = a.narrow == 0 && a.n_slices == 0 && a.D <= 4 * static_cast<int64_t>(sm_count()) && z_nw(a.K) == 0;
+    const ZStepKernel kern = few ? k_z_step<-1> : z_step_kernel(a.K);
+    if (few) allow_dynamic_smem(kern);
+    kern<<<grid, 32 * warps_per_block, z_step_smem(a.K, warps_per_block, a.narrow != 0), st>>>(a);
 }
 
 using ZMultiKernel = void (*)(const ZArgs *, const int2 *, int, int *, int, int);

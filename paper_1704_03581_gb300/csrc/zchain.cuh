@@ -521,7 +521,7 @@ __device__ __forceinline__ void z_doc_chain(const ZArgs &a, uint8_t *sm, DocRun 
     } else if (role == 2) {
         kd = static_cast<int>(__reduce_add_sync(0xFFFFFFFFu, static_cast<unsigned>(form.init_bits(m, sm + kChainCountOff + 2 * chain_count_sets(K) * PB, lane))));
     }
-    const int colmax = a.path == 1 ? 0x7FFFFFFF : -1;
+    const int colmax = -1;         // a row wherever there is one
     const uint32_t sweep_end = r.sweep + static_cast<uint32_t>(r.max_pass_end);
     bool stop = false;
     while (!stop && r.budget > 0 && r.sweep != sweep_end) {

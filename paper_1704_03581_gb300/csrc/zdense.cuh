@@ -309,8 +309,11 @@ __device__ __forceinline__ int column_draw(const ZArgs &a, const TokenDraw &t, i
 // A word with at most this many nonzero topics is summed over its column
 // even when it has a dense row: one or two entries per lane instead of the
 // whole row, which for such (rare) words mostly comes from beyond L1.
+// zstep_path 1 raises the limit, 2 takes the row wherever there is one.
 template <int NW>
 __device__ __forceinline__ constexpr int column_max() { return NW == 0 ? 128 : NW == 8 ? 64 : NW == 4 ? 32 : 0; }
+template <int NW>
+__device__ __forceinline__ int column_limit(int path) { return path == 1 ? 2 * column_max<NW>() + 32 : path == 2 ? -1 : column_max<NW>(); }
 
 // The staging records of a warp: where z_doc keeps them for its K.
 template <int NW>
@@ -437,7 +440,7 @@ __device__ __forceinline__ void z_doc_regs(const ZArgs &a, uint32_t *sm, DocRun 
     uint4 *rec = token_records<NW>(sm, a);
     uint32_t *drow_of = reinterpret_cast<uint32_t *>(rec + 64);
     const uint32_t sweep_end = rs.sweep + static_cast<uint32_t>(rs.max_pass_end);
-    const int colmax = a.path == 1 ? 0x7FFFFFFF : a.path == 2 ? -1 : column_max<NW>();
+    const int colmax = column_limit<NW>(a.path);
     bool first = true;
     while (rs.budget > 0 && rs.sweep != sweep_end) {
         if (rs.deadline != ~0ull && !first) {
@@ -489,6 +492,35 @@ __device__ __forceinline__ u64 big_plane_dot(const uint8_t *row, const uint8_t *
     return static_cast<u64>(s0) + (static_cast<u64>(s1) << 8) + (static_cast<u64>(s2) << 16);
 }
 
+// U chunks of a row from chunk c0 on, and their sum over planes 0 to lvl: for
+// few documents at a time, where nothing else hides a load.
+template <int U>
+__device__ __forceinline__ void big_load(const uint8_t *row, int PB, int C, int c0, int lane, uint4 (&q)[U][3]) {
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+            q[u][p] = c0 + u < C ? *reinterpret_cast<const uint4 *>(row + 16 * lane + 512 * (c0 + u) + p * PB) : make_uint4(0u, 0u, 0u, 0u);
+}
+template <int U>
+__device__ __forceinline__ u64 big_dot(const uint4 (&q)[U][3], const DocCounts &m, int PB, int C, int c0, int lane) {
+    u64 acc = 0;
+#pragma unroll 1
+    for (int pl = 0; pl <= m.lvl; ++pl) {
+        uint32_t s[3] = {0, 0, 0};
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (c0 + u >= C) continue;
+            const uint4 w = *reinterpret_cast<const uint4 *>(m.b + 16 * lane + pl * PB + 512 * (c0 + u));
+#pragma unroll
+            for (int p = 0; p < 3; ++p)
+                s[p] = __dp4a(w.w, q[u][p].w, __dp4a(w.z, q[u][p].z, __dp4a(w.y, q[u][p].y, __dp4a(w.x, q[u][p].x, s[p]))));
+        }
+        acc += (static_cast<u64>(s[0]) + (static_cast<u64>(s[1]) << 8) + (static_cast<u64>(s[2]) << 16)) << (8 * pl);
+    }
+    return acc;
+}
+
 // K > 1024: the topic of lane L's 16 C whose running sum passes res (position,
 // or -1): its 2 C groups of eight, one per lane, then the group's topics.
 __device__ __forceinline__ int big_find(int L, u64 res, const uint8_t *row, const DocCounts &m, int PB, int C, int lane) {
@@ -518,6 +550,9 @@ __device__ __forceinline__ int big_find(int L, u64 res, const uint8_t *row, cons
 // in C chunks of one 16-byte load per plane.  A lane holds no row and no
 // group sums: it accumulates its chunks, and the found lane's 2 C groups of
 // eight topics are summed again, one group per lane.
+// U > 0: for few documents at a time, the next token's first U chunks loaded
+// while this one is drawn.
+template <int U>
 __device__ __forceinline__ void z_doc_big(const ZArgs &a, uint32_t *sm, DocRun &r, u64 *wcnt, const uint32_t *m0) {
     const int lane = threadIdx.x & 31;
     const int C = (a.K + 511) >> 9;
@@ -550,7 +585,7 @@ __device__ __forceinline__ void z_doc_big(const ZArgs &a, uint32_t *sm, DocRun &
     uint4 *rec = token_records<0>(sm, a);
     uint32_t *drow_of = reinterpret_cast<uint32_t *>(rec + 64);
     const uint32_t sweep_end = rs.sweep + static_cast<uint32_t>(rs.max_pass_end);
-    const int colmax = a.path == 1 ? 0x7FFFFFFF : a.path == 2 ? -1 : column_max<0>();
+    const int colmax = column_limit<0>(a.path);
     bool first = true;
     while (rs.budget > 0 && rs.sweep != sweep_end) {
         if (rs.deadline != ~0ull && !first) {
@@ -565,6 +600,12 @@ __device__ __forceinline__ void z_doc_big(const ZArgs &a, uint32_t *sm, DocRun &
         if (lane < cnt) stage_token(a, rs, i0 + lane, rec + 2 * lane, drow_of + lane, colmax, pos);
         __syncwarp();
         uint32_t c_min = 0, c_cnt = 0, c_int = 0;      // as above, this lane's share of |J| in c_int
+        uint4 ahead[U > 0 ? U : 1][3];
+        auto load_ahead = [&](int tt) {
+            const uint32_t dn = tt < cnt ? drow_of[tt] : 0xFFFFFFFFu;
+            if (U > 0 && dn != 0xFFFFFFFFu) big_load(a.qrow + static_cast<size_t>(dn) * (3u * PB), PB, C, 0, lane, ahead);
+        };
+        load_ahead(0);
         for (int tt = 0; tt < cnt; ++tt) {
             const uint4 t0 = rec[2 * tt], t1 = rec[2 * tt + 1];
             TokenDraw t;
@@ -594,14 +635,27 @@ __device__ __forceinline__ void z_doc_big(const ZArgs &a, uint32_t *sm, DocRun &
             }
             c_min += static_cast<uint32_t>(kd < n_w ? kd : n_w);
             c_cnt += kd < n_w ? 1u : 0u;
+            // the word's bits, counted after the draw: nothing waits for their loads
             const uint16_t *wb = reinterpret_cast<const uint16_t *>(a.bits + static_cast<int64_t>(t1.z) * a.KWp) + C * lane;
-            for (int c = 0; c < C; ++c) c_int += static_cast<uint32_t>(__popc(wb[c] & mb[32 * c]));
+            constexpr int kEarly = 6;
+            uint32_t early[kEarly];
+#pragma unroll
+            for (int c = 0; c < kEarly; ++c) early[c] = c < C ? wb[c] : 0u;
             const uint32_t d = drow_of[tt];
             int knew = -1;
             if (d != 0xFFFFFFFFu) {
                 const uint8_t *row = a.qrow + static_cast<size_t>(d) * (3u * PB);
                 u64 acc = 0;
-                for (int pl = 0; pl <= m.lvl; ++pl) acc += big_plane_dot(row, m.b + pl * PB, PB, C, lane) << (8 * pl);
+                if constexpr (U > 0) {
+                    acc = big_dot(ahead, m, PB, C, 0, lane);
+                    for (int c0 = U; c0 < C; c0 += U) {
+                        big_load(row, PB, C, c0, lane, ahead);
+                        acc += big_dot(ahead, m, PB, C, c0, lane);
+                    }
+                    load_ahead(tt + 1);
+                } else {
+                    for (int pl = 0; pl <= m.lvl; ++pl) acc += big_plane_dot(row, m.b + pl * PB, PB, C, lane) << (8 * pl);
+                }
                 const u64 incl = warp_incl_scan(acc);
                 u64 rb;
                 knew = split_draw(t, __shfl_sync(0xFFFFFFFFu, incl, 31), rb, c_cnt);
@@ -617,9 +671,14 @@ __device__ __forceinline__ void z_doc_big(const ZArgs &a, uint32_t *sm, DocRun &
                 }
             } else {
                 const int64_t col = static_cast<int64_t>((static_cast<u64>(t0.y & 0xFFFFu) << 32) | t0.x);
+                load_ahead(tt + 1);
                 knew = column_draw(a, t, col, n_w, m, lane, c_cnt, pos);
             }
             __syncwarp();
+#pragma unroll
+            for (int c = 0; c < kEarly; ++c)
+                if (c < C) c_int += static_cast<uint32_t>(__popc(early[c] & mb[32 * c]));
+            for (int c = kEarly; c < C; ++c) c_int += static_cast<uint32_t>(__popc(wb[c] & mb[32 * c]));
             {
                 const int p = knew;
                 bool born = false;
@@ -653,10 +712,10 @@ __device__ __forceinline__ void z_doc_big(const ZArgs &a, uint32_t *sm, DocRun &
     __syncwarp();
 }
 
-// NW = dense_words(K) for K <= 1024, 0 above.
+// NW = dense_words(K) for K <= 1024, 0 above, -1 above for few documents at a time.
 template <int NW>
 __device__ __forceinline__ void z_doc(const ZArgs &a, uint32_t *sm, DocRun &r, u64 *wcnt, const uint32_t *m0) {
-    if constexpr (NW == 0) z_doc_big(a, sm, r, wcnt, m0);
+    if constexpr (NW <= 0) z_doc_big<NW == 0 ? 0 : 8>(a, sm, r, wcnt, m0);
     else z_doc_regs<NW>(a, sm, r, wcnt, m0);
 }
 
