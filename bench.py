@@ -41,16 +41,18 @@ K_TOPICS = 1000
 ALPHA, BETA = 0.1, 0.01
 def kernels_per_sweep(w: np.ndarray, phi_mode: int, layout: dict | None = None, slice_docs: int = 0) -> int:
     """Library kernels one sweep launches: the frequent-word histogram (when a
-    word has more than 2^17 tokens), then Polya urn: counts+draws, dead-row
+    word has more than N / 1024 tokens, within 4,096 and 2^17), then Polya urn: counts+draws, dead-row
     fix-up, column scan, per-word tables; Dirichlet: counts, Gamma draws, two
     row-sum passes, selection, column scan, per-word tables; then the z-step
-    as the handle laid it out (pulda_z_layout): its main kernel, the
-    cooperative kernel when some document is on CTAs, the one-warp kernel for
+    as the handle laid it out (pulda_z_layout): its main kernel unless every
+    document is on a CTA, the CTAs' kernel when some are, the one-warp kernel for
     documents too long for four per warp, or the pass-start counts before a
     z-step in slices."""
     heavy = 1 if np.bincount(w).max(initial=0) > min(max(len(w) // 1024, 4096), 1 << 17) else 0
     extra = 1 if slice_docs > 0 else 0
     if layout is not None:
+        if layout["docs_per_warp"] != 4 and layout["one_warp_docs"] == 0 and layout["coop_docs"] > 0:
+            extra -= 1
         extra += (1 if layout["coop_docs"] > 0 else 0)
         if layout["docs_per_warp"] == 4:
             extra += 1 if layout["one_warp_docs"] > 0 else 0
@@ -192,7 +194,7 @@ def code_hash(text: str) -> str:
 
 
 # The sources the one-warp z-step kernel is compiled from.
-Z_STEP_SOURCES = ("kernels.cu", "zstep.cuh", "device_rng.cuh", "checks.cuh", "pulda_internal.h")
+Z_STEP_SOURCES = ("kernels.cu", "zpair.cuh", "zdense.cuh", "zstep.cuh", "device_rng.cuh", "checks.cuh", "pulda_internal.h")
 
 
 def kernel_source_hash() -> str:

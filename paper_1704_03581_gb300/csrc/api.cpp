@@ -125,7 +125,7 @@ cudaError_t clear_z_counters(pulda_handle *h) {
     return e;
 }
 
-// Documents in decreasing length (ties by index), so the persistent z-step
+// Documents in decreasing length (ties by index), so the z-step
 // starts the long ones first.
 std::vector<int32_t> length_order(const int64_t *off, int64_t D) {
     std::vector<int32_t> o(D);

@@ -1,7 +1,7 @@
 // Many independent chains (corpora of uneven D, N, K, V) advanced together:
 // every kernel of a sweep runs once over all chains' work items, and a sweep
-// (six launches, or one persistent launch) is captured once into a CUDA graph
-// and replayed.  The z-step CTA size, the launch form and then the alias
+// (a launch or a few per phase, or one persistent launch for the Phi-step) is
+// captured once into a CUDA graph and replayed.  The z-step CTA size, the launch form and then the alias
 // tables' layout are picked by timing the candidates on the first sweeps
 // (none of them changes a result, so tuning costs no extra sweeps); the
 // longest documents go to CTAs of their own, the others one per warp, the chains
@@ -28,7 +28,7 @@ struct pulda_batch {
     BatchLaunch bl{};
     int sms = 1;
     int64_t sweep = 0;
-    // tuning candidates (z-step warps per CTA, cooperative threshold; 0 = none),
+    // tuning candidates (z-step warps per CTA, the threshold of documents on CTAs; 0 = none),
     // timed on real sweeps: first the CTA sizes, then thresholds at the best size
     // The candidates are timed twice, in order and then in reverse, so the
     // falling cost of the first sweeps after the uniform start does not favour
@@ -43,7 +43,7 @@ struct pulda_batch {
     // the alias layout is timed after the launch form: the best form with the
     // threshold and topic arrays, then with the packed slots
     bool tune_layout = false, layout_phase = false;
-    bool one_launch = false;        // in use: one persistent launch per sweep
+    bool one_launch = false;        // in use: one persistent launch for the Phi-step
     bool packed = false;            // in use: the chains' tables carry packed alias slots
     std::vector<PhiArgs> hp;        // the chains' descriptors (host copies of phi / z below)
     std::vector<ZArgs> hz;
@@ -366,7 +366,7 @@ pulda_status pulda_batch_init(pulda_batch **out, const pulda_chain_desc *chains,
         if (std::any_of(b->form_len.begin(), b->form_len.end(), [&](int64_t n) { return n >= L && n <= kNarrowMaxLen; })) fixed_coop = L;
     }
     // Launch forms: a launch or a few per phase with a CTA size for the z-step, and
-    // (without documents on CTAs) one persistent launch; tuned forms are timed.
+    // (without documents on CTAs) one persistent launch for the Phi-step; tuned forms are timed.
     const bool one_ok = bl.persist_grid > 0 && fixed_coop == 0;
     int one_warps = kMultiWarps;
     while (one_warps > 1 && z_step_smem(kmax, one_warps, narrow) > 160 * 1024) one_warps >>= 1;

@@ -29,7 +29,7 @@ struct pulda_handle {
     int64_t n_wide = 0;         // documents of 2^16 tokens or more (first in doc_order)
     int64_t n_coop = 0;         // documents the long-document z-step takes (next in doc_order)
     int coop_grid = 0;
-    cudaStream_t stream2 = nullptr;                       // the one-warp z-step beside the cooperative one
+    cudaStream_t stream2 = nullptr;                       // the one-warp z-step beside the CTAs'
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     std::vector<void *> allocs;
     // corpus and state

@@ -1,8 +1,8 @@
 // CUDA kernels of the Polya-urn partially collapsed LDA sampler, sm_103a.
 //
 // One sweep = Algorithm 2 (Section 3):
-//   Phi-step  k_heavy_hist   words with more than 2^17 tokens histogrammed in
-//                            chunks by many CTAs.
+//   Phi-step  k_heavy_hist   the most frequent words histogrammed in chunks by
+//                            many CTAs.
 //             k_phi_counts   per word v: rebuild n_{.,v} from z (shared-memory
 //                            histogram over the word's tokens), draw
 //                            c_{k,v} ~ Pois(beta + n_{k,v}) for every k (Eq. 9,
@@ -13,14 +13,14 @@
 //             k_phi_tables   phi = c/S, fixed-point weights, sigma_a, the
 //                            per-word alias table, bitmaps and dense q rows
 //                            ("Efficient sampling of z").
-//   z-step    k_z_step       one warp per document, tokens in order, the
-//                            doubly sparse a/b draw (k_slice_counts first
+//   z-step    k_z_step       one warp per document, tokens in order, the a/b
+//                            draw over dense rows of weights (k_slice_counts first
 //                            when long documents run in stale-count slices).
 // The *_multi kernels do the same over many chains; k_serve_step folds in
-// requests; the longest documents go to the cooperative z-step (one CTA per
-// document, coop.cu); Algorithm 1's Dirichlet Phi-step is in dirichlet.cu.
+// requests; k_z_step_pairs takes two documents per warp; the longest documents
+// go to CTAs of their own (coop.cu); Algorithm 1's Dirichlet Phi-step is in dirichlet.cu.
 // The arithmetic that decides any draw is integer or IEEE double with
-// explicit rounding, so results are independent of launch shapes.
+// explicit rounding (or integers that give the double's value), so results are independent of launch shapes.
 #include <algorithm>
 #include <atomic>
 #include <cstdint>
@@ -343,15 +343,13 @@ __device__ void phi_word(const PhiArgs &a, int v, bool do_draw, uint32_t *hist, 
 // topics of its bitmap words in ascending order, then the lanes share out the
 // list, so the draws and the stores do not wait on the lane of the most topics.
 // pk and the bitmaps are zero between words; kmax lays them out, the same for
-// every word of a launch.
-#ifndef PULDA_WARP_WORD
-#define PULDA_WARP_WORD 256
-#endif
-#ifndef PULDA_WARP_MAXK
-#define PULDA_WARP_MAXK 4096
-#endif
-constexpr int64_t kWarpWord = PULDA_WARP_WORD;
-constexpr int kWarpWordMaxK = PULDA_WARP_MAXK;
+// every word of a launch.  (100,000 words, 12.4 M tokens, K = 1000: the pass
+// took 600 us with a CTA per word and 500 with these warps; the rest of the way
+// to 200 is heavy_word's.  Limits of 64 to 1,024 tokens differ by less than the
+// runs do.  K = 3000: 0.28 ms less; above 4,096 topics a CTA's warps no longer
+// have room beside another CTA.)
+constexpr int64_t kWarpWord = 256;
+constexpr int kWarpWordMaxK = 4096;
 __host__ __device__ __forceinline__ int warp_word_words(int K) {
     return ((K + 3) & ~3) + 2 * (((K + 31) / 32 + 3) & ~3) + (((K + 1) / 2 + 3) & ~3);
 }
@@ -780,16 +778,6 @@ __device__ __forceinline__ uint32_t fixed_weight(long long pbits, int e) {
     return q < 1 ? 1u : static_cast<uint32_t>(q);
 }
 
-__device__ __forceinline__ u64 warp_incl_scan64(u64 x) {
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const u64 y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-        if (lane >= o) x += y;
-    }
-    return x;
-}
-
 __device__ void phi_tables_word_warp(const PhiArgs &a, int v, uint8_t *stage, uint8_t *scratch) {
     const int lane = threadIdx.x & 31;
     const int n = a.nnz_c[v];
@@ -924,7 +912,7 @@ __device__ void phi_tables_word_warp(const PhiArgs &a, int v, uint8_t *stage, ui
             const bool small = in && P < asum, large = in && !small;
             const uint32_t bs = __ballot_sync(0xFFFFFFFFu, small), bl = __ballot_sync(0xFFFFFFFFu, large);
             const uint32_t below = (1u << lane) - 1u;
-            const u64 d = D + warp_incl_scan64(small ? asum - P : 0), e = E + warp_incl_scan64(large ? P - asum : 0);
+            const u64 d = D + warp_incl_scan(small ? asum - P : 0), e = E + warp_incl_scan(large ? P - asum : 0);
             if (in) {
                 const int at = small ? ns + __popc(bs & below) : n - 1 - (nl + __popc(bl & below));
                 X[at] = small ? d : e;

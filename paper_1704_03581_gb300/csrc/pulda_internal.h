@@ -361,7 +361,7 @@ cudaError_t launch_barrier_selftest(GridBarrier *bar, int blocks, int missing, i
 int batch_phi_blocks_per_sm(int kmax);
 int batch_z_blocks_per_sm(int kmax, int warps, bool narrow);
 int batch_coop_blocks_per_sm(int kmax);
-// The cooperative z-step over (chain, document) items (coop.cu).
+// Documents on CTAs over (chain, document) items (coop.cu).
 void launch_z_step_coop_multi(const ZArgs *chains, const int2 *items, int n_items, int *work, int kmax, int grid,
                               cudaStream_t st);
 
@@ -382,7 +382,7 @@ void launch_serve_step(const ZArgs &a, ServeSlot *slots, const int32_t *active, 
                        int16_t *arena_z, int64_t slice, int *work, int warps_per_block, int grid, uint64_t window_ns,
                        bool narrow, cudaStream_t st);
 int serve_blocks_per_sm(int K, int warps_per_block);
-// The same with one CTA (the cooperative z-step) per slot, for long requests.
+// The same with one CTA per slot, for long requests.
 void launch_serve_step_coop(const ZArgs &a, ServeSlot *slots, const int32_t *active, int n_active,
                             const int32_t *arena_w, int16_t *arena_z, int64_t slice, int *work, int grid,
                             uint64_t window_ns, cudaStream_t st);

@@ -3,8 +3,8 @@
 // arrive.  A worker thread owns the GPU side: it admits waiting requests while
 // a slot and a contiguous range of the token arena are free (memory-based
 // admission, first come first served), advances every admitted request by up
-// to `slice` tokens per launch -- one warp per request (one CTA of the
-// cooperative z-step per long request, on a second stream), passes continuing
+// to `slice` tokens per launch -- one warp per request (a CTA per
+// long request, on a second stream), passes continuing
 // within the launch -- and hands finished requests back.  With the automatic
 // slice a launch instead runs every request for a 2 ms window, so each
 // advances as far as its own speed allows.  Each request's
@@ -82,7 +82,7 @@ constexpr size_t kMaxPending = size_t(1) << 22;
 struct pulda_server {
     pulda_handle *h = nullptr;
     int device = 0;
-    cudaStream_t stream = nullptr, stream2 = nullptr;   // the cooperative launch, the one-warp launch
+    cudaStream_t stream = nullptr, stream2 = nullptr;   // the CTAs' launch, the one-warp launch
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     int64_t budget = 0, slice = 0;
     int64_t coop_len = 0;                 // requests at least this long go to CTAs (0 = none)

@@ -145,13 +145,11 @@ struct DenseGeo {
     static constexpr int STRIDE = NW == 8 ? 16 : TPL;
 };
 
-// The lane's sum of q m over its topics: S is 32 bits for a document whose
-// total is below 2^32 and whose counts take one plane.
-template <int NW, typename S>
-__device__ __forceinline__ S dense_dot(const uint32_t (&q)[3][NW], const DocCounts &m, int lane) {
-    S sum = 0;
-    const int top = sizeof(S) == 4 ? 0 : m.lvl;
-    for (int p = 0; p <= top; ++p) {
+// The lane's sum of q m over its topics.
+template <int NW>
+__device__ __forceinline__ u64 dense_dot(const uint32_t (&q)[3][NW], const DocCounts &m, int lane) {
+    u64 sum = 0;
+    for (int p = 0; p <= m.lvl; ++p) {
         uint32_t w[NW];
         load_words<NW>(m.b + p * (128 * NW), lane, w);
         uint32_t s0 = 0, s1 = 0, s2 = 0;        // at most 32 topics of 255^2 each
@@ -161,7 +159,7 @@ __device__ __forceinline__ S dense_dot(const uint32_t (&q)[3][NW], const DocCoun
             s1 = __dp4a(w[x], q[1][x], s1);
             s2 = __dp4a(w[x], q[2][x], s2);
         }
-        sum += (static_cast<S>(s0 + (s1 << 8)) + (static_cast<S>(s2) << 16)) << (8 * p);
+        sum += (static_cast<u64>(s0 + (s1 << 8)) + (static_cast<u64>(s2) << 16)) << (8 * p);
     }
     return sum;
 }
@@ -169,8 +167,8 @@ __device__ __forceinline__ S dense_dot(const uint32_t (&q)[3][NW], const DocCoun
 // Lane j's prefix of q m over the first j + 1 topics of a group (its bytes
 // at off of every plane; lanes past the group repeat it): the counts of the
 // later topics are masked off.  Every lane reads the same words.
-template <int GW, typename S>
-__device__ __forceinline__ S group_prefix(const uint8_t *row, int PB, const DocCounts &m, int off, int lane) {
+template <int GW>
+__device__ __forceinline__ u64 group_prefix(const uint8_t *row, int PB, const DocCounts &m, int off, int lane) {
     const int j = lane & (4 * GW - 1);
     uint32_t mask[GW];
 #pragma unroll
@@ -188,9 +186,8 @@ __device__ __forceinline__ S group_prefix(const uint8_t *row, int PB, const DocC
             q[p][0] = *reinterpret_cast<const uint32_t *>(row + p * PB + off);
         }
     }
-    S sum = 0;
-    const int top = sizeof(S) == 4 ? 0 : m.lvl;
-    for (int pl = 0; pl <= top; ++pl) {
+    u64 sum = 0;
+    for (int pl = 0; pl <= m.lvl; ++pl) {
         uint32_t s0 = 0, s1 = 0, s2 = 0;
 #pragma unroll
         for (int x = 0; x < GW; ++x) {
@@ -199,7 +196,7 @@ __device__ __forceinline__ S group_prefix(const uint8_t *row, int PB, const DocC
             s1 = __dp4a(w, q[1][x], s1);
             s2 = __dp4a(w, q[2][x], s2);
         }
-        sum += (static_cast<S>(s0 + (s1 << 8)) + (static_cast<S>(s2) << 16)) << (8 * pl);
+        sum += (static_cast<u64>(s0 + (s1 << 8)) + (static_cast<u64>(s2) << 16)) << (8 * pl);
     }
     return sum;
 }
@@ -238,31 +235,24 @@ __device__ __forceinline__ int fine_search(S p, S res) {
 
 // The new topic (position) from the lanes' sums of q m: the lane whose prefix
 // passes the draw, then its TPL topics, one per lane.
-template <int NW, typename S>
-__device__ __forceinline__ int dense_draw(const ZArgs &a, S sum, const TokenDraw &t, const uint8_t *row, const DocCounts &m,
+template <int NW>
+__device__ __forceinline__ int dense_draw(const ZArgs &a, u64 sum, const TokenDraw &t, const uint8_t *row, const DocCounts &m,
                                           int fine, uint32_t &c_cnt) {
     using G = DenseGeo<NW>;
     constexpr int W = G::TPL;
-    const S incl = warp_incl_scan<32>(sum);
-    u64 rb64;
-    const int settled = split_draw(t, __shfl_sync(0xFFFFFFFFu, incl, 31), rb64, c_cnt);
+    const u64 incl = warp_incl_scan<32>(sum);
+    u64 rb;
+    const int settled = split_draw(t, __shfl_sync(0xFFFFFFFFu, incl, 31), rb, c_cnt);
     if (settled >= 0) return settled;
-    const S rb = static_cast<S>(rb64);
     const int L = __ffs(__ballot_sync(0xFFFFFFFFu, rb < incl)) - 1;      // rb < B: some lane passes it
-    const S res = __shfl_sync(0xFFFFFFFFu, rb - (incl - sum), L);
+    const u64 res = __shfl_sync(0xFFFFFFFFu, rb - (incl - sum), L);
     const int at = fine + L * G::STRIDE;                                 // this lane's topic of lane L's
     const uint32_t q = row[at] | (static_cast<uint32_t>(row[at + G::PB]) << 8) | (static_cast<uint32_t>(row[at + 2 * G::PB]) << 16);
-    int f;
-    if constexpr (sizeof(S) == 4) {
-        f = fine_search<W, uint32_t>(q * m.b[at], res);
-    } else {
-        const u64 p = static_cast<u64>(q) * m.get(at);
-        // lane L's topics sum to less than 2^32 but for counts in the hundreds
-        if (__shfl_sync(0xFFFFFFFFu, static_cast<uint32_t>(sum >> 32), L) == 0)
-            f = fine_search<W, uint32_t>(static_cast<uint32_t>(p), static_cast<uint32_t>(res));
-        else
-            f = fine_search<W, u64>(p, res);
-    }
+    const u64 p = static_cast<u64>(q) * m.get(at);
+    // lane L's topics sum to less than 2^32 but for counts in the hundreds
+    const int f = __shfl_sync(0xFFFFFFFFu, static_cast<uint32_t>(sum >> 32), L) == 0
+                      ? fine_search<W, uint32_t>(static_cast<uint32_t>(p), static_cast<uint32_t>(res))
+                      : fine_search<W, u64>(p, res);
     if (f >= W) {
         if ((threadIdx.x & 31) == 0) atomicOr(&a.stats[ST_ERROR], ERR_INTERNAL);
         return t.kold;
@@ -334,9 +324,8 @@ __device__ __forceinline__ void add_block_counts(u64 *wcnt, int lane, int cnt, u
 
 // The tokens of one 32-token block, in order.  Every lane carries out the
 // count updates (the same byte, the same value), so they need neither a branch
-// nor a vote.  S = uint32_t: a document whose counts fit one plane and whose
-// sums fit 32 bits for good.
-template <int NW, typename S>
+// nor a vote.
+template <int NW>
 __device__ __forceinline__ int z_block(const ZArgs &a, DocCounts &m, const uint4 *rec, const uint32_t *drow_of, int cnt,
                                        uint32_t &mbits, int &kd, uint32_t &c_min, uint32_t &c_cnt) {
     using G = DenseGeo<NW>;
@@ -364,10 +353,9 @@ __device__ __forceinline__ int z_block(const ZArgs &a, DocCounts &m, const uint4
         t.ka = static_cast<int>(t0.y >> 16);
         // remove the token: m^{-i}
         {
-            const uint32_t c = (sizeof(S) == 4 ? m.b[t.kold] : m.get(t.kold)) - 1u;
+            const uint32_t c = m.get(t.kold) - 1u;
             __syncwarp();
-            if (sizeof(S) == 4) m.b[t.kold] = static_cast<uint8_t>(c);
-            else m.set(t.kold, c);
+            m.set(t.kold, c);
             if (c == 0) {
                 --kd;
                 if (lane == G::owner(t.kold)) mbits &= ~(1u << G::bit(t.kold));
@@ -380,10 +368,10 @@ __device__ __forceinline__ int z_block(const ZArgs &a, DocCounts &m, const uint4
         const uint32_t dn = more ? drow_of[tt + 1] : 0xFFFFFFFFu;
         int knew;
         if (d != 0xFFFFFFFFu) {
-            const S sum = dense_dot<NW, S>(q, m, lane);
+            const u64 sum = dense_dot<NW>(q, m, lane);
             const uint8_t *r0 = row;
             fetch_row(dn);                  // the next token's row, while this one is drawn
-            knew = dense_draw<NW, S>(a, sum, t, r0, m, fine, c_cnt);
+            knew = dense_draw<NW>(a, sum, t, r0, m, fine, c_cnt);
         } else {
             const int64_t col = static_cast<int64_t>((static_cast<u64>(t0.y & 0xFFFFu) << 32) | t0.x);
             knew = column_draw(a, t, col, n_w, m, lane, c_cnt, [](int k) { return G::pos(k); });
@@ -392,14 +380,10 @@ __device__ __forceinline__ int z_block(const ZArgs &a, DocCounts &m, const uint4
         d = dn;
         // add it back with its new topic
         {
-            const uint32_t c = (sizeof(S) == 4 ? m.b[knew] : m.get(knew)) + 1u;
+            const uint32_t c = m.get(knew) + 1u;
             __syncwarp();
-            if (sizeof(S) == 4) {
-                m.b[knew] = static_cast<uint8_t>(c);
-            } else {
-                m.set(knew, c);
-                if (c == 256u || c == 65536u) m.lvl = max(m.lvl, count_level(c));
-            }
+            m.set(knew, c);
+            if (c == 256u || c == 65536u) m.lvl = max(m.lvl, count_level(c));
             if (c == 1) {
                 ++kd;
                 if (lane == G::owner(knew)) mbits |= 1u << G::bit(knew);
@@ -458,7 +442,7 @@ __device__ __forceinline__ void z_doc_regs(const ZArgs &a, uint32_t *sm, DocRun 
         // zero-mass tokens in 12-17 (each at most 32), this lane's share of
         // |J| (at most 32 x 32) from bit 18
         uint32_t c_min = 0, c_cnt = 0;
-        const int znew = z_block<NW, u64>(a, m, rec, drow_of, cnt, mbits, kd, c_min, c_cnt);
+        const int znew = z_block<NW>(a, m, rec, drow_of, cnt, mbits, kd, c_min, c_cnt);
         if (lane < cnt) rs.z[i0 + lane] = static_cast<int16_t>(guard_index(G::topic(znew), a.K, a.stats));
         add_block_counts(wcnt, lane, cnt, c_min, c_cnt, c_cnt >> 18);
         __syncwarp();
@@ -528,7 +512,7 @@ __device__ __forceinline__ int big_find(int L, u64 res, const uint8_t *row, cons
     for (int g0 = 0; g0 < 2 * C; g0 += 32) {
         const int gi = g0 + lane;
         u64 gs = 0;
-        if (gi < 2 * C) gs = group_prefix<2, u64>(row, PB, m, ((gi >> 1) << 9) + (L << 4) + ((gi & 1) << 3), 7);
+        if (gi < 2 * C) gs = group_prefix<2>(row, PB, m, ((gi >> 1) << 9) + (L << 4) + ((gi & 1) << 3), 7);
         const u64 gin = warp_incl_scan<32>(gs);
         const uint32_t f = __ballot_sync(0xFFFFFFFFu, res < gin);
         if (f) {
@@ -541,7 +525,7 @@ __device__ __forceinline__ int big_find(int L, u64 res, const uint8_t *row, cons
     }
     if (grp < 0) return -1;
     const int off = ((grp >> 1) << 9) + (L << 4) + ((grp & 1) << 3);
-    const u64 p = group_prefix<2, u64>(row, PB, m, off, lane);
+    const u64 p = group_prefix<2>(row, PB, m, off, lane);
     const uint32_t f = __ballot_sync(0xFFFFFFFFu, res < p) & 0xFFu;
     return f ? off + __ffs(f) - 1 : -1;
 }

@@ -24,7 +24,7 @@
 //
 // Requires K <= kMaxKGrouped, a dense q row for every word, and documents of at
 // most kMaxGroupDocLen tokens (uint16 counts); the host routes anything else to
-// the one-warp and cooperative kernels.
+// the one-warp kernels and those with a CTA per document.
 #include <algorithm>
 #include <cstdint>
 
