@@ -19,6 +19,10 @@
 // Warp 0 finds the topic within the found lane by masked dp4a, every lane
 // summing the lane's topics up to its own, without a scan.  Warps 0 and 3 meet
 // once per token, all four once per group of tokens.
+// About 640 cycles per token (K = 1000: 0.95 us with four warps sharing one
+// token's sparse walk, 0.33 so), which warps 0 and 3 both fill: work moved from
+// either to the other made a token longer (the draw's product prepared by
+// warp 3 +10%, two of its scan steps left to warp 0 +5%).
 #pragma once
 #include <cstdint>
 

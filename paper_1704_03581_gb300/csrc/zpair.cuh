@@ -8,6 +8,9 @@
 // consecutive), and so has two sums: the prefix in topic order runs over the
 // sixteen lanes' first sums, then over their second ones.  The sums, draws and
 // topics are those of the one-document form.
+// 236 warp instructions per token against 321 of the sparse walk; 99 M tokens
+// at K = 1000: 32.2 ms with a document per warp, 27.8 with two (0.67 of the
+// issue peak; without the accesses to the second count plane the same).
 #pragma once
 #include <cstdint>
 
