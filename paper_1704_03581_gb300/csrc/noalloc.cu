@@ -28,24 +28,16 @@ namespace {
 // Largest number of documents one call may carry.
 constexpr int64_t kNoAllocMaxDocs = 65536;
 
-// Length classes of documents, eight to an octave and the longest first: those
-// of 2^16 tokens or more (one warp each), then those of at least coop_len (a
-// CTA each), then the rest.  So the schedule is longest first, but for lengths
-// within an eighth of each other; in any order within the three groups, a long
-// document taken up late was the end of the pass (4,096 documents: 2.10 ms).
-constexpr int kLengthKeys = 112;
-constexpr int kClasses = 1 + 2 * kLengthKeys;
-
 // Layout of the scratch array (bytes).
 constexpr size_t kOffStats = 0;                                       // u64[ST_TOTAL_SLOTS]
 constexpr size_t kOffWork = 256;                                      // int[5]: z-step work counters
-constexpr size_t kOffCount = 320;                                     // int[kClasses]: documents by length class
+constexpr size_t kOffCount = 320;                                     // int[kLengthClasses]: documents by length class
 constexpr size_t kOffFlag = 1280;                                     // u64[2]: first bad token, first bad document
 constexpr size_t kOffOrder = 1536;                                    // int32[kNoAllocMaxDocs]
 constexpr size_t kScratchBytes = kOffOrder + sizeof(int32_t) * kNoAllocMaxDocs;   // 263,680 bytes
 static_assert(ST_TOTAL_SLOTS * sizeof(unsigned long long) <= kOffWork, "the counters overlap the work counter");
 static_assert(5 * sizeof(int) <= kOffCount - kOffWork, "the work counters overlap the class counts");
-static_assert(kClasses * sizeof(int) <= kOffFlag - kOffCount, "the class counts overlap the input check");
+static_assert(kLengthClasses * sizeof(int) <= kOffFlag - kOffCount, "the class counts overlap the input check");
 static_assert(2 * sizeof(unsigned long long) <= kOffOrder - kOffFlag, "the input check overlaps the schedule");
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
@@ -73,15 +65,9 @@ cudaError_t scratch_on_device(int dev, unsigned char **out) {
     return cudaSuccess;
 }
 
-__device__ __forceinline__ int length_class(int64_t len, int64_t coop_len) {
-    if (len > kNarrowMaxLen) return 0;
-    const int n = static_cast<int>(len), e = 31 - __clz(n | 1);
-    const int key = n < 8 ? n : 8 * (e - 2) + ((n >> (e - 3)) & 7);       // at most 111
-    return (len >= coop_len ? 1 : 1 + kLengthKeys) + kLengthKeys - 1 - key;
-}
-
 // Checks the caller's device inputs (ids in [0, V), offsets nondecreasing from
-// 0 to N) and counts the documents of each length class.  first[0] becomes the
+// 0 to N) and counts the documents of each length class, those with good
+// offsets only: another's length may be any number.  first[0] becomes the
 // smallest position of a word id outside [0, V), first[1] the smallest
 // document with bad offsets; both start at ~0 (none).
 __global__ void k_noalloc_check(const int32_t *w, int64_t N, const int64_t *off, int64_t D, int V,
@@ -94,7 +80,8 @@ __global__ void k_noalloc_check(const int32_t *w, int64_t N, const int64_t *off,
         const int64_t a = off[d], b = off[d + 1];
         if (a < 0 || b < a || b > N || (d == 0 && a != 0) || (d == D - 1 && b != N) || b - a > (int64_t(1) << 22))
             atomicMin(&first[1], static_cast<unsigned long long>(d));
-        atomicAdd(&count[length_class(b - a, coop_len)], 1);
+        else
+            atomicAdd(&count[length_class(b - a, coop_len)], 1);
     }
 }
 
@@ -154,7 +141,7 @@ extern "C" pulda_status pulda_infer_noalloc(pulda_handle *h, const int32_t *word
         k_noalloc_check<<<64, 256, 0, st>>>(word_ids_dev, N_new, doc_offsets_dev, D_new, hv.V, first, count, coop_len);
         e = cudaGetLastError();
     }
-    int hcount[kClasses] = {};
+    int hcount[kLengthClasses] = {};
     if (e == cudaSuccess) e = cudaMemcpyAsync(hcount, count, sizeof hcount, cudaMemcpyDeviceToHost, st);
     unsigned long long hfirst[2] = {~0ull, ~0ull};
     if (e == cudaSuccess) e = cudaMemcpyAsync(hfirst, first, sizeof hfirst, cudaMemcpyDeviceToHost, st);
@@ -172,8 +159,8 @@ extern "C" pulda_status pulda_infer_noalloc(pulda_handle *h, const int32_t *word
         return static_cast<pulda_status>(handle_fail(h, PULDA_ERR_INVALID, msg));
     }
     const int n_wide = hcount[0];
-    int n_coop = 0, cursor[kClasses], run = 0;
-    for (int c = 0; c < kClasses; ++c) {
+    int n_coop = 0, cursor[kLengthClasses], run = 0;
+    for (int c = 0; c < kLengthClasses; ++c) {
         cursor[c] = run;
         run += hcount[c];
         if (c >= 1 && c <= kLengthKeys) n_coop += hcount[c];

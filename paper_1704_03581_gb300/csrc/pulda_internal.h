@@ -275,6 +275,23 @@ constexpr int kMaxGroupDocLen = 65535;
 // A one-warp z-step launch whose documents have at most this many tokens each
 // keeps m_d's counts in 16 bits (ZArgs::narrow).
 constexpr int64_t kNarrowMaxLen = 65535;
+// Length classes of documents (fold-in without allocation), eight to an octave
+// and the longest first: those of 2^16 tokens or more (one warp each), then
+// those of at least coop_len (a CTA each), then the rest.  So the schedule is
+// longest first, but for lengths within an eighth of each other; in any order
+// within the three groups, a long document taken up late was the end of the
+// pass (4,096 documents: 2.10 ms).  A class is in [0, kLengthClasses) whatever
+// the length.
+constexpr int kLengthKeys = 112;
+constexpr int kLengthClasses = 1 + 2 * kLengthKeys;
+__host__ __device__ inline int length_class(int64_t len, int64_t coop_len) {
+    if (len > kNarrowMaxLen) return 0;
+    const int n = len < 0 ? 0 : static_cast<int>(len);
+    int e = 3;                                                   // n < 2^(e + 1), e >= 3
+    while (n >> (e + 1)) ++e;
+    const int key = n < 8 ? n : 8 * (e - 2) + ((n >> (e - 3)) & 7);       // at most 111
+    return (len >= coop_len ? 1 : 1 + kLengthKeys) + kLengthKeys - 1 - key;
+}
 void launch_z_step_groups(const ZArgs &a, int grid, cudaStream_t st);
 int z_groups_blocks_per_sm(int K);
 int phi_counts_blocks_per_sm(int K);

@@ -127,3 +127,28 @@ def test_noalloc_matches_infer_when_infer_uses_its_other_kernels(kw):
         zo = O.infer(ch.tables, w[a:b], np.array([0, b - a], np.int64), 4, 21, index_base=a)
         assert np.array_equal(z_ref[a:b], zo), int(d)
     s.close()
+
+
+@pytest.mark.parametrize("off", [
+    [0, 50, 45, 60],                        # a fall of a few tokens
+    [0, 50, 32, 60],
+    [0, 100000, 10000, 200000],             # of more than 2^16
+    [0, 200000, 0, 200000],
+    [0, 40, -(1 << 33), 60],                # of more than 2^32
+    [0, 40, -(1 << 62), 60],
+])
+def test_noalloc_refuses_falling_offsets(chain, off):
+    """Offsets that fall, by a few tokens or by many: refused with the first bad
+    document named, and the next call's topics are pulda_infer's."""
+    import torch
+    P, s, c = chain
+    n = off[-1]
+    w = torch.zeros(n, dtype=torch.int32, device="cuda")
+    z = torch.full((n,), -1, dtype=torch.int16, device="cuda")
+    torch.cuda.synchronize()
+    with pytest.raises(P.PuldaError) as e:
+        P.pulda_infer_noalloc(s.h, w, torch.tensor(off, dtype=torch.int64, device="cuda"), 1, 0, z)
+    assert e.value.status == -1 and "first bad document: 1" in str(e.value)
+    assert bool((z == -1).all())
+    new = c.slice_docs(10, 60)
+    assert np.array_equal(_noalloc(P, s, new.w, new.doc_off, 3, 8), s.infer(new.w, new.doc_off, 3, seed=8))
