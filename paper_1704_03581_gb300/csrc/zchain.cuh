@@ -698,7 +698,8 @@ __device__ __forceinline__ void z_doc_chain(const ZArgs &a, uint8_t *sm, DocRun 
                     __syncwarp();
                 }
                 if (g + 2 < ng) ok = landed(g + 2);
-                const bool late = ((t0 + cnt) & 31) == 0 && r.deadline != ~0ull && global_ns() >= r.deadline;
+                // the deadline, after every block of 32 and every pass (a document may be shorter than a block)
+                const bool late = (((t0 + cnt) & 31) == 0 || g + 1 == ng) && r.deadline != ~0ull && global_ns() >= r.deadline;
                 const bool mix = g + 1 < ng && mixed(g + 1);
                 if (lane == 0) ctl.after[g & 1] = (late || !ok ? kStop : 0) | (mix ? kMixed : 0);
             } else if (g > 0) {

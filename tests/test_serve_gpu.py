@@ -157,3 +157,29 @@ def test_cooperative_requests_equal_each_alone(trained, coop, slice_):
         zo = O.infer(ch.tables, r["words"], np.array([0, len(r["words"])]), r["sweeps"], r["seed"])
         assert np.array_equal(got[r["id"]], zo)
     s.close()
+
+
+@pytest.mark.parametrize("coop", [0, 1, -1])
+@pytest.mark.parametrize("length", [1, 20, 40])
+def test_short_requests_keep_the_launch_window(trained, length, coop):
+    """With the automatic slice a launch is a window of 2 ms whatever the
+    requests' lengths: one shorter than a block of 32 tokens, resampled many
+    times, does not keep the others waiting.  The bound leaves five windows for
+    a launch's fixed part."""
+    P, s0, ch, c = trained
+    s = P.Sampler(c.w, c.doc_off, 20, c.V, 0.1, 0.01, seed=3, coop_min_len=coop).sweep(3)
+    words = np.random.default_rng(length).integers(0, c.V, length).astype(np.int32)
+    sweeps = 100_000 // length
+    srv = P.Server(s, token_budget=1000, max_slots=4, slice_tokens=0)
+    srv.submit(1, 5, words, sweeps)
+    got = []
+    t0 = time.time()
+    while not got:
+        got = srv.poll(timeout_ms=200)
+        assert time.time() - t0 < 60, "server made no progress"
+    st = srv.stats()
+    srv.close()
+    assert got[0]["status"] == 0
+    assert st["kernel_ns"] <= 10_000_000 * st["launches"], st
+    assert np.array_equal(got[0]["z"], s0.infer(words, np.array([0, length]), sweeps, seed=5))
+    s.close()
