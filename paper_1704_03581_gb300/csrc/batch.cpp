@@ -298,12 +298,13 @@ pulda_status pulda_batch_init(pulda_batch **out, const pulda_chain_desc *chains,
     for (const auto &x : di) n_tokens += x.first;
     // the documents form by form: the order is stable, so longest first in each
     std::vector<int2> flist;
-    for (int nw : {8, 4, 2, 1, 0}) {        // the form of the most work per token first; 0 = above 1,024 topics
+    auto form_of = [](int K) { return K > kChainMaxK ? -1 : K > 1024 ? 0 : dense_words(K); };
+    for (int nw : {8, 4, 2, 1, 0, -1}) {    // the form of the most work per token first, but for those above 1,024 topics
         BatchForm F{};
         F.first = static_cast<int>(flist.size());
         for (const auto &x : di) {
             const int K = b->ch[x.second.x]->K;
-            if ((K <= 1024 ? dense_words(K) : 0) != nw) continue;
+            if (form_of(K) != nw) continue;
             F.kmax = std::max(F.kmax, K);
             if (x.first > kNarrowMaxLen) ++F.n_wide;
             flist.push_back(x.second);

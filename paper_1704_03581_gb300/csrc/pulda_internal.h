@@ -52,6 +52,9 @@ __host__ __device__ inline int dense_pos(int K, int k) {
     const int l = k / tpl, b = k - l * tpl;
     return ((b >> 4) << 9) + (l << 4) + (b & 15);
 }
+// A document on a CTA of its own: a chain of warps up to here (zchain.cuh), all
+// warps on each token above (zsplit.cuh).
+constexpr int kChainMaxK = 8192;
 // Warps per CTA of the warp-per-document z-step: the default and the largest
 // accepted (the kernel's launch bounds are sized for it).
 #ifndef PULDA_ZWARPS
@@ -327,9 +330,9 @@ struct GridBarrier {
 };
 
 // The chains of one form of the z-step (dense_words up to 1,024 topics, one
-// form above): their documents, n from `first` on in the form order, the n_wide
+// form to kChainMaxK and one above): their documents, n from `first` on in the form order, the n_wide
 // widest (2^16 tokens or more) one per warp, the next n_coop on CTAs.
-constexpr int kMaxForms = 5;
+constexpr int kMaxForms = 6;
 struct BatchForm {
     int kmax, first, n;
     int n_wide, n_coop;

@@ -23,6 +23,7 @@
 // token's sparse walk, 0.33 so), which warps 0 and 3 both fill: work moved from
 // either to the other made a token longer (the draw's product prepared by
 // warp 3 +10%, two of its scan steps left to warp 0 +5%).
+// Up to kChainMaxK topics; zsplit.cuh above.
 #pragma once
 #include <cstdint>
 
@@ -47,20 +48,21 @@ __host__ __device__ __forceinline__ int chain_group(int K) {
 // column's start}.
 constexpr int kChainRecWords = 12;
 
-// Warp 3 has counts of its own up to here; above, where they no longer fit,
-// warp 0 takes the next token's sum itself.
-constexpr int kChainAheadMaxK = 8192;
-__host__ __device__ __forceinline__ int chain_count_sets(int K) { return K <= kChainAheadMaxK ? 3 : 2; }
+// Above kChainMaxK the counts of three warps and the ring no longer fit a CTA
+// and zsplit.cuh takes over; the layout functions here hold for any K.
+__host__ __device__ __forceinline__ int chain_count_sets(int K) { return K <= kChainMaxK ? 3 : 2; }
 
 // Shared memory of a CTA, in bytes: the barriers and counters; the drawn
 // topics of two groups; the coming token's sums; three blocks of records; the
 // sets of counts (two planes each) and, above 1024 topics, the lanes' bits; the
 // ring.
-struct ChainCtl {
-    u64 full[3];                // a group's rows have arrived
+struct CtaCtl {                 // what every kernel with a CTA per document has
+    u64 full[3];                // a group's rows (zsplit.cuh: a row) have arrived
     u64 cnt[6];                 // the counters
     u64 deadline;
     int item, stop;
+};
+struct ChainCtl : CtaCtl {
     int after[2];               // after an even / odd group (a fast warp may already set the next one):
                                 // kStop, kMixed: the next group holds a token without a dense row
     uint32_t drawn[16];         // two groups: position | flags
@@ -79,7 +81,7 @@ __host__ __device__ __forceinline__ int chain_smem_bytes(int K) { return chain_r
 // take less room than the longer ones below them).
 __host__ __device__ __forceinline__ int chain_smem_bytes_upto(int kmax) {
     int most = 0;
-    const int edge[4] = {512, 1024, kChainAheadMaxK, kMaxK};
+    const int edge[4] = {512, 1024, kChainMaxK, kMaxK};
     for (int e : edge) {
         const int b = chain_smem_bytes(kmax < e ? kmax : e);
         most = b > most ? b : most;
@@ -129,18 +131,12 @@ __device__ __forceinline__ uint32_t row_weight(const uint8_t *row, int PB, int p
     return row[p] | (static_cast<uint32_t>(row[p + PB]) << 8) | (static_cast<uint32_t>(row[p + 2 * PB]) << 16);
 }
 
-__device__ __forceinline__ u64 shfl_up64(u64 v, int o) {
-    const uint32_t lo = __shfl_up_sync(0xFFFFFFFFu, static_cast<uint32_t>(v), o);
-    const uint32_t hi = __shfl_up_sync(0xFFFFFFFFu, static_cast<uint32_t>(v >> 32), o);
-    return (static_cast<u64>(hi) << 32) | lo;
-}
-
 // What the two ranges of K do differently: NW words per lane and plane, or
 // (NW = 0, K > 1024) C chunks of four.
 template <int NW>
 struct ChainForm {
     using G = DenseGeo<NW>;
-    uint32_t mbits;             // this lane's topics with m > 0 (warp 1)
+    uint32_t mbits;             // this lane's topics with m > 0 (warp 2)
     __device__ __forceinline__ ChainForm(int) {}
     __device__ __forceinline__ static constexpr int plane() { return G::PB; }
     __device__ __forceinline__ static int pos(int k) { return G::pos(k); }
@@ -244,7 +240,7 @@ template <>
 struct ChainForm<0> {
     int C, TPL, PB;
     uint32_t recip;
-    uint16_t *mb;               // this lane's bits (warp 1), chunk c at mb[32 c]
+    uint16_t *mb;               // this lane's bits (warp 2), chunk c at mb[32 c]
     __device__ __forceinline__ ChainForm(int K) {
         C = (K + 511) >> 9;
         TPL = 16 * C;
@@ -302,7 +298,6 @@ struct ChainState {
                                 // start the first token's topic, taken out of the counts)
     uint32_t top;               // a bound on every count
     uint32_t bad;               // a draw found no topic
-    u64 incl, below;            // without warp 3: the coming token's prefixes, without `prev`
 };
 
 // The last token's topic into the counts, this one's out.  Every lane stores
@@ -438,30 +433,25 @@ __device__ __forceinline__ void chain_run_fast(const ChainForm<NW> &form, uint8_
 // The same for any group: tokens without a dense row among them, or K > 1024.
 template <int NW, int P>
 __device__ __forceinline__ void chain_group_any(const ZArgs &a, const ChainForm<NW> &form, uint8_t *sm, ChainCtl &ctl, uint8_t *m, int t,
-                                                int cnt, bool paired, uint32_t *drawn, ChainState &st) {
+                                                int cnt, uint32_t *drawn, ChainState &st) {
     const int lane = threadIdx.x & 31;
     const int PB = form.plane();
     const uint4 *recs = reinterpret_cast<const uint4 *>(sm + kChainRecOff);
 #pragma unroll 1
     for (int u = 0; u < cnt; ++u, ++t) {
         const uint4 *rec = recs + 3 * (t % 96);
-        const uint4 r0 = rec[0], r1 = rec[1], n1 = recs[3 * ((t + 1) % 96) + 1];
+        const uint4 r0 = rec[0], r1 = rec[1];
         const u64 At = (static_cast<u64>(r0.y) << 32) | r0.x, U = (static_cast<u64>(r0.w) << 32) | r0.z;
         const int kold = static_cast<int>(r1.x & 0xFFFFu);
         const bool dense = r1.y != 0xFFFFFFFFu;
         const uint8_t *row = sm + r1.y;
         const uint32_t delta = dense ? form.weight(row, st.prev) : 0u;
         const int ow = form.owner(st.prev);
-        const ulonglong2 mine = paired ? ctl.ahead[t & 1][lane] : make_ulonglong2(st.incl, st.below);
+        const ulonglong2 mine = ctl.ahead[t & 1][lane];
         chain_update<P>(m, PB, kold, st);
         __syncwarp();
         const u64 upto = mine.x + (lane >= ow ? delta : 0u), below = mine.y + (lane > ow ? delta : 0u);
         uint32_t knew;
-        if (!paired && n1.y != 0xFFFFFFFFu) {
-            const ulonglong2 x = chain_sums<NW, P>(form, sm, m, n1, lane);
-            st.incl = x.x;
-            st.below = x.y;
-        }
         if (dense) {
             const u64 rr = __umul64hi(U, At + (__shfl_sync(0xFFFFFFFFu, upto, 31) << kFracBits));
             if (rr < At) {
@@ -490,7 +480,7 @@ __device__ __forceinline__ void chain_group_any(const ZArgs &a, const ChainForm<
         drawn[u] = knew;
         st.prev = static_cast<int>(knew & 0x3FFFu);
         ctl.last[t & 1] = st.prev;
-        if (paired) pair_barrier();
+        pair_barrier();
         __syncwarp();
     }
 }
@@ -511,21 +501,20 @@ __device__ __forceinline__ void z_doc_chain(const ZArgs &a, uint8_t *sm, DocRun 
     const int PB = form.plane();
     auto pos = [&](int k) { return form.pos(k); };
     // warps 0, 2 and 3 each keep the document's counts
-    const bool paired = K <= kChainAheadMaxK;
     DocCounts m{sm + kChainCountOff + (role == 0 ? 0 : role == 2 ? 2 * PB : 4 * PB), PB, 0};
-    if (role == 0 || role == 2 || (role == 3 && paired)) build_counts(a, m, r, nullptr, 2, pos);
+    if (role != 1) build_counts(a, m, r, nullptr, 2, pos);
     ChainState st{};
     st.prev = -1;
     bool begun = false;
     int kd = 0;
-    if (role == 0 || (role == 3 && paired)) {
+    if (role == 0 || role == 3) {
         uint32_t top = 0;
         for (int p = lane; p < PB; p += 32) top = max(top, m.b[p] | (static_cast<uint32_t>(m.b[p + PB]) << 8));
         st.top = __reduce_max_sync(0xFFFFFFFFu, top);
     } else if (role == 2) {
         kd = static_cast<int>(__reduce_add_sync(0xFFFFFFFFu, static_cast<unsigned>(form.init_bits(m, sm + kChainCountOff + 2 * chain_count_sets(K) * PB, lane))));
     }
-    const int colmax = -1;         // a row wherever there is one
+    constexpr int colmax = -1;     // a row wherever there is one
     const uint32_t sweep_end = r.sweep + static_cast<uint32_t>(r.max_pass_end);
     bool stop = false;
     while (!stop && r.budget > 0 && r.sweep != sweep_end) {
@@ -647,7 +636,7 @@ __device__ __forceinline__ void z_doc_chain(const ZArgs &a, uint8_t *sm, DocRun 
         }
         __syncthreads();
         ChainPass ps{n, ng, G, 0, 0, ctl.stop};
-        if ((role == 0 || (role == 3 && paired)) && ps.more()) {
+        if ((role == 0 || role == 3) && ps.more()) {
             const uint4 r1 = recs[1];
             if (!begun) {
                 st.prev = static_cast<int>(r1.x & 0xFFFFu);
@@ -656,12 +645,7 @@ __device__ __forceinline__ void z_doc_chain(const ZArgs &a, uint8_t *sm, DocRun 
                 chain_set<2>(m.b, PB, st.prev, c);
                 __syncwarp();
             }
-            if (r1.y != 0xFFFFFFFFu && (role == 3) == paired) {
-                const ulonglong2 x = chain_sums<NW, 2>(form, sm, m.b, r1, lane);
-                st.incl = x.x;
-                st.below = x.y;
-                if (paired) ctl.ahead[0][lane] = x;
-            }
+            if (r1.y != 0xFFFFFFFFu && role == 3) ctl.ahead[0][lane] = chain_sums<NW, 2>(form, sm, m.b, r1, lane);
             begun = true;
         }
         __syncthreads();
@@ -676,17 +660,15 @@ __device__ __forceinline__ void z_doc_chain(const ZArgs &a, uint8_t *sm, DocRun 
                         else chain_run_fast<NW, 2>(form, sm, ctl, m.b, ps, st);
                         continue;
                     }
-                    chain_group_any<NW, 2>(a, form, sm, ctl, m.b, t0, cnt, paired, drawn, st);
+                    chain_group_any<NW, 2>(a, form, sm, ctl, m.b, t0, cnt, drawn, st);
                 } else {
-                    if (one) chain_group_any<NW, 1>(a, form, sm, ctl, m.b, t0, cnt, paired, drawn, st);
-                    else chain_group_any<NW, 2>(a, form, sm, ctl, m.b, t0, cnt, paired, drawn, st);
+                    if (one) chain_group_any<NW, 1>(a, form, sm, ctl, m.b, t0, cnt, drawn, st);
+                    else chain_group_any<NW, 2>(a, form, sm, ctl, m.b, t0, cnt, drawn, st);
                 }
             } else if (role == 3) {
-                if (paired) {
-                    if (one) chain_run_ahead<NW, 1>(form, sm, ctl, m.b, ps, st);
-                    else chain_run_ahead<NW, 2>(form, sm, ctl, m.b, ps, st);
-                    continue;
-                }
+                if (one) chain_run_ahead<NW, 1>(form, sm, ctl, m.b, ps, st);
+                else chain_run_ahead<NW, 2>(form, sm, ctl, m.b, ps, st);
+                continue;
             } else if (role == 1) {
                 if (g + 2 < ng) fetch(g + 2);
                 // block b - 1 was drawn before this block's second group, and is
@@ -720,8 +702,8 @@ __device__ __forceinline__ void z_doc_chain(const ZArgs &a, uint8_t *sm, DocRun 
 }
 
 // Before the first document: the groups' barriers and the counters.
-__device__ __forceinline__ void chain_begin(uint8_t *sm) {
-    ChainCtl &ctl = *reinterpret_cast<ChainCtl *>(sm);
+__device__ __forceinline__ void cta_begin(uint8_t *sm) {
+    CtaCtl &ctl = *reinterpret_cast<CtaCtl *>(sm);
     if (threadIdx.x == 0) {
         for (int s = 0; s < 3; ++s) bar_init(&ctl.full[s]);
         for (int s = 0; s < 6; ++s) ctl.cnt[s] = 0;
