@@ -61,8 +61,8 @@ typedef struct {
     int32_t docs_per_warp;  /* z-step documents per warp: 0 = auto (two at K <= 1024 in passes
                                over many documents, else one), 1 = one, 4 = four (needs
                                K <= 1024; falls back to one when V K 4-byte weights do not fit
-                               2 GB); documents longer than 65,535 tokens still go one per warp,
-                               the longest to CTAs as coop_min_len says; results are identical */
+                               2 GB); the longest go to CTAs as coop_min_len says, others longer
+                               than 65,535 tokens one per warp; results are identical */
     int32_t phi_mode;       /* 0 = Poisson Polya urn (Algorithm 2), 1 = Dirichlet (Algorithm 1:
                                phi_k ~ Dir(n_k + beta) through Gamma draws, entries below 2^-24
                                of their column's maximum dropped); the batched form takes 0 only */
@@ -74,11 +74,11 @@ typedef struct {
                                slices, a different sampler from the paper's (AD-LDA's
                                approximation within a document).  Needs docs_per_warp 0 or 1;
                                fold-in, serving and the batched form ignore/reject it */
-    int32_t coop_min_len;   /* z-step and fold-in: a document of at least this many tokens (and
-                               at most 65,535) gets a CTA of its own, in which one warp draws
-                               the tokens and two others prepare and record them -- the least
-                               time per token -- concurrently with the other documents' one-warp
-                               kernel; results are identical.
+    int32_t coop_min_len;   /* z-step and fold-in: a document of at least this many tokens gets
+                               a CTA of its own, in which one warp draws the tokens and three
+                               others prepare, sum ahead and record them (above 8,192 topics
+                               four draw) -- the least time per token -- concurrently with the
+                               other documents' one-warp kernel; results are identical.
                                0 = auto (documents longer than max(256, N / 4500) tokens,
                                N / 9000 or N / 16000 beside two or four documents per warp: those that would
                                outlast the rest of the pass; where a pass has at most two

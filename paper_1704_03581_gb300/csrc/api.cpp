@@ -135,20 +135,19 @@ std::vector<int32_t> length_order(const int64_t *off, int64_t D) {
 }
 
 // Number of leading documents of a length-ordered schedule with 2^16 tokens
-// or more: their counts take three planes, which the one-warp kernel alone has.
+// or more: their counts take three planes.
 int64_t count_wide(const int64_t *off, const std::vector<int32_t> &order) {
     int64_t n = 0;
     while (n < static_cast<int64_t>(order.size()) && off[order[n] + 1] - off[order[n]] > kNarrowMaxLen) ++n;
     return n;
 }
 
-// Number of documents, after the n_wide widest of a length-ordered schedule,
-// that the long-document z-step takes.
-int64_t count_coop(const pulda_handle *h, const int64_t *off, const std::vector<int32_t> &order, int64_t n_wide, int64_t N) {
+// Number of leading documents that the long-document z-step takes.
+int64_t count_coop(const pulda_handle *h, const int64_t *off, const std::vector<int32_t> &order, int64_t N) {
     const int64_t L = long_document_tokens(h, static_cast<int64_t>(order.size()), N);
-    int64_t n = n_wide;
+    int64_t n = 0;
     while (n < static_cast<int64_t>(order.size()) && off[order[n] + 1] - off[order[n]] >= L) ++n;
-    return n - n_wide;
+    return n;
 }
 
 }  // namespace
@@ -226,9 +225,10 @@ int64_t long_document_tokens(const pulda_handle *h, int64_t D, int64_t N) {
     return std::max<int64_t>(kCoopAutoMin, N / div + 1);
 }
 
-// The n_wide widest documents one per warp, the next n_coop on a CTA each,
-// both on the handle's stream; beside them, on a second stream joined back
-// before the next step, the rest four per warp (grouped) or one per warp.
+// The first n_coop documents on a CTA each, on the handle's stream; beside
+// them, on a second stream joined back before the next step, the rest four per
+// warp (grouped), two or one; those of 2^16 tokens or more among the rest one
+// per warp, where the others go several, in a launch of their own.
 // Few documents (at most two for every CTA the GPU holds) all go to CTAs: each
 // is a chain of its own, and there a token takes a third of the time (1,000
 // documents of 100 tokens at K = 20: 85 us against 136).
@@ -236,37 +236,37 @@ cudaError_t run_z(pulda_handle *h, ZArgs a, int64_t n_wide, int64_t n_coop, int 
     cudaError_t e = cudaMemsetAsync(work, 0, 5 * sizeof(int), h->stream);
     if (e != cudaSuccess) return e;
     const int64_t D = a.D;
-    if (h->opt.coop_min_len == 0 && h->opt.slice_len == 0 && !h->z_groups && D - n_wide <= 2 * static_cast<int64_t>(h->coop_grid))
-        n_coop = D - n_wide;
-    const int64_t n_head = n_wide + n_coop;
-    const bool pairs = pairs_of_documents(h, D);
+    if (h->opt.coop_min_len == 0 && h->opt.slice_len == 0 && !h->z_groups && D <= 2 * static_cast<int64_t>(h->coop_grid)) n_coop = D;
     const int32_t *order = a.doc_order;
+    const bool pairs = pairs_of_documents(h, D);
+    // documents [n_coop, n_apart) one per warp beside the CTAs
+    const int64_t n_apart = h->z_groups || pairs ? std::max(n_coop, n_wide) : n_coop;
     auto launch_rest = [&](cudaStream_t st) {
-        if (D <= n_head) return;
+        if (D <= n_apart) return;
         ZArgs ar = a;
-        ar.doc_order = order + n_head;
-        ar.D = D - n_head;
-        ar.narrow = 1;
+        ar.doc_order = order + n_apart;
+        ar.D = D - n_apart;
+        ar.narrow = n_wide <= n_apart ? 1 : 0;
         ar.work = work + (h->z_groups ? 1 : 0);
         if (h->z_groups) launch_z_step_groups(ar, h->zg_grid, st);
         else if (pairs) launch_z_step_pairs(ar, h->z_warps, h->pair_grid, st);
         else launch_z_step(ar, h->z_warps, h->z_grid, st);
     };
     auto launch_head = [&](cudaStream_t st) {
-        if (n_wide > 0) {
+        if (n_coop > 0) {
+            const bool wide = n_wide > 0;
+            launch_z_step_coop(a, static_cast<int>(n_coop), wide, work + 3, wide ? h->coop_grid_wide : h->coop_grid, st);
+        }
+        if (n_apart > n_coop) {
             ZArgs aw = a;
-            aw.D = n_wide;
+            aw.doc_order = order + n_coop;
+            aw.D = n_apart - n_coop;
             aw.narrow = 0;
             aw.work = work + 2;
             launch_z_step(aw, h->z_warps, h->z_grid, st);
         }
-        if (n_coop > 0) {
-            ZArgs ac = a;
-            ac.doc_order = order + n_wide;
-            launch_z_step_coop(ac, static_cast<int>(n_coop), work + 3, h->coop_grid, st);
-        }
     };
-    if (n_head > 0 && n_head < D) {
+    if (n_apart > 0 && n_apart < D) {
         if ((e = cudaEventRecord(h->ev_fork, h->stream)) != cudaSuccess) return e;
         launch_head(h->stream);
         if ((e = cudaStreamWaitEvent(h->stream2, h->ev_fork, 0)) != cudaSuccess) return e;
@@ -526,9 +526,10 @@ pulda_status pulda_init(pulda_handle **out, const int32_t *word_ids, const int64
     h->z_grid = sms * z_step_blocks_per_sm(K, wpb, true);
     h->pair_grid = sms * z_pair_blocks_per_sm(K, wpb);
     h->n_wide = count_wide(doc_offsets, dord);
-    h->n_coop = count_coop(h, doc_offsets, dord, h->n_wide, N);
+    h->n_coop = count_coop(h, doc_offsets, dord, N);
     CUI(cudaGetLastError());
-    h->coop_grid = sms * z_coop_blocks_per_sm(K);
+    h->coop_grid = sms * z_coop_blocks_per_sm(K, false);
+    h->coop_grid_wide = sms * z_coop_blocks_per_sm(K, true);
     CUI(cudaGetLastError());
     CUI(cudaStreamCreateWithFlags(&h->stream2, cudaStreamNonBlocking));
     CUI(cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
@@ -789,7 +790,7 @@ pulda_status pulda_infer(pulda_handle *h, const int32_t *word_ids, const int64_t
     launch_init_z(N, h->K, seed, 0, dz, st);
     CU(h, clear_z_counters(h));
     const int64_t n_wide = count_wide(doc_offsets, ord);
-    const int64_t n_coop = count_coop(h, doc_offsets, ord, n_wide, N);
+    const int64_t n_coop = count_coop(h, doc_offsets, ord, N);
     for (int32_t sw = 1; sw <= n_sweeps; ++sw)
         CU(h, run_z(h, z_args(h, doff, dord, D_new, dw, dz, seed, static_cast<uint32_t>(sw), 0), n_wide, n_coop, h->work + 1));
     if (z_out) CU(h, cudaMemcpyAsync(z_out, dz, sizeof(int16_t) * N, cudaMemcpyDeviceToHost, st));
@@ -806,7 +807,7 @@ pulda_status pulda_z_layout(pulda_handle *h, int32_t *docs_per_warp, int64_t *co
     if (!h) return PULDA_ERR_INVALID;
     if (docs_per_warp) *docs_per_warp = h->z_groups ? 4 : pairs_of_documents(h, h->D) ? 2 : 1;
     if (coop_docs) *coop_docs = h->n_coop;
-    if (one_warp_docs) *one_warp_docs = h->z_groups ? h->n_wide : h->D - h->n_coop;
+    if (one_warp_docs) *one_warp_docs = h->z_groups ? std::max<int64_t>(0, h->n_wide - h->n_coop) : h->D - h->n_coop;
     return PULDA_OK;
 }
 

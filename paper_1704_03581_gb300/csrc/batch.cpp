@@ -83,14 +83,13 @@ cudaError_t balloc(pulda_batch *b, T **p, size_t n) {
 thread_local std::string g_batch_init_error;
 
 // Sets how many of each form's documents the long-document z-step takes at
-// threshold L (a form's list is longest first; the n_wide widest are the
-// one-warp kernel's).
+// threshold L (a form's list is longest first).
 void set_coop_items(pulda_batch *b, int64_t L) {
     for (int f = 0; f < b->bl.n_forms; ++f) {
         BatchForm &F = b->bl.form[f];
-        int n = F.n_wide;
+        int n = 0;
         while (L > 0 && n < F.n && b->form_len[F.first + n] >= L) ++n;
-        F.n_coop = n - F.n_wide;
+        F.n_coop = n;
     }
 }
 
@@ -312,7 +311,7 @@ pulda_status pulda_batch_init(pulda_batch **out, const pulda_chain_desc *chains,
         }
         F.n = static_cast<int>(flist.size()) - F.first;
         if (F.n == 0) continue;
-        F.coop_grid = b->sms * batch_coop_blocks_per_sm(F.kmax);
+        F.coop_grid = b->sms * batch_coop_blocks_per_sm(F.kmax, F.n_wide > 0);
         b->bl.form[b->bl.n_forms++] = F;
     }
     int2 *d_wl = nullptr, *d_fl = nullptr;
@@ -364,7 +363,7 @@ pulda_status pulda_batch_init(pulda_batch **out, const pulda_chain_desc *chains,
     int64_t fixed_coop = o.coop_min_len > 0 ? o.coop_min_len : 0;
     if (o.coop_min_len == 0) {
         const int64_t L = std::max<int64_t>(kCoopAutoMin, n_tokens / kBatchCoopDiv + 1);
-        if (std::any_of(b->form_len.begin(), b->form_len.end(), [&](int64_t n) { return n >= L && n <= kNarrowMaxLen; })) fixed_coop = L;
+        if (std::any_of(b->form_len.begin(), b->form_len.end(), [&](int64_t n) { return n >= L; })) fixed_coop = L;
     }
     // Launch forms: a launch or a few per phase with a CTA size for the z-step, and
     // (without documents on CTAs) one persistent launch for the Phi-step; tuned forms are timed.

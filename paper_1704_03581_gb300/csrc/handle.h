@@ -27,8 +27,8 @@ struct pulda_handle {
     bool z_groups = false;      // grouped z-step (four documents per warp) in use
     int zg_grid = 0;
     int64_t n_wide = 0;         // documents of 2^16 tokens or more (first in doc_order)
-    int64_t n_coop = 0;         // documents the long-document z-step takes (next in doc_order)
-    int coop_grid = 0;
+    int64_t n_coop = 0;         // documents the long-document z-step takes (first in doc_order)
+    int coop_grid = 0, coop_grid_wide = 0;      // its grid, and with documents of 2^16 tokens or more
     cudaStream_t stream2 = nullptr;                       // the one-warp z-step beside the CTAs'
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     std::vector<void *> allocs;
@@ -106,7 +106,7 @@ int64_t long_document_tokens(const pulda_handle *h, int64_t D, int64_t N);
 // Whether a pass over D documents takes them two per warp.
 bool pairs_of_documents(const pulda_handle *h, int64_t D);
 // One z-step over a's documents doc_order[0 .. D) on the handle's streams: the
-// first n_wide have 2^16 tokens or more, the next n_coop go to a CTA each, and
+// first n_wide have 2^16 tokens or more, the first n_coop go to a CTA each, and
 // so do the others when they are few.  work: five counters.
 cudaError_t run_z(pulda_handle *h, ZArgs a, int64_t n_wide, int64_t n_coop, int *work);
 PhiArgs phi_args(pulda_handle *h);

@@ -1458,15 +1458,15 @@ static void launch_batch_z(const BatchLaunch &b, cudaStream_t st) {
     for (int f = 0; f < b.n_forms; ++f) {
         const BatchForm &F = b.form[f];
         const int2 *items = b.form_items + F.first;
-        if (F.n_wide + F.n_coop > 0)
+        if (std::max(F.n_wide, F.n_coop) > 0)
             branch([&](cudaStream_t s) {
-                launch_z_step_multi(b, F, items, F.n_wide, false, b.work + 2 + 3 * f, s);
-                launch_z_step_coop_multi(b.z, items + F.n_wide, F.n_coop, b.work + 3 + 3 * f, F.kmax, F.coop_grid, s);
+                launch_z_step_coop_multi(b.z, items, F.n_coop, F.n_wide > 0, b.work + 3 + 3 * f, F.kmax, F.coop_grid, s);
+                launch_z_step_multi(b, F, items + F.n_coop, F.n_wide - F.n_coop, false, b.work + 2 + 3 * f, s);
             });
     }
     for (int f = 0; f < b.n_forms; ++f) {
         const BatchForm &F = b.form[f];
-        const int head = F.n_wide + F.n_coop;
+        const int head = std::max(F.n_wide, F.n_coop);
         if (F.n > head)
             branch([&](cudaStream_t s) {
                 launch_z_step_multi(b, F, b.form_items + F.first + head, F.n - head, true, b.work + 4 + 3 * f, s);

@@ -158,12 +158,13 @@ extern "C" pulda_status pulda_infer_noalloc(pulda_handle *h, const int32_t *word
         snprintf(msg, sizeof msg, "the word id at token %llu is outside [0, %d)", hfirst[0], hv.V);
         return static_cast<pulda_status>(handle_fail(h, PULDA_ERR_INVALID, msg));
     }
+    // (the documents of 2^16 tokens or more all go to CTAs, where any do)
     const int n_wide = hcount[0];
     int n_coop = 0, cursor[kLengthClasses], run = 0;
     for (int c = 0; c < kLengthClasses; ++c) {
         cursor[c] = run;
         run += hcount[c];
-        if (c >= 1 && c <= kLengthKeys) n_coop += hcount[c];
+        if (c == 0 ? coop_len != INT64_MAX : c <= kLengthKeys) n_coop += hcount[c];
     }
     e = cudaMemcpyAsync(count, cursor, sizeof cursor, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) {

@@ -55,6 +55,10 @@ __host__ __device__ inline int dense_pos(int K, int k) {
 // A document on a CTA of its own: a chain of warps up to here (zchain.cuh), all
 // warps on each token above (zsplit.cuh).
 constexpr int kChainMaxK = 8192;
+// With documents of 2^16 tokens or more, whose counts take a second plane, the
+// line lies here (one of 90,000 beside 500 others, ms per sweep, chain / split:
+// K = 4,200 86 / 112, 6,000 103 / 112, 8,000 128 / 112).
+constexpr int kChainWideMaxK = 6656;
 // Warps per CTA of the warp-per-document z-step: the default and the largest
 // accepted (the kernel's launch bounds are sized for it).
 #ifndef PULDA_ZWARPS
@@ -234,10 +238,11 @@ void launch_z_step(const ZArgs &a, int warps_per_block, int grid, cudaStream_t s
 // fits), documents of at most kNarrowMaxLen tokens, no slices.
 void launch_z_step_pairs(const ZArgs &a, int warps_per_block, int grid, cudaStream_t st);
 int z_pair_blocks_per_sm(int K, int warps_per_block);
-// The documents doc_order[0 .. n_coop), of at most kNarrowMaxLen tokens, one
-// CTA each (zchain.cuh); `work` is a counter zeroed before the launch.
-void launch_z_step_coop(const ZArgs &a, int n_coop, int *work, int grid, cudaStream_t st);
-int z_coop_blocks_per_sm(int K);
+// The documents doc_order[0 .. n_coop), one CTA each (zchain.cuh, zsplit.cuh);
+// `wide`: one of them has more than kNarrowMaxLen tokens; `work` is a counter
+// zeroed before the launch.
+void launch_z_step_coop(const ZArgs &a, int n_coop, bool wide, int *work, int grid, cudaStream_t st);
+int z_coop_blocks_per_sm(int K, bool wide);
 // Automatic threshold of the long-document z-step: a document on one warp
 // among 27 others on its SM takes about 1 us per token while the pass streams
 // a token in 0.32 ns (K = 1000), so one longer than N / 3100 tokens would
@@ -279,12 +284,12 @@ constexpr int kMaxGroupDocLen = 65535;
 // keeps m_d's counts in 16 bits (ZArgs::narrow).
 constexpr int64_t kNarrowMaxLen = 65535;
 // Length classes of documents (fold-in without allocation), eight to an octave
-// and the longest first: those of 2^16 tokens or more (one warp each), then
-// those of at least coop_len (a CTA each), then the rest.  So the schedule is
-// longest first, but for lengths within an eighth of each other; in any order
-// within the three groups, a long document taken up late was the end of the
-// pass (4,096 documents: 2.10 ms).  A class is in [0, kLengthClasses) whatever
-// the length.
+// and the longest first: those of 2^16 tokens or more, then those of at least
+// coop_len (a CTA each, as the ones before), then the rest.  So the schedule is
+// longest first, but for lengths within an eighth of each other or past 2^16; in
+// any order within the three groups, a long document taken up late was the end
+// of the pass (4,096 documents: 2.10 ms).  A class is in [0, kLengthClasses)
+// whatever the length.
 constexpr int kLengthKeys = 112;
 constexpr int kLengthClasses = 1 + 2 * kLengthKeys;
 __host__ __device__ inline int length_class(int64_t len, int64_t coop_len) {
@@ -330,8 +335,9 @@ struct GridBarrier {
 };
 
 // The chains of one form of the z-step (dense_words up to 1,024 topics, one
-// form to kChainMaxK and one above): their documents, n from `first` on in the form order, the n_wide
-// widest (2^16 tokens or more) one per warp, the next n_coop on CTAs.
+// form to kChainMaxK and one above): their documents, n from `first` on in the form order,
+// longest first: the first n_coop on CTAs, the others one per warp; the first
+// n_wide have 2^16 tokens or more.
 constexpr int kMaxForms = 6;
 struct BatchForm {
     int kmax, first, n;
@@ -380,9 +386,9 @@ cudaError_t launch_barrier_selftest(GridBarrier *bar, int blocks, int missing, i
                                     unsigned *passed, cudaStream_t st);
 int batch_phi_blocks_per_sm(int kmax);
 int batch_z_blocks_per_sm(int kmax, int warps, bool narrow);
-int batch_coop_blocks_per_sm(int kmax);
+int batch_coop_blocks_per_sm(int kmax, bool wide);
 // Documents on CTAs over (chain, document) items (coop.cu).
-void launch_z_step_coop_multi(const ZArgs *chains, const int2 *items, int n_items, int *work, int kmax, int grid,
+void launch_z_step_coop_multi(const ZArgs *chains, const int2 *items, int n_items, bool wide, int *work, int kmax, int grid,
                               cudaStream_t st);
 
 // A request being folded in by the server (device slot table entry).
@@ -402,11 +408,12 @@ void launch_serve_step(const ZArgs &a, ServeSlot *slots, const int32_t *active, 
                        int16_t *arena_z, int64_t slice, int *work, int warps_per_block, int grid, uint64_t window_ns,
                        bool narrow, cudaStream_t st);
 int serve_blocks_per_sm(int K, int warps_per_block);
-// The same with one CTA per slot, for long requests.
-void launch_serve_step_coop(const ZArgs &a, ServeSlot *slots, const int32_t *active, int n_active,
+// The same with one CTA per slot, for long requests; `wide`: one has more than
+// kNarrowMaxLen tokens.
+void launch_serve_step_coop(const ZArgs &a, ServeSlot *slots, const int32_t *active, int n_active, bool wide,
                             const int32_t *arena_w, int16_t *arena_z, int64_t slice, int *work, int grid,
                             uint64_t window_ns, cudaStream_t st);
-int serve_coop_blocks_per_sm(int K);
+int serve_coop_blocks_per_sm(int K, bool wide);
 // With the handle's coop_min_len 0 (automatic), requests at least this long
 // are served on CTAs, and all of them while a CTA is free for each.
 constexpr int64_t kServeCoopAuto = 1024;

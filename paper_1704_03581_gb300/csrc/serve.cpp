@@ -89,7 +89,7 @@ struct pulda_server {
     bool coop_auto = false;               // every request while a CTA is free for each
     uint64_t window_ns = 0;               // automatic slice: the launch's time window
     int32_t max_slots = 0;
-    int z_warps = 8, grid = 1, coop_grid = 1;
+    int z_warps = 8, grid = 1, coop_grid = 1, coop_grid_wide = 1;
     ZArgs tabs{};
     // device state
     int32_t *arena_w = nullptr;
@@ -189,9 +189,13 @@ void worker_loop(pulda_server *s) {
         const bool coop = s->coop_len > 0;
         const int64_t coop_len = s->coop_auto && n <= s->coop_grid ? 1 : s->coop_len;
         int nc = 0;
-        auto on_cta = [&](int32_t slot) { return coop && s->h_slots_len[slot] >= coop_len && s->h_slots_len[slot] <= kNarrowMaxLen; };
+        bool wide = false;      // a request on CTAs has 2^16 tokens or more
+        auto on_cta = [&](int32_t slot) { return coop && s->h_slots_len[slot] >= coop_len; };
         for (int32_t slot : s->active)
-            if (on_cta(slot)) s->h_active[nc++] = slot;
+            if (on_cta(slot)) {
+                s->h_active[nc++] = slot;
+                wide = wide || s->h_slots_len[slot] > kNarrowMaxLen;
+            }
         int j = nc;
         bool narrow = true;     // every request on the one-warp kernel fits 16-bit counts
         for (int32_t slot : s->active)
@@ -204,8 +208,8 @@ void worker_loop(pulda_server *s) {
         cudaEventRecord(s->ev0, s->stream);
         if (nc > 0) {
             cudaEventRecord(s->ev_fork, s->stream);
-            launch_serve_step_coop(s->tabs, s->d_slots, s->d_active, nc, s->arena_w, s->arena_z, s->slice,
-                                   s->d_work + 1, s->coop_grid, s->window_ns, s->stream);
+            launch_serve_step_coop(s->tabs, s->d_slots, s->d_active, nc, wide, s->arena_w, s->arena_z, s->slice,
+                                   s->d_work + 1, wide ? s->coop_grid_wide : s->coop_grid, s->window_ns, s->stream);
             cudaStreamWaitEvent(s->stream2, s->ev_fork, 0);
             launch_serve_step(s->tabs, s->d_slots, s->d_active + nc, n - nc, s->arena_w, s->arena_z, s->slice,
                               s->d_work, s->z_warps, s->grid, s->window_ns, narrow, s->stream2);
@@ -348,7 +352,8 @@ pulda_status pulda_serve_open(pulda_handle *h, int64_t token_budget, int32_t max
     int sms = 1;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->device);
     s->grid = sms * serve_blocks_per_sm(hv.K, hv.z_warps);
-    s->coop_grid = sms * serve_coop_blocks_per_sm(hv.K);
+    s->coop_grid = sms * serve_coop_blocks_per_sm(hv.K, false);
+    s->coop_grid_wide = sms * serve_coop_blocks_per_sm(hv.K, true);
     if ((e = cudaGetLastError()) != cudaSuccess) return bad(e, "set-up failed");
     s->worker = std::thread(worker_loop, s);
     *out = s;

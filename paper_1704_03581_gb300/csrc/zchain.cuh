@@ -54,8 +54,8 @@ __host__ __device__ __forceinline__ int chain_count_sets(int K) { return K <= kC
 
 // Shared memory of a CTA, in bytes: the barriers and counters; the drawn
 // topics of two groups; the coming token's sums; three blocks of records; the
-// sets of counts (two planes each) and, above 1024 topics, the lanes' bits; the
-// ring.
+// sets of counts (two planes each; three where a document of the launch has 2^16
+// tokens or more) and, above 1024 topics, the lanes' bits; the ring.
 struct CtaCtl {                 // what every kernel with a CTA per document has
     u64 full[3];                // a group's rows (zsplit.cuh: a row) have arrived
     u64 cnt[6];                 // the counters
@@ -73,17 +73,19 @@ constexpr int kChainRecOff = 1280;
 static_assert(sizeof(ChainCtl) <= kChainRecOff, "the control block must fit");
 constexpr int kChainCountOff = kChainRecOff + 3 * 32 * 4 * kChainRecWords;
 static_assert(kChainCountOff % 16 == 0, "counts and rows are read 16 bytes at a time");
-__host__ __device__ __forceinline__ int chain_ring_off(int K) {
-    return kChainCountOff + 2 * chain_count_sets(K) * 128 * dense_words(K) + (K > 1024 ? 16 * dense_words(K) : 0);
+__host__ __device__ __forceinline__ int chain_ring_off(int K, int planes = 2) {
+    return kChainCountOff + planes * chain_count_sets(K) * 128 * dense_words(K) + (K > 1024 ? 16 * dense_words(K) : 0);
 }
-__host__ __device__ __forceinline__ int chain_smem_bytes(int K) { return chain_ring_off(K) + 3 * chain_group(K) * dense_row_bytes(K); }
+__host__ __device__ __forceinline__ int chain_smem_bytes(int K, int planes = 2) {
+    return chain_ring_off(K, planes) + 3 * chain_group(K) * dense_row_bytes(K);
+}
 // The same for chains of any K up to kmax in one launch (shorter groups can
 // take less room than the longer ones below them).
-__host__ __device__ __forceinline__ int chain_smem_bytes_upto(int kmax) {
+__host__ __device__ __forceinline__ int chain_smem_bytes_upto(int kmax, int planes = 2) {
     int most = 0;
     const int edge[4] = {512, 1024, kChainMaxK, kMaxK};
     for (int e : edge) {
-        const int b = chain_smem_bytes(kmax < e ? kmax : e);
+        const int b = chain_smem_bytes(kmax < e ? kmax : e, planes);
         most = b > most ? b : most;
     }
     return most;
@@ -117,15 +119,24 @@ __device__ __forceinline__ void bar_expect(u64 *bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
 }
 
-// Counts of the chain: one plane, or two (P = 2), with no test in between.
+// Counts of the chain: P planes, with no test in between.
 template <int P>
 __device__ __forceinline__ uint32_t chain_count(const uint8_t *m, int PB, int p) {
-    return P == 1 ? m[p] : m[p] | (static_cast<uint32_t>(m[p + PB]) << 8);
+    uint32_t c = m[p];
+    if (P > 1) c |= static_cast<uint32_t>(m[p + PB]) << 8;
+    if (P > 2) c |= static_cast<uint32_t>(m[p + 2 * PB]) << 16;
+    return c;
 }
 template <int P>
 __device__ __forceinline__ void chain_set(uint8_t *m, int PB, int p, uint32_t c) {
     m[p] = static_cast<uint8_t>(c);
-    if (P == 2) m[p + PB] = static_cast<uint8_t>(c >> 8);
+    if (P > 1) m[p + PB] = static_cast<uint8_t>(c >> 8);
+    if (P > 2) m[p + 2 * PB] = static_cast<uint8_t>(c >> 16);
+}
+// Whether a group of G tokens keeps counts of at most `top` in P of PL planes.
+template <int P, int PL>
+__device__ __forceinline__ bool chain_fits(uint32_t top, int G) {
+    return P == PL || top + static_cast<uint32_t>(G) <= (P == 1 ? 255u : 65535u);
 }
 __device__ __forceinline__ uint32_t row_weight(const uint8_t *row, int PB, int p) {
     return row[p] | (static_cast<uint32_t>(row[p + PB]) << 8) | (static_cast<uint32_t>(row[p + 2 * PB]) << 16);
@@ -281,7 +292,8 @@ struct ChainForm<0> {
     template <int P>
     __device__ __forceinline__ u64 dot(const uint8_t *row, const uint8_t *m, int lane) const {
         u64 sum = big_plane_dot(row, m, PB, C, lane);
-        if (P == 2) sum += big_plane_dot(row, m + PB, PB, C, lane) << 8;
+        if (P > 1) sum += big_plane_dot(row, m + PB, PB, C, lane) << 8;
+        if (P > 2) sum += big_plane_dot(row, m + 2 * PB, PB, C, lane) << 16;
         return sum;
     }
     template <int P>
@@ -339,7 +351,7 @@ struct ChainPass {
 
 // Warp 3: the sums of the token after each of the coming groups' tokens, while
 // that one is drawn; for as long as counts stay in P planes.
-template <int NW, int P>
+template <int NW, int P, int PL>
 __device__ __forceinline__ void chain_run_ahead(const ChainForm<NW> &form, uint8_t *sm, ChainCtl &ctl, uint8_t *m, ChainPass &ps,
                                                 ChainState &st) {
     const int lane = threadIdx.x & 31;
@@ -374,12 +386,12 @@ __device__ __forceinline__ void chain_run_ahead(const ChainForm<NW> &form, uint8
             pair_barrier();
         }
         ps.meet(ctl);
-    } while (ps.more() && (P == 2 || st.top + static_cast<uint32_t>(ps.G) <= 255u));
+    } while (ps.more() && chain_fits<P, PL>(st.top, ps.G));
 }
 
 // Warp 0: the coming groups, while every token of theirs has a dense row and
 // counts stay in P planes.
-template <int NW, int P>
+template <int NW, int P, int PL>
 __device__ __forceinline__ void chain_run_fast(const ChainForm<NW> &form, uint8_t *sm, ChainCtl &ctl, uint8_t *m, ChainPass &ps,
                                                ChainState &st) {
     using G = DenseGeo<NW>;
@@ -427,7 +439,7 @@ __device__ __forceinline__ void chain_run_fast(const ChainForm<NW> &form, uint8_
             pair_barrier();
         }
         ps.meet(ctl);
-    } while (ps.more() && !(ps.after & kMixed) && (P == 2 || st.top + static_cast<uint32_t>(ps.G) <= 255u));
+    } while (ps.more() && !(ps.after & kMixed) && chain_fits<P, PL>(st.top, ps.G));
 }
 
 // The same for any group: tokens without a dense row among them, or K > 1024.
@@ -485,10 +497,52 @@ __device__ __forceinline__ void chain_group_any(const ZArgs &a, const ChainForm<
     }
 }
 
+// A run's topics counted by every thread of the CTA, K 32-bit counts in `hist`:
+// shared memory that bulk copies write later, behind async_reuse() and a barrier.
+// Warps that each count the tokens for themselves wait on one load per 32: 1 us
+// of them, so 3 ms for 90,000 tokens, in every launch of a request that long (us
+// per token of 66,000, K = 1,000: 0.312 -> 0.297).  The counts' way through K
+// words costs more where documents are short (K = 3,000, 200 tokens 0.742 ->
+// 0.758, 1,000 0.662 -> 0.656; K = 8,000, 600 tokens 0.874 -> 0.889).
+__device__ __forceinline__ int chain_hist_tokens(int K) { return 128 + K / 8; }
+constexpr int kCtaHistBatch = 8;
+__device__ __forceinline__ void cta_histogram(const ZArgs &a, const DocRun &r, uint32_t *hist) {
+    for (int k = threadIdx.x; k < a.K; k += blockDim.x) hist[k] = 0;
+    __syncthreads();
+    const int T = blockDim.x;
+    int i = threadIdx.x;
+    for (; i + (kCtaHistBatch - 1) * T < r.len; i += kCtaHistBatch * T) {
+        int k[kCtaHistBatch];
+#pragma unroll
+        for (int u = 0; u < kCtaHistBatch; ++u) k[u] = r.z[i + u * T];
+#pragma unroll
+        for (int u = 0; u < kCtaHistBatch; ++u) atomicAdd(&hist[guard_index(k[u], a.K, a.stats)], 1u);
+    }
+    for (; i < r.len; i += T) atomicAdd(&hist[guard_index(r.z[i], a.K, a.stats)], 1u);
+    __syncthreads();
+}
+__device__ __forceinline__ void async_reuse() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+// One warp's counts from them: PL planes, and lvl.
+template <int PL, typename Pos>
+__device__ __forceinline__ void counts_from(const uint32_t *hist, int K, DocCounts &m, Pos pos) {
+    const int lane = threadIdx.x & 31;
+    for (int i = lane; i < PL * m.PB / 16; i += 32) reinterpret_cast<uint4 *>(m.b)[i] = make_uint4(0u, 0u, 0u, 0u);
+    __syncwarp();
+    int top = 0;
+    for (int k = lane; k < K; k += 32) {
+        const uint32_t c = hist[k];
+        if (c) chain_set<PL>(m.b, m.PB, pos(k), c);
+        top = max(top, count_level(c));
+    }
+    m.lvl = static_cast<int>(__reduce_max_sync(0xFFFFFFFFu, static_cast<unsigned>(top)));
+    __syncwarp();
+}
+
 // All threads of the CTA; sm: chain_smem_bytes(K) bytes.  phases: the parities
-// of the groups' barriers, kept from one document to the next.  Documents of
-// at most kNarrowMaxLen tokens.
-template <int NW>
+// of the groups' barriers, kept from one document to the next.  PL planes of
+// counts: two for documents of at most kNarrowMaxLen tokens, three for any.
+template <int NW, int PL>
 __device__ __forceinline__ void z_doc_chain(const ZArgs &a, uint8_t *sm, DocRun &r, uint32_t &phases) {
     const int lane = threadIdx.x & 31;
     const int role = threadIdx.x >> 5;      // 0: the chain, 1: records and rows, 2: counters and topics, 3: sums ahead
@@ -496,23 +550,30 @@ __device__ __forceinline__ void z_doc_chain(const ZArgs &a, uint8_t *sm, DocRun 
     if (r.len == 0 || r.budget <= 0) return;
     ChainCtl &ctl = *reinterpret_cast<ChainCtl *>(sm);
     uint4 *recs = reinterpret_cast<uint4 *>(sm + kChainRecOff);
-    const int ring = chain_ring_off(K), RB = dense_row_bytes(K), G = chain_group(K);
+    const int ring = chain_ring_off(K, PL), RB = dense_row_bytes(K), G = chain_group(K);
     ChainForm<NW> form(K);
     const int PB = form.plane();
     auto pos = [&](int k) { return form.pos(k); };
     // warps 0, 2 and 3 each keep the document's counts
-    DocCounts m{sm + kChainCountOff + (role == 0 ? 0 : role == 2 ? 2 * PB : 4 * PB), PB, 0};
-    if (role != 1) build_counts(a, m, r, nullptr, 2, pos);
+    DocCounts m{sm + kChainCountOff + (role == 0 ? 0 : role == 2 ? PL * PB : 2 * PL * PB), PB, 0};
+    if (r.len >= chain_hist_tokens(K)) {
+        uint32_t *hist = reinterpret_cast<uint32_t *>(sm + ring);
+        cta_histogram(a, r, hist);
+        if (role != 1) counts_from<PL>(hist, K, m, pos);
+        async_reuse();
+    } else if (role != 1) {
+        build_counts(a, m, r, nullptr, PL, pos);
+    }
     ChainState st{};
     st.prev = -1;
     bool begun = false;
     int kd = 0;
     if (role == 0 || role == 3) {
         uint32_t top = 0;
-        for (int p = lane; p < PB; p += 32) top = max(top, m.b[p] | (static_cast<uint32_t>(m.b[p + PB]) << 8));
+        for (int p = lane; p < PB; p += 32) top = max(top, chain_count<PL>(m.b, PB, p));
         st.top = __reduce_max_sync(0xFFFFFFFFu, top);
     } else if (role == 2) {
-        kd = static_cast<int>(__reduce_add_sync(0xFFFFFFFFu, static_cast<unsigned>(form.init_bits(m, sm + kChainCountOff + 2 * chain_count_sets(K) * PB, lane))));
+        kd = static_cast<int>(__reduce_add_sync(0xFFFFFFFFu, static_cast<unsigned>(form.init_bits(m, sm + kChainCountOff + PL * chain_count_sets(K) * PB, lane))));
     }
     constexpr int colmax = -1;     // a row wherever there is one
     const uint32_t sweep_end = r.sweep + static_cast<uint32_t>(r.max_pass_end);
@@ -593,18 +654,18 @@ __device__ __forceinline__ void z_doc_chain(const ZArgs &a, uint8_t *sm, DocRun 
                 const uint4 r2 = recs[3 * ((t0 + u) % 96) + 2];
                 const uint32_t x = ctl.drawn[8 * (g & 1) + u];
                 const int knew = static_cast<int>(x & 0x3FFFu), n_w = static_cast<int>(r2.z);
-                const uint32_t co = chain_count<2>(m.b, PB, kold) - 1u;
+                const uint32_t co = chain_count<PL>(m.b, PB, kold) - 1u;
                 __syncwarp();
-                chain_set<2>(m.b, PB, kold, co);
+                chain_set<PL>(m.b, PB, kold, co);
                 if (co == 0) --kd;
                 form.flip(kold, lane, co == 0);
                 c_min += static_cast<uint32_t>(kd < n_w ? kd : n_w);
                 c_cnt += (kd < n_w ? 1u : 0u) + (x & kDrawnAlias ? 1u << 6 : 0u) + (x & kDrawnZero ? 1u << 12 : 0u);
                 if constexpr (NW > 0) c_int += static_cast<uint32_t>(__popc(bits & form.mbits));
                 else c_int += form.shared_topics(a.bits + static_cast<int64_t>(r2.w) * a.KWp, lane);
-                const uint32_t cn = chain_count<2>(m.b, PB, knew) + 1u;
+                const uint32_t cn = chain_count<PL>(m.b, PB, knew) + 1u;
                 __syncwarp();
-                chain_set<2>(m.b, PB, knew, cn);
+                chain_set<PL>(m.b, PB, knew, cn);
                 if (cn == 1) ++kd;
                 form.flip(knew, lane, cn == 1);
             };
@@ -640,34 +701,38 @@ __device__ __forceinline__ void z_doc_chain(const ZArgs &a, uint8_t *sm, DocRun 
             const uint4 r1 = recs[1];
             if (!begun) {
                 st.prev = static_cast<int>(r1.x & 0xFFFFu);
-                const uint32_t c = chain_count<2>(m.b, PB, st.prev) - 1u;
+                const uint32_t c = chain_count<PL>(m.b, PB, st.prev) - 1u;
                 __syncwarp();
-                chain_set<2>(m.b, PB, st.prev, c);
+                chain_set<PL>(m.b, PB, st.prev, c);
                 __syncwarp();
             }
-            if (r1.y != 0xFFFFFFFFu && role == 3) ctl.ahead[0][lane] = chain_sums<NW, 2>(form, sm, m.b, r1, lane);
+            if (r1.y != 0xFFFFFFFFu && role == 3) ctl.ahead[0][lane] = chain_sums<NW, PL>(form, sm, m.b, r1, lane);
             begun = true;
         }
         __syncthreads();
         while (ps.more()) {
             const int g = ps.g, t0 = g * G, cnt = ps.group_tokens();
-            const bool one = st.top + static_cast<uint32_t>(G) <= 255u;      // counts stay in one plane
+            // counts stay in one plane, or two
+            const bool one = chain_fits<1, PL>(st.top, G), two = chain_fits<2, PL>(st.top, G);
             if (role == 0) {
                 uint32_t *drawn = ctl.drawn + 8 * (g & 1);
                 if constexpr (NW > 0) {
                     if (!(ps.after & kMixed)) {
-                        if (one) chain_run_fast<NW, 1>(form, sm, ctl, m.b, ps, st);
-                        else chain_run_fast<NW, 2>(form, sm, ctl, m.b, ps, st);
+                        if (one) chain_run_fast<NW, 1, PL>(form, sm, ctl, m.b, ps, st);
+                        else if (two) chain_run_fast<NW, 2, PL>(form, sm, ctl, m.b, ps, st);
+                        else chain_run_fast<NW, PL, PL>(form, sm, ctl, m.b, ps, st);
                         continue;
                     }
-                    chain_group_any<NW, 2>(a, form, sm, ctl, m.b, t0, cnt, drawn, st);
+                    chain_group_any<NW, PL>(a, form, sm, ctl, m.b, t0, cnt, drawn, st);
                 } else {
                     if (one) chain_group_any<NW, 1>(a, form, sm, ctl, m.b, t0, cnt, drawn, st);
-                    else chain_group_any<NW, 2>(a, form, sm, ctl, m.b, t0, cnt, drawn, st);
+                    else if (two) chain_group_any<NW, 2>(a, form, sm, ctl, m.b, t0, cnt, drawn, st);
+                    else chain_group_any<NW, PL>(a, form, sm, ctl, m.b, t0, cnt, drawn, st);
                 }
             } else if (role == 3) {
-                if (one) chain_run_ahead<NW, 1>(form, sm, ctl, m.b, ps, st);
-                else chain_run_ahead<NW, 2>(form, sm, ctl, m.b, ps, st);
+                if (one) chain_run_ahead<NW, 1, PL>(form, sm, ctl, m.b, ps, st);
+                else if (two) chain_run_ahead<NW, 2, PL>(form, sm, ctl, m.b, ps, st);
+                else chain_run_ahead<NW, PL, PL>(form, sm, ctl, m.b, ps, st);
                 continue;
             } else if (role == 1) {
                 if (g + 2 < ng) fetch(g + 2);

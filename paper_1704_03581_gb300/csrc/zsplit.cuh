@@ -79,10 +79,14 @@ __device__ __forceinline__ bool z_doc_split(const ZArgs &a, uint8_t *sm, DocRun 
     auto col_of = [&](int t) { return sm + kSplitColOff + (t & 1) * kSplitColBytes; };
     const int planes = r.len <= kNarrowMaxLen ? 2 : 3;
     DocCounts all{counts, PB, planes - 1};
-    if (warp == 0) build_counts(a, all, r, nullptr, planes, pos);
+    for (int i = threadIdx.x; i < planes * PB / 16; i += kSplitThreads) reinterpret_cast<uint4 *>(counts)[i] = make_uint4(0u, 0u, 0u, 0u);
+    uint32_t *hist = reinterpret_cast<uint32_t *>(ring);
+    cta_histogram(a, r, hist);
+    for (int k = threadIdx.x; k < K; k += kSplitThreads)
+        if (hist[k]) all.set(pos(k), hist[k]);
+    async_reuse();
     if (threadIdx.x == 0) x.kd = x.high = x.bad[0] = x.bad[1] = 0;
     __syncthreads();
-    all.lvl = planes - 1;
     // this thread's topics: lane `lane`'s chunks [c0, c1), and the planes they take
     const int per = (C + kSplitWarps - 1) / kSplitWarps, c0 = min(C, warp * per), c1 = min(C, c0 + per);
     auto mine = [&](int p) { return ((p >> 4) & 31) == lane && static_cast<unsigned>((p >> 9) - c0) < static_cast<unsigned>(c1 - c0); };

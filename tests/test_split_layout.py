@@ -39,6 +39,13 @@ int main() {
         CHECK(next == C, "K=%d: %d of %d chunks", K, next, C);
         CHECK(bitmap_row_words(K) <= kSplitMapWords && bitmap_row_words(K) % 4 == 0, "K=%d: bitmap row", K);
     }
+    // the chain with three count planes
+    for (int K = 1; K <= kChainMaxK; ++K) {
+        const int ring = chain_ring_off(K, 3), pb = 128 * dense_words(K);
+        CHECK(ring % 16 == 0 && kChainCountOff + 3 * chain_count_sets(K) * pb + (K > 1024 ? 64 * ((K + 511) / 512) : 0) <= ring, "K=%d: ring at %d", K, ring);
+        CHECK(chain_smem_bytes(K, 3) == ring + 3 * chain_group(K) * 3 * pb && chain_smem_bytes(K, 3) <= 227 * 1024, "K=%d: %d bytes", K, chain_smem_bytes(K, 3));
+        CHECK(chain_smem_bytes_upto(K, 3) >= chain_smem_bytes(K, 3), "chains up to K=%d", K);
+    }
     std::printf("violations %d\n", bad);
     return bad != 0;
 }
