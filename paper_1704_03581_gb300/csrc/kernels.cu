@@ -1415,10 +1415,12 @@ void launch_slice_counts(const int64_t *doc_off, const int32_t *sliced_docs, int
 }
 
 void launch_z_step(const ZArgs &a, int warps_per_block, int grid, cudaStream_t st) {
-    // documents of 2^16 tokens or more are few, and each is bound by its loads'
-    // latency: above 1,024 topics they take the form that has more of them in
-    // flight
-    const bool few = a.narrow == 0 && a.n_slices == 0 && a.D <= 4 * static_cast<int64_t>(sm_count()) && z_nw(a.K) == 0;
+    // Few documents, each bound by its loads' latency, take the form that has more
+    // of them in flight: above 1,024 topics where one has 2^16 tokens or more,
+    // above 4,096 always (100 documents of 200 tokens, ms: K = 8,000 1.55 -> 1.15,
+    // K = 16,384 4.4 -> 2.7; 700 beside documents on CTAs, whose SMs it shares
+    // worse: K = 3,000 0.64 -> 0.80, K = 8,000 1.07 -> 0.86)
+    const bool few = (a.K > 4096 || a.narrow == 0) && a.n_slices == 0 && a.D <= 4 * static_cast<int64_t>(sm_count()) && z_nw(a.K) == 0;
     const ZStepKernel kern = few ? k_z_step<-1> : z_step_kernel(a.K);
     if (few) allow_dynamic_smem(kern);
     kern<<<grid, 32 * warps_per_block, z_step_smem(a.K, warps_per_block, a.narrow != 0), st>>>(a);

@@ -485,7 +485,7 @@ __device__ __forceinline__ void chain_group_any(const ZArgs &a, const ChainForm<
             uint32_t c = 0;
             DocCounts mc{m, PB, P - 1};
             const TokenDraw td{At, U, static_cast<int>(r1.x >> 16), kold};
-            const int k = column_draw(a, td, static_cast<int64_t>((static_cast<u64>(r2.y) << 32) | r2.x), static_cast<int>(r2.z), mc, lane, c,
+            const int k = column_draw<4>(a, td, static_cast<int64_t>((static_cast<u64>(r2.y) << 32) | r2.x), static_cast<int>(r2.z), mc, lane, c,
                                       [&](int x) { return form.pos(x); });
             knew = static_cast<uint32_t>(k) | (c & (1u << 6) ? kDrawnAlias : 0u) | (c & (1u << 12) ? kDrawnZero : 0u);
         }

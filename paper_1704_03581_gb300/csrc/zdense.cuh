@@ -116,6 +116,17 @@ __device__ __forceinline__ void build_counts(const ZArgs &a, DocCounts &m, const
     __syncwarp();
 }
 
+// Which of the sixteen topics from position p on (one chunk of a lane) have m > 0.
+__device__ __forceinline__ uint32_t nonzero_topics(const DocCounts &m, int p, int planes) {
+    uint4 v = *reinterpret_cast<const uint4 *>(m.b + p);
+    for (int pl = 1; pl < planes; ++pl) {
+        const uint4 u = *reinterpret_cast<const uint4 *>(m.b + p + pl * m.PB);
+        v = make_uint4(v.x | u.x, v.y | u.y, v.z | u.z, v.w | u.w);
+    }
+    auto four = [](uint32_t x) { return ((__vcmpne4(x, 0u) & 0x01010101u) * 0x01020408u) >> 24 & 15u; };
+    return four(v.x) | four(v.y) << 4 | four(v.z) << 8 | four(v.w) << 12;
+}
+
 // NW words of a plane (bytes of this lane's topics) from p, one to eight.
 template <int NW>
 __device__ __forceinline__ void load_words(const uint8_t *p, int lane, uint32_t (&w)[NW]) {
@@ -265,49 +276,78 @@ __device__ __forceinline__ int dense_draw(const ZArgs &a, u64 sum, const TokenDr
 }
 
 // The same over the word's column (words with few topics, or without a dense
-// row): lane l takes a contiguous share of its n_w entries.
-template <typename Pos>
+// row): lane l takes a contiguous share of its n_w entries, B of them loaded at
+// once; a found lane's share of more than B is shared out, an entry per lane (a
+// lane that walked it waited on a load per entry).
+template <int B, typename Pos>
 __device__ __forceinline__ int column_draw(const ZArgs &a, const TokenDraw &t, int64_t col, int n_w, const DocCounts &m,
                                            int lane, uint32_t &c_cnt, Pos pos) {
     __syncwarp();                                        // the column reads every lane's counts
-    const uint32_t *qcol = a.q + col;
-    const uint16_t *tcol = a.topic + col;
     const int seg = (n_w + 31) >> 5;
     const int j0 = min(seg * lane, n_w), j1 = min(j0 + seg, n_w);
-    u64 acc = 0;
-#pragma unroll 4
-    for (int j = j0; j < j1; ++j)
-        acc += static_cast<u64>(qcol[j]) * m.get(pos(guard_index(tcol[j], a.K, a.stats)));
+    u64 acc = 0, term[B];
+    int at[B];
+    for (int j = j0; j == j0 || j < j1; j += B) {
+        uint32_t q[B];
+        int k[B];
+#pragma unroll
+        for (int i = 0; i < B; ++i) {
+            q[i] = j + i < j1 ? a.q[col + j + i] : 0u;
+            k[i] = j + i < j1 ? a.topic[col + j + i] : 0;
+        }
+#pragma unroll
+        for (int i = 0; i < B; ++i) {
+            at[i] = pos(guard_index(k[i], a.K, a.stats));
+            term[i] = static_cast<u64>(q[i]) * m.get(at[i]);
+            acc += term[i];
+        }
+    }
     const u64 incl = warp_incl_scan(acc);
     u64 rb;
     const int settled = split_draw(t, __shfl_sync(0xFFFFFFFFu, incl, 31), rb, c_cnt);
     if (settled >= 0) return settled;
     const int L = __ffs(__ballot_sync(0xFFFFFFFFu, rb < incl)) - 1;
-    int f = -1;
-    if (lane == L) {
-        u64 run = incl - acc;
-        for (int j = j0; j < j1; ++j) {
-            const int k = pos(guard_index(tcol[j], a.K, a.stats));
-            run += static_cast<u64>(qcol[j]) * m.get(k);
-            if (rb < run) { f = k; break; }
+    u64 res = __shfl_sync(0xFFFFFFFFu, rb - (incl - acc), L);
+    if (seg <= B) {
+        int f = -1;
+        u64 upto = acc;
+#pragma unroll
+        for (int i = B - 1; i >= 0; --i) {
+            if (res < upto) f = at[i];
+            upto -= term[i];
         }
+        f = __shfl_sync(0xFFFFFFFFu, f, L);
+        if (f >= 0) return f;
     }
-    f = __shfl_sync(0xFFFFFFFFu, f, L);
-    if (f < 0) {
-        if (lane == 0) atomicOr(&a.stats[ST_ERROR], ERR_INTERNAL);
-        return t.kold;
+    const int end = min(seg * L + seg, n_w);
+    for (int i0 = seg <= B ? end : seg * L; i0 < end; i0 += 32) {
+        const int j = i0 + lane;
+        const int k = pos(guard_index(j < end ? a.topic[col + j] : 0, a.K, a.stats));
+        const u64 p = j < end ? static_cast<u64>(a.q[col + j]) * m.get(k) : 0;
+        const u64 upto = warp_incl_scan(p);
+        const uint32_t f = __ballot_sync(0xFFFFFFFFu, res < upto);
+        if (f) return __shfl_sync(0xFFFFFFFFu, k, __ffs(f) - 1);
+        res -= __shfl_sync(0xFFFFFFFFu, upto, 31);
     }
-    return f;
+    if (lane == 0) atomicOr(&a.stats[ST_ERROR], ERR_INTERNAL);
+    return t.kold;
 }
 
 // A word with at most this many nonzero topics is summed over its column
 // even when it has a dense row: one or two entries per lane instead of the
-// whole row, which for such (rare) words mostly comes from beyond L1.
+// whole row, which for such (rare) words mostly comes from beyond L1.  Above
+// 1,024 topics a row's work grows with K: with a limit of 128, K / 16, K / 10 and
+// K / 6 a pass over 12,000 documents of 200 tokens, one per warp, takes 3.2, 3.1,
+// 3.0 and 3.0 ms at K = 3,000, 6.5, 5.5, 5.3 and 5.5 at 8,000, 24.8, 16.5, 16.1 and
+// 16.2 at 16,384.
 // zstep_path 1 raises the limit, 2 takes the row wherever there is one.
 template <int NW>
 __device__ __forceinline__ constexpr int column_max() { return NW == 0 ? 128 : NW == 8 ? 64 : NW == 4 ? 32 : 0; }
 template <int NW>
-__device__ __forceinline__ int column_limit(int path) { return path == 1 ? 2 * column_max<NW>() + 32 : path == 2 ? -1 : column_max<NW>(); }
+__device__ __forceinline__ int column_limit(int path, int K) {
+    const int most = NW > 0 ? column_max<NW>() : max(column_max<NW>(), K / 10);
+    return path == 1 ? 2 * most + 32 : path == 2 ? -1 : most;
+}
 
 // The staging records of a warp: where z_doc keeps them for its K.
 template <int NW>
@@ -378,7 +418,7 @@ __device__ __forceinline__ int z_block(const ZArgs &a, DocCounts &m, const uint4
             knew = dense_draw<NW>(a, sum, t, r0, m, fine, c_cnt);
         } else {
             const int64_t col = static_cast<int64_t>((static_cast<u64>(t0.y & 0xFFFFu) << 32) | t0.x);
-            knew = column_draw(a, t, col, n_w, m, lane, c_cnt, [](int k) { return G::pos(k); });
+            knew = column_draw<2>(a, t, col, n_w, m, lane, c_cnt, [](int k) { return G::pos(k); });
             fetch_row(dn);
         }
         d = dn;
@@ -428,7 +468,7 @@ __device__ __forceinline__ void z_doc_regs(const ZArgs &a, uint32_t *sm, DocRun 
     uint4 *rec = token_records<NW>(sm, a);
     uint32_t *drow_of = reinterpret_cast<uint32_t *>(rec + 64);
     const uint32_t sweep_end = rs.sweep + static_cast<uint32_t>(rs.max_pass_end);
-    const int colmax = column_limit<NW>(a.path);
+    const int colmax = column_limit<NW>(a.path, a.K);
     bool first = true;
     while (rs.budget > 0 && rs.sweep != sweep_end) {
         if (rs.deadline != ~0ull && !first) {
@@ -537,7 +577,10 @@ __device__ __forceinline__ int big_find(int L, u64 res, const uint8_t *row, cons
 // The same for K > 1024: 512 C topics, lane l owning the 16 C from 16 C l on,
 // in C chunks of one 16-byte load per plane.  A lane holds no row and no
 // group sums: it accumulates its chunks, and the found lane's 2 C groups of
-// eight topics are summed again, one group per lane.
+// eight topics are summed again, one group per lane.  The topics that document and
+// word share are counted over words in topic order, 16 bytes a lane (over every
+// lane's 2 C bytes, two at a time, they took half of a token's time at K =
+// 16,384: 24.3 -> 14.0 ms with the column limit for 12,000 documents).
 // U > 0: for few documents at a time, the next token's first U chunks loaded
 // while this one is drawn.
 template <int U>
@@ -555,25 +598,30 @@ __device__ __forceinline__ void z_doc_big(const ZArgs &a, uint32_t *sm, DocRun &
     const int planes = z_count_planes(a.narrow != 0);
     DocCounts m{reinterpret_cast<uint8_t *>(sm), PB, 0};
     build_counts(a, m, r, m0, planes, pos);
-    // the lane's topics with m > 0, 16 bits per chunk, in shared memory (only
-    // this lane touches them)
-    uint16_t *mb = reinterpret_cast<uint16_t *>(m.b + planes * PB) + lane;
+    // the topics with m > 0 as bits in topic order, in shared memory: words
+    // 128 i + 4 lane to + 3 are this lane's (only it touches them)
+    uint32_t *map = reinterpret_cast<uint32_t *>(m.b + planes * PB);
     int kd = 0;
-    for (int c = 0; c < C; ++c) {
-        uint32_t bits = 0;
-        for (int b = 0; b < 16; ++b)
-            if (m.get(512 * c + 16 * lane + b) > 0) bits |= 1u << b;
-        mb[32 * c] = static_cast<uint16_t>(bits);
-        kd += __popc(bits);
-    }
+    for (int w0 = 4 * lane; w0 < 16 * C; w0 += 128)
+        for (int w = w0; w < w0 + 4; ++w) {
+            map[w] = nonzero_topics(m, pos(32 * w), planes) | nonzero_topics(m, pos(32 * w + 16), planes) << 16;
+            kd += __popc(map[w]);
+        }
     kd = static_cast<int>(__reduce_add_sync(0xFFFFFFFFu, static_cast<unsigned>(kd)));
+    auto flip = [&](int p) {
+        const int k = ((p >> 4) & 31) * TPL + ((p >> 9) << 4) + (p & 15), w = k >> 5;
+        if (((w >> 2) & 31) == lane) map[w] ^= 1u << (k & 31);
+    };
+    auto common = [](const uint4 x, const uint4 y) {
+        return static_cast<uint32_t>(__popc(x.x & y.x) + __popc(x.y & y.y) + __popc(x.z & y.z) + __popc(x.w & y.w));
+    };
     DocRun &rs = *z_warp_run(wcnt);
     if (lane == 0) rs = r;
     __syncwarp();
     uint4 *rec = token_records<0>(sm, a);
     uint32_t *drow_of = reinterpret_cast<uint32_t *>(rec + 64);
     const uint32_t sweep_end = rs.sweep + static_cast<uint32_t>(rs.max_pass_end);
-    const int colmax = column_limit<0>(a.path);
+    const int colmax = column_limit<0>(a.path, a.K);
     bool first = true;
     while (rs.budget > 0 && rs.sweep != sweep_end) {
         if (rs.deadline != ~0ull && !first) {
@@ -617,18 +665,17 @@ __device__ __forceinline__ void z_doc_big(const ZArgs &a, uint32_t *sm, DocRun &
                     const uint32_t c = m.get(p) - 1u;
                     m.set(p, c);
                     died = c == 0;
-                    if (died) mb[(p >> 9) << 5] &= static_cast<uint16_t>(~(1u << (p & 15)));
                 }
-                kd -= __any_sync(0xFFFFFFFFu, died) ? 1 : 0;
+                if (__any_sync(0xFFFFFFFFu, died)) {
+                    --kd;
+                    flip(p);
+                }
             }
             c_min += static_cast<uint32_t>(kd < n_w ? kd : n_w);
             c_cnt += kd < n_w ? 1u : 0u;
             // the word's bits, counted after the draw: nothing waits for their loads
-            const uint16_t *wb = reinterpret_cast<const uint16_t *>(a.bits + static_cast<int64_t>(t1.z) * a.KWp) + C * lane;
-            constexpr int kEarly = 6;
-            uint32_t early[kEarly];
-#pragma unroll
-            for (int c = 0; c < kEarly; ++c) early[c] = c < C ? wb[c] : 0u;
+            const uint32_t *wb = a.bits + static_cast<int64_t>(t1.z) * a.KWp;
+            const uint4 early = 4 * lane < 16 * C ? *reinterpret_cast<const uint4 *>(wb + 4 * lane) : make_uint4(0u, 0u, 0u, 0u);
             const uint32_t d = drow_of[tt];
             int knew = -1;
             if (d != 0xFFFFFFFFu) {
@@ -660,13 +707,12 @@ __device__ __forceinline__ void z_doc_big(const ZArgs &a, uint32_t *sm, DocRun &
             } else {
                 const int64_t col = static_cast<int64_t>((static_cast<u64>(t0.y & 0xFFFFu) << 32) | t0.x);
                 load_ahead(tt + 1);
-                knew = column_draw(a, t, col, n_w, m, lane, c_cnt, pos);
+                knew = column_draw<4>(a, t, col, n_w, m, lane, c_cnt, pos);
             }
             __syncwarp();
-#pragma unroll
-            for (int c = 0; c < kEarly; ++c)
-                if (c < C) c_int += static_cast<uint32_t>(__popc(early[c] & mb[32 * c]));
-            for (int c = kEarly; c < C; ++c) c_int += static_cast<uint32_t>(__popc(wb[c] & mb[32 * c]));
+            if (4 * lane < 16 * C) c_int += common(early, *reinterpret_cast<const uint4 *>(map + 4 * lane));
+            for (int w = 128 + 4 * lane; w < 16 * C; w += 128)
+                c_int += common(*reinterpret_cast<const uint4 *>(wb + w), *reinterpret_cast<const uint4 *>(map + w));
             {
                 const int p = knew;
                 bool born = false;
@@ -676,9 +722,11 @@ __device__ __forceinline__ void z_doc_big(const ZArgs &a, uint32_t *sm, DocRun &
                     m.set(p, c);
                     lv = count_level(c);
                     born = c == 1;
-                    if (born) mb[(p >> 9) << 5] |= static_cast<uint16_t>(1u << (p & 15));
                 }
-                kd += __any_sync(0xFFFFFFFFu, born) ? 1 : 0;
+                if (__any_sync(0xFFFFFFFFu, born)) {
+                    ++kd;
+                    flip(p);
+                }
                 if (__any_sync(0xFFFFFFFFu, lv > m.lvl)) ++m.lvl;
             }
             if (lane == tt) znew = knew;

@@ -107,7 +107,7 @@ __device__ __forceinline__ void z_pair(const ZArgs &a, uint32_t *sm, const DocRu
     for (int o = 8; o; o >>= 1) kd += __shfl_xor_sync(0xFFFFFFFFu, kd, o);
     if (s == 0) rs = r;
     __syncwarp();
-    const int colmax = column_limit<NW>(a.path);
+    const int colmax = column_limit<NW>(a.path, K);
     const int fine = s & (G::TPL - 1);
     for (int i0 = 0; i0 < most; i0 += 16) {
         const int cnt = min(16, rs.len - i0);       // this document's tokens in the block (0 or less: none)

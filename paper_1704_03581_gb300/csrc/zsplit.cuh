@@ -99,17 +99,7 @@ __device__ __forceinline__ bool z_doc_split(const ZArgs &a, uint8_t *sm, DocRun 
     if (m.lvl > 0) atomicMax(&x.high, m.lvl);
     // the document's topics as bits, in topic order
     for (int w = threadIdx.x; w < kSplitMapWords; w += kSplitThreads) {
-        uint32_t bits = 0;
-        for (int h = 0; h < 2 && 32 * w + 16 * h < K; ++h) {        // sixteen topics' bytes lie together
-            const uint8_t *p = counts + pos(32 * w + 16 * h);
-            uint4 v = *reinterpret_cast<const uint4 *>(p);
-            for (int pl = 1; pl < planes; ++pl) {
-                const uint4 u = *reinterpret_cast<const uint4 *>(p + pl * PB);
-                v = make_uint4(v.x | u.x, v.y | u.y, v.z | u.z, v.w | u.w);
-            }
-            auto nonzero = [](uint32_t x) { return ((__vcmpne4(x, 0u) & 0x01010101u) * 0x01020408u) >> 24 & 15u; };
-            bits |= (nonzero(v.x) | nonzero(v.y) << 4 | nonzero(v.z) << 8 | nonzero(v.w) << 12) << (16 * h);
-        }
+        const uint32_t bits = w < 16 * C ? nonzero_topics(all, pos(32 * w), planes) | nonzero_topics(all, pos(32 * w + 16), planes) << 16 : 0u;
         map[w] = bits;
         if (bits) atomicAdd(&x.kd, __popc(bits));
     }
