@@ -639,11 +639,8 @@ pulda_status pulda_sync(pulda_handle *h) {
     CU(h, cudaStreamSynchronize(h->stream));
     unsigned long long e = 0;
     CU(h, cudaMemcpy(&e, h->stats + ST_ERROR, sizeof e, cudaMemcpyDeviceToHost));
-    if (e & ERR_DEGENERATE) return fail(h, PULDA_ERR_DEGENERATE, "a Phi row stayed all-zero after 2^20 redraws");
-    if (e & ERR_INTERNAL) return fail(h, PULDA_ERR_CUDA, "z-step invariant violated (draw beyond the total mass)");
-    if (e & ERR_GAMMA) return fail(h, PULDA_ERR_DEGENERATE, "a Gamma draw was rejected 2^16 times");
-    if (e & ERR_BOUNDS) return fail(h, PULDA_ERR_CUDA, "an index read from device data was out of range (checked build)");
-    if (e & ERR_BARRIER) return fail(h, PULDA_ERR_TIMEOUT, "a grid barrier of the one-launch batched sweep waited 2 s");
+    const DeviceError err = device_error(e);
+    if (err.status != PULDA_OK) return fail(h, err.status, "%s", err.message);
     return PULDA_OK;
 }
 

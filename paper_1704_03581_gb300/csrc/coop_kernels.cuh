@@ -33,16 +33,11 @@ __device__ __forceinline__ int next_item(CtaCtl &ctl, int *work) {
     return ctl.item;
 }
 
-// One document, by the CTA, its counts in PL planes; false where its copies
-// failed, and the CTA stops.
+// One document, by the CTA, its counts in PL planes.
 template <int NW, int PL>
-__device__ __forceinline__ bool z_doc_cta(const ZArgs &a, uint8_t *sm, DocRun &r, uint32_t &phases) {
-    if constexpr (NW < 0) {
-        return z_doc_split(a, sm, r, phases);
-    } else {
-        z_doc_chain<NW, PL>(a, sm, r, phases);
-        return true;
-    }
+__device__ __forceinline__ void z_doc_cta(const ZArgs &a, uint8_t *sm, DocRun &r, uint32_t &phases) {
+    if constexpr (NW < 0) z_doc_split(a, sm, r, phases);
+    else z_doc_chain<NW, PL>(a, sm, r, phases);
 }
 
 // The longest documents of a pass (dynamically scheduled, longest first):
@@ -61,7 +56,8 @@ __global__ void __launch_bounds__(NW < 0 ? kSplitThreads : kChainThreads, NW < 0
         const int64_t s = a.doc_off[d];
         const int len = static_cast<int>(a.doc_off[d + 1] - s);
         DocRun r{a.w + s, a.z + s, len, a.seed, a.index_base + s, sweep, 0, len, 1};
-        if (!z_doc_cta<NW, PL>(a, csm, r, phases)) break;
+        z_doc_cta<NW, PL>(a, csm, r, phases);
+        if (ctl.failed) break;
     }
     if (threadIdx.x < 32) flush_warp_counters(a.stats, ctl.cnt);
 }
@@ -83,7 +79,8 @@ __global__ void __launch_bounds__(NW < 0 ? kSplitThreads : kChainThreads, NW < 0
         const int64_t s = a.doc_off[it.y];
         const int len = static_cast<int>(a.doc_off[it.y + 1] - s);
         DocRun r{a.w + s, a.z + s, len, a.seed, a.index_base + s, sweep_of(a), 0, len, 1};
-        if (!z_doc_cta<NW, PL>(a, csm, r, phases)) break;
+        z_doc_cta<NW, PL>(a, csm, r, phases);
+        if (ctl.failed) break;
         if (threadIdx.x < 32) flush_warp_counters(a.stats, ctl.cnt);
     }
 }
@@ -120,12 +117,12 @@ __global__ void __launch_bounds__(NW < 0 ? kSplitThreads : kChainThreads, NW < 0
         }
         DocRun r{arena_w + sl.off, z, sl.len, sl.seed, 0, sweep, pos, slice,
                  static_cast<int>(sl.sweep_end - sweep), deadline};
-        const bool ok = z_doc_cta<NW, PL>(a, csm, r, phases);
+        z_doc_cta<NW, PL>(a, csm, r, phases);
         if (threadIdx.x == 0) {         // a request that failed is handed back, with the error
-            slots[idx].sweep = ok ? r.sweep : sl.sweep_end;
+            slots[idx].sweep = ctl.failed ? slots[idx].sweep_end : r.sweep;
             slots[idx].pos = r.pos;
         }
-        if (!ok) break;
+        if (ctl.failed) break;
     }
     if (threadIdx.x < 32) flush_warp_counters(a.stats, ctl.cnt);
 }

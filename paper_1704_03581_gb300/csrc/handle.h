@@ -100,6 +100,21 @@ struct DevTemp {
         return e;
     }
 };
+// What the error word of a chain's counters says: the status and its message
+// (PULDA_OK and "" where no bit is set).
+struct DeviceError {
+    pulda_status status;
+    const char *message;
+};
+inline DeviceError device_error(unsigned long long bits) {
+    if (bits & ERR_DEGENERATE) return {PULDA_ERR_DEGENERATE, "a Phi row stayed all-zero after 2^20 redraws"};
+    if (bits & ERR_COPY) return {PULDA_ERR_TIMEOUT, "a word's dense row did not arrive in a z-step CTA's shared memory"};
+    if (bits & ERR_INTERNAL) return {PULDA_ERR_CUDA, "z-step invariant violated (draw beyond the total mass)"};
+    if (bits & ERR_GAMMA) return {PULDA_ERR_DEGENERATE, "a Gamma draw was rejected 2^16 times"};
+    if (bits & ERR_BOUNDS) return {PULDA_ERR_CUDA, "an index read from device data was out of range (checked build)"};
+    if (bits & ERR_BARRIER) return {PULDA_ERR_TIMEOUT, "a grid barrier of the one-launch batched sweep waited 2 s"};
+    return {PULDA_OK, ""};
+}
 // Tokens from which a document of a pass over D documents and N tokens goes to
 // a CTA of its own (INT64_MAX: none do).
 int64_t long_document_tokens(const pulda_handle *h, int64_t D, int64_t N);

@@ -189,6 +189,7 @@ extern "C" pulda_status pulda_infer_noalloc(pulda_handle *h, const int32_t *word
     if (e == cudaSuccess) e = cudaMemcpyAsync(&err, stats + ST_ERROR, sizeof err, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return static_cast<pulda_status>(handle_fail(h, PULDA_ERR_CUDA, cudaGetErrorString(e)));
-    if (err) return static_cast<pulda_status>(handle_fail(h, PULDA_ERR_CUDA, "z-step invariant violated"));
+    const DeviceError de = device_error(err);
+    if (de.status != PULDA_OK) return static_cast<pulda_status>(handle_fail(h, de.status, de.message));
     return PULDA_OK;
 }

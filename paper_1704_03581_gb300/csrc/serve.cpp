@@ -264,7 +264,7 @@ void worker_loop(pulda_server *s) {
             Request &r = s->slot_req[slot];
             pulda_result res{};
             res.req_id = r.id;
-            res.status = err ? PULDA_ERR_CUDA : PULDA_OK;
+            res.status = device_error(err).status;
             res.len = static_cast<int32_t>(r.words.size());
             res.submit_ns = r.submit_ns;
             res.done_ns = t;

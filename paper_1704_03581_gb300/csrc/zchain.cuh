@@ -61,6 +61,7 @@ struct CtaCtl {                 // what every kernel with a CTA per document has
     u64 cnt[6];                 // the counters
     u64 deadline;
     int item, stop;
+    int failed;                 // 1 + the barrier of a copy that did not arrive: the CTA takes no more documents
 };
 struct ChainCtl : CtaCtl {
     int after[2];               // after an even / odd group (a fast warp may already set the next one):
@@ -539,6 +540,14 @@ __device__ __forceinline__ void counts_from(const uint32_t *hist, int K, DocCoun
     __syncwarp();
 }
 
+// A copy did not arrive in time (one warp): the error, and the CTA gives up, but
+// not before the copy, if it comes.
+__device__ __forceinline__ void cta_failed(const ZArgs &a, CtaCtl &ctl, uint32_t phases) {
+    if ((threadIdx.x & 31) == 0) atomicOr(&a.stats[ST_ERROR], ERR_COPY);
+    const int s = ctl.failed - 1;
+    bar_wait(&ctl.full[s], (phases >> s) & 1u);
+}
+
 // All threads of the CTA; sm: chain_smem_bytes(K) bytes.  phases: the parities
 // of the groups' barriers, kept from one document to the next.  PL planes of
 // counts: two for documents of at most kNarrowMaxLen tokens, three for any.
@@ -619,8 +628,8 @@ __device__ __forceinline__ void z_doc_chain(const ZArgs &a, uint8_t *sm, DocRun 
         auto landed = [&](int g) {
             const int s = g % 3;
             const bool ok = bar_wait(&ctl.full[s], (phases >> s) & 1u);
-            phases ^= 1u << s;
-            if (!ok && lane == 0) atomicOr(&a.stats[ST_ERROR], ERR_BARRIER);
+            if (ok) phases ^= 1u << s;
+            else if (lane == 0) ctl.failed = 1 + s;
             // the weights of the tokens' own and previous topics, now that their rows are here
             const int t = g * G + lane;
             if (ok && lane < G && t < n) {
@@ -764,6 +773,7 @@ __device__ __forceinline__ void z_doc_chain(const ZArgs &a, uint8_t *sm, DocRun 
         if (r.pos == r.len) { r.pos = 0; r.sweep += 1; }
     }
     __syncthreads();
+    if (role == 1 && ctl.failed) cta_failed(a, ctl, phases);
 }
 
 // Before the first document: the groups' barriers and the counters.
@@ -772,7 +782,7 @@ __device__ __forceinline__ void cta_begin(uint8_t *sm) {
     if (threadIdx.x == 0) {
         for (int s = 0; s < 3; ++s) bar_init(&ctl.full[s]);
         for (int s = 0; s < 6; ++s) ctl.cnt[s] = 0;
-        ctl.stop = 0;
+        ctl.stop = ctl.failed = 0;
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     __syncthreads();

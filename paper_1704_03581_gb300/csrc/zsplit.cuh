@@ -63,11 +63,11 @@ __host__ __device__ __forceinline__ int split_smem_bytes(int K) { return kSplitC
 
 __device__ __forceinline__ void split_barrier() { asm volatile("bar.sync 1, 128;" ::: "memory"); }     // the four warps
 
-__device__ __forceinline__ bool z_doc_split(const ZArgs &a, uint8_t *sm, DocRun &r, uint32_t &phases) {
+__device__ __forceinline__ void z_doc_split(const ZArgs &a, uint8_t *sm, DocRun &r, uint32_t &phases) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool service = warp >= kSplitWarps;
     const int K = a.K;
-    if (r.len == 0 || r.budget <= 0) return true;
+    if (r.len == 0 || r.budget <= 0) return;
     SplitCtl &x = *reinterpret_cast<SplitCtl *>(sm);
     uint32_t *map = reinterpret_cast<uint32_t *>(sm + kSplitMapOff);
     const ChainForm<0> form(K);
@@ -142,8 +142,8 @@ __device__ __forceinline__ bool z_doc_split(const ZArgs &a, uint8_t *sm, DocRun 
             if (t >= n || *row_of(t) == 0xFFFFFFFFu) return true;
             const int s = t % 3;
             const bool here = bar_wait(&x.full[s], (phases >> s) & 1u);
-            if (!here) bar_wait(&x.full[s], (phases >> s) & 1u);        // the CTA gives up, but not before the copy
-            phases ^= 1u << s;
+            if (here) phases ^= 1u << s;
+            else if (lane == 0) x.failed = 1 + s;
             return here;
         };
         // the service warp's: the word's bits of token t, and the counters
@@ -440,15 +440,13 @@ __device__ __forceinline__ bool z_doc_split(const ZArgs &a, uint8_t *sm, DocRun 
         if (warp == kSplitWarps && done > 0 && ok) count(done - 1);
         // the copy in flight where the pass ended early
         if (warp == kSplitWarps && !landed(done + (ok ? 1 : 2))) ok = false;
-        if (!ok) {
-            if (warp == kSplitWarps && lane == 0) atomicOr(&a.stats[ST_ERROR], ERR_BARRIER);
-            stop = true;
-        }
+        if (!ok) stop = true;
         r.budget -= done;
         r.pos += done;
         if (r.pos == r.len) { r.pos = 0; r.sweep += 1; }
     }
-    return __syncthreads_and(ok) != 0;
+    __syncthreads();
+    if (warp == kSplitWarps && x.failed) cta_failed(a, x, phases);
 }
 
 }  // namespace pulda
