@@ -39,6 +39,13 @@ sys.path.insert(0, ROOT)
 METRIC = "z-step tokens/s/GPU at K=1000 (% HBM roofline); serving p50/p99 vs plain"
 K_TOPICS = 1000
 ALPHA, BETA = 0.1, 0.01
+
+
+def every_document_on_a_cta(layout: dict) -> bool:
+    """As pulda_z_layout reports it: no document left for the warps."""
+    return layout["docs_per_warp"] != 4 and layout["one_warp_docs"] == 0
+
+
 def kernels_per_sweep(w: np.ndarray, phi_mode: int, layout: dict | None = None, slice_docs: int = 0) -> int:
     """Library kernels one sweep launches: the frequent-word histogram (when a
     word has more than N / 1024 tokens, within 4,096 and 2^17), then Polya urn: counts+draws, dead-row
@@ -51,9 +58,8 @@ def kernels_per_sweep(w: np.ndarray, phi_mode: int, layout: dict | None = None, 
     heavy = 1 if np.bincount(w).max(initial=0) > min(max(len(w) // 1024, 4096), 1 << 17) else 0
     extra = 1 if slice_docs > 0 else 0
     if layout is not None:
-        if layout["docs_per_warp"] != 4 and layout["one_warp_docs"] == 0 and layout["coop_docs"] > 0:
-            extra -= 1
-        extra += (1 if layout["coop_docs"] > 0 else 0)
+        if not every_document_on_a_cta(layout):
+            extra += 1 if layout["coop_docs"] > 0 else 0
         if layout["docs_per_warp"] == 4:
             extra += 1 if layout["one_warp_docs"] > 0 else 0
     return heavy + (4 if phi_mode == 0 else 7) + 1 + extra
@@ -523,7 +529,8 @@ def run_pulda(args, corpus, rank: int, world: int):
         "roofline_issue": issue_roofline(K * corpus.N / (z_ms / 1000.0), (clk or {}).get("sm_mhz")),
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic,
-                     "kernel": {1: "k_z_step", 2: "k_z_step_pairs", 4: "k_z_step_grouped"}[layout["docs_per_warp"]],
+                     "kernel": ("k_z_step_coop" if every_document_on_a_cta(layout) else
+                                {1: "k_z_step", 2: "k_z_step_pairs", 4: "k_z_step_grouped"}[layout["docs_per_warp"]]),
                      "peak_kind": f"{peak_kind} HBM copy bandwidth",
                      "algorithmic_bytes_per_launch": zbytes / K,
                      "bytes_model": "12 B per token + 6 B per min(K_d, K_v) element + 8 B per alias draw + "
@@ -533,7 +540,7 @@ def run_pulda(args, corpus, rank: int, world: int):
                                                    "min(K_d, K_v) element + 6 B per alias draw + 8 B per document"},
         "gpu_launches": kernels_per_sweep(corpus.w, args.phi_mode, layout,
                                           int(args.slice_len > 0 and np.diff(corpus.doc_off).max() > args.slice_len)) * K,
-        "z_kernel": (f"{ {1: 'one document', 2: 'two documents', 4: 'four documents'}[layout['docs_per_warp']] } per warp; "
+        "z_kernel": ("every document on a CTA" if every_document_on_a_cta(layout) else f"{ {1: 'one document', 2: 'two documents', 4: 'four documents'}[layout['docs_per_warp']] } per warp; "
                      f"{layout['coop_docs']} longest documents on one CTA each"),
         "clocks": clk,
         "cpu_baseline": cpu,

@@ -403,9 +403,10 @@ pulda_status pulda_serve_close(pulda_server *s);
 
 /* pulda_z_layout -- how the handle's corpus z-step is laid out (launch shape
  * only: results never depend on it): documents per warp of the main z-step
- * kernel (1, 2 or 4), the number of (longest) documents that coop_min_len
- * puts on CTAs of their own, and, beside four per warp, the documents too long
- * for it that run one per warp (otherwise every document not on a CTA).  Any
+ * kernel (1, 2 or 4), the number of (longest) documents that are long enough
+ * for CTAs of their own by coop_min_len, and, beside four per warp, the
+ * documents too long for it that run one per warp, otherwise every document not
+ * on a CTA: 0 where a corpus has so few documents that all go to CTAs.  Any
  * pointer may be NULL.
  * Errors: PULDA_ERR_INVALID (NULL handle). */
 pulda_status pulda_z_layout(pulda_handle *h, int32_t *docs_per_warp, int64_t *coop_docs, int64_t *one_warp_docs);

@@ -225,18 +225,22 @@ int64_t long_document_tokens(const pulda_handle *h, int64_t D, int64_t N) {
     return std::max<int64_t>(kCoopAutoMin, N / div + 1);
 }
 
+// Few documents all go to CTAs: at most two for every CTA the GPU holds.  Each is
+// a chain of its own, and there a token takes a third of the time (1,000
+// documents of 100 tokens at K = 20: 85 us against 136).
+bool few_documents(const pulda_handle *h, int64_t D) {
+    return h->opt.coop_min_len == 0 && h->opt.slice_len == 0 && !h->z_groups && D <= 2 * static_cast<int64_t>(h->coop_grid);
+}
+
 // The first n_coop documents on a CTA each, on the handle's stream; beside
 // them, on a second stream joined back before the next step, the rest four per
 // warp (grouped), two or one; those of 2^16 tokens or more among the rest one
 // per warp, where the others go several, in a launch of their own.
-// Few documents (at most two for every CTA the GPU holds) all go to CTAs: each
-// is a chain of its own, and there a token takes a third of the time (1,000
-// documents of 100 tokens at K = 20: 85 us against 136).
 cudaError_t run_z(pulda_handle *h, ZArgs a, int64_t n_wide, int64_t n_coop, int *work) {
     cudaError_t e = cudaMemsetAsync(work, 0, 5 * sizeof(int), h->stream);
     if (e != cudaSuccess) return e;
     const int64_t D = a.D;
-    if (h->opt.coop_min_len == 0 && h->opt.slice_len == 0 && !h->z_groups && D <= 2 * static_cast<int64_t>(h->coop_grid)) n_coop = D;
+    if (few_documents(h, D)) n_coop = D;
     const int32_t *order = a.doc_order;
     const bool pairs = pairs_of_documents(h, D);
     // documents [n_coop, n_apart) one per warp beside the CTAs
@@ -804,7 +808,8 @@ pulda_status pulda_z_layout(pulda_handle *h, int32_t *docs_per_warp, int64_t *co
     if (!h) return PULDA_ERR_INVALID;
     if (docs_per_warp) *docs_per_warp = h->z_groups ? 4 : pairs_of_documents(h, h->D) ? 2 : 1;
     if (coop_docs) *coop_docs = h->n_coop;
-    if (one_warp_docs) *one_warp_docs = h->z_groups ? std::max<int64_t>(0, h->n_wide - h->n_coop) : h->D - h->n_coop;
+    if (one_warp_docs)
+        *one_warp_docs = few_documents(h, h->D) ? 0 : h->z_groups ? std::max<int64_t>(0, h->n_wide - h->n_coop) : h->D - h->n_coop;
     return PULDA_OK;
 }
 

@@ -500,7 +500,7 @@ pulda_status pulda_batch_tuning(pulda_batch *b, int32_t *z_warps, int32_t *coop_
     if (!b) return PULDA_ERR_INVALID;
     if (one_launch) *one_launch = b->one_launch ? 1 : 0;
     if (alias_layout) *alias_layout = b->packed ? 2 : 1;
-    if (z_warps) *z_warps = b->one_launch ? kMultiWarps : b->bl.z_warps;
+    if (z_warps) *z_warps = b->bl.z_warps;
     if (coop_min_len) *coop_min_len = static_cast<int32_t>(b->coop_len > 0 ? b->coop_len : -1);
     if (tuned) *tuned = b->tuned ? 1 : 0;
     return PULDA_OK;

@@ -120,6 +120,8 @@ inline DeviceError device_error(unsigned long long bits) {
 int64_t long_document_tokens(const pulda_handle *h, int64_t D, int64_t N);
 // Whether a pass over D documents takes them two per warp.
 bool pairs_of_documents(const pulda_handle *h, int64_t D);
+// Whether a pass over D documents takes them all on CTAs.
+bool few_documents(const pulda_handle *h, int64_t D);
 // One z-step over a's documents doc_order[0 .. D) on the handle's streams: the
 // first n_wide have 2^16 tokens or more, the first n_coop go to a CTA each, and
 // so do the others when they are few.  work: five counters.
