@@ -94,7 +94,7 @@ def parse():
     ap.add_argument("--serve-high-seconds", type=float, default=2.0, help="serving keys: its arrival window")
     ap.add_argument("--batch-steps", type=int, default=10, help="batched keys: timed sweeps of each arm")
     ap.add_argument("--batch-form", type=int, default=0, choices=[0, 1, 2],
-                    help="batched launch form: 0 tuned, 1 six launches per sweep, 2 one persistent launch")
+                    help="batched launch form: 0 tuned, 1 a launch or a few per phase, 2 the Phi-step as one persistent launch")
     ap.add_argument("--alias-layout", type=int, default=0, choices=[0, 1, 2],
                     help="alias tables: 1 threshold and topic arrays, 2 packed slots, 0 = arrays for the sweep "
                          "form and tuned for the batched one")
@@ -740,7 +740,7 @@ def batched_probe(scale: float, steps: int, warmup: int, coop_min_len: int, cloc
             "sequential_ms_per_sweep": ms_s / K, "speedup_vs_sequential": ms_s / ms_b,
             "identical_topics": same, "z_warps_tuned": warps, "coop_min_len_tuned": coop_len,
             "alias_layout": "packed 8-byte slots" if layout == 2 else "threshold and topic arrays",
-            "launch_form": "one persistent launch per sweep" if one_launch else "six launches per sweep (a graph)",
+            "launch_form": "the Phi-step as one persistent launch" if one_launch else "a launch or a few per phase (a graph)",
             "gpu_launches": (1 if one_launch else 6 + (1 if coop_len > 0 else 0)) * K, "generation_s": t_gen,
             "clocks": clk}
 

@@ -92,8 +92,8 @@ typedef struct {
                                of every token's key w K + z and its runs (needs V K < 2^32; the
                                batched form takes 0); the counts are identical */
     int32_t batch_form;     /* batched form only: how a sweep is launched -- 0 = tuned (timed on
-                               the first sweeps with the CTA sizes), 1 = six launches (a CUDA
-                               graph), 2 = the Phi-step as one persistent cooperative launch
+                               the first sweeps with the CTA sizes), 1 = a launch or a few per phase
+                               (a CUDA graph), 2 = the Phi-step as one persistent cooperative launch
                                whose phases are separated by grid barriers (every document
                                one per warp; not with coop_min_len > 0); the chains' results
                                are identical */
@@ -277,8 +277,8 @@ pulda_status pulda_infer_noalloc(pulda_handle *h, const int32_t *word_ids_dev, c
  * Many independent chains advanced together (the batched form of Algorithm
  * 2): each chain is exactly the chain a handle with the same arguments would
  * run -- bit for bit -- but every kernel of a sweep runs once over all chains'
- * words and documents (longest first across chains), and the six launches of
- * a sweep are captured into one CUDA graph that is replayed every sweep.  The
+ * words and documents (longest first across chains), and the launches of a
+ * sweep (one or a few per phase) are captured into one CUDA graph that is replayed every sweep.  The
  * z-step CTA size is chosen by timing the candidates on the first sweeps
  * (launch shapes never change results).  Chains may differ in D, N, K, V,
  * alpha, beta and seed; all share the batch's stream. */
@@ -321,7 +321,8 @@ pulda_status pulda_batch_get_z(pulda_batch *b, int32_t chain, int16_t *z_host);
 pulda_status pulda_batch_stats(pulda_batch *b, int32_t chain, pulda_sweep_stats *out);
 /* pulda_batch_tuning -- the z-step warps per CTA and the cooperative
  * threshold in use (-1 = none), whether tuning is over, whether a sweep is
- * one persistent launch (1) or six launches (0), and the alias layout in use
+ * one persistent launch for the Phi-step and the z-step's own (1) or a launch or a
+ * few per phase (0), and the alias layout in use
  * (1 = threshold and topic arrays, 2 = packed slots; see pulda_options); any
  * pointer may be NULL. */
 pulda_status pulda_batch_tuning(pulda_batch *b, int32_t *z_warps, int32_t *coop_min_len, int32_t *tuned,

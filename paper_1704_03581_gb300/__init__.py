@@ -514,7 +514,7 @@ class Batch:
 
     def __init__(self, chains: list[dict], stream=None, warps_per_block: int = 0, coop_min_len: int = 0,
                  allocator=None, batch_form: int = 0, alias_layout: int = 0):
-        """batch_form 0: the launch form is tuned; 1: six launches per sweep; 2: one persistent launch.
+        """batch_form 0: the launch form is tuned; 1: a launch or a few per phase; 2: the Phi-step as one persistent launch.
         alias_layout 0: tuned; 1: threshold and topic arrays; 2: packed slots."""
         self.sizes = [int(np.asarray(c["doc_off"])[-1]) for c in chains]
         self.b = None

@@ -194,7 +194,7 @@ pulda_status pulda_batch_init(pulda_batch **out, const pulda_chain_desc *chains,
         return bail(PULDA_ERR_INVALID);
     }
     if (o.batch_form < 0 || o.batch_form > 2 || (o.batch_form == 2 && o.coop_min_len > 0)) {
-        b->err = "batch_form must be 0 (tuned), 1 (six launches) or 2 (one launch, without coop_min_len > 0)";
+        b->err = "batch_form must be 0 (tuned), 1 (a launch or a few per phase) or 2 (one launch, without coop_min_len > 0)";
         return bail(PULDA_ERR_INVALID);
     }
     if (o.alias_layout < 0 || o.alias_layout > 2) {
@@ -260,7 +260,7 @@ pulda_status pulda_batch_init(pulda_batch **out, const pulda_chain_desc *chains,
     std::vector<HeavyChunk> heavy;
     std::vector<std::pair<int64_t, int2>> wi, di;    // (weight, (chain, item))
     int kmax = 1;
-    bool narrow = true;     // every document of every chain fits 16-bit counts
+    bool narrow = true;     // every document of every chain has fewer than 2^16 tokens
     for (int32_t c = 0; c < n_chains; ++c) {
         pulda_handle *h = b->ch[c];
         hp[c] = phi_args(h);
@@ -324,7 +324,6 @@ pulda_status pulda_batch_init(pulda_batch **out, const pulda_chain_desc *chains,
     }
     cudaStream_t st = b->stream;
     const uint32_t zero = 0;
-    for (ZArgs &z : hz) z.narrow = narrow ? 1 : 0;      // one width of the counts for the whole launch
     if (cudaMemcpyAsync(d_phi, hp.data(), sizeof(PhiArgs) * n_chains, cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaMemcpyAsync(d_z, hz.data(), sizeof(ZArgs) * n_chains, cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaMemcpyAsync(d_wl, wlist.data(), sizeof(int2) * wlist.size(), cudaMemcpyHostToDevice, st) != cudaSuccess ||
@@ -349,7 +348,6 @@ pulda_status pulda_batch_init(pulda_batch **out, const pulda_chain_desc *chains,
     bl.sweep = d_sweep;
     bl.work = d_work;
     bl.kmax = kmax;
-    bl.narrow = narrow ? 1 : 0;
     bl.phi_grid = b->sms * batch_phi_blocks_per_sm(kmax);
     const auto rare = std::partition_point(wi.begin(), wi.end(), [](const std::pair<int64_t, int2> &x) { return x.first > phi_warp_word_tokens(); });
     bl.n_big = phi_big_words(kmax, static_cast<int64_t>(wi.size()), rare - wi.begin(), bl.phi_grid);

@@ -567,10 +567,9 @@ __device__ void heavy_chunk(const PhiArgs *chains, const HeavyChunk &c, uint32_t
     __syncthreads();
 }
 
-__global__ void __launch_bounds__(kPhiBlock) k_heavy_hist(const PhiArgs *chains, const HeavyChunk *chunks, int kmax) {
+__global__ void __launch_bounds__(kPhiBlock) k_heavy_hist(const PhiArgs *chains, const HeavyChunk *chunks) {
     extern __shared__ uint32_t hs[];
     heavy_chunk(chains, chunks[blockIdx.x], hs);
-    (void)kmax;
 }
 
 // n_{k,v} from the compacted n column of word v (binary search), 0 if absent.
@@ -1357,7 +1356,7 @@ void launch_heavy_hist(const PhiArgs *chains, const HeavyChunk *chunks, int n_ch
     if (n_chunks <= 0) return;
     static bool opted_in = false;
     if (!opted_in) { allow_dynamic_smem(k_heavy_hist); opted_in = true; }
-    k_heavy_hist<<<n_chunks, kPhiBlock, sizeof(uint32_t) * static_cast<size_t>(kmax), st>>>(chains, chunks, kmax);
+    k_heavy_hist<<<n_chunks, kPhiBlock, sizeof(uint32_t) * static_cast<size_t>(kmax), st>>>(chains, chunks);
 }
 
 size_t z_step_smem(int K, int warps_per_block, bool narrow) {
@@ -1621,8 +1620,9 @@ static size_t batch_persistent_smem(int kmax, int stage) {
     return std::max(phi_counts_smem(kmax), static_cast<size_t>(kPersistWarps) * (stage + kTabScratch));
 }
 
-// 0 where the form is not offered: no room for a CTA, or K so large that the
-// counts of seven documents do not fit a CTA.
+// 0 where the form is not offered: no room for a CTA, or K above a limit kept
+// from when this launch ran the z-step too (seven documents' counts in a CTA), so
+// that what was refused stays refused.
 int batch_persistent_blocks_per_sm(int kmax, bool narrow, int *table_stage) {
     allow_dynamic_smem(k_batch_sweep_persistent);
     if (z_step_smem(kmax, kPersistWarps - 1, narrow) > static_cast<size_t>(smem_optin())) return 0;

@@ -219,7 +219,7 @@ struct ZArgs {
     uint32_t sweep;
     const uint32_t *sweep_ptr;  // if set, the sweep counter is read here (graph replay)
     int64_t index_base;         // RNG index of token 0
-    int path;                   // 0 auto, 1 column, 2 document topics
+    int path;                   // zstep_path: 0 auto, 1 a higher column limit, 2 the row wherever there is one
     int narrow;                 // 1: every document of the launch has fewer than 2^16 tokens (two count planes, else three)
     int *work;
     unsigned long long *stats;
@@ -280,8 +280,8 @@ int z_step_blocks_per_sm(int K, int warps_per_block, bool narrow = false);
 // kMaxKGrouped, documents of at most kMaxGroupDocLen tokens, every word with a
 // dense q row; the warps of a CTA are z_groups_warps().
 constexpr int kMaxGroupDocLen = 65535;
-// A one-warp z-step launch whose documents have at most this many tokens each
-// keeps m_d's counts in 16 bits (ZArgs::narrow).
+// A launch whose documents have at most this many tokens each keeps their counts
+// in two planes (ZArgs::narrow; the CTA kernels: !wide).
 constexpr int64_t kNarrowMaxLen = 65535;
 // Length classes of documents (fold-in without allocation), eight to an octave
 // and the longest first: those of 2^16 tokens or more, then those of at least
@@ -364,7 +364,6 @@ struct BatchLaunch {
     uint32_t *sweep;             // shared sweep counter, advanced by the first launch
     int *work;                   // [kBatchCounters] dynamic work queues
     int kmax;                    // largest K of the chains
-    int narrow;                  // 1: every document of every chain has fewer than 2^16 tokens
     int phi_grid, z_warps;
     // streams beside the batch's for the z-step's launches, forked and joined
     // with the events

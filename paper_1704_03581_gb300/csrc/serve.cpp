@@ -197,7 +197,7 @@ void worker_loop(pulda_server *s) {
                 wide = wide || s->h_slots_len[slot] > kNarrowMaxLen;
             }
         int j = nc;
-        bool narrow = true;     // every request on the one-warp kernel fits 16-bit counts
+        bool narrow = true;     // every request on the one-warp kernel has fewer than 2^16 tokens
         for (int32_t slot : s->active)
             if (!on_cta(slot)) {
                 s->h_active[j++] = slot;

@@ -452,10 +452,6 @@ __device__ __forceinline__ void z_doc_regs(const ZArgs &a, uint32_t *sm, DocRun 
     if (r.len == 0 || r.budget <= 0) return;
     DocCounts m{reinterpret_cast<uint8_t *>(sm), G::PB, 0};
     build_counts(a, m, r, m0, z_count_planes(a.narrow != 0), [](int k) { return G::pos(k); });
-    // counts of a document of at most 255 tokens fit one plane for good, and
-    // its sums 32 bits (q <= 2^24 - 1 in a dense row); slices start from the
-    // whole document's counts
-    const bool brief = r.len <= 255 && !m0;
     uint32_t mbits = 0;         // this lane's topics with m > 0
 #pragma unroll 1
     for (int b = 0; b < G::TPL; ++b)

@@ -17,12 +17,12 @@
 // updates need no warp barrier), the matching WPL words of the document's
 // nonzero-topic bitmap (registers) and of the token's word's bitmap row (one
 // aligned load, fetched a token ahead).  Per token each lane sums q_{k,v} m_k
-// over its part of the intersection, reading q from the word's dense row; an
+// over its part of the intersection, reading q by topic; an
 // 8-lane scan gives the prefix in ascending topic order, the draw
 // r = floor(u (A + 2^16 B)) takes the alias table when r < A, else the lane
 // whose prefix passes (r - A) / 2^16 walks its bits to the topic.
 //
-// Requires K <= kMaxKGrouped, a dense q row for every word, and documents of at
+// Requires K <= kMaxKGrouped, q by topic for every word (ZArgs::qdense), and documents of at
 // most kMaxGroupDocLen tokens (uint16 counts); the host routes anything else to
 // the one-warp kernels and those with a CTA per document.
 #include <algorithm>
@@ -93,7 +93,7 @@ __device__ __forceinline__ void load_bits(const uint32_t *p, uint32_t (&b)[WPL])
 
 // Stages token i (global index gi) of a document:
 //   rec[0] = {Philox x0, x1, sigma_a lo, hi}
-//   rec[1] = {offset of its word's dense q row, offset of its word's bitmap row, K_v | old topic << 16,
+//   rec[1] = {offset of its word's q by topic, offset of its word's bitmap row, K_v | old topic << 16,
 //             alias-table outcome}
 // and returns its current topic.
 __device__ __forceinline__ int zg_stage(const ZArgs &a, uint32_t sweep, int64_t gi, uint4 *rec) {
