@@ -208,7 +208,7 @@ pulda_status pulda_get_counts(pulda_handle *h, int32_t *n_kv_host, int32_t *m_dk
  *   out_host double[3] = {total, document sum, topic sum}
  * beta is the handle's float beta widened to double.  The counts are rebuilt
  * from the current z on the GPU and every sum runs in a fixed order, so equal
- * topics give equal bits.  Synchronous; uses 8 (D + V + 257 K + 4099) bytes
+ * topics give equal bits.  Synchronous; uses 8 (D + V + 258 K + 4142) bytes
  * of temporary device memory.  Errors: PULDA_ERR_INVALID (NULL out),
  * PULDA_ERR_CUDA. */
 pulda_status pulda_log_posterior(pulda_handle *h, double *out_host);

@@ -1401,6 +1401,7 @@ int z_step_blocks_per_sm(int K, int warps_per_block, bool narrow) {
     const size_t smem = z_step_smem(K, warps_per_block, narrow);
     ZStepKernel kern = z_step_kernel(K);
     allow_dynamic_smem(kern);
+    if (z_nw(K) == 0) allow_dynamic_smem(k_z_step<-1>);      // for launch_z_step, which loads no kernel
     int b = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kern, 32 * warps_per_block, smem);
     return b > 0 ? b : 1;
@@ -1421,7 +1422,6 @@ void launch_z_step(const ZArgs &a, int warps_per_block, int grid, cudaStream_t s
     // worse: K = 3,000 0.64 -> 0.80, K = 8,000 1.07 -> 0.86)
     const bool few = (a.K > 4096 || a.narrow == 0) && a.n_slices == 0 && a.D <= 4 * static_cast<int64_t>(sm_count()) && z_nw(a.K) == 0;
     const ZStepKernel kern = few ? k_z_step<-1> : z_step_kernel(a.K);
-    if (few) allow_dynamic_smem(kern);
     kern<<<grid, 32 * warps_per_block, z_step_smem(a.K, warps_per_block, a.narrow != 0), st>>>(a);
 }
 
