@@ -19,8 +19,8 @@
 // Warp 0 finds the topic within the found lane by masked dp4a, every lane
 // summing the lane's topics up to its own, without a scan.  Warps 0 and 3 meet
 // once per token, all four once per group of tokens.
-// About 640 cycles per token (K = 1000: 0.95 us with four warps sharing one
-// token's sparse walk, 0.33 so), which warps 0 and 3 both fill: work moved from
+// About 600 cycles per token (K = 1000, a document of 3,000 tokens: 1.10 us with
+// four warps sharing one token's sparse walk, 0.29 so), which warps 0 and 3 both fill: work moved from
 // either to the other made a token longer (the draw's product prepared by
 // warp 3 +10%, two of its scan steps left to warp 0 +5%).
 // Up to kChainMaxK topics; zsplit.cuh above.

@@ -126,3 +126,25 @@ def test_batch(coop):
         one.close()
         two.close()
     b.close()
+
+
+def test_batch_across_the_kernels_ranges():
+    """Chains on both sides of the line at which documents of 2^16 tokens or more
+    take the kernel with four warps on each token: in a batch they share one."""
+    import paper_1704_03581_gb300 as P
+    rng = np.random.default_rng(6)
+    for Ks in ([1100, 1500, 7000], [1100, 6000]):
+        chains = []
+        for i, K in enumerate(Ks):
+            w, off = corpus(rng, np.append(rng.integers(20, 400, size=40), [70000, 3000]), 30)
+            chains.append(dict(w=w, doc_off=off, K=K, V=30, alpha=few_topics(K), beta=0.01, seed=40 + i))
+        b = P.Batch(chains, coop_min_len=100)
+        b.sweep(2)
+        for i, c in enumerate(chains):
+            one = P.Sampler(c["w"], c["doc_off"], c["K"], c["V"], c["alpha"], 0.01, c["seed"], coop_min_len=-1).sweep(2)
+            assert np.array_equal(b.z(i), one.z()), (Ks, c["K"])
+            sb, ss = b.stats(i), one.stats()
+            for k in ("tokens", "a_branch", "sum_min", "zero_mass", "sum_inter", "docside"):
+                assert sb[k] == ss[k], (Ks, c["K"], k)
+            one.close()
+        b.close()
